@@ -36,6 +36,10 @@ struct de_handle {
   RunDesc* d_run = nullptr;
   int4* d_items = nullptr;  // FP64 generation kernel work list: (run, tile, first row, rows)
   int nitems = 0;
+  SlicePlan slices;           // FP64 rotations on the tensor cores (de_slice.cuh)
+  int2* d_shares = nullptr;   // sliced generation kernel: the items of each CTA
+  int nshares = 0;
+  int nsm = 1;
   int rows = 8;             // rows per tile of the FP64 generation kernel
   int threads = 256;
   size_t smem_gen = 0;
@@ -241,6 +245,8 @@ static size_t gen_smem(int rows, int dp, int ncomp = 1) {
   return (size_t)std::max(4, 1 + 2 * ncomp) * rows * dp * sizeof(double);
 }
 
+constexpr size_t kTileSmemMax = 200 * 1024;
+
 // Split every run into tiles of at most h->rows targets, of near-equal size.
 static de_status build_items(de_handle* h) {
   std::vector<int4> items;
@@ -248,7 +254,7 @@ static de_status build_items(de_handle* h) {
   for (int r = 0; r < h->nruns; ++r) {
     RunDesc& R = h->run[r];
     int rows = std::max(1, std::min(h->rows, 8));
-    while (rows > 1 && gen_smem(rows, R.dp, suite_comps(R)) > 200 * 1024) --rows;
+    while (rows > 1 && gen_smem(rows, R.dp, suite_comps(R)) + h->slices.smem_op > kTileSmemMax) --rows;
     const int nt = (R.np + rows - 1) / rows;
     R.rows = (R.np + nt - 1) / nt;  // the largest tile after even splitting
     R.ntiles = nt;
@@ -260,6 +266,36 @@ static de_status build_items(de_handle* h) {
   }
   h->smem_gen = smem;
   h->nitems = (int)items.size();
+  if (h->slices.on) {
+    // contiguous shares of about equal work (a coordinate's FP64 terms, times
+    // the components of a composition function; a row's draws and selection)
+    const int nct = std::min(h->nitems, h->nsm * h->slices.per_sm());
+    std::vector<double> acc(items.size() + 1, 0.0);
+    size_t tiles_smem = smem;
+    for (size_t k = 0; k < items.size(); ++k) {
+      const RunDesc& R = h->run[items[k].x];
+      acc[k + 1] = acc[k] + items[k].w * (suite_comps(R) * (double)R.d + 16.0);
+      if (R.sl && R.obj >= DE_OBJ_COMPOSITION1) tiles_smem = std::max(tiles_smem, slice_group_smem(R.dp));
+    }
+    std::vector<int2> shares(nct);
+    int at = 0;
+    for (int b = 0; b < nct; ++b) {
+      // at least one item each; the share ends where its work does
+      const double want = acc.back() * (b + 1) / nct;
+      int e = at + 1;
+      while (e < h->nitems - (nct - 1 - b) && 0.5 * (acc[e] + acc[e + 1]) <= want) ++e;
+      if (b == nct - 1) e = h->nitems;
+      shares[b] = make_int2(at, e);
+      at = e;
+    }
+    h->nshares = nct;
+    h->slices.smem = h->slices.smem_op + tiles_smem;
+    if (h->d_shares) cudaFree(h->d_shares);
+    h->d_shares = nullptr;
+    DE_CUDA(h, cudaMalloc(&h->d_shares, shares.size() * sizeof(int2)));
+    DE_CUDA(h, cudaMemcpyAsync(h->d_shares, shares.data(), shares.size() * sizeof(int2), cudaMemcpyHostToDevice,
+                               h->stream));
+  }
   if (h->d_items) cudaFree(h->d_items);
   h->d_items = nullptr;
   DE_CUDA(h, cudaMalloc(&h->d_items, items.size() * sizeof(int4)));
@@ -296,7 +332,10 @@ static de_status islands_resync(de_handle* h) {
 // Enqueue one generation of every run (the kernels skip stopped runs).
 static de_status launch_generation(de_handle* h, cudaStream_t s) {
   if (h->prec == DE_PREC_FP64) {
-    k_gen_fp64_launch(h->d_run, h->d_items, h->nitems, h->threads, h->smem_gen, h->variants, h->suite, s);
+    if (h->slices.on)
+      k_gen_fp64_tc_launch(h->d_run, h->d_items, h->d_shares, h->nshares, h->slices, h->variants, h->suite, s);
+    else
+      k_gen_fp64_launch(h->d_run, h->d_items, h->nitems, h->threads, h->smem_gen, h->variants, h->suite, s);
     if (h->islands) k_island_launch(h->d_run, h->d_isl, h->stage, h->nruns, true, h->isl.async != 0, s);
   } else {
     tc_generation_launch(h->tc, h->d_run, s);
@@ -327,10 +366,11 @@ static de_status enqueue_generations(de_handle* h, int64_t n) {
       const long long g = std::min<int64_t>(left, (int64_t)1 << 20);
       if (h->fp64_cluster)
         DE_CUDA(h, k_gen_fp64_cluster_launch(h->d_run, h->d_items, h->nitems, h->threads, h->smem_gen, h->variants,
-                                             h->suite, h->d_ctl64, g, h->stream));
+                                             h->suite, h->d_ctl64, g, h->stream, h->slices));
       else
         DE_CUDA(h, k_gen_fp64_persist_launch(h->d_run, h->d_items, h->nitems, h->nruns, h->threads, h->smem_gen,
-                                             h->variants, h->suite, h->d_ctl64, g, h->stream, h->test_grid_skip,
+                                             h->variants, h->suite, h->d_ctl64, g, h->stream, h->slices,
+                                             h->test_grid_skip,
                                              h->islands ? h->d_isl : nullptr, h->islands ? &h->stage : nullptr));
     }
     return DE_OK;
@@ -470,7 +510,7 @@ static std::string tune_key(const de_handle* h) {
     sum_d += (long long)R.np * R.d;
   }
   char b[256];
-  snprintf(b, sizeof b, "gen_fp64v4 runs=%d np0=%d d0=%d obj0=%d rot0=%d sumnp=%lld sumnd=%lld", h->nruns, h->run[0].np,
+  snprintf(b, sizeof b, "gen_fp64v5 runs=%d np0=%d d0=%d obj0=%d rot0=%d sumnp=%lld sumnd=%lld", h->nruns, h->run[0].np,
            h->run[0].d, h->run[0].obj, h->run[0].rotate, sum_np, sum_d);
   return b;
 }
@@ -537,7 +577,20 @@ static int heuristic_rows(const de_handle* h, int nsm) {
   long long np_total = 0;
   for (auto& R : h->run) np_total += R.np;
   // about one CTA per SM, at most 8 rows (one warp per target)
-  return (int)std::max(1LL, std::min(8LL, (np_total + nsm - 1) / nsm));
+  int rows = (int)std::max(1LL, std::min(8LL, (np_total + nsm - 1) / nsm));
+  if (h->slices.on) {
+    // the sliced cooperative kernel runs one CTA per SM: the fewest rows
+    // whose tiles all fit, where there are such
+    auto tiles = [&](int r) {
+      long long n = 0;
+      for (auto& R : h->run) n += (R.np + r - 1) / r;
+      return n;
+    };
+    int r = rows;
+    while (r < 8 && tiles(r) > nsm) ++r;
+    if (tiles(r) <= nsm) rows = r;
+  }
+  return rows;
 }
 
 // The cooperative persistent FP64 kernel applies to runs without a surrogate
@@ -548,13 +601,14 @@ static bool fp64_persist_ok(const de_handle* h) {
   if (h->prec != DE_PREC_FP64 || h->surr || (h->islands && h->suite) || !h->d_ctl64 || h->nitems >= 4096) return false;
   if (const char* e = getenv("DE_GB300_FP64_PERSIST"))
     if (e[0] == '0') return false;
-  return h->nitems <= k_gen_fp64_persist_capacity(h->threads, h->smem_gen, h->variants, h->suite, h->islands);
+  return h->nitems <= k_gen_fp64_persist_capacity(h->threads, h->smem_gen, h->variants, h->suite, h->slices,
+                                                  h->islands);
 }
 
 // ... and as one thread-block cluster: one run of at most 8 tiles.
 static bool fp64_cluster_ok(const de_handle* h) {
   return h->nruns == 1 && fp64_persist_ok(h) &&
-         k_gen_fp64_cluster_fits(h->nitems, h->threads, h->smem_gen, h->variants, h->suite);
+         k_gen_fp64_cluster_fits(h->nitems, h->threads, h->smem_gen, h->variants, h->suite, h->slices);
 }
 
 static de_status autotune_fp64(de_handle* h, int nsm) {
@@ -923,6 +977,7 @@ de_status de_destroy(de_handle* h) {
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   tc_plan_free(h->tc);
   if (h->d_items) cudaFree(h->d_items);
+  if (h->d_shares) cudaFree(h->d_shares);
   if (h->d_run) cudaFree(h->d_run);
   if (h->d_ctl64) cudaFree(h->d_ctl64);
   if (h->isl_mem) cudaFree(h->isl_mem);
@@ -993,6 +1048,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
   h->stream = (cudaStream_t)cuda_stream;
   h->device = dev;
   h->nruns = nruns;
+  h->nsm = nsm;
   h->prec = cfgs[0].precision;
   for (int r = 0; r < nruns; ++r) {
     h->variants = h->variants || cfgs[r].strategy != DE_RAND1BIN || cfgs[r].jde;
@@ -1016,7 +1072,10 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
     return o;
   };
   struct Offs {
-    size_t X0, X1, f0, f1, fx0, fx1, o, MT, Mr, st, part, T, ref, jF0, jF1, jC0, jC1, perm;
+    size_t X0, X1, f0, f1, fx0, fx1, o, MT, Mr, sl, slx;
+    bool sliced;
+    int32_t qmin[5];
+    size_t st, part, T, ref, jF0, jF1, jC0, jC1, perm;
     size_t dbg_idx, dbg_jrand, dbg_mask, dbg_trial, dbg_ftrial, dbg_accept, dbg_fp64, dbg_cand;
   };
   std::vector<Offs> offs(nruns);
@@ -1037,6 +1096,11 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
     O.MT = c.rot ? take((size_t)pairs * c.d * c.d * sizeof(double)) : 0;
     O.perm = suite_spec(c.objective).kind == 1 ? take((size_t)c.d * sizeof(int32_t)) : 0;
     O.Mr = (c.rot && c.precision != DE_PREC_FP64) ? take((size_t)c.d * c.d * sizeof(double)) : 0;
+    // the rotation as digit slices, where it applies (FP64)
+    memset(O.qmin, 0, sizeof O.qmin);
+    O.sliced = c.rot && c.precision == DE_PREC_FP64 && slice_plan(c.rot, pairs, c.d, O.qmin);
+    O.sl = O.sliced ? take((size_t)pairs * slice_matrix_bytes(c.d)) : 0;
+    O.slx = O.sliced ? take((size_t)pairs * kSliceExp * sizeof(int32_t)) : 0;
     O.st = states_off + (size_t)r * sizeof(RunState);
     O.part = take((size_t)2 * c.np * sizeof(BestPartial));  // double buffered by generation parity
     const bool split = c.precision != DE_PREC_FP64;
@@ -1209,8 +1273,28 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
         rn = std::max(rn, std::sqrt(s));
       }
       R.rownorm = (float)rn;
+      if (O.sliced) {
+        R.sl = (const uint8_t*)(A + O.sl);
+        R.slx = (const int32_t*)(A + O.slx);
+        R.sl_kpad = slice_kpad_of(c.d);
+        memcpy(R.sl_qmin, O.qmin, sizeof R.sl_qmin);
+        k_slice_m_launch(R.MT, pairs, c.d, (uint8_t*)R.sl, (int32_t*)R.slx, h->stream);
+        h->slices.on = true;
+        h->slices.kpad = std::max(h->slices.kpad, R.sl_kpad);
+        h->slices.cols = std::max(h->slices.cols, slice_kernel_cols(R.sl_kpad));
+        h->slices.smem_op = std::max(h->slices.smem_op, slice_kernel_smem(R.sl_kpad));
+      }
     } else {
       R.rownorm = 1.0f;
+    }
+  }
+  if (h->slices.on) {
+    // every run's smallest tile has to fit beside the operands
+    bool fits = true;
+    for (auto& R : h->run) fits = fits && gen_smem(1, R.dp, suite_comps(R)) + h->slices.smem_op <= kTileSmemMax;
+    if (!fits) {
+      h->slices = SlicePlan{};
+      for (auto& R : h->run) R.sl = nullptr;
     }
   }
   if (h->prec != DE_PREC_FP64) {

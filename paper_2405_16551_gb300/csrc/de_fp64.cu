@@ -30,6 +30,7 @@
 #include "de_common.cuh"
 #include "de_internal.cuh"
 #include "de_device.cuh"
+#include "de_gen_tile.cuh"
 #include "de_island_dev.cuh"
 #include "de_kernels.h"
 #include "de_suite.cuh"
@@ -177,195 +178,6 @@ __global__ void k_best_init(const RunDesc* __restrict__ runs, int run) {
 }
 
 // ------------------------------------------------------------------ generation
-// Q groups of 32 flattened outputs (row r, coordinate j) of the tile's
-// rotation, one per accumulator chain: z[r][j] = sum_k M^T[k][j] y[r][k].
-template <int Q>
-__device__ __forceinline__ void rotate_groups(const RunDesc& R, const double* __restrict__ Y, double* __restrict__ Z,
-                                              int w0, int stride, int lane, int nout, int dp) {
-  const int d = R.d;
-  int rr[Q], jj[Q];
-  bool ok[Q];
-  double acc[Q];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const int e = (w0 + q * stride) * 32 + lane;
-    ok[q] = e < nout;
-    const int ec = ok[q] ? e : nout - 1;
-    rr[q] = ec / d;
-    jj[q] = ec - rr[q] * d;
-    acc[q] = 0.0;
-  }
-  for (int k = 0; k < d; ++k) {
-    const double* mk = R.MT + (size_t)k * d;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) acc[q] = fma(__ldg(mk + jj[q]), Y[rr[q] * dp + k], acc[q]);
-  }
-#pragma unroll
-  for (int q = 0; q < Q; ++q)
-    if (ok[q]) Z[rr[q] * dp + jj[q]] = acc[q];
-}
-
-// One tile of generation g: the trials of targets row0 .. row0 + nrows - 1
-// (a warp per target), their fitness, and greedy selection into the other
-// population buffer.  Shared memory sm: T (trials), Y (shifted trials), Z
-// (rotated), W (second term sum of Ackley), each rows_max x dp doubles.
-// best: the current population's best row (DE/best/1).  Returns the calling
-// warp's best (f, index) over the tile's new population rows (the same in
-// every lane).  Population rows, fitness and jDE parameters of generation
-// g - 1 are read at L2.
-// VAR / SUITE: strategy variants and jDE / the benchmark suite's objectives.
-template <bool VAR, bool SUITE>
-__device__ __forceinline__ Best gen_tile(const RunDesc& R, int64_t g, int row0, int nrows, int rows_max, int best,
-                                         double* sm, double* s_fsuite, double (*s_comp)[10]) {
-  const int cur = (int)((g - 1) & 1), nxt = cur ^ 1;
-  const double* X = R.X[cur];
-  double* __restrict__ Xn = R.X[nxt];
-  const double* fX = R.f[cur];
-  double* __restrict__ fn = R.f[nxt];
-  const int d = R.d, dp = R.dp;
-  double* T = sm;
-  double* Y = T + rows_max * dp;
-  double* Z = Y + rows_max * dp;
-  double* W = Z + rows_max * dp;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = blockDim.x >> 5;
-
-  // ---- trials (a warp per target)
-  const bool var = VAR && (R.strategy != 0 || R.jde);
-  const double* jFc = VAR && R.jde ? R.jF[cur] : nullptr;
-  const double* jCRc = VAR && R.jde ? R.jCR[cur] : nullptr;
-  if (var) {
-    for (int rl = warp; rl < nrows; rl += nwarps)
-      build_trial_row<true>(R, X, (uint32_t)(row0 + rl), g, lane, T + rl * dp, Y + rl * dp, best, jFc, jCRc);
-  } else if (R.unit_scale) {
-    // a unit domain scale: no multiplication on the FP64 pipe (the compiler
-    // would otherwise run it speculatively)
-    for (int rl = warp; rl < nrows; rl += nwarps)
-      build_trial_row<false, true>(R, X, (uint32_t)(row0 + rl), g, lane, T + rl * dp, Y + rl * dp);
-  } else {
-    for (int rl = warp; rl < nrows; rl += nwarps)
-      build_trial_row<false>(R, X, (uint32_t)(row0 + rl), g, lane, T + rl * dp, Y + rl * dp);
-  }
-  __syncthreads();
-
-  const int nout = nrows * d;
-  const bool suite = SUITE && suite_objective(R.obj);
-  if (suite) {
-    // ---- the proposed benchmark's functions (Sec. 7.3, Table 2)
-    const int ncomp = R.obj >= kObjComposition1 ? R.nc : 1;  // Y and Z hold every component of the tile
-    suite_tile(R, T, dp, nrows, Y, Y + (size_t)ncomp * rows_max * dp, s_fsuite, s_comp);
-  } else if (R.obj == kObjOde) {
-    // ---- ODE objective: a warp integrates one trial's chain; f to W[row][0]
-    for (int rl = warp; rl < nrows; rl += nwarps) {
-      const double s = warp_sum(ode_chain(T + rl * dp, lane, R.ode_ref, nullptr));
-      if (lane == 0) W[rl * dp] = s / (double)(kOdeSteps * kOdeN);
-    }
-    __syncthreads();
-  } else {
-    // ---- rotation, flattened over (row, output): output e = 32 w + lane of
-    // warp-group w; a warp takes groups warp, warp + 8, ... and runs up to four
-    // of them at once (independent accumulator chains)
-    if (R.rotate) {
-      const int ngroups = (nout + 31) / 32;
-      for (int w0 = warp; w0 < ngroups; w0 += 4 * nwarps) {
-        const int qn = min(4, (ngroups - w0 + nwarps - 1) / nwarps);  // uniform in the warp
-        if (qn == 4) rotate_groups<4>(R, Y, Z, w0, nwarps, lane, nout, dp);
-        else if (qn == 3) rotate_groups<3>(R, Y, Z, w0, nwarps, lane, nout, dp);
-        else if (qn == 2) rotate_groups<2>(R, Y, Z, w0, nwarps, lane, nout, dp);
-        else rotate_groups<1>(R, Y, Z, w0, nwarps, lane, nout, dp);
-      }
-    } else {
-      for (int e = tid; e < nout; e += blockDim.x) {
-        const int r = e / d, j = e - r * d;
-        Z[r * dp + j] = Y[r * dp + j];
-      }
-    }
-    __syncthreads();
-
-    // ---- objective terms, flattened; Y and W receive the per-coordinate terms
-    for (int e = tid; e < nout; e += blockDim.x) {
-      const int r = e / d, j = e - r * d;
-      const double z = Z[r * dp + j];
-      double t1 = 0.0, t2 = 0.0;
-      if (R.obj == kObjSphere) {
-        t1 = z * z;
-      } else if (R.obj == kObjRastrigin) {
-        t1 = z * z - 10.0 * cos2pi_f64_horner(z) + 10.0;
-      } else if (R.obj == kObjAckley) {
-        t1 = z * z;
-        t2 = cos2pi_f64_horner(z);
-      } else if (R.obj == kObjRosenbrock) {
-        if (j + 1 < d) {
-          const double t0 = z + 1.0, tn = Z[r * dp + j + 1] + 1.0;
-          const double a = tn - t0 * t0, b = t0 - 1.0;
-          t1 = 100.0 * a * a + b * b;
-        }
-      } else {
-        t1 = CUDART_NAN;
-      }
-      Y[r * dp + j] = t1;
-      W[r * dp + j] = t2;
-    }
-    __syncthreads();
-  }
-
-  // ---- row sums, greedy selection, best partial (a warp per row)
-  Best bb;
-  bb.init();
-  for (int rl = warp; rl < nrows; rl += nwarps) {
-    const int i = row0 + rl;
-    double ft;
-    if (suite) {
-      ft = s_fsuite[rl];
-    } else if (R.obj == kObjOde) {
-      ft = W[rl * dp];
-    } else {
-      double s1 = 0.0, s2 = 0.0;
-      for (int j = lane; j < d; j += 32) {
-        s1 += Y[rl * dp + j];
-        s2 += W[rl * dp + j];
-      }
-      s1 = warp_sum(s1);
-      s2 = warp_sum(s2);
-      ft = R.obj == kObjAckley ? 20.0 + 2.718281828459045 - 20.0 * exp(-0.2 * sqrt(s1 / d)) - exp(s2 / d) : s1;
-    }
-    const double fi = __ldcg(fX + i);
-    const bool acc = fit_key(ft) <= fit_key(fi) && fit_key(ft) != 0x7FFFFFFFFFFFFFFFLL;  // ft <= fi, NaN never
-    double2* dst = reinterpret_cast<double2*>(Xn + (size_t)i * dp);
-    if (acc) {
-      const double2* src = reinterpret_cast<const double2*>(T + rl * dp);
-      for (int j = lane; j < dp / 2; j += 32) dst[j] = src[j];
-    } else {
-      const double2* src = reinterpret_cast<const double2*>(X + (size_t)i * dp);
-      for (int j = lane; j < dp / 2; j += 32) dst[j] = __ldcg(src + j);
-    }
-    const double fnew = acc ? ft : fi;
-    if (VAR && R.jde && lane == 0) {
-      // jDE: an accepted trial passes its F_i and CR_i on
-      double Fi = __ldcg(jFc + i), CRi = __ldcg(jCRc + i);
-      if (acc) jde_params(R, (uint32_t)i, g, jFc, jCRc, Fi, CRi);
-      R.jF[nxt][i] = Fi;
-      R.jCR[nxt][i] = CRi;
-    }
-    if (lane == 0) {
-      fn[i] = fnew;
-      if (R.dbg_ftrial) {
-        R.dbg_ftrial[i] = ft;
-        R.dbg_accept[i] = acc ? 1 : 0;
-        R.dbg_fp64[i] = 1;
-      }
-    }
-    bb.offer(fnew, i);
-  }
-  return bb;
-}
-
-// Copy of a run descriptor into shared memory (its fields are read in every
-// phase, after barriers that would force global reloads).
-__device__ __forceinline__ void load_desc(RunDesc& sR, const RunDesc* src) {
-  for (int q = threadIdx.x; q < (int)(sizeof(RunDesc) / 8); q += blockDim.x)
-    reinterpret_cast<uint64_t*>(&sR)[q] = reinterpret_cast<const uint64_t*>(src)[q];
-}
-
 // items: (run, tile, first row, rows); the rows of all runs are spread over
 // about one CTA per SM so that every SM's FP64 pipe gets the same work.
 // VAR: some run of the launch uses a strategy variant or jDE; SUITE: some
@@ -445,12 +257,18 @@ constexpr long long kFp64Spin = 1LL << 22;
 
 // ISL: the runs are islands (an instance of its own, so that the other
 // instances keep their register allocation)
-template <bool VAR, bool SUITE, bool ISL>
+// TC: some run's rotation is sliced (de_slice.cuh); each CTA keeps its run's
+// matrix resident for the whole launch (a composition function's matrices
+// take turns).  kpad, cols: the launch's operand sizes.
+template <bool VAR, bool SUITE, bool ISL, bool TC>
 __global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restrict__ runs,
                                                           const int4* __restrict__ items, int nruns,
                                                           PersistCtl* ctl, long long gens, int clustered,
-                                                          IslandCtl* isl, IslandStage stage) {
-  extern __shared__ __align__(16) double sm[];
+                                                          IslandCtl* isl, IslandStage stage, int kpad,
+                                                          uint32_t cols) {
+  extern __shared__ __align__(1024) uint8_t smem_p[];
+  double* sm = reinterpret_cast<double*>(smem_p + (TC ? slice_smem(kpad) : 0u));
+  __shared__ SliceShared s_sl;
   __shared__ int s_stop, s_best, s_abort, s_done;
   __shared__ unsigned s_below;
   __shared__ long long s_gen, s_evals;
@@ -483,6 +301,8 @@ __global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restr
   __syncthreads();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = blockDim.x >> 5;
   if (nruns == 1 && s_stop) return;
+  SliceCtx sc;
+  if constexpr (TC) slice_begin(sc, smem_p, kpad, cols, s_sl);
   unsigned nstopped = 0;  // runs known stopped (thread 0)
   // the failure-detection test (off in normal launches): this CTA may leave
   // out its first arrival, and the barrier may give up sooner
@@ -534,9 +354,19 @@ __global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restr
     const bool live = !s_stop;
     const int64_t g = s_gen + 1;
     if (live) {
-      Best bb = gen_tile<VAR, SUITE>(R, g, it.z, it.w, R.rows, max(s_best, 0), sm, s_fsuite, s_comp);
+      Best bb = gen_tile<VAR, SUITE, TC>(R, g, it.z, it.w, R.rows, max(s_best, 0), sm, s_fsuite, s_comp, &sc);
       if (lane == 0) { s_bf[warp] = bb.f; s_bk[warp] = bb.k; s_bi[warp] = bb.i; }
       __syncthreads();
+      if (TC && tid == 0 && s_sl.fail) {
+        // a wait for the products gave up: every CTA leaves after this
+        // generation's barrier (which this one does not join; a cluster's
+        // members are told before theirs)
+        atomicExch(&ctl->abort, 1);
+        atomicOr(&st->err, kErrTimeout);
+        s_abort = 1;
+        if (clustered)
+          for (unsigned q = 0; q < nct; ++q) *cg::this_cluster().map_shared_rank(&s_abort, q) = 1;
+      }
       if (tid == 0) {
         bb.init();
         for (int w = 0; w < nwarps; ++w) bb.take(s_bf[w], s_bk[w], s_bi[w]);
@@ -552,7 +382,8 @@ __global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restr
       cg::this_cluster().sync();
     } else if (warp == 0) {
       // arrive, then wait for every CTA of this iteration
-      const bool ok = grid_sync();
+      __syncwarp();
+      const bool ok = (!TC || *(volatile int*)&s_abort == 0) && grid_sync();
       if (lane == 0) {
         if (!ok) {
           atomicExch(&ctl->abort, 1);
@@ -657,6 +488,9 @@ __global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restr
       __syncthreads();
     }
   }
+  if constexpr (TC) {
+    slice_end(sc);
+  }
 }
 
 }  // namespace de
@@ -664,104 +498,128 @@ __global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restr
 // ------------------------------------------------------------------ launchers
 namespace de {
 
+// The instance of the cooperative kernel (islands of the suite's objectives
+// run generation by generation).
+static const void* persist_kernel(bool var, bool suite, bool isl, bool tc) {
+  if (tc)
+    return isl ? (var ? (const void*)k_gen_fp64_persist<true, false, true, true>
+                      : (const void*)k_gen_fp64_persist<false, false, true, true>)
+           : var && suite ? (const void*)k_gen_fp64_persist<true, true, false, true>
+           : var          ? (const void*)k_gen_fp64_persist<true, false, false, true>
+           : suite        ? (const void*)k_gen_fp64_persist<false, true, false, true>
+                          : (const void*)k_gen_fp64_persist<false, false, false, true>;
+  return isl ? (var ? (const void*)k_gen_fp64_persist<true, false, true, false>
+                    : (const void*)k_gen_fp64_persist<false, false, true, false>)
+         : var && suite ? (const void*)k_gen_fp64_persist<true, true, false, false>
+         : var          ? (const void*)k_gen_fp64_persist<true, false, false, false>
+         : suite        ? (const void*)k_gen_fp64_persist<false, true, false, false>
+                        : (const void*)k_gen_fp64_persist<false, false, false, false>;
+}
+
+// Dynamic shared memory of a cooperative (or one-cluster) launch.  The
+// sliced instances take all of an SM's shared memory: their CTAs wait for one
+// another, so no other kernel that allocates tensor memory may share an SM
+// with them (two such grids, each holding the columns the other waits for,
+// would never finish).
+static size_t persist_smem(const void* k, size_t smem, bool tc) {
+  if (!tc) return smem;
+  cudaFuncAttributes a{};
+  int dev = 0, most = 0;
+  if (cudaFuncGetAttributes(&a, k) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return smem;
+  }
+  return std::max(smem, (size_t)most - a.sharedSizeBytes);
+}
+
 void k_configure(size_t smem_gen) {
   const int smem = (int)std::max<size_t>(smem_gen, 1);
   cudaFuncSetAttribute(k_gen_fp64<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   cudaFuncSetAttribute(k_gen_fp64<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   cudaFuncSetAttribute(k_gen_fp64<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   cudaFuncSetAttribute(k_gen_fp64<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_gen_fp64_persist<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_gen_fp64_persist<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_gen_fp64_persist<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_gen_fp64_persist<true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_gen_fp64_persist<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_gen_fp64_persist<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  for (int q = 0; q < 12; ++q) {
+    const bool tc = (q & 1) != 0, var = (q & 2) != 0, suite = q / 4 == 1, isl = q / 4 == 2;
+    const void* k = persist_kernel(var, suite, isl, tc);
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)persist_smem(k, smem, tc));
+  }
+  k_tc_configure();
   cudaFuncSetAttribute(k_eval_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
 cudaError_t k_gen_fp64_persist_launch(const RunDesc* runs, const int4* items, int nitems, int nruns, int threads,
                                       size_t smem, bool var, bool suite, PersistCtl* ctl, long long gens,
-                                      cudaStream_t s, int test_skip, IslandCtl* isl, const IslandStage* stage) {
+                                      cudaStream_t s, const SlicePlan& sp, int test_skip, IslandCtl* isl,
+                                      const IslandStage* stage) {
   cudaError_t e = persist_ctl_reset(ctl, test_skip, s);
   if (e != cudaSuccess) return e;
-  int clustered = 0;
+  int clustered = 0, kpad = sp.kpad;
+  uint32_t cols = sp.cols;
   IslandStage st{};
   if (stage) st = *stage;
   void* args[] = {(void*)&runs, (void*)&items, (void*)&nruns, (void*)&ctl, (void*)&gens, (void*)&clustered,
-                  (void*)&isl, (void*)&st};
+                  (void*)&isl, (void*)&st, (void*)&kpad, (void*)&cols};
   const dim3 grid((unsigned)nitems), block((unsigned)threads);
   if (isl && suite) return cudaErrorInvalidValue;  // islands of the suite's objectives run generation by generation
-  const void* k = isl ? (var ? (const void*)k_gen_fp64_persist<true, false, true>
-                             : (const void*)k_gen_fp64_persist<false, false, true>)
-                  : var && suite ? (const void*)k_gen_fp64_persist<true, true, false>
-                  : var          ? (const void*)k_gen_fp64_persist<true, false, false>
-                  : suite        ? (const void*)k_gen_fp64_persist<false, true, false>
-                                 : (const void*)k_gen_fp64_persist<false, false, false>;
-  return cudaLaunchCooperativeKernel(k, grid, block, args, smem, s);
+  const void* k = persist_kernel(var, suite, isl != nullptr, sp.on);
+  return cudaLaunchCooperativeKernel(k, grid, block, args, persist_smem(k, smem + sp.smem_op, sp.on), s);
 }
 
 // The same kernel as one cluster of nitems CTAs (nitems <= 8, one run).
-template <bool VAR, bool SUITE>
-static cudaError_t fp64_cluster_launch(const RunDesc* runs, const int4* items, int nitems, int threads, size_t smem,
-                                       PersistCtl* ctl, long long gens, cudaStream_t s, bool query_only,
-                                       int* nclusters) {
+static cudaLaunchConfig_t cluster_config(int nitems, int threads, size_t smem, cudaStream_t s, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)nitems);
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)nitems;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = (unsigned)nitems;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (query_only) return cudaOccupancyMaxActiveClusters(nclusters, k_gen_fp64_persist<VAR, SUITE, false>, &cfg);
-  const int nruns = 1, clustered = 1;
-  IslandCtl* isl = nullptr;
-  const IslandStage stage{};
-  return cudaLaunchKernelEx(&cfg, k_gen_fp64_persist<VAR, SUITE, false>, runs, items, nruns, ctl, gens, clustered, isl,
-                            stage);
+  return cfg;
 }
 
 cudaError_t k_gen_fp64_cluster_launch(const RunDesc* runs, const int4* items, int nitems, int threads, size_t smem,
-                                      bool var, bool suite, PersistCtl* ctl, long long gens, cudaStream_t s) {
+                                      bool var, bool suite, PersistCtl* ctl, long long gens, cudaStream_t s,
+                                      const SlicePlan& sp) {
   cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(PersistCtl), s);
   if (e != cudaSuccess) return e;
-  if (var && suite) return fp64_cluster_launch<true, true>(runs, items, nitems, threads, smem, ctl, gens, s, false, nullptr);
-  if (var) return fp64_cluster_launch<true, false>(runs, items, nitems, threads, smem, ctl, gens, s, false, nullptr);
-  if (suite) return fp64_cluster_launch<false, true>(runs, items, nitems, threads, smem, ctl, gens, s, false, nullptr);
-  return fp64_cluster_launch<false, false>(runs, items, nitems, threads, smem, ctl, gens, s, false, nullptr);
+  cudaLaunchAttribute attr[1];
+  const void* k = persist_kernel(var, suite, false, sp.on);
+  cudaLaunchConfig_t cfg = cluster_config(nitems, threads, persist_smem(k, smem + sp.smem_op, sp.on), s, attr);
+  int nruns = 1, clustered = 1, kpad = sp.kpad;
+  uint32_t cols = sp.cols;
+  IslandCtl* isl = nullptr;
+  IslandStage stage{};
+  void* args[] = {(void*)&runs, (void*)&items, (void*)&nruns, (void*)&ctl, (void*)&gens, (void*)&clustered,
+                  (void*)&isl, (void*)&stage, (void*)&kpad, (void*)&cols};
+  return cudaLaunchKernelExC(&cfg, k, args);
 }
 
-bool k_gen_fp64_cluster_fits(int nitems, int threads, size_t smem, bool var, bool suite) {
+bool k_gen_fp64_cluster_fits(int nitems, int threads, size_t smem, bool var, bool suite, const SlicePlan& sp) {
   if (nitems < 1 || nitems > 8) return false;
   int n = 0;
-  cudaError_t e;
-  if (var && suite) e = fp64_cluster_launch<true, true>(nullptr, nullptr, nitems, threads, smem, nullptr, 0, 0, true, &n);
-  else if (var) e = fp64_cluster_launch<true, false>(nullptr, nullptr, nitems, threads, smem, nullptr, 0, 0, true, &n);
-  else if (suite) e = fp64_cluster_launch<false, true>(nullptr, nullptr, nitems, threads, smem, nullptr, 0, 0, true, &n);
-  else e = fp64_cluster_launch<false, false>(nullptr, nullptr, nitems, threads, smem, nullptr, 0, 0, true, &n);
-  if (e != cudaSuccess) {
+  cudaLaunchAttribute attr[1];
+  const void* k = persist_kernel(var, suite, false, sp.on);
+  cudaLaunchConfig_t cfg = cluster_config(nitems, threads, persist_smem(k, smem + sp.smem_op, sp.on), 0, attr);
+  if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
   return n >= 1;
 }
 
-int k_gen_fp64_persist_capacity(int threads, size_t smem, bool var, bool suite, bool isl) {
+int k_gen_fp64_persist_capacity(int threads, size_t smem, bool var, bool suite, const SlicePlan& sp, bool isl) {
   int per_sm = 0, dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (isl && suite) return 0;  // islands of the suite's objectives run generation by generation
-  const void* f = isl ? (var ? (const void*)k_gen_fp64_persist<true, false, true>
-                             : (const void*)k_gen_fp64_persist<false, false, true>)
-                  : var && suite ? (const void*)k_gen_fp64_persist<true, true, false>
-                  : var          ? (const void*)k_gen_fp64_persist<true, false, false>
-                  : suite        ? (const void*)k_gen_fp64_persist<false, true, false>
-                                 : (const void*)k_gen_fp64_persist<false, false, false>;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, smem) != cudaSuccess) {
+  const void* k = persist_kernel(var, suite, isl, sp.on);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, persist_smem(k, smem + sp.smem_op, sp.on)) !=
+      cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -798,6 +656,10 @@ void k_init_population_launch(const RunDesc* runs, int run, int np, int dp, cuda
 void k_eval_rows_launch(const RunDesc* runs, int run, const RunDesc& Rh, const double* x, int64_t ld, int n,
                         double* f, uint8_t* fx, cudaStream_t s) {
   if (n <= 0) return;
+  if (Rh.sl) {
+    k_eval_rows_tc_launch(runs, run, Rh, x, ld, n, f, fx, s);
+    return;
+  }
   if (Rh.obj == kObjOde) {
     // a warp per row, few rows per CTA: the rows spread over every SM (an
     // SM's FP64 pipe, not the latency of one chain, bounds a CTA of 8 chains)

@@ -90,6 +90,13 @@ struct RunDesc {
   const double* o;
   const double* MT;
   const double* Mrow;  // d x d, row-major M (z_j = sum_k M[j][k] y_k), split path FP64 band
+  // FP64 rotation on the tensor cores (de_slice.cuh): nc matrices as digit
+  // slices in operand layout, their row exponents (128 per matrix), and the
+  // least count of large coordinates a row needs (0: the run's rotation is the
+  // DFMA chain)
+  const uint8_t* sl;
+  const int32_t* slx;
+  int32_t sl_kpad, sl_qmin[5];
   const double* ode_ref;  // ODE objective: kOdeSteps x 10 positions of the hidden parameter vector o
   RunState* st;
   BestPartial* part;

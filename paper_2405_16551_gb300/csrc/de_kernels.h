@@ -39,6 +39,33 @@ void k_configure(size_t smem_gen);
 // objective of the proposed benchmark (5..20)
 void k_gen_fp64_launch(const RunDesc* runs, const int4* items, int nitems, int threads, size_t smem, bool var,
                        bool suite, cudaStream_t s);
+// FP64 rotations as exact digit products on the tensor cores (de_slice.cuh,
+// de_fp64_tc.cu): what the kernels of a handle with such runs are launched
+// with (on = some run's rotation is sliced)
+struct SlicePlan {
+  bool on = false;
+  int kpad = 0;         // the largest padded d of the sliced runs
+  uint32_t cols = 0;    // tensor-memory columns a CTA allocates
+  size_t smem = 0;      // dynamic shared memory of k_gen_fp64_tc
+  size_t smem_op = 0;   // ... of which operands
+  int per_sm() const { return (int)(512u / cols); }
+};
+// eligibility of nc row-major d x d matrices, and the least count of large
+// coordinates a row of y needs for each
+bool slice_plan(const double* M, int nc, int d, int32_t qmin[5]);
+size_t slice_matrix_bytes(int d);  // digit slices of one matrix
+int slice_kpad_of(int d);
+uint32_t slice_kernel_cols(int kpad);
+size_t slice_kernel_smem(int kpad);
+size_t slice_group_smem(int dp);   // tile buffers of a composition function's row group
+constexpr int kSliceExp = 128;     // row exponents per matrix
+void k_slice_m_launch(const double* MT, int nc, int d, uint8_t* sl, int32_t* fexp, cudaStream_t s);
+// one generation: nct CTAs, CTA b works through items [shares[b].x, shares[b].y)
+void k_gen_fp64_tc_launch(const RunDesc* runs, const int4* items, const int2* shares, int nct, const SlicePlan& p,
+                          bool var, bool suite, cudaStream_t s);
+void k_eval_rows_tc_launch(const RunDesc* runs, int run, const RunDesc& Rh, const double* x, int64_t ld, int n,
+                           double* f, uint8_t* fx, cudaStream_t s);
+void k_tc_configure();
 // the generation loop of FP64 runs in one cooperative launch (every item
 // co-resident: nitems <= k_gen_fp64_persist_capacity; gens <= 2^20)
 // test_skip > 0: the grid-barrier failure test (PersistCtl::test_skip)
@@ -48,15 +75,16 @@ struct IslandCtl;
 struct IslandStage;
 cudaError_t k_gen_fp64_persist_launch(const RunDesc* runs, const int4* items, int nitems, int nruns, int threads,
                                       size_t smem, bool var, bool suite, PersistCtl* ctl, long long gens,
-                                      cudaStream_t s, int test_skip = 0, IslandCtl* isl = nullptr,
+                                      cudaStream_t s, const SlicePlan& sp, int test_skip = 0, IslandCtl* isl = nullptr,
                                       const IslandStage* stage = nullptr);
 // CTAs of the cooperative FP64 kernel that fit at once (isl: the island instance)
-int k_gen_fp64_persist_capacity(int threads, size_t smem, bool var, bool suite, bool isl = false);
+int k_gen_fp64_persist_capacity(int threads, size_t smem, bool var, bool suite, const SlicePlan& sp, bool isl = false);
 // the same loop as one thread-block cluster of nitems CTAs (one run,
 // nitems <= 8), the cluster barrier between generations
 cudaError_t k_gen_fp64_cluster_launch(const RunDesc* runs, const int4* items, int nitems, int threads, size_t smem,
-                                      bool var, bool suite, PersistCtl* ctl, long long gens, cudaStream_t s);
-bool k_gen_fp64_cluster_fits(int nitems, int threads, size_t smem, bool var, bool suite);
+                                      bool var, bool suite, PersistCtl* ctl, long long gens, cudaStream_t s,
+                                      const SlicePlan& sp);
+bool k_gen_fp64_cluster_fits(int nitems, int threads, size_t smem, bool var, bool suite, const SlicePlan& sp);
 void k_init_population_launch(const RunDesc* runs, int run, int np, int dp, cudaStream_t s);
 // f (and, when fx is not NULL, the FP64 flags) of n rows of x; Rh is the
 // host copy of run `run`'s descriptor

@@ -1,0 +1,344 @@
+// de_slice.cuh -- the FP64 rotation z = M y as exact integer products on the
+// tensor cores (an Ozaki-type splitting; Ozaki, Ogita, Oishi, Rump, Numerical
+// Algorithms 59 (2012), with signed 8-bit digits in BF16 operands).
+//
+// Why: a DFMA warp instruction occupies a sub-partition's FP64 unit for 64
+// cycles on this part (1.06 TFLOP/s in all), and the rotation is 2 d of the
+// about 2 d + 55 FP64 operations of a coordinate.  BF16 tensor products run
+// about 1800 times faster, so 43 digit products per FP64 product cost 2% of it.
+//
+// Arithmetic.  With 2^e > max_k |y_k| and 2^f_j > max_k |M_jk|,
+//   U_k = round(y_k 2^(62 - e)),  V_jk = round(M_jk 2^(62 - f_j)),  |U|, |V| <= 2^62,
+// each written in 8 signed digits of 8 bits (base 256, the digits in
+// [-128, 127], the leading one in [-65, 65]).  A digit is exact in BF16, a
+// product of two is exact, and for d <= 128 the sum over k of all digit
+// products of one weight group g = s + t <= 8 stays below 2^24 in size, so
+// its FP32 accumulation in tensor memory is exact:
+//   P_g = sum_k sum_{s + t = g} u_s,k v_t,jk,   z_j = 2^(e + f_j - 76) sum_{g <= 8} 256^(8 - g) P_g
+// with one rounding at the end (H = P_0 .. P_4 and L = P_5 .. P_8 are integers
+// below 2^51; z = fma(H, 2^32, L)).  What is lost: bits of y_k (M_jk) below
+// 2^-63 of the row's largest, and the groups g >= 9, together about 2^-64 of
+// 2^(e + f_j), where a chain of d DFMAs loses about 2^-52 of the products it
+// sums.
+//
+// A row is computed this way only when that comparison holds: with at least
+// qmin = cM + ceil(d / 8) coordinates of size >= 2^-6 max|y| (cM: the most
+// entries below 1/8 of a row of M's largest), every z_j sums at least d / 8
+// products of size >= 2^-9 of the largest possible one.  Other rows (and rows
+// with non-finite, subnormal or extreme values) take the DFMA chain
+// (rows_dfma), and matrices whose cM leaves no room (sparse ones) are not
+// sliced at all, so no row is computed less precisely than by the chain.
+//
+// Operands: A = M (128 rows, rows past d zero), one slice per digit t,
+// resident for as long as the CTA works on that matrix: the first nsm
+// slices in shared memory (their products are the widest, which hides the
+// 4 KB of A each reads), the others in tensor memory.  B = the digits of up to
+// 8 rows of y: row 8 s + r holds digit s of tile row r, so that one product
+// of slice t with digits 0 .. 8 - t adds its sums to the groups t .. 8, which
+// lie side by side in tensor memory (10 groups x 8 columns).  8 products
+// per 16 coordinates; 20 to 33 cycles each when issued from warp-uniform code
+// under elect.sync (60 to 80 from a divergent branch).
+#pragma once
+#include <cuda_runtime.h>
+
+#include "de_device.cuh"
+#include "de_tcgen05.cuh"
+
+namespace de {
+
+constexpr int kSlices = 8;          // digits per number
+constexpr int kSliceRows = 8;       // rows of y per product
+constexpr int kSliceDMin = 16;
+constexpr int kSliceDMax = 128;     // largest d (the exactness bound and the 128 rows of A)
+constexpr uint32_t kSliceKg = 1296; // bytes between 8-coordinate groups of B: 80 rows x 16, + 16 against bank conflicts
+constexpr uint32_t kSliceAcc = 80;  // accumulator columns: 10 groups x 8 rows
+
+__host__ __device__ inline int slice_kpad(int d) { return (d + 15) / 16 * 16; }
+// bytes of one slice of M: kpad / 8 groups of 128 rows x 16 bytes
+__host__ __device__ inline uint32_t slice_bytes(int kpad) { return (uint32_t)(kpad / 8) * 2048u; }
+// slices kept in shared memory (the others fit tensor memory's 512 columns)
+__host__ __device__ inline int slice_nsm(int kpad) {
+  const int fit = (int)(512u - kSliceAcc) / (kpad / 2);
+  return fit >= kSlices ? 0 : kSlices - fit;
+}
+__host__ __device__ inline uint32_t slice_tmem_cols(int kpad) {
+  const uint32_t need = kSliceAcc + (uint32_t)(kSlices - slice_nsm(kpad)) * (uint32_t)(kpad / 2);
+  return need <= 128u ? 128u : need <= 256u ? 256u : 512u;
+}
+// shared memory of the operands: B, then the resident slices
+__host__ __device__ inline uint32_t slice_b_bytes(int kpad) { return ((uint32_t)(kpad / 8) * kSliceKg + 1023u) / 1024u * 1024u; }
+__host__ __device__ inline uint32_t slice_smem(int kpad) { return slice_b_bytes(kpad) + (uint32_t)slice_nsm(kpad) * slice_bytes(kpad); }
+
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred P;\n elect.sync _|P, 0xffffffff;\n selp.u32 %0, 1, 0, P;\n}\n" : "=r"(p));
+  return p != 0u;
+}
+
+// One CTA's state of the sliced rotation (the same in every thread).
+struct SliceCtx {
+  uint8_t* sB;       // B operand (1024-byte aligned)
+  uint8_t* sA;       // slices resident in shared memory
+  uint32_t tmem;     // accumulators at column 0, slices from column kSliceAcc on
+  uint32_t bar;      // mbarrier of the products
+  uint32_t phase;
+  int* s_exp;        // per tile row: e
+  uint32_t* s_bad;   // bit r: tile row r takes the DFMA chain
+  int* s_fail;       // set when a wait for the products gave up
+  const uint8_t* cur;  // the matrix loaded (its slices in global memory)
+  uint32_t cols;       // tensor-memory columns allocated
+};
+
+// The slices of one matrix (global layout = operand layout) into shared and
+// tensor memory, by all threads of the CTA (256).
+__device__ __forceinline__ void slice_load_m(SliceCtx& c, const uint8_t* __restrict__ sl, int kpad) {
+  const int nsm = slice_nsm(kpad), tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t sbytes = slice_bytes(kpad);
+  __syncthreads();  // no product of the previous matrix is in flight and none of its slices is being read
+  for (uint32_t q = (uint32_t)tid * 16u; q < (uint32_t)nsm * sbytes; q += blockDim.x * 16u)
+    *reinterpret_cast<uint4*>(c.sA + q) = __ldg(reinterpret_cast<const uint4*>(sl + q));
+  // row r of a slice in lane r, 4 columns per 8-coordinate group; warps w and
+  // w + 4 share the lanes 32 (w mod 4) .. + 31 and take alternate groups
+  const int q4 = warp & 3, r = 32 * q4 + lane, nkg = kpad / 8;
+  const uint32_t ta0 = c.tmem + ((uint32_t)(32 * q4) << 16) + kSliceAcc;
+  const uint8_t* src = sl + (size_t)nsm * sbytes + (size_t)r * 16u;
+  const int n = (kSlices - nsm) * nkg;  // slices are contiguous, so the groups are too
+#pragma unroll 8
+  for (int g = warp >> 2; g < n; g += 2) {
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(src + (size_t)g * 2048u));
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ta0 + 4u * (uint32_t)g), "r"(v.x),
+                 "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
+  }
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  c.cur = sl;
+}
+
+// Allocates tensor memory, sets up the barrier and the zero rows of B; by
+// all threads, before any other use.  kpad: the largest of the matrices this
+// CTA will load (smem holds slice_smem(kpad) bytes), cols: their columns.
+struct SliceShared {
+  uint64_t bar;
+  uint32_t tmem, bad;
+  int fail;
+  int exp[kSliceRows];
+};
+
+__device__ __forceinline__ void slice_begin(SliceCtx& c, uint8_t* smem, int kpad, uint32_t cols, SliceShared& sh) {
+  uint32_t* s_tmem = &sh.tmem;
+  uint64_t* s_bar = &sh.bar;
+  int* s_exp = sh.exp;
+  uint32_t* s_bad = &sh.bad;
+  int* s_fail = &sh.fail;
+  c.cols = cols;
+  c.sB = smem;
+  c.sA = smem + slice_b_bytes(kpad);
+  c.bar = smem_u32(s_bar);
+  c.phase = 0;
+  c.s_exp = s_exp;
+  c.s_bad = s_bad;
+  c.s_fail = s_fail;
+  c.cur = nullptr;
+  if (threadIdx.x == 0) {
+    mbar_init(c.bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    *s_bad = 0u;
+    *s_fail = 0;
+  }
+  if (threadIdx.x < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)),
+                 "r"(cols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  for (uint32_t q = threadIdx.x * 16u; q < slice_b_bytes(kpad); q += blockDim.x * 16u)
+    *reinterpret_cast<uint4*>(smem + q) = make_uint4(0u, 0u, 0u, 0u);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  c.tmem = *s_tmem;
+}
+
+// Waits (bounded) for products still in flight after a failed wait, then
+// frees tensor memory; by all threads.
+__device__ __forceinline__ void slice_end(SliceCtx& c) {
+  if (threadIdx.x == 0 && *c.s_fail) mbar_wait(c.bar, c.phase ^ 1u);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x < 32)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(c.tmem), "r"(c.cols));
+}
+
+// Digits of one row of y into row r of the tile (one warp; lane L holds
+// coordinates 4 L .. 4 L + 3, zero past d).
+__device__ __forceinline__ void slice_digits(const SliceCtx& c, int r, int lane, int kpad, int qmin,
+                                             const double (&y)[4]) {
+  uint32_t hw[4], mx = 0u;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    hw[m] = (uint32_t)__double2hiint(y[m]) & 0x7FFFFFFFu;
+    mx = max(mx, hw[m]);
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  const int ex = (int)(mx >> 20);  // 2^(ex - 1022) exceeds every |y_k|
+  // coordinates of at least 2^-6 of the largest (by the high words)
+  const uint32_t thr = mx > (6u << 20) ? mx - (6u << 20) : 1u;
+  int q = 0;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) q += __popc(__ballot_sync(0xffffffffu, hw[m] >= thr));
+  // a row of zeros is exact; z stays in the normal range for e in [-800, 800]
+  const bool zero = mx == 0u && __all_sync(0xffffffffu, ((__double2loint(y[0]) | __double2loint(y[1]) |
+                                                         __double2loint(y[2]) | __double2loint(y[3])) == 0));
+  const bool bad = !zero && (q < qmin || ex < 1022 - 800 || ex > 1022 + 800);
+  if (lane == 0) {
+    c.s_exp[r] = ex - 1022;
+    if (bad) atomicOr(c.s_bad, 1u << r);
+  }
+  if (4 * lane >= kpad) return;
+  uint32_t lo[4], hi[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const long long b = __double_as_longlong(y[m]);
+    const int ek = (int)(hw[m] >> 20);
+    // significand at bits 9 .. 61, shifted down to the row's exponent with
+    // rounding (an exact shift by up to 9 bits)
+    unsigned long long u = (((unsigned long long)b & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL) << 9;
+    const int sh = ex - ek;
+    if (ek == 0 || sh > 62) u = 0ULL;
+    else if (sh > 0) u = (u + (1ULL << (sh - 1))) >> sh;
+    const long long v = (b < 0 ? -(long long)u : (long long)u) + (long long)0x8080808080808080ULL;
+    lo[m] = (uint32_t)v;
+    hi[m] = (uint32_t)((unsigned long long)v >> 32);
+  }
+  // byte s of v (from the top) is digit s plus 128; in the low byte of
+  // 2^23 + byte, minus 2^23 + 128, it is the digit in FP32, whose upper half
+  // is its exact BF16 form
+  uint8_t* dst = c.sB + (uint32_t)(lane >> 1) * kSliceKg + (uint32_t)r * 16u + (uint32_t)(lane & 1) * 8u;
+#pragma unroll
+  for (int s = 0; s < kSlices; ++s) {
+    float f[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const uint32_t w = s < 4 ? hi[m] : lo[m];
+      f[m] = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7550u | (uint32_t)(3 - (s & 3)))) - 8388736.0f;
+    }
+    uint2 p;
+    p.x = __byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632u);
+    p.y = __byte_perm(__float_as_uint(f[2]), __float_as_uint(f[3]), 0x7632u);
+    *reinterpret_cast<uint2*>(dst + s * 128) = p;
+  }
+}
+
+// The products of the tile's digits with the loaded matrix, then z into
+// Z[r][j] (row stride dp) for the tile's nrows rows; by all threads of the
+// CTA, after a CTA barrier that follows the digits.  fexp: f_j per output.
+// The caller's CTA barrier makes Z visible.  Y: the FP64 rows (stride dp), for
+// rows that take the DFMA chain over MT.
+__device__ __forceinline__ void slice_rotate(SliceCtx& c, int kpad, const int32_t* __restrict__ fexp,
+                                             const double* __restrict__ MT, const double* __restrict__ Y,
+                                             double* __restrict__ Z, int nrows, int d, int dp) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const int nsm = slice_nsm(kpad), ksteps = kpad / 16;
+    const uint32_t sbytes = slice_bytes(kpad);
+    const uint64_t db0 = smem_desc(smem_u32(c.sB), kSliceKg, 128u);
+    const uint64_t da0 = smem_desc(smem_u32(c.sA), 2048u, 128u);
+    constexpr uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTileM >> 4) << 24);
+    constexpr uint32_t bstep = (2u * kSliceKg) >> 4, astep = 4096u >> 4;
+    if (elect_one()) {
+#pragma unroll
+      for (int t = 0; t < kSlices; ++t) {
+        // digits 0 .. 8 - t (at most 8 of them, an even number: N is a multiple of 16)
+        const uint32_t ns = t <= 2 ? 8u : (uint32_t)((10 - t) / 2 * 2);
+        const uint32_t idesc = idesc0 | (ns << 17);
+        const uint32_t dcol = c.tmem + (uint32_t)t * 8u;
+        for (int ks = 0; ks < ksteps; ++ks) {
+          const uint64_t db = db0 + (uint64_t)(bstep * (uint32_t)ks);
+          // the first product also covers groups 8 and 9 (B's zero rows), so
+          // that every group starts at zero
+          const uint32_t id = t == 0 && ks == 0 ? (idesc0 | (10u << 17)) : idesc;
+          const uint32_t acc = t == 0 && ks == 0 ? 0u : 1u;
+          if (t < nsm)
+            mma_split<2>(dcol, da0 + (uint64_t)((uint32_t)t * (sbytes >> 4) + astep * (uint32_t)ks), db, id, acc);
+          else
+            mma_split_ta<2>(dcol, c.tmem + kSliceAcc + (uint32_t)(t - nsm) * (uint32_t)(kpad / 2) + 8u * (uint32_t)ks, db,
+                            id, acc);
+        }
+      }
+      mma_commit(c.bar);
+    }
+    __syncwarp();
+    const bool ok = mbar_wait(c.bar, c.phase);
+    if (!__all_sync(0xffffffffu, ok) && lane == 0) *c.s_fail = 1;
+  }
+  c.phase ^= 1u;
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  // warp w: outputs 32 (w mod 4) .. + 31 (lanes), tile rows 4 (w / 4) .. + 3
+  const int q4 = warp & 3, r0 = 4 * (warp >> 2), j = 32 * q4 + lane;
+  if (r0 < nrows && 32 * q4 < d) {
+    float p[9][4];
+    const uint32_t ta = c.tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)r0;
+#pragma unroll
+    for (int g = 0; g < 9; ++g) {
+      uint32_t v[4];
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                   : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                   : "r"(ta + 8u * (uint32_t)g));
+#pragma unroll
+      for (int e = 0; e < 4; ++e) p[g][e] = __uint_as_float(v[e]);
+    }
+    // the values are used only after the wait (the operands tie them to it)
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(p[0][0]), "+f"(p[0][1]), "+f"(p[0][2]), "+f"(p[0][3]), "+f"(p[1][0]), "+f"(p[1][1]),
+                   "+f"(p[1][2]), "+f"(p[1][3]), "+f"(p[2][0]), "+f"(p[2][1]), "+f"(p[2][2]), "+f"(p[2][3]),
+                   "+f"(p[3][0]), "+f"(p[3][1]), "+f"(p[3][2]), "+f"(p[3][3])::"memory");
+    asm volatile(""
+                 : "+f"(p[4][0]), "+f"(p[4][1]), "+f"(p[4][2]), "+f"(p[4][3]), "+f"(p[5][0]), "+f"(p[5][1]),
+                   "+f"(p[5][2]), "+f"(p[5][3]), "+f"(p[6][0]), "+f"(p[6][1]), "+f"(p[6][2]), "+f"(p[6][3]),
+                   "+f"(p[7][0]), "+f"(p[7][1]), "+f"(p[7][2]), "+f"(p[7][3]), "+f"(p[8][0]), "+f"(p[8][1]),
+                   "+f"(p[8][2]), "+f"(p[8][3])::"memory");
+    const int fj = j < d ? __ldg(fexp + j) : 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (r0 + e < nrows) {
+        int P[9];
+#pragma unroll
+        for (int g = 0; g < 9; ++g) P[g] = __float2int_rn(p[g][e]);
+        const int a = P[0] * 256 + P[1], b = P[2] * 256 + P[3];
+        const long long H = (long long)a * 16777216LL + ((long long)b * 256LL + P[4]);
+        const long long L = ((long long)P[5] * 256LL + P[6]) * 65536LL + ((long long)P[7] * 256LL + P[8]);
+        // |H|, |L| < 2^51: exact in the significand of 1.5 2^52 + n
+        const double C = 6755399441055744.0;
+        const double h = __dsub_rn(__longlong_as_double(H + 0x4338000000000000LL), C);
+        const double l = __dsub_rn(__longlong_as_double(L + 0x4338000000000000LL), C);
+        const double z = __fma_rn(h, 4294967296.0, l);
+        // times 2^(e + f_j - 76), on the exponent field (z is 0 or normal)
+        const int hz = __double2hiint(z), sc = (c.s_exp[r0 + e] + fj - 76) * 1048576;
+        if (j < d) Z[(r0 + e) * dp + j] = __hiloint2double((hz & 0x7FF00000) ? hz + sc : hz, __double2loint(z));
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  const uint32_t bad = *c.s_bad;
+  if (bad) {
+    // rows outside the splitting's comparison: one DFMA chain per output
+    __syncthreads();
+    if (tid == 0) *c.s_bad = 0u;
+    for (int e = tid; e < nrows * d; e += (int)blockDim.x) {
+      const int r = e / d, jj = e - r * d;
+      if (!((bad >> r) & 1u)) continue;
+      double s = 0.0;
+      for (int k = 0; k < d; ++k) s = fma(__ldg(MT + (size_t)k * d + jj), Y[r * dp + k], s);
+      Z[r * dp + jj] = s;
+    }
+  }
+}
+
+}  // namespace de

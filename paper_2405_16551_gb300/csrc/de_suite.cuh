@@ -15,6 +15,7 @@
 #include "de_common.cuh"
 #include "de_device.cuh"
 #include "de_internal.cuh"
+#include "de_slice.cuh"
 
 namespace de {
 
@@ -235,6 +236,96 @@ __device__ __forceinline__ void comp_rotate(const double* __restrict__ MT, const
   }
 }
 
+// y = (x - o) s of tile row r (one warp; src: the row of x), stored as FP64
+// row Yr and as digits of the sliced rotation; returns |x - o|^2 (every lane).
+__device__ __forceinline__ double suite_digits(const RunDesc& R, const SliceCtx& c, int r, int lane, const double* src,
+                                               const double* __restrict__ o, double sc, int qmin,
+                                               double* __restrict__ Yr) {
+  double y[4] = {0.0, 0.0, 0.0, 0.0};
+  double dd = 0.0;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const int j = 4 * lane + m;
+    if (j < R.d) {
+      const double t = __dsub_rn(src[j], o[j]);
+      dd += t * t;
+      y[m] = __dmul_rn(t, sc);
+    }
+  }
+  if (4 * lane < R.dp) {
+    *reinterpret_cast<double2*>(Yr + 4 * lane) = make_double2(y[0], y[1]);
+    *reinterpret_cast<double2*>(Yr + 4 * lane + 2) = make_double2(y[2], y[3]);
+  }
+  slice_digits(c, r, lane, R.sl_kpad, qmin, y);
+  return warp_sum(dd);
+}
+
+// Weights and mixture of a composition function from g_c (comp[0..4]) and
+// D_c (comp[5..9]) of one row.
+__device__ __forceinline__ double comp_mix(const RunDesc& R, const double* comp) {
+  const int nc = R.nc, d = R.d;
+  int hit = -1;
+  for (int c = 0; c < nc; ++c)
+    if (comp[5 + c] == 0.0 && hit < 0) hit = c;
+  double om[5], m = -CUDART_INF, sum = 0.0;
+  for (int c = 0; c < nc; ++c) {
+    const double D = comp[5 + c];
+    om[c] = -0.5 * log(D) - D / (2.0 * d * R.ssigma[c] * R.ssigma[c]);
+    m = fmax(m, om[c]);
+  }
+  for (int c = 0; c < nc; ++c) {
+    om[c] = hit >= 0 ? (c == hit ? 1.0 : 0.0) : exp(om[c] - m);
+    sum += om[c];
+  }
+  double acc = 0.0;
+  for (int c = 0; c < nc; ++c) acc += om[c] / sum * (R.slambda[c] * comp[c] + R.sbias[c]);
+  return acc;
+}
+
+// Composition function of nrows rows of src with the sliced rotation: one
+// component's matrix at a time is resident for all rows (a matrix is 229 KB at
+// d = 100, so it is loaded once per component and call, not per 8 rows).
+// Y, Z: 8 x dp doubles; comp: nrows x 10.
+static __device__ __noinline__ void suite_comp_sliced(const RunDesc& R, const double* src, int64_t ld, int nrows,
+                                                     double* __restrict__ Y, double* __restrict__ Z,
+                                                     double* __restrict__ f, double (*comp)[10], SliceCtx& sc) {
+  const int d = R.d, dp = R.dp, kpad = R.sl_kpad;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int c = 0; c < R.nc; ++c) {
+    slice_load_m(sc, R.sl + (size_t)c * kSlices * slice_bytes(kpad), kpad);
+    const int fn = R.sfn[c];
+    const bool costly = basic_has_costly(fn);
+    for (int t0 = 0; t0 < nrows; t0 += kSliceRows) {
+      const int nr = min(kSliceRows, nrows - t0);
+      if (warp < nr) {
+        const double dd = suite_digits(R, sc, warp, lane, src + (size_t)(t0 + warp) * ld, R.o + (size_t)c * dp,
+                                       R.sscale[c], R.sl_qmin[c], Y + warp * dp);
+        if (lane == 0) comp[t0 + warp][5 + c] = dd;
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncthreads();
+      slice_rotate(sc, kpad, R.slx + c * kSliceDMax, R.MT + (size_t)c * d * d, Y, Z, nr, d, dp);
+      __syncthreads();
+      if (costly) {
+        for (int e = tid; e < nr * dp; e += blockDim.x) {
+          const int r = e / dp, j = e - r * dp;
+          if (j >= d) continue;
+          const double* zr = Z + r * dp;
+          Y[e] = basic_costly(fn, zr[j], zr[j + 1 < d ? j + 1 : 0], j, d, R.skex[c]);
+        }
+        __syncthreads();
+      }
+      if (warp < nr) {
+        const double g = basic_fn_warp(fn, Z + warp * dp, nullptr, 0, d, 1.0, Y + warp * dp, lane);
+        if (lane == 0) comp[t0 + warp][c] = g;
+      }
+      __syncthreads();
+    }
+  }
+  for (int r = tid; r < nrows; r += blockDim.x) f[r] = comp_mix(R, comp[r]);
+  __syncthreads();
+}
+
 // Objective of the suite for nrows rows of src (row stride ld, in shared or
 // global memory); the whole CTA calls it.  Y, Z: shared buffers of
 // nrows x dp doubles, nc times that for a composition function;
@@ -250,9 +341,15 @@ __device__ __forceinline__ void comp_rotate(const double* __restrict__ MT, const
 //                   logarithms; at x = o_c the weight is 1 for the first such c.
 constexpr int kSuiteMaxRows = 8;
 
+// TC: the run's rotation may be sliced (sc; R.sl != NULL then).
+template <bool TC = false>
 static __device__ __noinline__ void suite_tile(const RunDesc& R, const double* src, int64_t ld, int nrows,
                                               double* __restrict__ Y, double* __restrict__ Z, double* __restrict__ f,
-                                              double (*comp)[10]) {
+                                              double (*comp)[10], SliceCtx* sc = nullptr) {
+  if (TC && R.sl && R.obj >= kObjComposition1) {
+    suite_comp_sliced(R, src, ld, nrows, Y, Z, f, comp, *sc);
+    return;
+  }
   const int d = R.d, dp = R.dp;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   const bool is_comp = R.obj >= kObjComposition1;
@@ -310,38 +407,30 @@ static __device__ __noinline__ void suite_tile(const RunDesc& R, const double* s
       }
     }
     __syncthreads();
-    for (int r = threadIdx.x; r < nrows; r += blockDim.x) {
-      int hit = -1;
-      for (int c = 0; c < nc; ++c)
-        if (comp[r][5 + c] == 0.0 && hit < 0) hit = c;
-      double om[5], m = -CUDART_INF, sum = 0.0;
-      for (int c = 0; c < nc; ++c) {
-        const double D = comp[r][5 + c];
-        om[c] = -0.5 * log(D) - D / (2.0 * d * R.ssigma[c] * R.ssigma[c]);
-        m = fmax(m, om[c]);
-      }
-      for (int c = 0; c < nc; ++c) {
-        om[c] = hit >= 0 ? (c == hit ? 1.0 : 0.0) : exp(om[c] - m);
-        sum += om[c];
-      }
-      double acc = 0.0;
-      for (int c = 0; c < nc; ++c) acc += om[c] / sum * (R.slambda[c] * comp[r][c] + R.sbias[c]);
-      f[r] = acc;
-    }
+    for (int r = threadIdx.x; r < nrows; r += blockDim.x) f[r] = comp_mix(R, comp[r]);
     __syncthreads();
     return;
   }
   // basic and hybrid functions: one shift and one rotation
-  for (int e = threadIdx.x; e < nrows * dp; e += blockDim.x) {
-    const int r = e / dp, j = e - r * dp;
-    double y = 0.0;
-    if (j < d) y = __dmul_rn(__dsub_rn(src[(size_t)r * ld + j], R.o[j]), R.scale);
-    Y[e] = y;
+  if (TC && R.sl) {
+    if (sc->cur != R.sl) slice_load_m(*sc, R.sl, R.sl_kpad);
+    if (warp < nrows)
+      suite_digits(R, *sc, warp, lane, src + (size_t)warp * ld, R.o, R.scale, R.sl_qmin[0], Y + warp * dp);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    slice_rotate(*sc, R.sl_kpad, R.slx, R.MT, Y, Z, nrows, d, dp);
+  } else {
+    for (int e = threadIdx.x; e < nrows * dp; e += blockDim.x) {
+      const int r = e / dp, j = e - r * dp;
+      double y = 0.0;
+      if (j < d) y = __dmul_rn(__dsub_rn(src[(size_t)r * ld + j], R.o[j]), R.scale);
+      Y[e] = y;
+    }
+    __syncthreads();
+    if (R.rotate) suite_rotate(R.MT, Y, Z, nrows, d, dp);
+    else
+      for (int e = threadIdx.x; e < nrows * dp; e += blockDim.x) Z[e] = Y[e];
   }
-  __syncthreads();
-  if (R.rotate) suite_rotate(R.MT, Y, Z, nrows, d, dp);
-  else
-    for (int e = threadIdx.x; e < nrows * dp; e += blockDim.x) Z[e] = Y[e];
   __syncthreads();
   // the costly parts of every (row, position) over the whole CTA, into Y
   // (free after the rotation)
