@@ -51,19 +51,106 @@ __device__ __forceinline__ double cos2pi_f64(double z) {
   return odd ? -c : c;
 }
 
-// Same series by Horner's rule: fewer FP64 instructions than Estrin's
-// scheme, for kernels bound by FP64 throughput rather than latency.
-__device__ __forceinline__ double cos2pi_f64_horner(double z) {
-  const double sh = 6755399441055744.0;  // 1.5 * 2^52
-  const double tz = 2.0 * z;
-  const double t1 = __dadd_rn(tz, sh);
-  const double r = __dsub_rn(tz, __dsub_rn(t1, sh));
-  const bool odd = __double_as_longlong(t1) & 1;
-  const double u = r * r;
-  double c = cospi_taylor(10);
-#pragma unroll
-  for (int n = 9; n >= 0; --n) c = fma(c, u, cospi_taylor(n));
-  return odd ? -c : c;
+// 1 - cos(2 pi z) in fixed point on the integer pipe, in units of 2^-62
+// (0 .. 2^63): the FP64 series takes 15 FP64-pipe instructions of 64 cycles
+// each, this about 100 integer ones of 1 to 2.  2z = k + r with r, |r| <= 1/2,
+// a 64-bit fraction cut from the significand (exact down to 2^-64);
+// with v = (2r)^2, 1 - cos(pi r) = v (a_1 - v (a_2 - ...)), a_n = (pi/2)^(2n) /
+// (2n)!, all partial values positive.  The terms n >= 7 (below 2^-27) run in
+// 32 bits at units of 2^-59, the others in 64 bits at units of 2^-63, so the
+// sum is within 2^-58, against 2^-53 of the FP64 form.  *ok = false for a
+// non-finite z (whose cosine is NaN).
+__host__ __device__ constexpr double cos_term(int n) {  // (pi/2)^(2n) / (2n)!
+  double c = 1.0;
+  for (int k = 1; k <= n; ++k) c *= 2.4674011002723396547 / ((2.0 * k - 1.0) * (2.0 * k));
+  return c;
+}
+
+// a_1 .. a_6 in units of 2^-63: the leading factor pi^2/8 to 64 bits, then each
+// from the one before by 128-bit division (constant expressions)
+__host__ __device__ constexpr unsigned long long cos_fix(int n) {
+  // pi^2 / 4 = 2.4674011002723396547... = 2 + 0.4674011002723396547086...
+  unsigned __int128 q = ((unsigned __int128)2 << 124) + ((unsigned __int128)0x77A79937C8BBCB49ULL << 60);  // units of 2^-124
+  unsigned __int128 a = q / 2;
+  for (int k = 2; k <= n; ++k) {
+    // a * (pi^2 / 4) / ((2k - 1) 2k), the product on 62-bit halves
+    const unsigned __int128 hi = (a >> 62) * (q >> 62);
+    a = hi / ((2 * k - 1) * (2 * k));
+  }
+  return (unsigned long long)((a + ((unsigned __int128)1 << 60)) >> 61);
+}
+
+__device__ __forceinline__ unsigned long long omcos2pi_fix(double z, bool& ok) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(z);
+  const int ex = (int)((b >> 52) & 0x7FF);
+  ok = ex != 0x7FF;
+  // 2z = m 2^(ex - 1074): the bits below the point as a 64-bit fraction, and
+  // the lowest bit of the integer part
+  const unsigned long long m = (b & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL;
+  const int up = ex - 1074 + 64;  // the fraction is m 2^up modulo 2^64
+  unsigned long long fr = 0ULL;
+  unsigned int odd = 0u;
+  if (up >= 0) {
+    if (up < 64) fr = m << up;
+    const int ib = 64 - up;  // the integer part's lowest bit
+    if (ib >= 0 && ib < 53) odd = (unsigned int)(m >> ib) & 1u;
+  } else if (up > -64) {
+    fr = m >> -up;
+  }
+  // the sign of z does not matter; r = fr or fr - 1 (then k is one more)
+  odd ^= (unsigned int)(fr >> 63);
+  const unsigned long long r = (fr >> 63) ? 0ULL - fr : fr;  // |r| <= 2^63
+  const unsigned long long u = __umul64hi(r, r);             // r^2 <= 2^62
+  const unsigned long long v = u >= (1ULL << 62) ? ~0ULL : u << 2;
+  const unsigned int vh = (unsigned int)(v >> 32);
+  constexpr unsigned int t10 = (unsigned int)(cos_term(10) * 0x1p59), t9 = (unsigned int)(cos_term(9) * 0x1p59),
+                         t8 = (unsigned int)(cos_term(8) * 0x1p59), t7 = (unsigned int)(cos_term(7) * 0x1p59);
+  constexpr unsigned long long a6 = cos_fix(6), a5 = cos_fix(5), a4 = cos_fix(4), a3 = cos_fix(3), a2 = cos_fix(2),
+                               a1 = cos_fix(1);
+  unsigned int q32 = t9 - __umulhi(vh, t10);
+  q32 = t8 - __umulhi(vh, q32);
+  q32 = t7 - __umulhi(vh, q32);
+  unsigned long long q = a6 - __umul64hi(v, (unsigned long long)q32 << 4);
+  q = a5 - __umul64hi(v, q);
+  q = a4 - __umul64hi(v, q);
+  q = a3 - __umul64hi(v, q);
+  q = a2 - __umul64hi(v, q);
+  q = a1 - __umul64hi(v, q);
+  const unsigned long long x = (__umul64hi(v, q) + 1ULL) >> 1;  // 1 - cos(pi r), units of 2^-62
+  return odd ? (1ULL << 63) - x : x;
+}
+
+// w 2^e rounded to nearest even, on the integer pipe (the conversion
+// instruction occupies the FP64 pipe).
+__device__ __forceinline__ double f64_of_u64(unsigned long long w, int e) {
+  if (w == 0ULL) return 0.0;
+  const int lz = __clzll((long long)w);
+  const unsigned long long n = w << lz;
+  unsigned long long k = n >> 11;
+  const unsigned int rem = (unsigned int)n & 0x7FFu;
+  k += (rem > 0x400u || (rem == 0x400u && (k & 1ULL))) ? 1ULL : 0ULL;
+  // k carries the leading one, which adds 1 to the exponent field
+  return __longlong_as_double((long long)(((unsigned long long)(1023 + 62 - lz + e) << 52) + k));
+}
+
+// cos(2 pi z) rounded from the fixed-point form.
+__device__ __forceinline__ double cos2pi_fix(double z) {
+  bool ok;
+  const unsigned long long x = omcos2pi_fix(z, ok);
+  const bool neg = x > (1ULL << 62);
+  const double c = f64_of_u64(neg ? x - (1ULL << 62) : (1ULL << 62) - x, -62);
+  return ok ? (neg ? -c : c) : CUDART_NAN;
+}
+
+// 10 (1 - cos(2 pi z)), the periodic part of Rastrigin's term z^2 - 10 cos(2 pi
+// z) + 10: with it the term is one FP64 operation, without cancellation near
+// a minimum.
+__device__ __forceinline__ double rastrigin_w(double z) {
+  bool ok;
+  const unsigned long long x = omcos2pi_fix(z, ok);
+  // 10 x in units of 2^-59 (x 2^3 smaller, below 2^64)
+  const double w = f64_of_u64(((x + 4ULL) >> 3) * 10ULL, -59);
+  return ok ? w : CUDART_NAN;
 }
 
 __device__ __forceinline__ float cos2pi_f32(float z) {
@@ -175,7 +262,7 @@ __device__ __forceinline__ double row_objective_fp64(int obj, const double* __re
   } else if (obj == kObjRastrigin) {
     for (int j = lane; j < d; j += 32) {
       const double zj = z[j];
-      s1 += zj * zj - 10.0 * cos2pi_f64_horner(zj) + 10.0;
+      s1 += fma(zj, zj, rastrigin_w(zj));
     }
   } else if (obj == kObjRosenbrock) {
     for (int j = lane; j + 1 < d; j += 32) {
@@ -187,7 +274,7 @@ __device__ __forceinline__ double row_objective_fp64(int obj, const double* __re
     for (int j = lane; j < d; j += 32) {
       const double zj = z[j];
       s1 += zj * zj;
-      s2 += cos2pi_f64_horner(zj);
+      s2 += cos2pi_fix(zj);
     }
   } else {
     s1 = CUDART_NAN;

@@ -179,10 +179,10 @@ __device__ __forceinline__ Best gen_tile(const RunDesc& R, int64_t g, int row0, 
       if (R.obj == kObjSphere) {
         t1 = z * z;
       } else if (R.obj == kObjRastrigin) {
-        t1 = z * z - 10.0 * cos2pi_f64_horner(z) + 10.0;
+        t1 = fma(z, z, rastrigin_w(z));
       } else if (R.obj == kObjAckley) {
         t1 = z * z;
-        t2 = cos2pi_f64_horner(z);
+        t2 = cos2pi_fix(z);
       } else if (R.obj == kObjRosenbrock) {
         if (j + 1 < d) {
           const double t0 = z + 1.0, tn = Z[r * dp + j + 1] + 1.0;

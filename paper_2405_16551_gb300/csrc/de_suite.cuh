@@ -54,8 +54,8 @@ __device__ __forceinline__ double schwefel_term(double t, int n) {
 // Katsuura's exponent 10 / n^1.2 for this n (computed once per part).
 __device__ __forceinline__ double basic_costly(int fn, double w, double v, int l, int n, double kex) {
   switch (fn) {
-    case kObjRastrigin:
-    case kObjAckley: return cos2pi_f64_horner(w);
+    case kObjRastrigin: return rastrigin_w(w);
+    case kObjAckley: return cos2pi_fix(w);
     case kObjSchwefel: return schwefel_term(w + 420.9687462275036, n);
     case kObjSchafferF6: {
       const double s = w * w + v * v;
@@ -106,7 +106,7 @@ static __device__ __noinline__ double basic_fn_warp(int fn, const double* __rest
     const double w = W(l);
     switch (fn) {
       case kObjSphere: s1 += w * w; break;
-      case kObjRastrigin: s1 += w * w - 10.0 * E[l] + 10.0; break;
+      case kObjRastrigin: s1 += fma(w, w, E[l]); break;
       case kObjRosenbrock:
         if (l + 1 < n) {
           const double t0 = w + 1.0, t1 = W(l + 1) + 1.0;
