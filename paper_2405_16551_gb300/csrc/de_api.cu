@@ -39,6 +39,10 @@ struct de_handle {
   SlicePlan slices;           // FP64 rotations on the tensor cores (de_slice.cuh)
   int2* d_shares = nullptr;   // sliced generation kernel: the items of each CTA
   int nshares = 0;
+  // every run is sliced plain DE/rand/1/bin of objectives 0..3: the cooperative
+  // launch is k_gen_sliced (unit: every scale is 1)
+  bool sliced_loop = false, unit = true;
+  size_t smem_loop = 0;
   int nsm = 1;
   int rows = 8;             // rows per tile of the FP64 generation kernel
   int threads = 256;
@@ -367,6 +371,10 @@ static de_status enqueue_generations(de_handle* h, int64_t n) {
       if (h->fp64_cluster)
         DE_CUDA(h, k_gen_fp64_cluster_launch(h->d_run, h->d_items, h->nitems, h->threads, h->smem_gen, h->variants,
                                              h->suite, h->d_ctl64, g, h->stream, h->slices));
+      else if (h->sliced_loop)
+        DE_CUDA(h, k_gen_sliced_launch(h->d_run, h->d_items, h->nitems, h->nruns, h->d_ctl64, g, h->slices, h->unit,
+                                       h->smem_loop, h->stream, h->test_grid_skip, h->islands ? h->d_isl : nullptr,
+                                       h->islands ? &h->stage : nullptr));
       else
         DE_CUDA(h, k_gen_fp64_persist_launch(h->d_run, h->d_items, h->nitems, h->nruns, h->threads, h->smem_gen,
                                              h->variants, h->suite, h->d_ctl64, g, h->stream, h->slices,
@@ -601,6 +609,7 @@ static bool fp64_persist_ok(const de_handle* h) {
   if (h->prec != DE_PREC_FP64 || h->surr || (h->islands && h->suite) || !h->d_ctl64 || h->nitems >= 4096) return false;
   if (const char* e = getenv("DE_GB300_FP64_PERSIST"))
     if (e[0] == '0') return false;
+  if (h->sliced_loop) return h->nitems <= k_gen_sliced_capacity(h->islands, h->unit, h->smem_loop);
   return h->nitems <= k_gen_fp64_persist_capacity(h->threads, h->smem_gen, h->variants, h->suite, h->slices,
                                                   h->islands);
 }
@@ -1296,6 +1305,16 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
       h->slices = SlicePlan{};
       for (auto& R : h->run) R.sl = nullptr;
     }
+    h->sliced_loop = h->slices.on && !h->variants && !h->suite;
+    int dp_max = 0;
+    for (auto& R : h->run) {
+      // the loop's draws are made before the stop decision, which a debug
+      // capture must not see
+      h->sliced_loop = h->sliced_loop && R.sl && !R.dbg_trial;
+      h->unit = h->unit && R.unit_scale;
+      dp_max = std::max(dp_max, R.dp);
+    }
+    h->smem_loop = sliced_loop_smem(h->slices, dp_max);
   }
   if (h->prec != DE_PREC_FP64) {
     TRY(tc_plan_build(h->tc, h->run, cfgs, h->prec, h->stream, h->err));

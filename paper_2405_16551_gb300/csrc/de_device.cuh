@@ -88,15 +88,11 @@ __device__ __forceinline__ unsigned long long omcos2pi_fix(double z, bool& ok) {
   // the lowest bit of the integer part
   const unsigned long long m = (b & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL;
   const int up = ex - 1074 + 64;  // the fraction is m 2^up modulo 2^64
-  unsigned long long fr = 0ULL;
-  unsigned int odd = 0u;
-  if (up >= 0) {
-    if (up < 64) fr = m << up;
-    const int ib = 64 - up;  // the integer part's lowest bit
-    if (ib >= 0 && ib < 53) odd = (unsigned int)(m >> ib) & 1u;
-  } else if (up > -64) {
-    fr = m >> -up;
-  }
+  // (no branches, so that independent calls interleave)
+  const unsigned long long fl = up < 64 ? m << (up & 63) : 0ULL, fs = up > -64 ? m >> (-up & 63) : 0ULL;
+  const unsigned long long fr = up >= 0 ? fl : fs;
+  const int ib = 64 - up;  // the integer part's lowest bit
+  unsigned int odd = ib >= 0 && ib < 53 ? (unsigned int)(m >> (ib & 63)) & 1u : 0u;
   // the sign of z does not matter; r = fr or fr - 1 (then k is one more)
   odd ^= (unsigned int)(fr >> 63);
   const unsigned long long r = (fr >> 63) ? 0ULL - fr : fr;  // |r| <= 2^63
@@ -123,14 +119,14 @@ __device__ __forceinline__ unsigned long long omcos2pi_fix(double z, bool& ok) {
 // w 2^e rounded to nearest even, on the integer pipe (the conversion
 // instruction occupies the FP64 pipe).
 __device__ __forceinline__ double f64_of_u64(unsigned long long w, int e) {
-  if (w == 0ULL) return 0.0;
-  const int lz = __clzll((long long)w);
-  const unsigned long long n = w << lz;
+  const int lz = __clzll((long long)w);  // 64 for w = 0
+  const unsigned long long n = w << (lz & 63);
   unsigned long long k = n >> 11;
   const unsigned int rem = (unsigned int)n & 0x7FFu;
   k += (rem > 0x400u || (rem == 0x400u && (k & 1ULL))) ? 1ULL : 0ULL;
   // k carries the leading one, which adds 1 to the exponent field
-  return __longlong_as_double((long long)(((unsigned long long)(1023 + 62 - lz + e) << 52) + k));
+  const double r = __longlong_as_double((long long)(((unsigned long long)(1023 + 62 - lz + e) << 52) + k));
+  return w == 0ULL ? 0.0 : r;
 }
 
 // cos(2 pi z) rounded from the fixed-point form.

@@ -521,8 +521,7 @@ static const void* persist_kernel(bool var, bool suite, bool isl, bool tc) {
 // another, so no other kernel that allocates tensor memory may share an SM
 // with them (two such grids, each holding the columns the other waits for,
 // would never finish).
-static size_t persist_smem(const void* k, size_t smem, bool tc) {
-  if (!tc) return smem;
+size_t fp64_exclusive_smem(const void* k, size_t smem) {
   cudaFuncAttributes a{};
   int dev = 0, most = 0;
   if (cudaFuncGetAttributes(&a, k) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
@@ -532,6 +531,8 @@ static size_t persist_smem(const void* k, size_t smem, bool tc) {
   }
   return std::max(smem, (size_t)most - a.sharedSizeBytes);
 }
+
+static size_t persist_smem(const void* k, size_t smem, bool tc) { return tc ? fp64_exclusive_smem(k, smem) : smem; }
 
 void k_configure(size_t smem_gen) {
   const int smem = (int)std::max<size_t>(smem_gen, 1);

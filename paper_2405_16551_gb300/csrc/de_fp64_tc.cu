@@ -204,10 +204,8 @@ __global__ void __launch_bounds__(256, 1)
     }
     __syncthreads();
     if (!sc.cur) slice_load_m(sc, R.sl, kpad);
-    slice_rotate(sc, kpad, R.slx, R.MT, Y, Z, nr, d, dp);
-    __syncthreads();
+    const double f = slice_fitness(sc, R, Y, Z, nr);
     if (warp < nr) {
-      const double f = row_objective_fp64(obj, Z + warp * dp, d, lane);
       if (lane == 0) {
         fout[row0 + warp] = f;
         if (fx_out) fx_out[row0 + warp] = 1;

@@ -136,7 +136,11 @@ __device__ __forceinline__ Best gen_tile(const RunDesc& R, int64_t g, int row0, 
   __syncthreads();
 
   const int nout = nrows * d;
-  if (suite) {
+  double fsl = 0.0;
+  if (sliced) {
+    if (sc->cur != R.sl) slice_load_m(*sc, R.sl, R.sl_kpad);
+    fsl = slice_fitness(*sc, R, Y, Z, nrows);
+  } else if (suite) {
     // ---- the proposed benchmark's functions (Sec. 7.3, Table 2)
     const int ncomp = R.obj >= kObjComposition1 ? R.nc : 1;  // Y and Z hold every component of the tile
     suite_tile<TC>(R, T, dp, nrows, Y, Y + (size_t)ncomp * rows_max * dp, s_fsuite, s_comp, sc);
@@ -151,10 +155,7 @@ __device__ __forceinline__ Best gen_tile(const RunDesc& R, int64_t g, int row0, 
     // ---- rotation, flattened over (row, output): output e = 32 w + lane of
     // warp-group w; a warp takes groups warp, warp + 8, ... and runs up to four
     // of them at once (independent accumulator chains)
-    if (sliced) {
-      if (sc->cur != R.sl) slice_load_m(*sc, R.sl, R.sl_kpad);
-      slice_rotate(*sc, R.sl_kpad, R.slx, R.MT, Y, Z, nrows, d, dp);
-    } else if (R.rotate) {
+    if (R.rotate) {
       const int ngroups = (nout + 31) / 32;
       for (int w0 = warp; w0 < ngroups; w0 += 4 * nwarps) {
         const int qn = min(4, (ngroups - w0 + nwarps - 1) / nwarps);  // uniform in the warp
@@ -204,7 +205,9 @@ __device__ __forceinline__ Best gen_tile(const RunDesc& R, int64_t g, int row0, 
   for (int rl = warp; rl < nrows; rl += nwarps) {
     const int i = row0 + rl;
     double ft;
-    if (suite) {
+    if (sliced) {
+      ft = fsl;
+    } else if (suite) {
       ft = s_fsuite[rl];
     } else if (R.obj == kObjOde) {
       ft = W[rl * dp];

@@ -66,6 +66,17 @@ void k_gen_fp64_tc_launch(const RunDesc* runs, const int4* items, const int2* sh
 void k_eval_rows_tc_launch(const RunDesc* runs, int run, const RunDesc& Rh, const double* x, int64_t ld, int n,
                            double* f, uint8_t* fx, cudaStream_t s);
 void k_tc_configure();
+// Dynamic shared memory that gives a CTA of kernel k a whole SM (at least smem)
+size_t fp64_exclusive_smem(const void* k, size_t smem);
+// the generation loop of plain DE/rand/1/bin runs that are all sliced
+// (de_fp64_sliced.cu); unit: every run's scale is 1
+size_t sliced_loop_smem(const SlicePlan& p, int dp_max);
+int k_gen_sliced_capacity(bool isl, bool unit, size_t smem);
+struct IslandCtl;
+struct IslandStage;
+cudaError_t k_gen_sliced_launch(const RunDesc* runs, const int4* items, int nitems, int nruns, PersistCtl* ctl,
+                                long long gens, const SlicePlan& p, bool unit, size_t smem, cudaStream_t s,
+                                int test_skip, IslandCtl* isl, const IslandStage* stage);
 // the generation loop of FP64 runs in one cooperative launch (every item
 // co-resident: nitems <= k_gen_fp64_persist_capacity; gens <= 2^20)
 // test_skip > 0: the grid-barrier failure test (PersistCtl::test_skip)

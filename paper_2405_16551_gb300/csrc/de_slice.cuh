@@ -15,8 +15,7 @@
 // products of one weight group g = s + t <= 8 stays below 2^24 in size, so
 // its FP32 accumulation in tensor memory is exact:
 //   P_g = sum_k sum_{s + t = g} u_s,k v_t,jk,   z_j = 2^(e + f_j - 76) sum_{g <= 8} 256^(8 - g) P_g
-// with one rounding at the end (H = P_0 .. P_4 and L = P_5 .. P_8 are integers
-// below 2^51; z = fma(H, 2^32, L)).  What is lost: bits of y_k (M_jk) below
+// with one rounding at the end (in integers; the sum is below 2^83).  What is lost: bits of y_k (M_jk) below
 // 2^-63 of the row's largest, and the groups g >= 9, together about 2^-64 of
 // 2^(e + f_j), where a chain of d DFMAs loses about 2^-52 of the products it
 // sums.
@@ -41,11 +40,14 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "de_device.cuh"
 #include "de_tcgen05.cuh"
 
 namespace de {
 
+constexpr int kSliceIssuer = 7;     // the warp that issues the products
 constexpr int kSlices = 8;          // digits per number
 constexpr int kSliceRows = 8;       // rows of y per product
 constexpr int kSliceDMin = 16;
@@ -75,8 +77,19 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0u;
 }
 
+// Its part in static shared memory.
+struct SliceShared {
+  double sum[2][4][kSliceRows];  // per quarter of the outputs and tile row: term sums
+  double edge[4][kSliceRows];    // ... the quarter's first output (Rosenbrock)
+  uint64_t bar;
+  uint32_t tmem, bad;
+  int fail;
+  int exp[kSliceRows];
+};
+
 // One CTA's state of the sliced rotation (the same in every thread).
 struct SliceCtx {
+  SliceShared* sh;
   uint8_t* sB;       // B operand (1024-byte aligned)
   uint8_t* sA;       // slices resident in shared memory
   uint32_t tmem;     // accumulators at column 0, slices from column kSliceAcc on
@@ -121,36 +134,25 @@ __device__ __forceinline__ void slice_load_m(SliceCtx& c, const uint8_t* __restr
 // Allocates tensor memory, sets up the barrier and the zero rows of B; by
 // all threads, before any other use.  kpad: the largest of the matrices this
 // CTA will load (smem holds slice_smem(kpad) bytes), cols: their columns.
-struct SliceShared {
-  uint64_t bar;
-  uint32_t tmem, bad;
-  int fail;
-  int exp[kSliceRows];
-};
-
 __device__ __forceinline__ void slice_begin(SliceCtx& c, uint8_t* smem, int kpad, uint32_t cols, SliceShared& sh) {
-  uint32_t* s_tmem = &sh.tmem;
-  uint64_t* s_bar = &sh.bar;
-  int* s_exp = sh.exp;
-  uint32_t* s_bad = &sh.bad;
-  int* s_fail = &sh.fail;
+  c.sh = &sh;
   c.cols = cols;
   c.sB = smem;
   c.sA = smem + slice_b_bytes(kpad);
-  c.bar = smem_u32(s_bar);
+  c.bar = smem_u32(&sh.bar);
   c.phase = 0;
-  c.s_exp = s_exp;
-  c.s_bad = s_bad;
-  c.s_fail = s_fail;
+  c.s_exp = sh.exp;
+  c.s_bad = &sh.bad;
+  c.s_fail = &sh.fail;
   c.cur = nullptr;
   if (threadIdx.x == 0) {
     mbar_init(c.bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    *s_bad = 0u;
-    *s_fail = 0;
+    sh.bad = 0u;
+    sh.fail = 0;
   }
   if (threadIdx.x < 32) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)),
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem)),
                  "r"(cols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
@@ -160,7 +162,7 @@ __device__ __forceinline__ void slice_begin(SliceCtx& c, uint8_t* smem, int kpad
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  c.tmem = *s_tmem;
+  c.tmem = sh.tmem;
 }
 
 // Waits (bounded) for products still in flight after a failed wait, then
@@ -233,17 +235,12 @@ __device__ __forceinline__ void slice_digits(const SliceCtx& c, int r, int lane,
   }
 }
 
-// The products of the tile's digits with the loaded matrix, then z into
-// Z[r][j] (row stride dp) for the tile's nrows rows; by all threads of the
-// CTA, after a CTA barrier that follows the digits.  fexp: f_j per output.
-// The caller's CTA barrier makes Z visible.  Y: the FP64 rows (stride dp), for
-// rows that take the DFMA chain over MT.
-__device__ __forceinline__ void slice_rotate(SliceCtx& c, int kpad, const int32_t* __restrict__ fexp,
-                                             const double* __restrict__ MT, const double* __restrict__ Y,
-                                             double* __restrict__ Z, int nrows, int d, int dp) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-  if (warp == 0) {
+// Issues the products of the tile's digits with the loaded matrix and waits
+// for them; by all threads, after a CTA barrier that follows the digits.
+__device__ __forceinline__ void slice_products(SliceCtx& c, int kpad) {
+  const int lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
+  if (warp == kSliceIssuer) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const int nsm = slice_nsm(kpad), ksteps = kpad / 16;
     const uint32_t sbytes = slice_bytes(kpad);
@@ -280,50 +277,86 @@ __device__ __forceinline__ void slice_rotate(SliceCtx& c, int kpad, const int32_
   c.phase ^= 1u;
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  // warp w: outputs 32 (w mod 4) .. + 31 (lanes), tile rows 4 (w / 4) .. + 3
-  const int q4 = warp & 3, r0 = 4 * (warp >> 2), j = 32 * q4 + lane;
-  if (r0 < nrows && 32 * q4 < d) {
-    float p[9][4];
+}
+
+// The tile rows of warp w's threads: rows slice_row0 .. + slice_nrow - 1 (the
+// two halves of the warps share the tile's rows evenly), outputs
+// 32 (w mod 4) + lane.
+__device__ __forceinline__ int slice_row0(int warp, int nrows) { return (warp >> 2) * ((nrows + 1) >> 1); }
+__device__ __forceinline__ int slice_nrow(int warp, int nrows) {
+  return warp < 4 ? (nrows + 1) >> 1 : nrows >> 1;
+}
+
+// sum_g 256^(8 - g) P_g 2^sc rounded once to FP64, in integers (three FP64
+// operations would take 192 cycles of the FP64 pipe a warp and row).
+__device__ __forceinline__ double slice_combine(const float (&p)[9], int sc) {
+  int P[9];
+#pragma unroll
+  for (int g = 0; g < 9; ++g) P[g] = __float2int_rn(p[g]);
+  const int a = P[0] * 256 + P[1], b = P[2] * 256 + P[3];
+  const long long H = (long long)a * 16777216LL + ((long long)b * 256LL + P[4]);
+  const long long L = ((long long)P[5] * 256LL + P[6]) * 65536LL + ((long long)P[7] * 256LL + P[8]);
+  // T = H 2^32 + L, |T| < 2^83, as sign and magnitude (hi, lo); no branches,
+  // so that a thread's rows run interleaved
+  unsigned long long lo = ((unsigned long long)H << 32) + (unsigned long long)L;
+  unsigned long long hi = (unsigned long long)((H >> 32) + (L >> 63) + (lo < (unsigned long long)L ? 1LL : 0LL));
+  const bool neg = (long long)hi < 0;
+  const unsigned long long m = neg ? ~0ULL : 0ULL;
+  lo = (lo ^ m) + (neg ? 1ULL : 0ULL);
+  hi = (hi ^ m) + (neg && lo == 0ULL ? 1ULL : 0ULL);
+  // the leading 64 bits, with everything below as one sticky bit
+  const bool wide = hi != 0ULL;
+  const unsigned long long h2 = wide ? hi : lo, l2 = wide ? lo : 0ULL;
+  const int lz = __clzll((long long)h2);  // 64 for T = 0
+  const unsigned long long n = (h2 << (lz & 63)) | ((l2 >> 1) >> (63 - (lz & 63)));
+  const unsigned long long rest = l2 << (lz & 63);
+  unsigned long long k = n >> 11;
+  const unsigned int rem = ((unsigned int)n & 0x7FFu) | (rest ? 1u : 0u);
+  k += (rem > 0x400u || (rem == 0x400u && (k & 1ULL))) ? 1ULL : 0ULL;
+  const long long e = 1023 + 126 - 64 - lz + (wide ? 64 : 0) + sc;
+  const double z = __longlong_as_double((long long)(((unsigned long long)e << 52) + k) | (neg ? (long long)0x8000000000000000ULL : 0LL));
+  return h2 == 0ULL ? 0.0 : z;
+}
+
+// z of this thread's output and rows from the accumulators (after
+// slice_products); rows past the tile and outputs past d give 0.  A row that
+// takes the DFMA chain is computed over MT from Y (FP64 rows of stride dp)
+// into Zf (as Y).
+__device__ __forceinline__ void slice_z(SliceCtx& c, const int32_t* __restrict__ fexp, const double* __restrict__ MT,
+                                        const double* __restrict__ Y, double* __restrict__ Zf, int nrows, int d, int dp,
+                                        double (&z)[4]) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int q4 = warp & 3, r0 = slice_row0(warp, nrows), nr = slice_nrow(warp, nrows), j = 32 * q4 + lane;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) z[e] = 0.0;
+  if (nr > 0 && 32 * q4 < d) {
+    uint32_t v[9][4];
     const uint32_t ta = c.tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)r0;
 #pragma unroll
-    for (int g = 0; g < 9; ++g) {
-      uint32_t v[4];
+    for (int g = 0; g < 9; ++g)
       asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                   : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                   : "=r"(v[g][0]), "=r"(v[g][1]), "=r"(v[g][2]), "=r"(v[g][3])
                    : "r"(ta + 8u * (uint32_t)g));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    // the values are used only after the wait
 #pragma unroll
-      for (int e = 0; e < 4; ++e) p[g][e] = __uint_as_float(v[e]);
-    }
-    // the values are used only after the wait (the operands tie them to it)
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+f"(p[0][0]), "+f"(p[0][1]), "+f"(p[0][2]), "+f"(p[0][3]), "+f"(p[1][0]), "+f"(p[1][1]),
-                   "+f"(p[1][2]), "+f"(p[1][3]), "+f"(p[2][0]), "+f"(p[2][1]), "+f"(p[2][2]), "+f"(p[2][3]),
-                   "+f"(p[3][0]), "+f"(p[3][1]), "+f"(p[3][2]), "+f"(p[3][3])::"memory");
-    asm volatile(""
-                 : "+f"(p[4][0]), "+f"(p[4][1]), "+f"(p[4][2]), "+f"(p[4][3]), "+f"(p[5][0]), "+f"(p[5][1]),
-                   "+f"(p[5][2]), "+f"(p[5][3]), "+f"(p[6][0]), "+f"(p[6][1]), "+f"(p[6][2]), "+f"(p[6][3]),
-                   "+f"(p[7][0]), "+f"(p[7][1]), "+f"(p[7][2]), "+f"(p[7][3]), "+f"(p[8][0]), "+f"(p[8][1]),
-                   "+f"(p[8][2]), "+f"(p[8][3])::"memory");
+    for (int g = 0; g < 9; ++g)
+      asm volatile("" : "+r"(v[g][0]), "+r"(v[g][1]), "+r"(v[g][2]), "+r"(v[g][3]));
     const int fj = j < d ? __ldg(fexp + j) : 0;
+    // rows past the tile (at most one here) are computed and dropped
+    auto rows = [&](auto count) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      if (r0 + e < nrows) {
-        int P[9];
+      for (int e = 0; e < decltype(count)::value; ++e) {
+        float p[9];
 #pragma unroll
-        for (int g = 0; g < 9; ++g) P[g] = __float2int_rn(p[g][e]);
-        const int a = P[0] * 256 + P[1], b = P[2] * 256 + P[3];
-        const long long H = (long long)a * 16777216LL + ((long long)b * 256LL + P[4]);
-        const long long L = ((long long)P[5] * 256LL + P[6]) * 65536LL + ((long long)P[7] * 256LL + P[8]);
-        // |H|, |L| < 2^51: exact in the significand of 1.5 2^52 + n
-        const double C = 6755399441055744.0;
-        const double h = __dsub_rn(__longlong_as_double(H + 0x4338000000000000LL), C);
-        const double l = __dsub_rn(__longlong_as_double(L + 0x4338000000000000LL), C);
-        const double z = __fma_rn(h, 4294967296.0, l);
-        // times 2^(e + f_j - 76), on the exponent field (z is 0 or normal)
-        const int hz = __double2hiint(z), sc = (c.s_exp[r0 + e] + fj - 76) * 1048576;
-        if (j < d) Z[(r0 + e) * dp + j] = __hiloint2double((hz & 0x7FF00000) ? hz + sc : hz, __double2loint(z));
+        for (int g = 0; g < 9; ++g) p[g] = __uint_as_float(v[g][e]);
+        const double ze = slice_combine(p, c.s_exp[min(r0 + e, kSliceRows - 1)] + fj - 76);
+        z[e] = j < d && e < nr ? ze : 0.0;
       }
-    }
+    };
+    if (nr > 2) rows(std::integral_constant<int, 4>{});
+    else rows(std::integral_constant<int, 2>{});
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   const uint32_t bad = *c.s_bad;
@@ -336,9 +369,114 @@ __device__ __forceinline__ void slice_rotate(SliceCtx& c, int kpad, const int32_
       if (!((bad >> r) & 1u)) continue;
       double s = 0.0;
       for (int k = 0; k < d; ++k) s = fma(__ldg(MT + (size_t)k * d + jj), Y[r * dp + k], s);
-      Z[r * dp + jj] = s;
+      Zf[r * dp + jj] = s;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (e < nr && j < d && ((bad >> (r0 + e)) & 1u)) z[e] = Zf[(r0 + e) * dp + j];
+  }
+}
+
+// z into Z[r][j] (row stride dp) for the tile's rows.  The caller's CTA
+// barrier makes Z visible.
+__device__ __forceinline__ void slice_rotate(SliceCtx& c, int kpad, const int32_t* __restrict__ fexp,
+                                             const double* __restrict__ MT, const double* __restrict__ Y,
+                                             double* __restrict__ Z, int nrows, int d, int dp) {
+  const int warp = threadIdx.x >> 5, j = 32 * (warp & 3) + (threadIdx.x & 31);
+  slice_products(c, kpad);
+  double z[4];
+  slice_z(c, fexp, MT, Y, Z, nrows, d, dp, z);
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    if (e < slice_nrow(warp, nrows) && j < d) Z[(slice_row0(warp, nrows) + e) * dp + j] = z[e];
+}
+
+// Sums of 4 rows' values over the lanes of a warp: 6 FP64 additions (the lanes
+// of bit 16, then of bit 8, keep half of the rows each) instead of 20.  The lanes of
+// (bit 16, bit 8) return the sum of row 2 (bit 16) + (bit 8); a row's order of
+// additions does not depend on its place.
+__device__ __forceinline__ double slice_sum4(const double (&v)[4], int lane) {
+  const bool h = lane & 16, g = lane & 8;
+  const double b0 = h ? v[0] : v[2], b1 = h ? v[1] : v[3];
+  const double a0 = (h ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, b0, 16);
+  const double a1 = (h ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, b1, 16);
+  double s = (g ? a1 : a0) + __shfl_xor_sync(0xffffffffu, g ? a0 : a1, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// Fitness of the tile's rows (objectives 0 .. 3), after a CTA barrier that
+// follows the digits: products, z in registers, the objective's terms in the
+// thread that holds z, sums over lanes and then over the four quarters of
+// the outputs.  Warp r < nrows returns the fitness of row r (every lane).
+__device__ __forceinline__ double slice_fitness(SliceCtx& c, const RunDesc& R, const double* __restrict__ Y,
+                                                double* __restrict__ Zf, int nrows) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q4 = warp & 3;
+  const int d = R.d, dp = R.dp, obj = R.obj, j = 32 * q4 + lane;
+  const int r0 = slice_row0(warp, nrows), nr = slice_nrow(warp, nrows);
+  slice_products(c, R.sl_kpad);
+  double z[4], t[4], u[4];
+  slice_z(c, R.slx, R.MT, Y, Zf, nrows, d, dp, z);
+  if (obj == kObjRosenbrock) {
+    // the next quarter's first output
+    if (lane == 0) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (e < nr) c.sh->edge[q4][r0 + e] = z[e];
+    }
+    __syncthreads();
+  }
+  if (nr > 0 && 32 * q4 < d) {
+    const int srow = ((lane >> 4) & 1) * 2 + ((lane >> 3) & 1);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) t[e] = u[e] = 0.0;
+    // z is 0 past the tile's rows and past d, where every term but
+    // Rosenbrock's is 0 (Ackley's cosine is masked)
+    auto terms = [&](auto count) {
+      constexpr int N = decltype(count)::value;
+      if (obj == kObjRosenbrock) {
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+          double zn = __shfl_down_sync(0xffffffffu, z[e], 1);
+          if (lane == 31 && q4 < 3 && e < nr) zn = c.sh->edge[q4 + 1][r0 + e];
+          const double t0 = z[e] + 1.0, tn = zn + 1.0;
+          const double a = tn - t0 * t0, b = t0 - 1.0;
+          t[e] = e < nr && j + 1 < d ? 100.0 * a * a + b * b : 0.0;
+        }
+      } else if (obj == kObjRastrigin) {
+#pragma unroll
+        for (int e = 0; e < N; ++e) t[e] = fma(z[e], z[e], rastrigin_w(z[e]));
+      } else {
+#pragma unroll
+        for (int e = 0; e < N; ++e) t[e] = z[e] * z[e];
+        if (obj == kObjAckley) {
+#pragma unroll
+          for (int e = 0; e < N; ++e) {
+            const double w = cos2pi_fix(z[e]);
+            u[e] = e < nr && j < d ? w : 0.0;
+          }
+        }
+      }
+    };
+    if (nr > 2) terms(std::integral_constant<int, 4>{});
+    else terms(std::integral_constant<int, 2>{});
+    const double s = slice_sum4(t, lane);
+    if ((lane & 7) == 0 && srow < nr) c.sh->sum[0][q4][r0 + srow] = s;
+    if (obj == kObjAckley) {
+      const double s2 = slice_sum4(u, lane);
+      if ((lane & 7) == 0 && srow < nr) c.sh->sum[1][q4][r0 + srow] = s2;
     }
   }
+  __syncthreads();
+  if (warp >= nrows) return 0.0;
+  double s1 = c.sh->sum[0][0][warp];
+  for (int q = 1; 32 * q < d; ++q) s1 += c.sh->sum[0][q][warp];
+  if (obj != kObjAckley) return s1;
+  double s2 = c.sh->sum[1][0][warp];
+  for (int q = 1; 32 * q < d; ++q) s2 += c.sh->sum[1][q][warp];
+  return 20.0 + 2.718281828459045 - 20.0 * exp(-0.2 * sqrt(s1 / d)) - exp(s2 / d);
 }
 
 }  // namespace de
