@@ -76,6 +76,7 @@ struct de_handle {
   // run_id, precision, strategy, jDE, FP64 band policy, shift, rotation and
   // permutation), written to checkpoints and checked by de_load
   std::vector<uint64_t> fingerprint;
+  std::vector<bool> ode_ref_done;  // per run: the ODE objective's reference trajectory is in place
   std::string err;
 };
 
@@ -459,7 +460,11 @@ static de_status init_run(de_handle* h, int r) {
   st.evals = R.np;  // the initial population counts as NP evaluations
   DE_CUDA(h, cudaMemcpyAsync(R.st, &st, sizeof st, cudaMemcpyHostToDevice, h->stream));
   DE_CUDA(h, cudaMemsetAsync(R.X[0], 0, (size_t)R.np * R.dp * sizeof(double), h->stream));
-  if (R.obj == DE_OBJ_ODE) k_ode_reference_launch(h->d_run, r, const_cast<double*>(R.ode_ref), h->stream);
+  if (R.obj == DE_OBJ_ODE && !h->ode_ref_done[r]) {
+    // the hidden vector's trajectory depends on the run's shift only
+    k_ode_reference_launch(h->d_run, r, const_cast<double*>(R.ode_ref), h->stream);
+    h->ode_ref_done[r] = true;
+  }
   k_init_population_launch(h->d_run, r, R.np, R.dp, h->stream);
   if (R.jde) k_jde_init_launch(h->d_run, r, R.np, h->stream);
   if (h->prec == DE_PREC_FP64) {
@@ -1071,6 +1076,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
     c.perm = nullptr;
   }
   h->run.resize(nruns);
+  h->ode_ref_done.assign(nruns, false);
 
   // ---- arena layout
   size_t off = 0;
