@@ -13,13 +13,18 @@
 //                   output dot product in the TMEM epilogues
 //   k_mlp_pass<true>   one training step's forward and backward pass for one
 //                   128-row half of a 256-row minibatch: dZ2 = dy w3 relu',
-//                   dH1 = dZ2 W2 on the tensor cores, dZ1 = dH1 relu'; writes
-//                   the transposed operands of the weight gradients
-//   k_mlp_wgrad     weight gradients as products over the batch
-//                   (dW2 = dZ2^T H1 with a ones row for db2, dW1 = dZ1^T A1)
-//                   into the raw gradient vector
-//   k_mlp_adam      Adam on every FP32 master (one thread per parameter,
-//                   coalesced) and the BF16 operand copies of W1 | b1 and W2
+//                   dH1 = dZ2 W2 on the tensor cores, dZ1 = dH1 relu'; stores
+//                   H1, dZ2, dZ1 and the inputs as they are
+//   k_mlp_update    weight gradients as products over the batch
+//                   (dW2 = dZ2^T H1 with a ones row for db2, dW1 = dZ1^T A1),
+//                   each tile's Adam step on the FP32 masters, and the BF16
+//                   operand copies of W1 | b1 and W2
+//
+// A training step is a chain of latencies, not of work (3 GFLOP a step).  What
+// it cost before (48.5 + 11.4 + 3.7 us in three kernels): transposed 2-byte
+// stores of three activations, a 5-step shuffle sum per column of dw3, a second
+// copy of W2, FP64 conversions; now the weight gradients read the stored tiles
+// MN-major, and a step is two kernels chained by programmatic launches.
 //
 // Operand layout in shared and global memory: the canonical K-major, no
 // swizzle layout of de_tcgen05.cuh (core matrices of 8 rows x 16 bytes).
@@ -51,6 +56,14 @@ __device__ __forceinline__ uint32_t toff(int row, int k, int RG) {
 __device__ __forceinline__ uint32_t idesc_bf16(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
 }
+
+// A tile of RG row groups read the other way round: its columns as the rows of
+// the operand (M or N) and its rows as K ("MN-major": a core matrix holds 8
+// columns of 8 rows, the columns contiguous).  So the transposed products need
+// no transposed copy.  Byte strides: between 8-column groups RG * 128, between
+// 8-row groups 128.
+__device__ __forceinline__ uint64_t desc_mn(uint32_t addr, int rg) { return smem_desc(addr, 128u, (uint32_t)rg * 128u); }
+constexpr uint32_t kAMn = 1u << 15, kBMn = 1u << 16;  // instruction descriptor: A / B is MN-major
 
 // D (TMEM) = or += A (M = 128, K = 16 ksteps) B^T (N rows); A and B K-major
 // with RGa / RGb row groups.
@@ -103,8 +116,8 @@ __device__ __forceinline__ int batch_row(const MlpStepArgs& a, int m) {
 
 // ------------------------------------------------------------------ forward / backward
 // Shared memory of k_mlp_pass (dynamic, 1024-aligned).
-constexpr uint32_t kSBig = 0;                 // 128 KB: W2k; later dZ2 (A) + W2t half 0
-constexpr uint32_t kSH1 = 131072;             // 64 KB: H1 (A operand of layer 2); later W2t half 1
+constexpr uint32_t kSBig = 0;                 // 128 KB: W2k (layer 2, and read MN-major for dH1)
+constexpr uint32_t kSH1 = 131072;             // 64 KB: H1 (A operand of layer 2); later dZ2 (A operand of dH1)
 constexpr uint32_t kSW1 = 196608;             // 16 KB: W1k
 constexpr uint32_t kSA1 = 212992;             // 8 KB: A1 (inputs)
 constexpr uint32_t kMlpSmem = 221184;
@@ -116,10 +129,11 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
                                                      int64_t ld, int n, const float* __restrict__ t,
                                                      float* __restrict__ yout) {
   extern __shared__ __align__(1024) uint8_t smem[];
-  __shared__ __align__(8) uint64_t bars[3];  // weights, mma, W2t
+  __shared__ __align__(8) uint64_t bars[2];  // weights, mma
   __shared__ uint32_t s_tmem;
   __shared__ float s_y[2][kTileM];
   __shared__ float s_t[kTileM];
+  __shared__ float s_b2[kMlpH], s_w3[kMlpH];
   __shared__ float s_dw3[4][kMlpH];
   __shared__ float s_red[8][2];
   __shared__ int s_err;
@@ -128,19 +142,18 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
   const int m = 32 * q + lane;                 // tile row of this thread in the epilogues
   const int row0 = blockIdx.x * kTileM;
   const uint32_t sb = smem_u32(smem);
-  const uint32_t b_w = smem_u32(&bars[0]), b_mma = smem_u32(&bars[1]), b_w2t = smem_u32(&bars[2]);
+  const uint32_t b_w = smem_u32(&bars[0]), b_mma = smem_u32(&bars[1]);
 
   if (tid == 0) {
-    for (int k = 0; k < 3; ++k) mbar_init(smem_u32(&bars[k]), 1);
+    for (int k = 0; k < 2; ++k) mbar_init(smem_u32(&bars[k]), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_err = 0;
-    mbar_expect_tx(b_w, kMlpW1Bytes + kMlpW2Bytes);
-    bulk_g2s(sb + kSW1, P.w1k, kMlpW1Bytes, b_w);
-    bulk_g2s(sb + kSBig, P.w2k, kMlpW2Bytes, b_w);
   }
   if (warp == 0) tmem_alloc(&s_tmem, 512);
 
-  // ---- inputs: A1 row = (x / 100, 1, 0 ...) in bf16; two threads per row
+  // ---- inputs: A1 row = (x / 100, 1, 0 ...) in bf16; two threads per row.
+  // They do not depend on the weights: a training step reads them before it
+  // waits for the step before.
   {
     const int r = tid >> 1, half = tid & 1;
     const int grow = row0 + r;
@@ -153,20 +166,31 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
       const int col = 16 * half + c;
       float val = 0.f;
       if (src >= 0) {
-        if (col < kMlpIn) val = (float)(x[(size_t)src * ld + col] * 0.01);
+        if (col < kMlpIn) val = to_f32_rn(x[(size_t)src * ld + col] * 0.01);
         else if (col == kMlpIn) val = 1.f;
       }
       v[c] = val;
     }
     st_bf16x8(smem + kSA1, r, 16 * half, 16, v);
     st_bf16x8(smem + kSA1, r, 16 * half + 8, 16, v + 8);
+    if (TRAIN && half == 0) s_t[r] = src >= 0 ? t[src] : 0.f;
     if (TRAIN) {
-      // A1^T (32 x 256 batch, 4 row groups) for the W1 gradient
-#pragma unroll
-      for (int c = 0; c < 16; ++c) st_bf16(P.a1t, toff(16 * half + c, grow, 4), v[c]);
-      if (half == 0) s_t[r] = src >= 0 ? t[src] : 0.f;
+      pdl_wait();
+      // (after the wait: the update before this step no longer reads it)
+      st_bf16x8(P.a1 + (size_t)blockIdx.x * kMlpA1Bytes, r, 16 * half, 16, v);
+      st_bf16x8(P.a1 + (size_t)blockIdx.x * kMlpA1Bytes, r, 16 * half + 8, 16, v + 8);
+      pdl_launch_dependents();
     }
   }
+  if (tid == 0) {
+    // the operands were written by ordinary stores of the kernel before
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    mbar_expect_tx(b_w, kMlpW1Bytes + kMlpW2Bytes);
+    bulk_g2s(sb + kSW1, P.w1k, kMlpW1Bytes, b_w);
+    bulk_g2s(sb + kSBig, P.w2k, kMlpW2Bytes, b_w);
+  }
+  s_b2[tid] = P.b2[tid];
+  s_w3[tid] = P.w3[tid];
   fence_async_smem();
   tc_before_sync();
   __syncthreads();
@@ -187,7 +211,7 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
   tc_after_sync();
 
   // ---- epilogue 1: H1 = relu(Z1) to shared memory (A operand of layer 2);
-  // training: its transpose to global memory and the ReLU mask in registers
+  // training: also to global memory, and the ReLU mask in registers
   uint32_t mask[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
@@ -202,10 +226,9 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
     }
     mask[j] = mk;
 #pragma unroll
-    for (int e = 0; e < 32; e += 8) st_bf16x8(smem + kSH1, m, c0 + e, 16, v + e);
-    if (TRAIN) {
-#pragma unroll
-      for (int e = 0; e < 32; ++e) st_bf16(P.h1t, toff(c0 + e, row0 + m, 32), v[e]);
+    for (int e = 0; e < 32; e += 8) {
+      st_bf16x8(smem + kSH1, m, c0 + e, 16, v + e);
+      if (TRAIN) st_bf16x8(P.h1 + (size_t)blockIdx.x * kMlpActBytes, m, c0 + e, 16, v + e);
     }
   }
   fence_async_smem();
@@ -220,13 +243,6 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
   }
   if (!mbar_wait(b_mma, 1)) s_err = 1;
   tc_after_sync();
-  if (TRAIN && tid == 0) {
-    // W2k and H1 are consumed: stage W2^T (two 128-row halves) for dH1
-    mbar_expect_tx(b_w2t, kMlpW2Bytes);
-    bulk_g2s(sb + kSBig + 65536, P.w2t, kMlpW2Bytes / 2, b_w2t);
-    bulk_g2s(sb + kSH1, P.w2t + kMlpW2Bytes / 2, kMlpW2Bytes / 2, b_w2t);
-  }
-
   // ---- epilogue 2: y = w3 . relu(Z2 + b2) + b3
   float yp = 0.f;
 #pragma unroll
@@ -235,7 +251,7 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
     float v[32];
     tmem_ld_cols32(tmem + lane_base + 256u + (uint32_t)c0, v);
 #pragma unroll
-    for (int e = 0; e < 32; ++e) yp = fmaf(fmaxf(v[e] + P.b2[c0 + e], 0.f), P.w3[c0 + e], yp);
+    for (int e = 0; e < 32; ++e) yp = fmaf(fmaxf(v[e] + s_b2[c0 + e], 0.f), s_w3[c0 + e], yp);
   }
   s_y[h][m] = yp;
   __syncthreads();
@@ -246,25 +262,37 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
     // mean squared error over the 256-row minibatch
     const float r = y - s_t[m];
     const float dy = 2.f * r / (float)kMlpBatch;
-    // dZ2 = dy w3 relu'(Z2 + b2): A operand of dH1 (shared) and, transposed,
-    // of dW2 (global); dw3 = sum over rows of H2 dy
+    // dZ2 = dy w3 relu'(Z2 + b2): A operand of dH1 (in H1's place, which
+    // layer 2 has consumed) and of dW2 (global); dw3 = sum over rows of H2 dy
+#pragma unroll 1
     for (int j = 0; j < 4; ++j) {
       const int c0 = 128 * h + 32 * j;
       float v[32], dz[32];
       tmem_ld_cols32(tmem + lane_base + 256u + (uint32_t)c0, v);
 #pragma unroll
       for (int e = 0; e < 32; ++e) {
-        const float zb = v[e] + P.b2[c0 + e];
-        const float h2 = fmaxf(zb, 0.f);
-        dz[e] = zb > 0.f ? dy * P.w3[c0 + e] : 0.f;
-        float s = h2 * dy;  // row contribution to dw3[c0 + e]
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) s_dw3[q][c0 + e] = s;
-        st_bf16(P.dz2t + (size_t)((c0 + e) >> 7) * (kMlpW2Bytes / 2), toff((c0 + e) & 127, row0 + m, 16), dz[e]);
+        const float zb = v[e] + s_b2[c0 + e];
+        dz[e] = zb > 0.f ? dy * s_w3[c0 + e] : 0.f;
+        v[e] = fmaxf(zb, 0.f) * dy;  // row contribution to dw3[c0 + e]
       }
 #pragma unroll
-      for (int e = 0; e < 32; e += 8) st_bf16x8(smem + kSBig, m, c0 + e, 16, dz + e);
+      for (int e = 0; e < 32; e += 8) {
+        st_bf16x8(smem + kSH1, m, c0 + e, 16, dz + e);
+        st_bf16x8(P.dz2 + (size_t)blockIdx.x * kMlpActBytes, m, c0 + e, 16, dz + e);
+      }
+      // sums over the 32 rows of all 32 columns: at each step a lane keeps the
+      // columns whose index agrees with it in one bit, so 31 additions do
+      // (the pairs added are those of the xor tree)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int e = 0; e < o; ++e) {
+          const float keep = up ? v[e + o] : v[e], give = up ? v[e] : v[e + o];
+          v[e] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+      }
+      s_dw3[q][c0 + lane] = v[0];
     }
     // loss and db3 partials of this half
     float rs = r * r, ds = dy;
@@ -291,30 +319,27 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
       P.part[blockIdx.x * kMlpPart + kMlpH + 1] = ((s_red[0][0] + s_red[1][0]) + s_red[2][0]) + s_red[3][0];
     }
 
-    // ---- dH1 = dZ2 W2: A = dZ2 (shared), B = W2^T halves -> TMEM [0, 256)
+    // ---- dH1 = dZ2 W2: A = dZ2 (shared), B = W2 read MN-major -> TMEM [0, 256)
     if (tid == 0) {
-      if (!mbar_wait(b_w2t, 0)) s_err = 1;
-      else {
-        tc_after_sync();
-        mma_bf16(tmem, sb + kSBig, 16, sb + kSBig + 65536, 16, 16, 128, false);
-        mma_bf16(tmem + 128, sb + kSBig, 16, sb + kSH1, 16, 16, 128, false);
-      }
+      const uint32_t id = idesc_bf16(kMlpH) | kBMn;
+      for (int ks = 0; ks < 16; ++ks)
+        mma_split<2>(tmem, smem_desc(sb + kSH1 + (uint32_t)ks * 4096u, 2048u, 128u),
+                     desc_mn(sb + kSBig + (uint32_t)ks * 256u, 32), id, ks > 0 ? 1u : 0u);
       mma_commit(b_mma);
     }
     if (!mbar_wait(b_mma, 0)) s_err = 1;
     tc_after_sync();
 
-    // ---- epilogue 3: dZ1 = dH1 relu'(Z1), transposed to global memory
+    // ---- epilogue 3: dZ1 = dH1 relu'(Z1) to global memory
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int c0 = 128 * h + 32 * j;
       float v[32];
       tmem_ld_cols32(tmem + lane_base + (uint32_t)c0, v);
 #pragma unroll
-      for (int e = 0; e < 32; ++e) {
-        const float g = ((mask[j] >> e) & 1u) ? v[e] : 0.f;
-        st_bf16(P.dz1t + (size_t)((c0 + e) >> 7) * (kMlpW2Bytes / 2), toff((c0 + e) & 127, row0 + m, 16), g);
-      }
+      for (int e = 0; e < 32; ++e) v[e] = ((mask[j] >> e) & 1u) ? v[e] : 0.f;
+#pragma unroll
+      for (int e = 0; e < 32; e += 8) st_bf16x8(P.dz1 + (size_t)blockIdx.x * kMlpActBytes, m, c0 + e, 16, v + e);
     }
   }
   tc_before_sync();
@@ -337,9 +362,17 @@ __device__ __forceinline__ float adam_step(float w, float g, float* m, float* v,
   return w - A.lr * (mn / A.c1) / (sqrtf(vn / A.c2) + A.eps);
 }
 
-// Raw weight gradients of one step into P.grad.  Blocks 0, 1: rows
-// [128 b, 128 b + 128) of W2 and b2; block 2: W1, b1, w3, b3 and the loss.
-__global__ void __launch_bounds__(256, 1) k_mlp_wgrad(MlpDev P) {
+// Weight gradients of one step and their Adam update (apply = 0: into P.grad
+// only).  Blocks 0 .. 15: rows 128 (b / 8) .. + 127 of W2, columns 32 (b mod 8)
+// .. + 31 (the first column block also b2); blocks 16, 17: 128 rows of W1 and b1
+// (block 16 also w3, b3 and the loss).  The products leave a tile of 128 x 32
+// gradients in shared memory, from which each thread updates 8 consecutive
+// parameters at a time: coalesced masters and moments, 16-byte operand stores.
+constexpr uint32_t kUpA = 0, kUpB = 65536, kUpOnes = kUpB + 16384, kUpG = kUpOnes + 8192;
+constexpr int kUpStride = 36;  // floats per row of the gradient tile (16-byte rows, spread over the banks)
+constexpr uint32_t kUpSmem = kUpG + 128u * kUpStride * 4u;
+
+__global__ void __launch_bounds__(256, 1) k_mlp_update(MlpDev P, AdamArgs A, int apply) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ uint32_t s_tmem;
@@ -348,32 +381,39 @@ __global__ void __launch_bounds__(256, 1) k_mlp_wgrad(MlpDev P) {
   const int q = warp & 3, h = warp >> 2;
   const uint32_t sb = smem_u32(smem);
   const uint32_t b_ld = smem_u32(&bars[0]), b_mma = smem_u32(&bars[1]);
-  const bool w2 = blockIdx.x < 2;
-  const uint32_t ncols = w2 ? 512u : 64u;
+  const bool w2 = blockIdx.x < 16;
+  const int ob = w2 ? blockIdx.x >> 3 : blockIdx.x - 16, ig = w2 ? blockIdx.x & 7 : 0;
+  const bool bias = w2 && ig == 0;
+  float* gt = reinterpret_cast<float*>(smem + kUpG);
   if (tid == 0) {
     mbar_init(b_ld, 1);
     mbar_init(b_mma, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_err = 0;
-    if (w2) {
-      mbar_expect_tx(b_ld, kMlpW2Bytes / 2 + kMlpW2Bytes);
-      bulk_g2s(sb, P.dz2t + (size_t)blockIdx.x * (kMlpW2Bytes / 2), kMlpW2Bytes / 2, b_ld);
-      bulk_g2s(sb + 65536, P.h1t, kMlpW2Bytes, b_ld);
-    } else {
-      mbar_expect_tx(b_ld, kMlpW2Bytes + kMlpA1tBytes);
-      bulk_g2s(sb, P.dz1t, kMlpW2Bytes, b_ld);
-      bulk_g2s(sb + 131072, P.a1t, kMlpA1tBytes, b_ld);
+  }
+  if (warp == 0) tmem_alloc(&s_tmem, 64);
+  if (bias) {
+    // a ones row (row 0 of a 16-row operand): the sum over the batch, i.e. the
+    // gradient of b2
+    for (int e = tid; e < 16 * kMlpBatch / 8; e += blockDim.x) {
+      const int r = e & 15, k8 = e >> 4;
+      const uint32_t one = r == 0 ? 0x3F803F80u : 0u;
+      *reinterpret_cast<uint4*>(smem + kUpOnes + toff(r, 8 * k8, 2)) = make_uint4(one, one, one, one);
     }
   }
-  if (w2) {
-    // a ones row (row 0 of a 16-row operand) so that column 256 of the
-    // product is the sum over the batch, i.e. the gradient of b2
-    for (int e = tid; e < 16 * kMlpBatch; e += blockDim.x) {
-      const int r = e / kMlpBatch, k = e % kMlpBatch;
-      st_bf16(smem + 196608, toff(r, k, 2), r == 0 ? 1.f : 0.f);
+  // the next step's kernel may start (its inputs do not depend on this one)
+  pdl_launch_dependents();
+  pdl_wait();
+  if (tid == 0) {
+    const uint8_t *sa = w2 ? P.dz2 : P.dz1, *sbm = w2 ? P.h1 : P.a1;
+    const size_t bh = w2 ? kMlpActBytes : kMlpA1Bytes;  // bytes of one half of the batch
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    mbar_expect_tx(b_ld, 65536u + 16384u);
+    for (int f = 0; f < 2; ++f) {
+      bulk_g2s(sb + kUpA + 32768u * f, sa + (size_t)f * kMlpActBytes + (size_t)ob * 32768u, 32768u, b_ld);
+      bulk_g2s(sb + kUpB + 8192u * f, sbm + f * bh + (size_t)ig * 8192u, 8192u, b_ld);
     }
   }
-  if (warp == 0) tmem_alloc(&s_tmem, ncols);
   fence_async_smem();
   tc_before_sync();
   __syncthreads();
@@ -383,12 +423,13 @@ __global__ void __launch_bounds__(256, 1) k_mlp_wgrad(MlpDev P) {
     if (!mbar_wait(b_ld, 0)) s_err = 1;
     else {
       tc_after_sync();
-      if (w2) {
-        mma_bf16(tmem, sb, 16, sb + 65536, 32, 16, kMlpH, false);
-        mma_bf16(tmem + 256, sb, 16, sb + 196608, 2, 16, 16, false);
-      } else {
-        mma_bf16(tmem, sb, 16, sb + 131072, 4, 16, 32, false);
-        mma_bf16(tmem + 32, sb + 65536, 16, sb + 131072, 4, 16, 32, false);
+      for (int ks = 0; ks < 16; ++ks) {
+        const uint32_t f = ks >> 3, kk = (uint32_t)(ks & 7) * 256u;
+        const uint64_t da = desc_mn(sb + kUpA + 32768u * f + kk, 16);
+        mma_split<2>(tmem, da, desc_mn(sb + kUpB + 8192u * f + kk, 16), idesc_bf16(32) | kAMn | kBMn, ks > 0 ? 1u : 0u);
+        if (bias)
+          mma_split<2>(tmem + 32, da, smem_desc(sb + kUpOnes + (uint32_t)ks * 512u, 256u, 128u), idesc_bf16(16) | kAMn,
+                       ks > 0 ? 1u : 0u);
       }
     }
     mma_commit(b_mma);
@@ -396,57 +437,82 @@ __global__ void __launch_bounds__(256, 1) k_mlp_wgrad(MlpDev P) {
   if (!mbar_wait(b_mma, 0)) s_err = 1;
   tc_after_sync();
   const uint32_t lane_base = (uint32_t)(32 * q) << 16;
-
-  if (w2) {
-    const int o = 128 * blockIdx.x + 32 * q + lane;  // output unit of this thread
-    for (int j = 0; j < 4; ++j) {
-      const int c0 = 128 * h + 32 * j;
-      float g[32];
-      tmem_ld_cols32(tmem + lane_base + (uint32_t)c0, g);
-      float4* dst = reinterpret_cast<float4*>(P.grad + kMlpOffW2 + (size_t)o * kMlpH + c0);
+  // gradient tile: row 32 q + lane, 16 columns per half of the warps
+  {
+    float g[16];
+    tmem_ld_cols16(tmem + lane_base + 16u * (uint32_t)h, g);
+    float4* dst = reinterpret_cast<float4*>(gt + (32 * q + lane) * kUpStride + 16 * h);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) dst[e] = make_float4(g[4 * e], g[4 * e + 1], g[4 * e + 2], g[4 * e + 3]);
+    for (int e = 0; e < 4; ++e) dst[e] = make_float4(g[4 * e], g[4 * e + 1], g[4 * e + 2], g[4 * e + 3]);
+  }
+  const float gb = bias && h == 0 ? tmem_ld1(tmem + lane_base + 32u) : 0.f;
+  tc_before_sync();
+  __syncthreads();
+  // one parameter of the vector: its gradient, or its update
+  auto one = [&](int k, float g) -> float {
+    if (!apply) {
+      P.grad[k] = g;
+      return 0.f;
     }
-    if (h == 0) P.grad[kMlpOffB2 + o] = tmem_ld1(tmem + lane_base + 256u);
-  } else {
-    // W1 (and b1 in column 20): thread row o of half h
-    const int o = 128 * h + 32 * q + lane;
-    float g[32];
-    tmem_ld_cols32(tmem + lane_base + 32u * (uint32_t)h, g);
+    const float w = adam_step(P.W1[k], g, P.mW1 + k, P.vW1 + k, A);
+    P.W1[k] = w;
+    return w;
+  };
+  if (bias && h == 0) one(kMlpOffB2 + 128 * ob + 32 * q + lane, gb);
+  if (w2) {
+    // 128 x 32 parameters, 8 consecutive per thread and turn: 4 threads a row
 #pragma unroll
-    for (int c = 0; c < kMlpIn; ++c) P.grad[kMlpOffW1 + (size_t)o * kMlpIn + c] = g[c];
-    P.grad[kMlpOffB1 + o] = g[kMlpIn];
-    // w3 and b3 from the two halves' partial sums, in a fixed order
-    P.grad[kMlpOffW3 + tid] = P.part[tid] + P.part[kMlpPart + tid];
-    if (tid == 0) {
-      P.grad[kMlpOffB3] = P.part[kMlpH] + P.part[kMlpPart + kMlpH];
-      P.loss[0] = (P.part[kMlpH + 1] + P.part[kMlpPart + kMlpH + 1]) / (float)kMlpBatch;
+    for (int u = 0; u < 2; ++u) {
+      const int r = (tid >> 2) + 64 * u, c = 8 * (tid & 3);
+      const int o = 128 * ob + r, i = 32 * ig + c, k = kMlpOffW2 + o * kMlpH + i;
+      float g[8], w[8];
+      const float4* gs = reinterpret_cast<const float4*>(gt + r * kUpStride + c);
+      *reinterpret_cast<float4*>(g) = gs[0];
+      *reinterpret_cast<float4*>(g + 4) = gs[1];
+      if (!apply) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) P.grad[k + e] = g[e];
+        continue;
+      }
+      float mm[8], vv[8];
+      float4 *pw = reinterpret_cast<float4*>(P.W1 + k), *pm = reinterpret_cast<float4*>(P.mW1 + k),
+             *pv = reinterpret_cast<float4*>(P.vW1 + k);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        *reinterpret_cast<float4*>(w + 4 * e) = pw[e];
+        *reinterpret_cast<float4*>(mm + 4 * e) = pm[e];
+        *reinterpret_cast<float4*>(vv + 4 * e) = pv[e];
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) w[e] = adam_step(w[e], g[e], mm + e, vv + e, A);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        pw[e] = *reinterpret_cast<const float4*>(w + 4 * e);
+        pm[e] = *reinterpret_cast<const float4*>(mm + 4 * e);
+        pv[e] = *reinterpret_cast<const float4*>(vv + 4 * e);
+      }
+      st_bf16x8(P.w2k, o, i, 32, w);
+    }
+  } else {
+    // W1 (256 x 20) and, in column 20, b1
+    for (int e = tid; e < 128 * (kMlpIn + 1); e += blockDim.x) {
+      const int r = e / (kMlpIn + 1), c = e - r * (kMlpIn + 1), o = 128 * ob + r;
+      const float w = one(c < kMlpIn ? kMlpOffW1 + o * kMlpIn + c : kMlpOffB1 + o, gt[r * kUpStride + c]);
+      if (apply) st_bf16(P.w1k, toff(o, c, 32), w);
+    }
+    if (ob == 0) {
+      // w3 and b3 from the two halves' partial sums, in a fixed order
+      one(kMlpOffW3 + tid, P.part[tid] + P.part[kMlpPart + tid]);
+      if (tid == 0) {
+        one(kMlpOffB3, P.part[kMlpH] + P.part[kMlpPart + kMlpH]);
+        P.loss[0] = (P.part[kMlpH + 1] + P.part[kMlpPart + kMlpH + 1]) / (float)kMlpBatch;
+      }
     }
   }
   tc_before_sync();
   __syncthreads();
   if (s_err && tid == 0) atomicOr(P.err, 1);
-  if (warp == 0) tmem_free(tmem, ncols);
-}
-
-// Adam on parameter k of the FP32 vector (masters, moments and gradients are
-// laid out alike), then its BF16 operand copies (W1 | b1 and W2; b2, w3 and
-// b3 are read as FP32).
-__global__ void __launch_bounds__(256) k_mlp_adam(MlpDev P, AdamArgs A) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= kMlpParams) return;
-  float* W = P.W1;  // the parameter vector starts at W1
-  const float w = adam_step(W[k], P.grad[k], P.mW1 + k, P.vW1 + k, A);
-  W[k] = w;
-  if (k < kMlpOffB1) {
-    st_bf16(P.w1k, toff(k / kMlpIn, k % kMlpIn, 32), w);
-  } else if (k < kMlpOffW2) {
-    st_bf16(P.w1k, toff(k - kMlpOffB1, kMlpIn, 32), w);
-  } else if (k < kMlpOffB2) {
-    const int e = k - kMlpOffW2, o = e / kMlpH, i = e % kMlpH;
-    st_bf16(P.w2k, toff(o, i, 32), w);
-    st_bf16(P.w2t + (size_t)(i >> 7) * (kMlpW2Bytes / 2), toff(i & 127, o, 16), w);
-  }
+  if (warp == 0) tmem_free(tmem, 64);
 }
 
 // BF16 operand copies from the FP32 masters (after set-up or a parameter load).
@@ -459,9 +525,7 @@ __global__ void k_mlp_pack(MlpDev P) {
   }
   for (int e = tid; e < kMlpH * kMlpH; e += stride) {
     const int o = e / kMlpH, i = e % kMlpH;
-    const float v = P.W2[e];
-    st_bf16(P.w2k, toff(o, i, 32), v);
-    st_bf16(P.w2t + (size_t)(i >> 7) * (kMlpW2Bytes / 2), toff(i & 127, o, 16), v);
+    st_bf16(P.w2k, toff(o, i, 32), P.W2[e]);
   }
 }
 
@@ -469,7 +533,7 @@ __global__ void k_mlp_pack(MlpDev P) {
 void mlp_configure() {
   cudaFuncSetAttribute(k_mlp_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMlpSmem);
   cudaFuncSetAttribute(k_mlp_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMlpSmem);
-  cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  cudaFuncSetAttribute(k_mlp_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpSmem);
 }
 
 void mlp_pack_launch(const MlpDev& P, cudaStream_t s) { k_mlp_pack<<<64, 256, 0, s>>>(P); }
@@ -480,9 +544,10 @@ void mlp_forward_launch(const MlpDev& P, const double* x, int64_t ld, int n, flo
   k_mlp_pass<false><<<(n + kTileM - 1) / kTileM, 256, kMlpSmem, s>>>(P, a, x, ld, n, nullptr, y);
 }
 
+// chained: the launch before this one on the stream is a step's k_mlp_update,
+// whose tail this step's first kernel may overlap.
 void mlp_step_launch(const MlpDev& P, const MlpStepArgs& a, const double* x, int64_t ld, const float* t, float lr,
-                     bool apply, cudaStream_t s) {
-  k_mlp_pass<true><<<kMlpBatch / kTileM, 256, kMlpSmem, s>>>(P, a, x, ld, 0, t, nullptr);
+                     bool apply, bool chained, cudaStream_t s) {
   AdamArgs A;
   const double b1 = 0.9, b2 = 0.999;
   A.lr = lr;
@@ -493,8 +558,21 @@ void mlp_step_launch(const MlpDev& P, const MlpStepArgs& a, const double* x, int
   A.eps = 1e-8f;
   A.omb1 = (float)(1.0 - b1);
   A.omb2 = (float)(1.0 - b2);
-  k_mlp_wgrad<<<3, 256, 200 * 1024, s>>>(P);
-  if (apply) k_mlp_adam<<<(kMlpParams + 255) / 256, 256, 0, s>>>(P, A);
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.gridDim = dim3(kMlpBatch / kTileM);
+  cfg.dynamicSmemBytes = kMlpSmem;
+  cfg.numAttrs = chained ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, k_mlp_pass<true>, P, a, x, ld, 0, t, (float*)nullptr);
+  cfg.gridDim = dim3(18);
+  cfg.dynamicSmemBytes = kUpSmem;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_mlp_update, P, A, apply ? 1 : 0);
 }
 
 }  // namespace de
@@ -582,9 +660,9 @@ de_status mlp_create(uint64_t seed, cudaStream_t stream, de_mlp** out) {
   };
   const size_t pw = take(sizeof(float) * kMlpParams), pm = take(sizeof(float) * kMlpParams),
                pv = take(sizeof(float) * kMlpParams);
-  const size_t o_w1k = take(kMlpW1Bytes), o_w2k = take(kMlpW2Bytes), o_w2t = take(kMlpW2Bytes);
-  const size_t o_h1t = take(kMlpW2Bytes), o_dz2t = take(kMlpW2Bytes), o_dz1t = take(kMlpW2Bytes);
-  const size_t o_a1t = take(kMlpA1tBytes), o_part = take(sizeof(float) * 2 * kMlpPart);
+  const size_t o_w1k = take(kMlpW1Bytes), o_w2k = take(kMlpW2Bytes);
+  const size_t o_h1 = take(2 * kMlpActBytes), o_dz2 = take(2 * kMlpActBytes), o_dz1 = take(2 * kMlpActBytes);
+  const size_t o_a1 = take(2 * kMlpA1Bytes), o_part = take(sizeof(float) * 2 * kMlpPart);
   const size_t o_grad = take(sizeof(float) * kMlpParams), o_loss = take(sizeof(float)), o_err = take(sizeof(int));
   cudaError_t e = cudaMalloc(&m->arena, off);
   if (e != cudaSuccess) {
@@ -607,11 +685,10 @@ de_status mlp_create(uint64_t seed, cudaStream_t stream, de_mlp** out) {
   views((float*)(A + pv), P.vW1, P.vb1, P.vW2, P.vb2, P.vw3, P.vb3);
   P.w1k = A + o_w1k;
   P.w2k = A + o_w2k;
-  P.w2t = A + o_w2t;
-  P.h1t = A + o_h1t;
-  P.dz2t = A + o_dz2t;
-  P.dz1t = A + o_dz1t;
-  P.a1t = A + o_a1t;
+  P.h1 = A + o_h1;
+  P.dz2 = A + o_dz2;
+  P.dz1 = A + o_dz1;
+  P.a1 = A + o_a1;
   P.part = (float*)(A + o_part);
   P.grad = (float*)(A + o_grad);
   P.loss = (float*)(A + o_loss);
@@ -657,7 +734,7 @@ de_status mlp_train_rows(de_mlp* m, const double* x, int64_t ld, const float* t,
                          float lr) {
   for (int k = 0; k < steps; ++k) {
     MlpStepArgs a{m->seed, m->step, n, base, cap};
-    mlp_step_launch(m->P, a, x, ld, t, lr, true, m->stream);
+    mlp_step_launch(m->P, a, x, ld, t, lr, true, k > 0, m->stream);
     ++m->step;
   }
   cudaError_t e = cudaGetLastError();
@@ -714,7 +791,7 @@ de_status de_mlp_grad(de_mlp* m, const double* x_dev, int64_t ld, const float* t
   if (!mlp_dev_ptr(x_dev) || !mlp_dev_ptr(t_dev))
     return mlp_fail(m, DE_ERR_INVALID_ARG, "x_dev and t_dev must be device memory");
   MlpStepArgs a{m->seed, m->step, 0, 0, 1};
-  mlp_step_launch(m->P, a, x_dev, ld, t_dev, 0.f, false, m->stream);
+  mlp_step_launch(m->P, a, x_dev, ld, t_dev, 0.f, false, false, m->stream);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return mlp_fail(m, DE_ERR_CUDA, std::string("surrogate gradient: ") + cudaGetErrorString(e));
   de_status s = mlp_check(m);

@@ -22,14 +22,15 @@ constexpr int kMlpParams = kMlpOffB3 + 1;  // 71,425
 // BF16 operand copies (canonical K-major tiles)
 constexpr uint32_t kMlpW1Bytes = kMlpH * 32 * 2;       // W1 with b1 in column 20: 256 x 32
 constexpr uint32_t kMlpW2Bytes = kMlpH * kMlpH * 2;    // 256 x 256
-constexpr uint32_t kMlpA1tBytes = 32 * kMlpBatch * 2;  // inputs, transposed: 32 x 256
+constexpr uint32_t kMlpA1Bytes = 128 * 32 * 2;          // inputs of one 128-row half
+constexpr uint32_t kMlpActBytes = 128 * kMlpH * 2;       // an activation of one half: 128 x 256
 
 struct MlpDev {
   float *W1, *b1, *W2, *b2, *w3, *b3;        // FP32 masters (views into one vector)
   float *mW1, *mb1, *mW2, *mb2, *mw3, *mb3;  // Adam first moments
   float *vW1, *vb1, *vW2, *vb2, *vw3, *vb3;  // Adam second moments
-  uint8_t *w1k, *w2k, *w2t;                  // BF16 operands: W1|b1 (256 x 32), W2 (256 x 256), W2^T (2 x 128 x 256)
-  uint8_t *h1t, *dz2t, *dz1t, *a1t;          // transposed activations of one minibatch
+  uint8_t *w1k, *w2k;                        // BF16 operands: W1|b1 (256 x 32), W2 (256 x 256)
+  uint8_t *h1, *dz2, *dz1, *a1;              // activations of one minibatch, two 128-row halves each
   float* part;                               // 2 x kMlpPart partial sums
   float* grad;                               // kMlpParams raw gradients (gradient-only steps)
   float* loss;                               // loss of the last step
@@ -49,6 +50,6 @@ void mlp_configure();
 void mlp_pack_launch(const MlpDev& P, cudaStream_t s);
 void mlp_forward_launch(const MlpDev& P, const double* x, int64_t ld, int n, float* y, cudaStream_t s);
 void mlp_step_launch(const MlpDev& P, const MlpStepArgs& a, const double* x, int64_t ld, const float* t, float lr,
-                     bool apply, cudaStream_t s);
+                     bool apply, bool chained, cudaStream_t s);
 
 }  // namespace de
