@@ -106,6 +106,7 @@ struct RunDesc {
   double* T;          // np x dp trial rows
   float* ynorm;       // ntiles_tc * 128, |y|_2 of each trial (error bound of the split GEMM)
   float* tau;         // np, error bound of a split-precision f[i] (0 when f[i] is FP64)
+  uint8_t* acc;       // np, three-kernel path: 1 when the generation's trial replaces row i (moved by the band kernel)
   unsigned long long* stats;  // [0] FP64 re-evaluations, [1] trials evaluated
   uint8_t* A;         // tensor-core A operand, ntiles_tc tiles of a_tile_bytes
   const uint8_t* B;   // tensor-core B operand (M split), nn tiles of b_tile_bytes

@@ -173,6 +173,9 @@ struct TcPlan {
   int nitems_fit = 0;     // 128-row tiles over all runs
   int2* d_trial_items = nullptr;
   int2* d_fit_items = nullptr;
+  bool pair = false;      // generations: two row tiles per fitness CTA (d_pair_items: (run, tile pair))
+  int nitems_pair = 0;
+  int2* d_pair_items = nullptr;
   void* arena = nullptr;  // operand copies of M, the A tiles, |y|, tau, stats
   size_t smem_fit = 0;
   std::vector<int> fit_offset;  // first fit item of each run

@@ -17,13 +17,13 @@
 //                  a two-stage shared-memory pipeline; the objective terms are
 //                  evaluated from TMEM on the CUDA cores in FP32; then greedy
 //                  selection (Sec. 2) where the split-precision values decide
-//                  it within their error bound; accepted trials are copied
-//                  over their targets in place (the trial kernel of this
-//                  generation has finished reading donors).  Rows the split
-//                  values cannot decide, and trials that could become the new
-//                  best, go to a list for the FP64 band kernel.
+//                  it within their error bound (a flag per accepted row).
+//                  Rows the split values cannot decide, and trials that could
+//                  become the new best, go to a list for the FP64 band kernel.
 //
-//   k_band_fp64    the listed rows, spread over the whole GPU: FP64 rotation
+//   k_band_fp64    moves the accepted trials over their targets in place (the
+//                  trial kernel of this generation has finished reading
+//                  donors); the listed rows, spread over the whole GPU: FP64 rotation
 //                  and objective of the trial (and of the target when its
 //                  stored fitness is not FP64) in 32-column chunks, then the
 //                  FP64 selection decision.  The last CTA to finish a run's
@@ -178,26 +178,36 @@ __global__ void __launch_bounds__(256) k_prep_rows(const RunDesc* __restrict__ r
 // n_eval rows already converted by k_prep_rows, f written to fout; mode 2:
 // the same for the run's own population (n_eval = np), written as the
 // population's split fitness values with their error bounds (f, fx = 0, tau).
-template <int ESZ>
-__global__ void __launch_bounds__(kFitThreads, 1)
+//
+// MT = 2: a CTA takes two 128-row tiles (items = the run's tile pairs, 256
+// threads each) against one N tile of 256 columns, both accumulators in
+// tensor memory.  The products of a wide problem are bound by the operand
+// bytes each SM draws from L2: at D = 1000, K steps of 24 KB for 384 cycles of
+// products, i.e. all of the 64 B a clock an SM gets; the second tile shares
+// M's half of them (32 KB for 768 cycles).  Used when one-tile CTAs would
+// need more than one wave (tc_plan_build).
+constexpr int kPairKc = 64;      // bytes of a row per pipeline stage of the pair form (32 bf16 or 16 tf32)
+constexpr int kPairStages = 3;   // 64 KB each
+constexpr size_t kPairSmem = (size_t)kPairStages * 2 * kPairKc * (2 * kTileM + 256);
+
+template <int ESZ, int MT>
+__global__ void __launch_bounds__(kFitThreads* MT, 1)
     k_fit_tc(const RunDesc* __restrict__ runs, const int2* __restrict__ items, int mode, double* __restrict__ fout,
              int n_eval) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ __align__(8) uint64_t bars[2 * kMaxStages + 1];  // full[S], done[S], acc
   __shared__ uint32_t s_tmem;
-  __shared__ int s_stop, s_err, s_nlist, s_nacc, s_last;
+  __shared__ int s_stop, s_err, s_nlist[MT], s_last[MT];
   __shared__ long long s_gen;
   __shared__ double s_bestprev;
-  __shared__ float s_part[5][kTileM];
-  __shared__ double s_fnew[kTileM];
-  __shared__ double s_ftrial[kTileM];
-  __shared__ float s_taunew[kTileM];
-  __shared__ uint8_t s_flag[kTileM];  // bit 0 accept, bit 1 decided in FP64
-  __shared__ int s_list[kTileM];
-  __shared__ int s_acc[kTileM];
-  __shared__ double s_bf[8];
-  __shared__ long long s_bk[8];
-  __shared__ int s_bi[8];
+  __shared__ float s_part[MT][5][kTileM];
+  __shared__ double s_fnew[MT][kTileM];
+  __shared__ double s_ftrial[MT][kTileM];
+  __shared__ float s_taunew[MT][kTileM];
+  __shared__ uint8_t s_flag[MT][kTileM];  // bit 0 accept, bit 1 decided in FP64
+  __shared__ double s_bf[MT][8];
+  __shared__ long long s_bk[MT][8];
+  __shared__ int s_bi[MT][8];
 
   const int2 it = items[blockIdx.x];
   const RunDesc& R = runs[it.x];  // run descriptors are written once, at set-up
@@ -207,14 +217,17 @@ __global__ void __launch_bounds__(kFitThreads, 1)
   const bool split = gridDim.y > 1 && R.nn > 1;
   const int nt_lo = split ? (int)blockIdx.y : 0, nt_hi = split ? nt_lo + 1 : R.nn;
   RunState* st = R.st;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  pdl_launch_dependents();
+  const int tid = threadIdx.x, lane = tid & 31;
+  // this thread's row tile, and its place among the tile's 256 threads
+  const int mt = MT == 1 ? 0 : tid >> 8, lt = tid & (kFitThreads - 1), warp = lt >> 5;
+  const int tile = MT * it.y + mt;
+  if (MT == 1) pdl_launch_dependents();
 
   // ---- set-up that does not depend on the previous kernel: barriers, tensor
   // memory, and the constant B operand of the first pipeline stages
   // S-stage K pipeline: stage s is filled when full[s] completes and free
   // again when done[s] (the commit of its products) completes
-  const int S = R.nstage;
+  const int S = MT == 1 ? R.nstage : kPairStages;
   auto full_bar = [&](int sg) { return smem_u32(&bars[sg]); };
   auto done_bar = [&](int sg) { return smem_u32(&bars[kMaxStages + sg]); };
   const uint32_t b_acc = smem_u32(&bars[2 * kMaxStages]);
@@ -222,11 +235,10 @@ __global__ void __launch_bounds__(kFitThreads, 1)
     for (int k = 0; k < 2 * kMaxStages + 1; ++k) mbar_init(smem_u32(&bars[k]), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_err = 0;
-    s_nlist = 0;
-    s_nacc = 0;
+    for (int t = 0; t < MT; ++t) s_nlist[t] = 0;
   }
-  const uint32_t ncols = R.ntn <= 32 ? 32u : (R.ntn <= 64 ? 64u : (R.ntn <= 128 ? 128u : 256u));
-  if (warp == 0) {
+  const uint32_t ncols = MT == 2 ? 512u : R.ntn <= 32 ? 32u : (R.ntn <= 64 ? 64u : (R.ntn <= 128 ? 128u : 256u));
+  if (tid < 32) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
                  "r"(ncols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -234,10 +246,14 @@ __global__ void __launch_bounds__(kFitThreads, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = s_tmem;
+  const uint32_t tmem = s_tmem + (uint32_t)mt * 256u;
+  // (two-tile CTAs hold all of an SM's tensor memory: the next kernel may
+  // start once every CTA of this one has it)
+  if (MT == 2) pdl_launch_dependents();
 
   // ---- geometry of the K pipeline
-  const int kc = R.kc;
+  const int kc = MT == 1 ? R.kc : kPairKc / ESZ;
+  const int ntile = MT == 1 || MT * it.y + 1 < R.ntiles_tc ? MT : 1;  // row tiles of this CTA
   const int nkc = (R.kpad + kc - 1) / kc;
   const int nseq = (nt_hi - nt_lo) * nkc;
   const uint32_t a_part = (uint32_t)(R.a_tile_bytes / 2);
@@ -246,8 +262,9 @@ __global__ void __launch_bounds__(kFitThreads, 1)
   const uint32_t a_chunk = kg_chunk * 16u * 128u;
   const uint32_t bk = (uint32_t)(R.ntn / 8) * 128u;     // B k-group stride
   const uint32_t b_chunk = kg_chunk * bk;
-  const uint32_t stage_bytes = 2 * a_chunk + 2 * b_chunk;
-  const uint8_t* Atile = R.A + (size_t)it.y * R.a_tile_bytes;
+  const uint32_t a_bytes = (uint32_t)MT * 2u * a_chunk;  // the tiles' parts, then M's
+  const uint32_t stage_bytes = a_bytes + 2 * b_chunk;
+  const uint8_t* Atile = R.A + (size_t)(MT * it.y) * R.a_tile_bytes;
   const uint32_t sbase = smem_u32(smem);
   const uint32_t fmt = ESZ == 2 ? 1u : 2u;
   const uint32_t idesc =
@@ -261,11 +278,11 @@ __global__ void __launch_bounds__(kFitThreads, 1)
     const uint32_t ab = kgs * 16u * 128u, bb = kgs * bk;
     const uint32_t base = sbase + (uint32_t)sg * stage_bytes;
     const uint32_t bar = full_bar(sg);
-    mbar_expect_tx(bar, 2 * ab + 2 * bb);
+    mbar_expect_tx(bar, (uint32_t)ntile * 2 * ab + 2 * bb);
     const size_t b_off = (size_t)kci * b_chunk;
     const uint8_t* Bt = R.B + (size_t)nt * R.b_tile_bytes;
-    bulk_g2s(base + 2 * a_chunk, Bt + b_off, bb, bar);
-    bulk_g2s(base + 2 * a_chunk + b_chunk, Bt + b_part + b_off, bb, bar);
+    bulk_g2s(base + a_bytes, Bt + b_off, bb, bar);
+    bulk_g2s(base + a_bytes + b_chunk, Bt + b_part + b_off, bb, bar);
   };
   auto issue_load_a = [&](int q) {
     const int kci = q % nkc, sg = q % S;
@@ -274,8 +291,11 @@ __global__ void __launch_bounds__(kFitThreads, 1)
     const uint32_t base = sbase + (uint32_t)sg * stage_bytes;
     const uint32_t bar = full_bar(sg);
     const size_t a_off = (size_t)kci * a_chunk;
-    bulk_g2s(base, Atile + a_off, ab, bar);
-    bulk_g2s(base + a_chunk, Atile + a_part + a_off, ab, bar);
+    for (int t = 0; t < ntile; ++t) {
+      const uint8_t* At = Atile + (size_t)t * R.a_tile_bytes + a_off;
+      bulk_g2s(base + (uint32_t)(2 * t) * a_chunk, At, ab, bar);
+      bulk_g2s(base + (uint32_t)(2 * t + 1) * a_chunk, At + a_part, ab, bar);
+    }
   };
   const int npro = min(nseq, S);
   if (tid == 0)
@@ -295,11 +315,12 @@ __global__ void __launch_bounds__(kFitThreads, 1)
     if (tid == 0)
       for (int q = 0; q < npro; ++q) mbar_wait(full_bar(q), 0u);
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
+    if (tid < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(ncols));
     return;
   }
-  const int row0 = it.y * kTileM;
-  const int nrows = min(kTileM, (mode == 0 ? R.np : n_eval) - row0);
+  const int row0 = tile * kTileM;
+  const int nrows = max(0, min(kTileM, (mode == 0 ? R.np : n_eval) - row0));
+  const bool live = mt < ntile;  // a pair's second tile may be missing
 
   // per-thread epilogue state: row m (TMEM lane), column half h
   const int m = 32 * (warp & 3) + lane;
@@ -336,12 +357,13 @@ __global__ void __launch_bounds__(kFitThreads, 1)
         const uint32_t base = sbase + (uint32_t)sg * stage_bytes;
         const int ksteps = chunk_len(kci) * ESZ / 32;
         for (int ks = 0; ks < ksteps; ++ks) {
+          for (int t = 0; t < ntile; ++t)
 #pragma unroll
           for (int pass = 0; pass < 3; ++pass) {
-            const uint32_t a = base + (pass == 2 ? a_chunk : 0u) + (uint32_t)ks * 2u * 2048u;
-            const uint32_t b = base + 2 * a_chunk + (pass == 1 ? b_chunk : 0u) + (uint32_t)ks * 2u * bk;
+            const uint32_t a = base + (uint32_t)(2 * t + (pass == 2 ? 1 : 0)) * a_chunk + (uint32_t)ks * 2u * 2048u;
+            const uint32_t b = base + a_bytes + (pass == 1 ? b_chunk : 0u) + (uint32_t)ks * 2u * bk;
             const uint32_t accum = (kci > 0 || ks > 0 || pass > 0) ? 1u : 0u;
-            mma_split<ESZ>(tmem, smem_desc(a, 2048u, 128u), smem_desc(b, bk, 128u), idesc, accum);
+            mma_split<ESZ>(tmem + 256u * (uint32_t)t, smem_desc(a, 2048u, 128u), smem_desc(b, bk, 128u), idesc, accum);
           }
         }
         mma_commit(done_bar(sg));
@@ -366,7 +388,7 @@ __global__ void __launch_bounds__(kFitThreads, 1)
       if (!have) atomicOr(&s_err, 1);
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (have) {
+    if (have && live) {
       // ---- epilogue of N tile nt: objective terms from TMEM (FP32), 32 or 16
       // columns per load
       const int nbase = nt * R.ntn + cb;
@@ -408,36 +430,36 @@ __global__ void __launch_bounds__(kFitThreads, 1)
       for (int k = 0; k < loads_issued; ++k) mbar_wait(full_bar(k % S), (uint32_t)((k / S) & 1));
       for (int k = 0; k < mmas_committed; ++k) mbar_wait(done_bar(k % S), (uint32_t)((k / S) & 1));
     }
-    if (mode == 1 && tid < nrows) fout[row0 + tid] = __longlong_as_double(0x7FF8000000000000LL);
+    if (mode == 1 && lt < nrows) fout[row0 + lt] = __longlong_as_double(0x7FF8000000000000LL);
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
+    if (tid < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(ncols));
     return;
   }
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
+  if (tid < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(ncols));
 
   // ---- combine the two column halves of each row (fixed order)
   if (h == 1) {
-    s_part[0][m] = acc_.a1;
-    s_part[1][m] = acc_.a2;
-    s_part[2][m] = acc_.a3;
-    s_part[3][m] = acc_.aS;
-    s_part[4][m] = acc_.aG;
+    s_part[mt][0][m] = acc_.a1;
+    s_part[mt][1][m] = acc_.a2;
+    s_part[mt][2][m] = acc_.a3;
+    s_part[mt][3][m] = acc_.aS;
+    s_part[mt][4][m] = acc_.aG;
   }
   __syncthreads();
   float t1 = 0.f, t2 = 0.f, t3 = 0.f, tS = 0.f, tG = 0.f;
   if (h == 0) {
-    t1 = acc_.a1 + s_part[0][m];
-    t2 = acc_.a2 + s_part[1][m];
-    t3 = acc_.a3 + s_part[2][m];
-    tS = acc_.aS + s_part[3][m];
-    tG = acc_.aG + s_part[4][m];
+    t1 = acc_.a1 + s_part[mt][0][m];
+    t2 = acc_.a2 + s_part[mt][1][m];
+    t3 = acc_.a3 + s_part[mt][2][m];
+    tS = acc_.aS + s_part[mt][3][m];
+    tG = acc_.aG + s_part[mt][4][m];
   }
   if (split) {
     // partial sums of this N tile -> global; the tile's last CTA adds them up
     // in N-tile order (the same order whichever CTA finishes last)
     const size_t pstride = (size_t)5 * kTileM;
-    float* P = R.npart + ((size_t)it.y * R.nn + nt_lo) * pstride;
-    if (h == 0) {
+    float* P = R.npart + ((size_t)tile * R.nn + nt_lo) * pstride;
+    if (h == 0 && live) {
       P[0 * kTileM + m] = t1;
       P[1 * kTileM + m] = t2;
       P[2 * kTileM + m] = t3;
@@ -446,16 +468,21 @@ __global__ void __launch_bounds__(kFitThreads, 1)
     }
     __threadfence();
     __syncthreads();
-    if (tid == 0) {
-      const uint32_t tk = atomicAdd(&R.nticket[it.y], 1u);
-      s_last = (tk == (uint32_t)R.nn - 1u);
-      if (s_last) R.nticket[it.y] = 0u;  // every CTA of this tile has counted itself
+    if (lt == 0) {
+      bool lastc = false;
+      if (live) {
+        const uint32_t tk = atomicAdd(&R.nticket[tile], 1u);
+        lastc = (tk == (uint32_t)R.nn - 1u);
+        if (lastc) R.nticket[tile] = 0u;  // every CTA of this tile has counted itself
+      }
+      s_last[mt] = lastc;
     }
     __syncthreads();
-    if (!s_last) return;
+    if (MT == 1 && !s_last[0]) return;
+    if (MT == 2 && !s_last[0] && !s_last[MT - 1]) return;
     __threadfence();
-    if (h == 0) {
-      const float* Q = R.npart + (size_t)it.y * R.nn * pstride;
+    if (h == 0 && s_last[mt]) {
+      const float* Q = R.npart + (size_t)tile * R.nn * pstride;
       t1 = t2 = t3 = tS = tG = 0.f;
       for (int k = 0; k < R.nn; ++k, Q += pstride) {
         t1 += __ldcg(Q + 0 * kTileM + m);
@@ -466,7 +493,9 @@ __global__ void __launch_bounds__(kFitThreads, 1)
       }
     }
   }
-  if (h == 0 && m < nrows) {
+  // the tile's selection is this CTA's (a pair's tiles may end in different CTAs)
+  const bool own = live && (!split || s_last[mt]);
+  if (h == 0 && m < nrows && own) {
     const float s1 = t1, s2 = t2, s3 = t3;
     float S = tS, G = tG;
     float fs;
@@ -505,7 +534,7 @@ __global__ void __launch_bounds__(kFitThreads, 1)
           // needs FP64 for the stop rule: surely below (or above) decides it as well
           const bool may_stop = R.target > 0.0 && fs - tau < (float)R.target * 1.001f &&
                                 !(fs + tau < (float)R.target * 0.999f);
-      s_ftrial[m] = (double)fs;
+      s_ftrial[mt][m] = (double)fs;
       if ((ambiguous && (R.band_all || near)) || may_be_best || may_stop || !(fs == fs) || !(fif == fif)) {
         // the split values cannot decide (or the trial may become the best):
         // FP64 decision in k_band_fp64
@@ -513,34 +542,35 @@ __global__ void __launch_bounds__(kFitThreads, 1)
         R.band[e] = BandEntry{it.x, i, pf_fx ? 0 : 1, 0};
         atomicAdd(&st->band_n, 1);
         atomicAdd(&st->band_left, 1);
-        s_flag[m] = 4;
-        atomicAdd(&s_nlist, 1);
+        s_flag[mt][m] = 4;
+        atomicAdd(&s_nlist[mt], 1);
       } else {
         // decided on the split values (an undecidable comparison far from the
         // optimum goes to the smaller split value, ties to the trial)
         const bool acc = sure_accept || (ambiguous && fs <= fif);
-        s_flag[m] = acc ? 1 : 0;
-        s_fnew[m] = acc ? (double)fs : pf_fi;
-        s_taunew[m] = acc ? tau : tif;
+        s_flag[mt][m] = acc ? 1 : 0;
+        s_fnew[mt][m] = acc ? (double)fs : pf_fi;
+        s_taunew[mt][m] = acc ? tau : tif;
       }
     }
   }
   __syncthreads();
   if (mode != 0) return;
 
-  // ---- write back fitness, flags, debug; list the accepted rows
+  // ---- write back fitness, accept flags, debug
   Best bb;
   bb.init();
-  if (tid < nrows) {
-    const int mm = tid, i = row0 + mm;
-    const uint8_t fl = s_flag[mm];
+  if (lt < nrows && own) {
+    const int mm = lt, i = row0 + mm;
+    const uint8_t fl = s_flag[mt][mm];
+    if (fl & 4) R.acc[i] = 0;  // k_band_fp64 decides and moves the row
     if (!(fl & 4)) {  // rows sent to the FP64 band are finished by k_band_fp64
       const bool acc = fl & 1;
-      R.f[0][i] = s_fnew[mm];
+      R.f[0][i] = s_fnew[mt][mm];
+      R.acc[i] = acc ? 1 : 0;  // the band kernel moves the row
       if (acc) {
         R.fx[0][i] = 0;
-        R.tau[i] = s_taunew[mm];
-        s_acc[atomicAdd(&s_nacc, 1)] = mm;
+        R.tau[i] = s_taunew[mt][mm];
         if (R.jde) {
           // jDE: the accepted trial's F_i and CR_i replace the target's (in place)
           double Fi, CRi;
@@ -550,43 +580,32 @@ __global__ void __launch_bounds__(kFitThreads, 1)
         }
       }
       if (R.dbg_ftrial) {
-        R.dbg_ftrial[i] = s_ftrial[mm];
+        R.dbg_ftrial[i] = s_ftrial[mt][mm];
         R.dbg_accept[i] = acc ? 1 : 0;
         R.dbg_fp64[i] = 0;
       }
-      bb.offer(s_fnew[mm], i);
+      bb.offer(s_fnew[mt][mm], i);
     }
   }
-  if (tid == 0) {
-    atomicAdd(&R.stats[0], (unsigned long long)s_nlist);
+  if (lt == 0 && own) {
+    atomicAdd(&R.stats[0], (unsigned long long)s_nlist[mt]);
     atomicAdd(&R.stats[1], (unsigned long long)nrows);
   }
   __syncthreads();
-  // accepted trials replace their targets in place
-  {
-    const int na = s_nacc;
-    const int dp2 = R.dp / 2;
-    for (int e = warp; e < na; e += kFitThreads / 32) {
-      const int i = row0 + s_acc[e];
-      const double2* src = reinterpret_cast<const double2*>(R.T + (size_t)i * R.dp);
-      double2* dst = reinterpret_cast<double2*>(R.X[0] + (size_t)i * R.dp);
-      for (int j = lane; j < dp2; j += 32) dst[j] = src[j];
-    }
-  }
   // ---- best partial of the tile, then the last CTA of the run finishes the generation
   bb.warp_reduce();
   if (lane == 0) {
-    s_bf[warp] = bb.f;
-    s_bk[warp] = bb.k;
-    s_bi[warp] = bb.i;
+    s_bf[mt][warp] = bb.f;
+    s_bk[mt][warp] = bb.k;
+    s_bi[mt][warp] = bb.i;
   }
   __syncthreads();
-  if (tid == 0) {
+  if (lt == 0 && own) {
     bb.init();
-    for (int w = 0; w < kFitThreads / 32; ++w) bb.take(s_bf[w], s_bk[w], s_bi[w]);
+    for (int w = 0; w < kFitThreads / 32; ++w) bb.take(s_bf[mt][w], s_bk[mt][w], s_bi[mt][w]);
     // the band kernel that follows reduces the partials of every tile
-    R.part[it.y].f = bb.f;
-    R.part[it.y].idx = bb.i;
+    R.part[tile].f = bb.f;
+    R.part[tile].idx = bb.i;
   }
 }
 
@@ -599,7 +618,53 @@ __global__ void __launch_bounds__(kFitThreads, 1)
 // objective terms of the chunk; partial sums go to band_part.  The CTA
 // completing the last chunk of an entry decides the selection in FP64, the one
 // completing the last entry of a run finishes that run's generation.
+//
+// Before that, the accepted trials replace their targets in place (items: the
+// (run, 128-row tile) list), a warp for `unit` rows (32 of many short ones, 4
+// where the whole list has few), four rows' loads in flight:
+// here the whole chip moves them (the tile's fitness CTA alone, a row per warp
+// and one load in flight, took most of its time: NP = 8192, D = 1000, 250 of
+// 300 us while most trials are accepted).
+__device__ __forceinline__ void move_rows(const RunDesc& R, int row0, int rows, int lane) {
+  const int np = R.np, dp2 = R.dp / 2;
+  const int i = row0 + lane;
+  const bool on = lane < rows && i < np && R.acc[min(i, np - 1)] != 0;
+  uint32_t m = __ballot_sync(0xffffffffu, on);
+  if (on) R.acc[i] = 0;  // a run that has stopped writes no flags and moves nothing
+  const double2* T = reinterpret_cast<const double2*>(R.T);
+  double2* X = reinterpret_cast<double2*>(R.X[0]);
+  while (m) {
+    // up to four rows at a time, 32 lanes of 16 bytes along each
+    int r[4], n = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      r[q] = m ? row0 + __ffs(m) - 1 : -1;
+      n += m != 0;
+      m &= m - 1;
+    }
+    for (int j = lane; j < dp2; j += 64) {
+      double2 v[4], w[4];
+      const bool two = j + 32 < dp2;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (q < n) {
+          const double2* p = T + (size_t)r[q] * dp2 + j;
+          v[q] = __ldcs(p);
+          if (two) w[q] = __ldcs(p + 32);
+        }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (q < n) {
+          double2* p = X + (size_t)r[q] * dp2 + j;
+          p[0] = v[q];
+          if (two) p[32] = w[q];
+        }
+    }
+  }
+}
+
 __global__ void __launch_bounds__(256) k_band_fp64(const RunDesc* __restrict__ runs, int nruns,
+                                                   const int2* __restrict__ items, int nitems, int unit,
                                                    const BandEntry* __restrict__ band,
                                                    const uint32_t* __restrict__ band_cnt, int nch_max) {
   extern __shared__ __align__(16) double s_dyn[];
@@ -609,6 +674,11 @@ __global__ void __launch_bounds__(256) k_band_fp64(const RunDesc* __restrict__ r
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   pdl_launch_dependents();
   pdl_wait();
+  const int per = kTileM / unit;
+  for (int u = blockIdx.x * 8 + warp; u < per * nitems; u += gridDim.x * 8) {
+    const int2 it = items[u / per];
+    move_rows(runs[it.x], it.y * kTileM + unit * (u % per), unit, lane);
+  }
   const uint32_t n = *(volatile const uint32_t*)band_cnt;
   // runs that sent no row to the band finish their generation here
   for (int r = blockIdx.x; r < nruns; r += gridDim.x) {
@@ -849,10 +919,13 @@ de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* 
   for (const auto& R : runs) p.var = p.var || R.strategy != 0 || R.jde;
   const int esz = prec == DE_PREC_BF16X3 ? 2 : 4;
   size_t bytes = 0;
-  std::vector<size_t> offA(runs.size()), offB(runs.size()), offY(runs.size()), offT(runs.size()), offS(runs.size());
+  std::vector<size_t> offA(runs.size()), offB(runs.size()), offY(runs.size()), offT(runs.size()), offS(runs.size()),
+      offC(runs.size());
   std::vector<size_t> offP(runs.size(), 0), offK(runs.size(), 0);
   p.nsplit = 1;
-  std::vector<int2> trial_items, fit_items;
+  std::vector<int2> trial_items, fit_items, pair_items;
+  long long wide_ctas = 0;  // one-tile CTAs of the runs with several N tiles
+  bool all_wide = true;
   size_t smem = 0;
   p.fit_offset.assign(runs.size(), 0);
   for (size_t r = 0; r < runs.size(); ++r) {
@@ -903,6 +976,9 @@ de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* 
     offT[r] = bytes;
     bytes += (size_t)R.np * sizeof(float);
     bytes = round_up(bytes, 256);
+    offC[r] = bytes;
+    bytes += (size_t)R.np;
+    bytes = round_up(bytes, 256);
     offS[r] = bytes;
     bytes += 2 * sizeof(unsigned long long);
     if (R.nn > 1) {
@@ -916,15 +992,23 @@ de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* 
       p.nsplit = std::max(p.nsplit, R.nn);
     }
 
+    for (int t = 0; t < (R.ntiles_tc + 1) / 2; ++t) pair_items.push_back(make_int2((int)r, t));
+    wide_ctas += R.nn > 1 ? (long long)R.ntiles_tc * R.nn : 0;
+    all_wide = all_wide && R.nn > 1;
     p.fit_offset[r] = (int)fit_items.size();
     for (int t = 0; t < R.ntiles_tc; ++t) fit_items.push_back(make_int2((int)r, t));
   }
   p.smem_fit = smem;
   p.nruns = (int)runs.size();
-  // trial kernel: about one CTA per SM, at most 8 targets (warps) per CTA
+  // two row tiles per fitness CTA where every run has several N tiles and
+  // one-tile CTAs need a second wave: NP = 8192, D = 1000 (256 one-tile CTAs on
+  // 152 SMs) 150 -> 45 us; in one wave the pairs would only leave SMs idle
   int dev = 0, nsm = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  p.pair = all_wide && wide_ctas > nsm;
+  p.nitems_pair = (int)pair_items.size();
+  // trial kernel: about one CTA per SM, at most 8 targets (warps) per CTA
   {
     long long tot = 0;
     for (auto& R : runs) tot += R.np;
@@ -974,6 +1058,7 @@ de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* 
     R.B = base + offB[r];
     R.ynorm = (float*)(base + offY[r]);
     R.tau = (float*)(base + offT[r]);
+    R.acc = base + offC[r];
     R.stats = (unsigned long long*)(base + offS[r]);
     R.npart = R.nn > 1 ? (float*)(base + offP[r]) : nullptr;
     R.nticket = R.nn > 1 ? (uint32_t*)(base + offK[r]) : nullptr;
@@ -992,6 +1077,14 @@ de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* 
     e = cudaMemcpyAsync(p.d_trial_items, trial_items.data(), trial_items.size() * sizeof(int2), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(p.d_fit_items, fit_items.data(), fit_items.size() * sizeof(int2), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess && p.pair) {
+    e = cudaMalloc(&p.d_pair_items, pair_items.size() * sizeof(int2));
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(p.d_pair_items, pair_items.data(), pair_items.size() * sizeof(int2), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+      e = esz == 2 ? cudaFuncSetAttribute(k_fit_tc<2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem)
+                   : cudaFuncSetAttribute(k_fit_tc<4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   p.nitems_trial = (int)trial_items.size();
   p.nitems_fit = (int)fit_items.size();
@@ -1013,9 +1106,9 @@ de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* 
     e = cudaFuncSetAttribute(k_band_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(p.smem_band, 1));
   if (e == cudaSuccess) {
     if (esz == 2) {
-      e = cudaFuncSetAttribute(k_fit_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      e = cudaFuncSetAttribute(k_fit_tc<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     } else {
-      e = cudaFuncSetAttribute(k_fit_tc<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      e = cudaFuncSetAttribute(k_fit_tc<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
   }
   if (e != cudaSuccess) {
@@ -1047,8 +1140,8 @@ de_status tc_set_geometry(TcPlan& p, std::vector<RunDesc>& runs, int trial_rows,
     e = cudaMemcpyAsync(p.d_trial_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) {
-    e = esz == 2 ? cudaFuncSetAttribute(k_fit_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                 : cudaFuncSetAttribute(k_fit_tc<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = esz == 2 ? cudaFuncSetAttribute(k_fit_tc<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                 : cudaFuncSetAttribute(k_fit_tc<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   }
   if (e != cudaSuccess) {
     err = std::string("split-precision geometry: ") + cudaGetErrorString(e);
@@ -1065,7 +1158,9 @@ void tc_plan_free(TcPlan& p) {
   if (p.arena) cudaFree(p.arena);
   if (p.d_trial_items) cudaFree(p.d_trial_items);
   if (p.d_fit_items) cudaFree(p.d_fit_items);
+  if (p.d_pair_items) cudaFree(p.d_pair_items);
   p.arena = nullptr;
+  p.d_pair_items = nullptr;
   p.d_trial_items = nullptr;
   p.d_fit_items = nullptr;
 }
@@ -1097,17 +1192,26 @@ void tc_generation_launch(const TcPlan& p, const RunDesc* runs, cudaStream_t s) 
     else if (p.var) launch_pdl(k_trial_split<2, true, false>, gt, tb, 0, s, runs, ti);
     else if (p.trial_occ) launch_pdl(k_trial_split<2, false, true>, gt, tb, 0, s, runs, ti);
     else launch_pdl(k_trial_split<2, false, false>, gt, tb, 0, s, runs, ti);
-    launch_pdl(k_fit_tc<2>, dim3(p.nitems_fit, p.nsplit), kFitThreads, p.smem_fit, s, runs,
-               (const int2*)p.d_fit_items, 0, (double*)nullptr, 0);
+    if (p.pair)
+      launch_pdl(k_fit_tc<2, 2>, dim3(p.nitems_pair, p.nsplit), 2 * kFitThreads, kPairSmem, s, runs,
+                 (const int2*)p.d_pair_items, 0, (double*)nullptr, 0);
+    else
+      launch_pdl(k_fit_tc<2, 1>, dim3(p.nitems_fit, p.nsplit), kFitThreads, p.smem_fit, s, runs,
+                 (const int2*)p.d_fit_items, 0, (double*)nullptr, 0);
   } else {
     if (p.var && p.trial_occ) launch_pdl(k_trial_split<4, true, true>, gt, tb, 0, s, runs, ti);
     else if (p.var) launch_pdl(k_trial_split<4, true, false>, gt, tb, 0, s, runs, ti);
     else if (p.trial_occ) launch_pdl(k_trial_split<4, false, true>, gt, tb, 0, s, runs, ti);
     else launch_pdl(k_trial_split<4, false, false>, gt, tb, 0, s, runs, ti);
-    launch_pdl(k_fit_tc<4>, dim3(p.nitems_fit, p.nsplit), kFitThreads, p.smem_fit, s, runs,
-               (const int2*)p.d_fit_items, 0, (double*)nullptr, 0);
+    if (p.pair)
+      launch_pdl(k_fit_tc<4, 2>, dim3(p.nitems_pair, p.nsplit), 2 * kFitThreads, kPairSmem, s, runs,
+                 (const int2*)p.d_pair_items, 0, (double*)nullptr, 0);
+    else
+      launch_pdl(k_fit_tc<4, 1>, dim3(p.nitems_fit, p.nsplit), kFitThreads, p.smem_fit, s, runs,
+                 (const int2*)p.d_fit_items, 0, (double*)nullptr, 0);
   }
-  launch_pdl(k_band_fp64, dim3(p.grid_band), 256, p.smem_band, s, runs, p.nruns, (const BandEntry*)p.d_band,
+  launch_pdl(k_band_fp64, dim3(p.grid_band), 256, p.smem_band, s, runs, p.nruns, (const int2*)p.d_fit_items,
+             p.nitems_fit, p.nitems_fit * (kTileM / 32) >= 8 * p.grid_band ? 32 : 4, (const BandEntry*)p.d_band,
              (const uint32_t*)p.d_band_cnt, p.nch_max);
 }
 
@@ -1115,10 +1219,10 @@ void tc_init_eval_launch(const TcPlan& p, const RunDesc* runs, int run, const Ru
   const int2* items = p.d_fit_items + p.fit_offset[run];
   if (p.prec == DE_PREC_BF16X3) {
     k_prep_rows<2><<<(R.np + 7) / 8, 256, 0, s>>>(runs, run, R.X[0], R.dp, R.np);
-    k_fit_tc<2><<<R.ntiles_tc, kFitThreads, p.smem_fit, s>>>(runs, items, 2, (double*)nullptr, R.np);
+    k_fit_tc<2, 1><<<R.ntiles_tc, kFitThreads, p.smem_fit, s>>>(runs, items, 2, (double*)nullptr, R.np);
   } else {
     k_prep_rows<4><<<(R.np + 7) / 8, 256, 0, s>>>(runs, run, R.X[0], R.dp, R.np);
-    k_fit_tc<4><<<R.ntiles_tc, kFitThreads, p.smem_fit, s>>>(runs, items, 2, (double*)nullptr, R.np);
+    k_fit_tc<4, 1><<<R.ntiles_tc, kFitThreads, p.smem_fit, s>>>(runs, items, 2, (double*)nullptr, R.np);
   }
 }
 
@@ -1132,10 +1236,10 @@ de_status tc_eval_launch(const TcPlan& p, const RunDesc* runs, int run, const Ru
     const int2* items = p.d_fit_items + p.fit_offset[run];
     if (p.prec == DE_PREC_BF16X3) {
       k_prep_rows<2><<<(nb + 7) / 8, 256, 0, s>>>(runs, run, x + (size_t)r0 * ld, ld, nb);
-      k_fit_tc<2><<<tiles, kFitThreads, p.smem_fit, s>>>(runs, items, 1, f + r0, nb);
+      k_fit_tc<2, 1><<<tiles, kFitThreads, p.smem_fit, s>>>(runs, items, 1, f + r0, nb);
     } else {
       k_prep_rows<4><<<(nb + 7) / 8, 256, 0, s>>>(runs, run, x + (size_t)r0 * ld, ld, nb);
-      k_fit_tc<4><<<tiles, kFitThreads, p.smem_fit, s>>>(runs, items, 1, f + r0, nb);
+      k_fit_tc<4, 1><<<tiles, kFitThreads, p.smem_fit, s>>>(runs, items, 1, f + r0, nb);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -1149,18 +1253,18 @@ de_status tc_eval_launch(const TcPlan& p, const RunDesc* runs, int run, const Ru
 de_status tc_eval_rows(const RunDesc* desc, const int2* items, int tiles, int esz, size_t smem, const double* x,
                        int64_t ld, int n, double* f, cudaStream_t s, std::string& err) {
   cudaFuncAttributes fa{};
-  cudaError_t e = esz == 2 ? cudaFuncGetAttributes(&fa, k_fit_tc<2>) : cudaFuncGetAttributes(&fa, k_fit_tc<4>);
+  cudaError_t e = esz == 2 ? cudaFuncGetAttributes(&fa, k_fit_tc<2, 1>) : cudaFuncGetAttributes(&fa, k_fit_tc<4, 1>);
   if (e == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes < smem) {
-    e = esz == 2 ? cudaFuncSetAttribute(k_fit_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                 : cudaFuncSetAttribute(k_fit_tc<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = esz == 2 ? cudaFuncSetAttribute(k_fit_tc<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                 : cudaFuncSetAttribute(k_fit_tc<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   }
   if (e == cudaSuccess) {
     if (esz == 2) {
       k_prep_rows<2><<<(n + 7) / 8, 256, 0, s>>>(desc, 0, x, ld, n);
-      k_fit_tc<2><<<tiles, kFitThreads, smem, s>>>(desc, items, 1, f, n);
+      k_fit_tc<2, 1><<<tiles, kFitThreads, smem, s>>>(desc, items, 1, f, n);
     } else {
       k_prep_rows<4><<<(n + 7) / 8, 256, 0, s>>>(desc, 0, x, ld, n);
-      k_fit_tc<4><<<tiles, kFitThreads, smem, s>>>(desc, items, 1, f, n);
+      k_fit_tc<4, 1><<<tiles, kFitThreads, smem, s>>>(desc, items, 1, f, n);
     }
     e = cudaGetLastError();
   }
