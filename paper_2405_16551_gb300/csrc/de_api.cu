@@ -720,8 +720,8 @@ static de_status autotune_fp64(de_handle* h, int nsm) {
   return DE_OK;
 }
 
-// Split precisions, three-kernel path: targets per trial CTA and the K chunk
-// of the fitness kernel, timed on the handle's own problem and cached like
+// Split precisions, three-kernel path: the trial kernel's warps per CTA and
+// groups per warp and the K chunk of the fitness kernel, timed on the handle's own problem and cached like
 // the FP64 choice (neither changes results).  The persistent cluster kernel
 // takes its geometry from occupancy and is not tuned here.
 static std::string tune_key_split(const de_handle* h) {
@@ -731,7 +731,7 @@ static std::string tune_key_split(const de_handle* h) {
     sum_d += (long long)R.np * R.d;
   }
   char b[256];
-  snprintf(b, sizeof b, "split_v4 prec=%d runs=%d np0=%d d0=%d obj0=%d sumnp=%lld sumnd=%lld", h->prec, h->nruns,
+  snprintf(b, sizeof b, "split_v5 prec=%d runs=%d np0=%d d0=%d obj0=%d sumnp=%lld sumnd=%lld", h->prec, h->nruns,
            h->run[0].np, h->run[0].d, h->run[0].obj, sum_np, sum_d);
   return b;
 }
@@ -740,12 +740,17 @@ static de_status autotune_split(de_handle* h) {
   const char* env = getenv("DE_GB300_AUTOTUNE");
   if ((env && env[0] == '0') || h->tc.persist.ok) return DE_OK;
   const std::string key = tune_key_split(h);
-  // cached value: 1000 x trial-kernel instance (1: held to 85 registers) + 100
-  // x targets per trial CTA + 10 x K-chunk divisor + pipeline stages
+  // cached value, in decimal digits: trial-kernel instance (1: held to 85
+  // registers), warps per trial CTA, target groups per warp, K-chunk divisor,
+  // pipeline stages
+  auto set = [&](int code) {
+    h->tc.trial_occ = code / 10000;
+    return tc_set_geometry(h->tc, h->run, (code / 1000) % 10, (code / 100) % 10, (code / 10) % 10, code % 10, h->stream,
+                           h->err);
+  };
   int code = 0;
   if (tune_lookup(key, code)) {
-    h->tc.trial_occ = code / 1000;
-    de_status s = tc_set_geometry(h->tc, h->run, (code / 100) % 10, (code / 10) % 10, code % 10, h->stream, h->err);
+    de_status s = set(code);
     if (s == DE_OK) s = upload_desc(h);
     return s;
   }
@@ -761,32 +766,36 @@ static de_status autotune_split(de_handle* h) {
   float best_ms = 1e30f;
   int best = 0;
   de_status st_all = DE_OK;
-  for (int oc = 0; oc < 2 && st_all == DE_OK; ++oc)
-  for (int tr : {2, 4, 8}) {
-    h->tc.trial_occ = oc;
-    for (int kd : {1, 2, 4})
-      for (int ns : {2, 4}) {
-      st_all = tc_set_geometry(h->tc, h->run, tr, kd, ns, h->stream, h->err);
-      if (st_all == DE_OK) st_all = upload_desc(h);
-      if (st_all != DE_OK) break;
-      for (int r = 0; r < h->nruns; ++r) {
-        int32_t zero = 0;
-        DE_CUDA(h, cudaMemcpyAsync(&h->run[r].st->stop, &zero, sizeof zero, cudaMemcpyHostToDevice, h->stream));
-      }
-      launch_generation(h);
-      DE_CUDA(h, cudaEventRecord(e0, h->stream));
-      for (int k = 0; k < 6; ++k) launch_generation(h);
-      DE_CUDA(h, cudaEventRecord(e1, h->stream));
-      DE_CUDA(h, cudaEventSynchronize(e1));
-      float ms = 0.f;
-      DE_CUDA(h, cudaEventElapsedTime(&ms, e0, e1));
-      if (ms < best_ms * 0.97f) {
-        best_ms = ms;
-        best = oc * 1000 + tr * 100 + kd * 10 + ns;
-      }
-      }
-    if (st_all != DE_OK) break;
-  }
+  auto time_code = [&](int c) -> de_status {
+    de_status s = set(c);
+    if (s == DE_OK) s = upload_desc(h);
+    if (s != DE_OK) return s;
+    for (int r = 0; r < h->nruns; ++r) {
+      int32_t zero = 0;
+      DE_CUDA(h, cudaMemcpyAsync(&h->run[r].st->stop, &zero, sizeof zero, cudaMemcpyHostToDevice, h->stream));
+    }
+    launch_generation(h);
+    DE_CUDA(h, cudaEventRecord(e0, h->stream));
+    for (int k = 0; k < 6; ++k) launch_generation(h);
+    DE_CUDA(h, cudaEventRecord(e1, h->stream));
+    DE_CUDA(h, cudaEventSynchronize(e1));
+    float ms = 0.f;
+    DE_CUDA(h, cudaEventElapsedTime(&ms, e0, e1));
+    if (ms < best_ms * 0.97f) {
+      best_ms = ms;
+      best = c;
+    }
+    return DE_OK;
+  };
+  // the trial kernel's geometry first, then the fitness kernel's
+  for (int oc = 0; oc < 2; ++oc)
+    for (int tr : {2, 4, 8})
+      for (int per : {1, 2, 4, 8})
+        if (st_all == DE_OK) st_all = time_code(oc * 10000 + tr * 1000 + per * 100 + 12);
+  const int trial = best / 100 * 100;
+  for (int kd : {1, 2, 4})
+    for (int ns : {2, 4})
+      if (st_all == DE_OK && kd * 10 + ns != 12) st_all = time_code(trial + kd * 10 + ns);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   for (size_t r = 0; r < saved.size(); ++r) {
@@ -795,8 +804,7 @@ static de_status autotune_split(de_handle* h) {
   }
   h->run = saved;
   if (st_all != DE_OK) return st_all;
-  h->tc.trial_occ = best / 1000;
-  de_status s = tc_set_geometry(h->tc, h->run, (best / 100) % 10, (best / 10) % 10, best % 10, h->stream, h->err);
+  de_status s = set(best);
   if (s == DE_OK) s = upload_desc(h);
   if (s == DE_OK) tune_store(key, best);
   return s;

@@ -185,6 +185,7 @@ struct TcPlan {
   size_t smem_band = 0;
   int grid_band = 0;
   int trial_rows = 8;          // targets (warps) per trial CTA
+  int trial_per = 1;           // target groups per warp of the trial kernel
   int trial_occ = 0;           // 1: the trial kernel instance held to 85 registers (more warps per SM)
   int nsplit = 1;              // N tiles spread over CTAs of the fitness kernel (the largest N-tile count)
   int nruns = 0;
@@ -211,11 +212,11 @@ void k_persist_close_launch(const RunDesc* runs, const PersistCtl* ctl, cudaStre
 de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* cfgs, int prec, cudaStream_t s,
                         std::string& err);
 void tc_plan_free(TcPlan& p);
-// Launch geometry that leaves the results unchanged (autotuner): targets per
-// trial CTA, a divisor of the fitness kernel's default K chunk, and the
+// Launch geometry that leaves the results unchanged (autotuner): warps per
+// trial CTA and target groups per warp, a divisor of the fitness kernel's default K chunk, and the
 // stages of its K pipeline.
-de_status tc_set_geometry(TcPlan& p, std::vector<RunDesc>& runs, int trial_rows, int kc_div, int stages,
-                          cudaStream_t s, std::string& err);
+de_status tc_set_geometry(TcPlan& p, std::vector<RunDesc>& runs, int trial_rows, int trial_per, int kc_div,
+                          int stages, cudaStream_t s, std::string& err);
 void tc_generation_launch(const TcPlan& p, const RunDesc* runs, cudaStream_t s);
 // Split-precision evaluation of run `run`'s population X[0] into f[0] (fx = 0,
 // tau set): the initial evaluation of split-precision runs.

@@ -62,22 +62,30 @@ namespace de {
 // ------------------------------------------------------------------ trial kernel
 // items: (run, group); a warp holds 32 / R.lpt targets, R.lpt lanes each
 // (lane L: coordinates 4 (L % lpt) .. + 3 of each 4 lpt-wide chunk), so that
-// short rows do not leave most lanes of the FP64 instructions idle; warp w of
-// the CTA takes targets (group * warps + w) * (32 / lpt) + L / lpt.
+// short rows do not leave most lanes of the FP64 instructions idle.  Warp w of
+// the CTA takes the per consecutive target groups from (group * warps + w) * per
+// on, one step (a chunk of a group) at a time, with the next step's loads in
+// flight: also across groups, whose draws are made a step ahead.  A warp with
+// one group of one chunk (D <= 128) had nothing to overlap its loads with, and
+// a CTA of two such warps spent most of its life reading its descriptor
+// (512-run batch, 64,275 CTAs: 252 us for 100 us of FP64 instructions).
 // VAR: some run uses a strategy variant or jDE (a separate instance).
 // OCC: an instance held to 85 registers a thread (three 256-thread CTAs' worth
 // of warps per SM), which spills a little but keeps more loads in flight; the
-// other is held to 128 (no spills; left unbounded the compiler takes ~150 and
-// a quarter of the warps).  The autotuner times both on the handle's problem.
+// other is held to 128.  The autotuner times both, and per, on the handle's problem.
 template <int ESZ, bool VAR, bool OCC>
 __global__ void __launch_bounds__(256, OCC ? 3 : 2)
-    k_trial_split(const RunDesc* __restrict__ runs, const int2* __restrict__ items) {
+    k_trial_split(const RunDesc* __restrict__ runs, const int2* __restrict__ items, int per) {
+  __shared__ RunDesc sR;
   __shared__ int s_stop, s_best;
   __shared__ long long s_gen;
   const int2 it = items[blockIdx.x];
-  const RunDesc& R = runs[it.x];
+  for (int q = threadIdx.x; q < (int)(sizeof(RunDesc) / 8); q += blockDim.x)
+    reinterpret_cast<uint64_t*>(&sR)[q] = reinterpret_cast<const uint64_t*>(runs + it.x)[q];
+  const RunDesc& R = sR;
   pdl_launch_dependents();
   pdl_wait();
+  __syncthreads();
   // the previous generation's FP64 band kernel has finished: empty its list
   if (blockIdx.x == 0 && threadIdx.x == 0) *R.band_cnt = 0u;
   if (threadIdx.x == 0) {
@@ -89,62 +97,80 @@ __global__ void __launch_bounds__(256, OCC ? 3 : 2)
   if (s_stop) return;
   const int64_t g = s_gen + 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int lpt = R.lpt, sub = lane & (lpt - 1);
-  const int i0 = (it.y * (int)(blockDim.x >> 5) + warp) * (32 / lpt);
-  if (i0 >= R.np) return;  // the whole warp
-  const int iraw = i0 + lane / lpt;
-  const bool valid = iraw < R.np;
-  const int i = valid ? iraw : R.np - 1;  // idle segments repeat a valid target without writing
+  const int lpt = R.lpt, sub = lane & (lpt - 1), tpw = 32 / lpt, np = R.np, d = R.d, kpad = R.kpad;
   const double* X = R.X[0];
-  TrialVar v;
-  TrialSetup s;
-  if constexpr (VAR) s = trial_setup_var(R, (uint32_t)i, g, lane, s_best, R.jde ? R.jF[0] : nullptr,
-                                         R.jde ? R.jCR[0] : nullptr, v, lpt, valid);
-  else s = trial_setup(R, (uint32_t)i, g, sub, 0u, valid);
-  uint8_t* Ahi = R.A + (size_t)(i >> 7) * R.a_tile_bytes;
   const uint32_t a_part = (uint32_t)(R.a_tile_bytes / 2);
-  const int m = i & 127;
-  float yn2 = 0.f;
   const bool dbg = R.dbg_trial != nullptr;
   const int cw = 4 * lpt;  // coordinates per chunk
-  const int nchunks = (R.kpad + cw - 1) / cw;
-  // the loads of chunk c + 1 are issued before chunk c is computed; the loop
-  // is compiled twice, for a unit domain scale (no multiplication) and any other
-  ChunkIn cur, nxt;
-  if (4 * sub < R.d) trial_load(R, X, s, (uint32_t)i, g, 4 * sub, cur);
-  auto chunks = [&](auto unit) {
-  constexpr bool UNIT = decltype(unit)::value;
-  for (int c = 0; c < nchunks; ++c) {
-    const int j0 = cw * c + 4 * sub;
-    if (c + 1 < nchunks && j0 + cw < R.d) trial_load(R, X, s, (uint32_t)i, g, j0 + cw, nxt);
-    double t[4] = {0.0, 0.0, 0.0, 0.0};
-    uint32_t bits = 0;
-    if (j0 < R.d) {
-      if constexpr (VAR) bits = trial_compute(R, s, j0, cur, t, v.F, v.thr, v.L);
-      else bits = trial_compute(R, s, j0, cur, t);
-      if (valid) {
-        double* Trow = R.T + (size_t)i * R.dp + j0;
-        *reinterpret_cast<double2*>(Trow) = make_double2(t[0], t[1]);
-        *reinterpret_cast<double2*>(Trow + 2) = make_double2(t[2], t[3]);
-      }
-    }
-    if (j0 < R.kpad) {
-      float y[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        y[q] = (j0 + q < R.d) ? to_f32_rn(shifted_as<UNIT>(t[q], R.o[j0 + q], R.scale)) : 0.f;
-        yn2 += y[q] * y[q];
-      }
-      if (valid) store_split4<ESZ>(Ahi, a_part, m, j0, y);
-    }
-    if (dbg) trial_debug(R, (uint32_t)i, j0, lane, bits, t, lpt, valid);
-    cur = nxt;
-  }
+  const int nchunks = (kpad + cw - 1) / cw;
+  const int grp0 = (it.y * (int)(blockDim.x >> 5) + warp) * per;
+  // groups of this warp that have a target
+  const int ngrp = min(per, max(0, (np - grp0 * tpw + tpw - 1) / tpw));
+  if (ngrp <= 0) return;  // the whole warp
+  // a group's target of this lane's segment, its draws and control parameters
+  struct Grp {
+    TrialVar v;
+    TrialSetup s;
+    int i;
+    bool valid;
   };
-  if (R.unit_scale) chunks(std::true_type{});
-  else chunks(std::false_type{});
-  for (int o = lpt >> 1; o > 0; o >>= 1) yn2 += __shfl_xor_sync(0xffffffffu, yn2, o);
-  if (valid && sub == 0) R.ynorm[i] = sqrtf(yn2);
+  auto setup = [&](int k, Grp& G) {
+    const int iraw = (grp0 + k) * tpw + lane / lpt;
+    G.valid = iraw < np;
+    G.i = G.valid ? iraw : np - 1;  // idle segments repeat a valid target without writing
+    if constexpr (VAR) G.s = trial_setup_var(R, (uint32_t)G.i, g, lane, s_best, R.jde ? R.jF[0] : nullptr,
+                                             R.jde ? R.jCR[0] : nullptr, G.v, lpt, G.valid);
+    else G.s = trial_setup(R, (uint32_t)G.i, g, sub, 0u, G.valid);
+  };
+  // the loop is compiled twice, for a unit domain scale (no multiplication)
+  // and any other
+  auto steps = [&](auto unit) {
+    constexpr bool UNIT = decltype(unit)::value;
+    Grp G, H;
+    ChunkIn cur, nxt;
+    setup(0, G);
+    if (4 * sub < d) trial_load(R, X, G.s, (uint32_t)G.i, g, 4 * sub, cur);
+    for (int k = 0; k < ngrp; ++k) {
+      float yn2 = 0.f;
+      uint8_t* Ahi = R.A + (size_t)(G.i >> 7) * R.a_tile_bytes;
+      for (int c = 0; c < nchunks; ++c) {
+        const int j0 = cw * c + 4 * sub;
+        if (c + 1 < nchunks) {
+          if (j0 + cw < d) trial_load(R, X, G.s, (uint32_t)G.i, g, j0 + cw, nxt);
+        } else if (k + 1 < ngrp) {
+          setup(k + 1, H);
+          if (4 * sub < d) trial_load(R, X, H.s, (uint32_t)H.i, g, 4 * sub, nxt);
+        }
+        double t[4] = {0.0, 0.0, 0.0, 0.0};
+        uint32_t bits = 0;
+        if (j0 < d) {
+          if constexpr (VAR) bits = trial_compute(R, G.s, j0, cur, t, G.v.F, G.v.thr, G.v.L);
+          else bits = trial_compute(R, G.s, j0, cur, t);
+          if (G.valid) {
+            double* Trow = R.T + (size_t)G.i * R.dp + j0;
+            *reinterpret_cast<double2*>(Trow) = make_double2(t[0], t[1]);
+            *reinterpret_cast<double2*>(Trow + 2) = make_double2(t[2], t[3]);
+          }
+        }
+        if (j0 < kpad) {
+          float y[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            y[q] = (j0 + q < d) ? to_f32_rn(shifted_as<UNIT>(t[q], R.o[j0 + q], R.scale)) : 0.f;
+            yn2 += y[q] * y[q];
+          }
+          if (G.valid) store_split4<ESZ>(Ahi, a_part, G.i & 127, j0, y);
+        }
+        if (dbg) trial_debug(R, (uint32_t)G.i, j0, lane, bits, t, lpt, G.valid);
+        cur = nxt;
+      }
+      for (int o = lpt >> 1; o > 0; o >>= 1) yn2 += __shfl_xor_sync(0xffffffffu, yn2, o);
+      if (G.valid && sub == 0) R.ynorm[G.i] = sqrtf(yn2);
+      G = H;
+    }
+  };
+  if (R.unit_scale) steps(std::true_type{});
+  else steps(std::false_type{});
 }
 
 // Rows of caller memory -> A operand tiles and |y| (evaluation mode).
@@ -863,10 +889,10 @@ static int plan_kc(const RunDesc& R, int esz, int kc_div) {
 }
 
 // Work items of the trial kernel for one run: CTAs of `warps` warps, each
-// warp 32 / lpt targets.
-static int trial_groups(const RunDesc& R, int warps) {
-  const int per = warps * (32 / R.lpt);
-  return (R.np + per - 1) / per;
+// warp `per` groups of 32 / lpt targets.
+static int trial_groups(const RunDesc& R, int warps, int per) {
+  const int n = warps * per * (32 / R.lpt);
+  return (R.np + n - 1) / n;
 }
 
 // Stages of the K pipeline: one when the whole K of one N tile is one chunk,
@@ -1014,7 +1040,7 @@ de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* 
     for (auto& R : runs) tot += R.np;
     p.trial_rows = (int)std::max(1LL, std::min(8LL, (tot + nsm - 1) / nsm));
     for (size_t r = 0; r < runs.size(); ++r)
-      for (int gI = 0; gI < trial_groups(runs[r], p.trial_rows); ++gI)
+      for (int gI = 0; gI < trial_groups(runs[r], p.trial_rows, p.trial_per); ++gI)
         trial_items.push_back(make_int2((int)r, gI));
   }
   // FP64 band list shared by all runs of the handle
@@ -1118,7 +1144,7 @@ de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* 
   return DE_OK;
 }
 
-de_status tc_set_geometry(TcPlan& p, std::vector<RunDesc>& runs, int trial_rows, int kc_div, int stages,
+de_status tc_set_geometry(TcPlan& p, std::vector<RunDesc>& runs, int trial_rows, int trial_per, int kc_div, int stages,
                           cudaStream_t s, std::string& err) {
   const int esz = p.prec == DE_PREC_BF16X3 ? 2 : 4;
   size_t smem = 0;
@@ -1129,7 +1155,7 @@ de_status tc_set_geometry(TcPlan& p, std::vector<RunDesc>& runs, int trial_rows,
   }
   std::vector<int2> items;
   for (size_t r = 0; r < runs.size(); ++r)
-    for (int gI = 0; gI < trial_groups(runs[r], trial_rows); ++gI) items.push_back(make_int2((int)r, gI));
+    for (int gI = 0; gI < trial_groups(runs[r], trial_rows, trial_per); ++gI) items.push_back(make_int2((int)r, gI));
   cudaError_t e = cudaSuccess;
   if (items.size() != (size_t)p.nitems_trial) {
     if (p.d_trial_items) cudaFree(p.d_trial_items);
@@ -1149,6 +1175,7 @@ de_status tc_set_geometry(TcPlan& p, std::vector<RunDesc>& runs, int trial_rows,
   }
   p.nitems_trial = (int)items.size();
   p.trial_rows = trial_rows;
+  p.trial_per = trial_per;
   p.smem_fit = smem;
   return DE_OK;
 }
@@ -1188,10 +1215,10 @@ void tc_generation_launch(const TcPlan& p, const RunDesc* runs, cudaStream_t s) 
   const dim3 gt(p.nitems_trial);
   const int2* ti = p.d_trial_items;
   if (p.prec == DE_PREC_BF16X3) {
-    if (p.var && p.trial_occ) launch_pdl(k_trial_split<2, true, true>, gt, tb, 0, s, runs, ti);
-    else if (p.var) launch_pdl(k_trial_split<2, true, false>, gt, tb, 0, s, runs, ti);
-    else if (p.trial_occ) launch_pdl(k_trial_split<2, false, true>, gt, tb, 0, s, runs, ti);
-    else launch_pdl(k_trial_split<2, false, false>, gt, tb, 0, s, runs, ti);
+    if (p.var && p.trial_occ) launch_pdl(k_trial_split<2, true, true>, gt, tb, 0, s, runs, ti, p.trial_per);
+    else if (p.var) launch_pdl(k_trial_split<2, true, false>, gt, tb, 0, s, runs, ti, p.trial_per);
+    else if (p.trial_occ) launch_pdl(k_trial_split<2, false, true>, gt, tb, 0, s, runs, ti, p.trial_per);
+    else launch_pdl(k_trial_split<2, false, false>, gt, tb, 0, s, runs, ti, p.trial_per);
     if (p.pair)
       launch_pdl(k_fit_tc<2, 2>, dim3(p.nitems_pair, p.nsplit), 2 * kFitThreads, kPairSmem, s, runs,
                  (const int2*)p.d_pair_items, 0, (double*)nullptr, 0);
@@ -1199,10 +1226,10 @@ void tc_generation_launch(const TcPlan& p, const RunDesc* runs, cudaStream_t s) 
       launch_pdl(k_fit_tc<2, 1>, dim3(p.nitems_fit, p.nsplit), kFitThreads, p.smem_fit, s, runs,
                  (const int2*)p.d_fit_items, 0, (double*)nullptr, 0);
   } else {
-    if (p.var && p.trial_occ) launch_pdl(k_trial_split<4, true, true>, gt, tb, 0, s, runs, ti);
-    else if (p.var) launch_pdl(k_trial_split<4, true, false>, gt, tb, 0, s, runs, ti);
-    else if (p.trial_occ) launch_pdl(k_trial_split<4, false, true>, gt, tb, 0, s, runs, ti);
-    else launch_pdl(k_trial_split<4, false, false>, gt, tb, 0, s, runs, ti);
+    if (p.var && p.trial_occ) launch_pdl(k_trial_split<4, true, true>, gt, tb, 0, s, runs, ti, p.trial_per);
+    else if (p.var) launch_pdl(k_trial_split<4, true, false>, gt, tb, 0, s, runs, ti, p.trial_per);
+    else if (p.trial_occ) launch_pdl(k_trial_split<4, false, true>, gt, tb, 0, s, runs, ti, p.trial_per);
+    else launch_pdl(k_trial_split<4, false, false>, gt, tb, 0, s, runs, ti, p.trial_per);
     if (p.pair)
       launch_pdl(k_fit_tc<4, 2>, dim3(p.nitems_pair, p.nsplit), 2 * kFitThreads, kPairSmem, s, runs,
                  (const int2*)p.d_pair_items, 0, (double*)nullptr, 0);
