@@ -452,56 +452,74 @@ static de_status check_device_errors(de_handle* h) {
   return DE_OK;
 }
 
-// (Re)initialise run r's population from the INIT stream and evaluate it.
-static de_status init_run(de_handle* h, int r) {
-  RunDesc& R = h->run[r];
-  RunState st{};
-  st.best_idx = -1;
-  st.evals = R.np;  // the initial population counts as NP evaluations
-  DE_CUDA(h, cudaMemcpyAsync(R.st, &st, sizeof st, cudaMemcpyHostToDevice, h->stream));
-  DE_CUDA(h, cudaMemsetAsync(R.X[0], 0, (size_t)R.np * R.dp * sizeof(double), h->stream));
-  if (R.obj == DE_OBJ_ODE && !h->ode_ref_done[r]) {
-    // the hidden vector's trajectory depends on the run's shift only
-    k_ode_reference_launch(h->d_run, r, const_cast<double*>(R.ode_ref), h->stream);
-    h->ode_ref_done[r] = true;
+// Shared memory of the FP64 evaluation kernels' tiles (8 rows, fewer where
+// they do not fit) over the runs run0 .. run0 + n - 1.
+static size_t eval_smem(const de_handle* h, int run0, int n) {
+  size_t most = 1;
+  for (int r = run0; r < run0 + n; ++r) {
+    const RunDesc& R = h->run[r];
+    size_t one = (size_t)2 * suite_comps(R) * R.dp * sizeof(double);
+    int rows = 8;
+    while (rows > 1 && rows * one > kTileSmemMax) rows >>= 1;
+    most = std::max(most, rows * one);
   }
-  k_init_population_launch(h->d_run, r, R.np, R.dp, h->stream);
-  if (R.jde) k_jde_init_launch(h->d_run, r, R.np, h->stream);
-  if (h->prec == DE_PREC_FP64) {
-    k_eval_rows_launch(h->d_run, r, R, R.X[0], R.dp, R.np, R.f[0], R.fx[0], h->stream);
-  } else {
+  return most;
+}
+
+// (Re)initialise the populations of the runs run0 .. run0 + n - 1 from the INIT
+// stream and evaluate them, in one launch per step (a batch of 512 runs took
+// 3000 launches, 16 ms, run by run).
+static de_status init_runs(de_handle* h, int run0, int n) {
+  int np_max = 0, dp_max = 0;
+  bool jde = false, plain = false;
+  for (int r = run0; r < run0 + n; ++r) {
+    const RunDesc& R = h->run[r];
+    np_max = std::max(np_max, R.np);
+    dp_max = std::max(dp_max, R.dp);
+    jde = jde || R.jde;
+    plain = plain || (!R.sl && R.obj != DE_OBJ_ODE);
+    if (R.obj == DE_OBJ_ODE && !h->ode_ref_done[r]) {
+      // the hidden vector's trajectory depends on the run's shift only
+      k_ode_reference_launch(h->d_run, r, const_cast<double*>(R.ode_ref), h->stream);
+      h->ode_ref_done[r] = true;
+    }
+  }
+  k_reset_states_launch(h->d_run, run0, n, h->stream);
+  k_init_population_launch(h->d_run, run0, n, np_max, dp_max, h->stream);
+  if (jde) k_jde_init_launch(h->d_run, run0, n, np_max, h->stream);
+  const bool all = n == h->nruns && n > 1;
+  if (h->prec != DE_PREC_FP64) {
     // split precisions evaluate the initial population in their own precision
     // (values with error bounds, like accepted trials); the best record is
     // made FP64 when a caller reads it
-    tc_init_eval_launch(h->tc, h->d_run, r, R, h->stream);
+    if (all) tc_init_eval_all_launch(h->tc, h->d_run, h->stream);
+    else
+      for (int r = run0; r < run0 + n; ++r) tc_init_eval_launch(h->tc, h->d_run, r, h->run[r], h->stream);
+  } else {
+    if (all && h->slices.on)
+      k_eval_pops_tc_launch(h->d_run, h->d_items, h->d_shares, h->nshares, h->slices, dp_max, h->stream);
+    if (all && plain) k_eval_pops_launch(h->d_run, run0, n, np_max, eval_smem(h, run0, n), h->stream);
+    for (int r = run0; r < run0 + n; ++r) {
+      const RunDesc& R = h->run[r];
+      if (!all || R.obj == DE_OBJ_ODE)
+        k_eval_rows_launch(h->d_run, r, R, R.X[0], R.dp, R.np, R.f[0], R.fx[0], h->stream);
+    }
   }
-  k_best_init_launch(h->d_run, r, h->stream);
+  k_best_init_launch(h->d_run, run0, n, h->stream);
   DE_CUDA(h, cudaGetLastError());
   return DE_OK;
 }
 
 // Split precisions keep some fitness values in split precision; the best
-// record handed to a caller is made FP64 here (the best row is evaluated in
-// FP64 when its stored value is not).
-static de_status exact_best(de_handle* h, int r) {
+// records handed to a caller are made FP64 here (a best row is evaluated in
+// FP64 when its stored value is not), and the mirror of the states read.
+static de_status exact_best(de_handle* h, int run0, int n) {
   if (h->prec == DE_PREC_FP64) return DE_OK;
-  RunState& st = h->h_state[r];
-  if (st.best_idx < 0) return DE_OK;
-  const RunDesc& R = h->run[r];
-  const int cur = cur_buf(h, st.gen);
-  uint8_t fx = 1;
-  DE_CUDA(h, cudaMemcpyAsync(&fx, R.fx[cur] + st.best_idx, 1, cudaMemcpyDeviceToHost, h->stream));
-  DE_CUDA(h, cudaStreamSynchronize(h->stream));
-  if (fx) return DE_OK;
-  double* fb = R.f[cur] + st.best_idx;
-  k_eval_rows_launch(h->d_run, r, R, R.X[cur] + (size_t)st.best_idx * R.dp, R.dp, 1, fb,
-                     R.fx[cur] + st.best_idx, h->stream);
+  int dp_max = 0;
+  for (int r = run0; r < run0 + n; ++r) dp_max = std::max(dp_max, h->run[r].dp);
+  k_best_exact_launch(h->d_run, run0, n, dp_max, h->stream);
   DE_CUDA(h, cudaGetLastError());
-  DE_CUDA(h, cudaMemcpyAsync(&st.best_f, fb, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  DE_CUDA(h, cudaStreamSynchronize(h->stream));
-  DE_CUDA(h, cudaMemcpyAsync(&R.st->best_f, &st.best_f, sizeof(double), cudaMemcpyHostToDevice, h->stream));
-  DE_CUDA(h, cudaStreamSynchronize(h->stream));
-  return DE_OK;
+  return read_states(h);
 }
 
 // ---------------------------------------------------------------- autotuner
@@ -1338,7 +1356,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
   TRY(build_items(h));
   TRY(upload_desc(h));
   k_configure(h->smem_gen);
-  for (int r = 0; r < nruns; ++r) TRY(init_run(h, r));
+  TRY(init_runs(h, 0, nruns));
   if (h->prec == DE_PREC_FP64 && cfgs[0].surrogate_k < 2) {
     ce = cudaMalloc(&h->d_ctl64, sizeof(PersistCtl));
     if (ce != cudaSuccess) return fin(fail(h, DE_ERR_OOM, "cudaMalloc(persistent control) failed"));
@@ -1356,7 +1374,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
     // the failure-detection test applies to the generations after set-up
     // (not to the autotuner's timing launches)
     if (const char* v = getenv("DE_GB300_TEST_GRID_TIMEOUT")) h->test_grid_skip = std::max(0, atoi(v));
-    for (int r = 0; r < nruns; ++r) TRY(init_run(h, r));
+    TRY(init_runs(h, 0, nruns));
   } else if (h->prec != DE_PREC_FP64) {
     if (h->tc.persist.ok) {
       TRY(autotune_persist(h));
@@ -1366,8 +1384,8 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
     }
     // the failure-detection test applies to the generations after set-up
     if (const char* v = getenv("DE_GB300_TEST_GRID_TIMEOUT")) h->test_grid_skip = std::max(0, atoi(v));
+    TRY(init_runs(h, 0, nruns));
     for (int r = 0; r < nruns; ++r) {
-      TRY(init_run(h, r));
       // the counters start after the timing generations
       if (h->run[r].stats) {
         ce = cudaMemsetAsync(h->run[r].stats, 0, 2 * sizeof(unsigned long long), h->stream);
@@ -1395,10 +1413,8 @@ de_status de_reset(de_handle* h, int32_t run) {
   if (!h) return fail(nullptr, DE_ERR_INVALID_ARG, "handle is NULL");
   if (run < -1 || run >= h->nruns) return fail(h, DE_ERR_INVALID_ARG, "run out of range");
   h->err.clear();
-  for (int r = (run < 0 ? 0 : run); r < (run < 0 ? h->nruns : run + 1); ++r) {
-    de_status s = init_run(h, r);
-    if (s != DE_OK) return s;
-  }
+  const de_status st = run < 0 ? init_runs(h, 0, h->nruns) : init_runs(h, run, 1);
+  if (st != DE_OK) return st;
   if (h->surr) {
     const de_status s = surr_reset(*h->surr, h->stream, h->err);
     if (s != DE_OK) return fail(h, s, h->err);
@@ -1511,8 +1527,8 @@ de_status de_run(de_handle* h, de_result* out) {
     if (s != DE_OK) return s;
     chunk = std::min<int64_t>(chunk * 2, 1024);
   }
-  for (int r = 0; r < h->nruns && out; ++r) {
-    s = exact_best(h, r);
+  if (out) {
+    s = exact_best(h, 0, h->nruns);
     if (s != DE_OK) return s;
   }
   const double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
@@ -1599,7 +1615,7 @@ de_status de_set_population(de_handle* h, int32_t run, const double* x_host, con
   } else {
     k_eval_rows_launch(h->d_run, run, R, R.X[cur], R.dp, R.np, R.f[cur], R.fx[cur], h->stream);
   }
-  k_best_init_launch(h->d_run, run, h->stream);
+  k_best_init_launch(h->d_run, run, 1, h->stream);
   DE_CUDA(h, cudaGetLastError());
   s = islands_resync(h);
   if (s != DE_OK) return s;
@@ -1630,7 +1646,7 @@ de_status de_set_generation(de_handle* h, int32_t run, int64_t generation) {
   DE_CUDA(h, cudaMemcpyAsync(&R.st->gen, &generation, sizeof generation, cudaMemcpyHostToDevice, h->stream));
   int64_t ev = (int64_t)R.np * (1 + generation);
   DE_CUDA(h, cudaMemcpyAsync(&R.st->evals, &ev, sizeof ev, cudaMemcpyHostToDevice, h->stream));
-  k_best_init_launch(h->d_run, run, h->stream);
+  k_best_init_launch(h->d_run, run, 1, h->stream);
   DE_CUDA(h, cudaGetLastError());
   s = islands_resync(h);
   if (s != DE_OK) return s;
@@ -1682,7 +1698,7 @@ de_status de_get_best(de_handle* h, int32_t run, double* best_f, int32_t* best_i
   const RunDesc& R = h->run[run];
   de_status s = read_states(h);
   if (s != DE_OK) return s;
-  s = exact_best(h, run);
+  s = exact_best(h, run, 1);
   if (s != DE_OK) return s;
   const RunState& st = h->h_state[run];
   if (best_x) {

@@ -42,8 +42,9 @@ namespace de {
 // ------------------------------------------------------------------ init
 // Parameter j of individual i: x = lo + (hi - lo) u with u from draws 2j, 2j+1
 // of the INIT stream; one Philox block serves parameters 2b and 2b + 1.
-__global__ void k_init_population(const RunDesc* __restrict__ runs, int run) {
-  const RunDesc& R = runs[run];
+// blockIdx.y: the run, from `run0` on.
+__global__ void k_init_population(const RunDesc* __restrict__ runs, int run0) {
+  const RunDesc& R = runs[run0 + blockIdx.y];
   const int64_t nblk = (int64_t)R.np * (R.dp / 2);
   const double span = R.hi - R.lo;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nblk; t += (int64_t)gridDim.x * blockDim.x) {
@@ -61,20 +62,15 @@ __global__ void k_init_population(const RunDesc* __restrict__ runs, int run) {
 }
 
 // ------------------------------------------------------------------ eval
-// f of n rows of x (row stride ld) with run `run`'s objective; CTA per tile
-// of `rows` rows.  Shared memory: 2 * rows * dp doubles.
-__global__ void k_eval_rows(const RunDesc* __restrict__ runs, int run, const double* __restrict__ x, int64_t ld,
-                            int n, int rows, double* __restrict__ fout, uint8_t* __restrict__ fx_out) {
-  extern __shared__ __align__(16) double sm[];
-  const RunDesc& R = runs[run];
+// f of rows row0 .. row0 + nrows - 1 of x (row stride ld), a tile of at most
+// `rows` rows.  Shared memory: 2 * rows * dp doubles (times the components).
+__device__ __forceinline__ void eval_tile(const RunDesc& R, const double* __restrict__ x, int64_t ld, int row0, int nrows,
+                                          int rows, double* __restrict__ fout, uint8_t* __restrict__ fx_out, double* sm) {
   const int d = R.d, dp = R.dp;
   // a composition function keeps every component's rows at once
   const int ncomp = R.obj >= kObjComposition1 ? R.nc : 1;
   double* Y = sm;
   double* Z = Y + ncomp * rows * dp;
-  const int row0 = blockIdx.x * rows;
-  const int nrows = min(rows, n - row0);
-  if (nrows <= 0) return;
   if (suite_objective(R.obj)) {
     // the proposed benchmark's functions (Sec. 7.3, Table 2)
     __shared__ double s_f[kSuiteMaxRows];
@@ -121,11 +117,60 @@ __global__ void k_eval_rows(const RunDesc* __restrict__ runs, int run, const dou
   }
 }
 
+// n rows of x with run `run`'s objective; CTA per tile of `rows` rows.
+__global__ void k_eval_rows(const RunDesc* __restrict__ runs, int run, const double* __restrict__ x, int64_t ld,
+                            int n, int rows, double* __restrict__ fout, uint8_t* __restrict__ fx_out) {
+  extern __shared__ __align__(16) double sm[];
+  const int row0 = blockIdx.x * rows, nrows = min(rows, n - row0);
+  if (nrows > 0) eval_tile(runs[run], x, ld, row0, nrows, rows, fout, fx_out, sm);
+}
+
+// The populations X[0] of the runs whose rotation is not sliced (but for the
+// ODE objective): blockIdx.y is the run, blockIdx.x the tile of 8 rows (fewer
+// where eval_smem says so).
+__global__ void __launch_bounds__(256) k_eval_pops(const RunDesc* __restrict__ runs, int run0, size_t smem) {
+  extern __shared__ __align__(16) double sm[];
+  const RunDesc& R = runs[run0 + blockIdx.y];
+  if (R.sl || R.obj == kObjOde) return;
+  const int ncomp = R.obj >= kObjComposition1 ? R.nc : 1;
+  int rows = 8;
+  while (rows > 1 && (size_t)2 * ncomp * rows * R.dp * sizeof(double) > smem) rows >>= 1;
+  for (int row0 = blockIdx.x * rows; row0 < R.np; row0 += gridDim.x * rows) {
+    eval_tile(R, R.X[0], R.dp, row0, min(rows, R.np - row0), rows, R.f[0], R.fx[0], sm);
+    __syncthreads();
+  }
+}
+
+// The runs' states after (re)initialisation: generation 0, NP evaluations.
+__global__ void k_reset_states(const RunDesc* __restrict__ runs, int run0, int n) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= n) return;
+  const RunDesc& R = runs[run0 + r];
+  RunState st = {};
+  st.best_idx = -1;
+  st.evals = R.np;
+  *R.st = st;
+}
+
+// Split precisions: the best individual's fitness in FP64 where it is stored
+// as a split value (blockIdx.x: the run, from run0 on).
+__global__ void __launch_bounds__(256) k_best_exact(const RunDesc* __restrict__ runs, int run0) {
+  extern __shared__ __align__(16) double sm[];
+  const RunDesc& R = runs[run0 + blockIdx.x];
+  RunState* st = R.st;
+  const int i = st->best_idx, cur = R.dbuf ? (int)(st->gen & 1) : 0;
+  if (i < 0 || R.fx[cur][i]) return;
+  eval_tile(R, R.X[cur], R.dp, i, 1, 1, R.f[cur], R.fx[cur], sm);
+  // (the warp that evaluated the row wrote its fitness)
+  __syncthreads();
+  if (threadIdx.x == 0) st->best_f = R.f[cur][i];
+}
+
 // jDE: every F_i and CR_i of generation 0 set to the run's F and CR.
-__global__ void k_jde_init(const RunDesc* __restrict__ runs, int run) {
-  const RunDesc& R = runs[run];
+__global__ void k_jde_init(const RunDesc* __restrict__ runs, int run0) {
+  const RunDesc& R = runs[run0 + blockIdx.y];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < R.np) {
+  if (R.jde && i < R.np) {
     R.jF[0][i] = R.F;
     R.jCR[0][i] = R.CR;
   }
@@ -139,8 +184,8 @@ __global__ void k_ode_reference(const RunDesc* __restrict__ runs, int run, doubl
 
 // Reduce f[0..np) of the current generation into the run's best record and
 // set the stop flag; single CTA per run.  Used after (re)initialisation.
-__global__ void k_best_init(const RunDesc* __restrict__ runs, int run) {
-  const RunDesc& R = runs[run];
+__global__ void k_best_init(const RunDesc* __restrict__ runs, int run0) {
+  const RunDesc& R = runs[run0 + blockIdx.x];
   RunState* st = R.st;
   // double-buffered paths alternate buffers by generation; the three-kernel
   // split path updates X[0] in place
@@ -547,6 +592,8 @@ void k_configure(size_t smem_gen) {
   }
   k_tc_configure();
   cudaFuncSetAttribute(k_eval_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  cudaFuncSetAttribute(k_eval_pops, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  cudaFuncSetAttribute(k_best_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
 cudaError_t k_gen_fp64_persist_launch(const RunDesc* runs, const int4* items, int nitems, int nruns, int threads,
@@ -647,11 +694,27 @@ void k_gen_fp64_launch(const RunDesc* runs, const int4* items, int nitems, int t
   else cudaLaunchKernelEx(&cfg, k_gen_fp64<false, false>, runs, items);
 }
 
-void k_init_population_launch(const RunDesc* runs, int run, int np, int dp, cudaStream_t s) {
-  const long long n = (long long)np * (dp / 2);
+void k_reset_states_launch(const RunDesc* runs, int run0, int n, cudaStream_t s) {
+  k_reset_states<<<(n + 127) / 128, 128, 0, s>>>(runs, run0, n);
+}
+
+void k_init_population_launch(const RunDesc* runs, int run0, int n, int np_max, int dp_max, cudaStream_t s) {
+  const long long m = (long long)np_max * (dp_max / 2);
   const int threads = 256;
-  const int blocks = (int)std::min<long long>((n + threads - 1) / threads, 152LL * 16);
-  k_init_population<<<blocks, threads, 0, s>>>(runs, run);
+  const int blocks = (int)std::max(1LL, std::min<long long>((m + threads - 1) / threads, 152LL * 16 / std::min(n, 16)));
+  for (int r = 0; r < n; r += 65535)
+    k_init_population<<<dim3((unsigned)blocks, (unsigned)std::min(n - r, 65535)), threads, 0, s>>>(runs, run0 + r);
+}
+
+// Populations of the runs run0 .. run0 + n - 1 that k_eval_pops serves.
+void k_eval_pops_launch(const RunDesc* runs, int run0, int n, int np_max, size_t smem, cudaStream_t s) {
+  const int tiles = std::min((np_max + 7) / 8, std::max(1, 152 * 64 / std::max(1, std::min(n, 512))));
+  for (int r = 0; r < n; r += 65535)
+    k_eval_pops<<<dim3((unsigned)tiles, (unsigned)std::min(n - r, 65535)), 256, smem, s>>>(runs, run0 + r, smem);
+}
+
+void k_best_exact_launch(const RunDesc* runs, int run0, int n, int dp_max, cudaStream_t s) {
+  k_best_exact<<<n, 256, (size_t)2 * dp_max * sizeof(double), s>>>(runs, run0);
 }
 
 void k_eval_rows_launch(const RunDesc* runs, int run, const RunDesc& Rh, const double* x, int64_t ld, int n,
@@ -678,10 +741,13 @@ void k_eval_rows_launch(const RunDesc* runs, int run, const RunDesc& Rh, const d
   k_eval_rows<<<(n + rows - 1) / rows, 256, smem, s>>>(runs, run, x, ld, n, rows, f, fx);
 }
 
-void k_best_init_launch(const RunDesc* runs, int run, cudaStream_t s) { k_best_init<<<1, 256, 0, s>>>(runs, run); }
+void k_best_init_launch(const RunDesc* runs, int run0, int n, cudaStream_t s) {
+  k_best_init<<<n, 256, 0, s>>>(runs, run0);
+}
 
-void k_jde_init_launch(const RunDesc* runs, int run, int np, cudaStream_t s) {
-  k_jde_init<<<(np + 255) / 256, 256, 0, s>>>(runs, run);
+void k_jde_init_launch(const RunDesc* runs, int run0, int n, int np_max, cudaStream_t s) {
+  for (int r = 0; r < n; r += 65535)
+    k_jde_init<<<dim3((unsigned)((np_max + 255) / 256), (unsigned)std::min(n - r, 65535)), 256, 0, s>>>(runs, run0 + r);
 }
 
 void k_ode_reference_launch(const RunDesc* runs, int run, double* ref, cudaStream_t s) {

@@ -155,28 +155,15 @@ __global__ void __launch_bounds__(256, 1)
   slice_end(sc);
 }
 
-// f of n rows of x (row stride ld); a warp per row of the 8-row tiles.
-__global__ void __launch_bounds__(256, 1)
-    k_eval_rows_tc(const RunDesc* __restrict__ runs, int run, const double* __restrict__ x, int64_t ld, int n,
-                   double* __restrict__ fout, uint8_t* __restrict__ fx_out, int kpad, uint32_t cols) {
-  extern __shared__ __align__(1024) uint8_t smem_tc[];
-  __shared__ SliceShared s_sl;
-  __shared__ RunDesc sR;
-  __shared__ double s_f[kCompGroup];
-  __shared__ double s_comp[kCompGroup][10];
-  load_desc(sR, runs + run);
-  SliceCtx sc;
-  slice_begin(sc, smem_tc, kpad, cols, s_sl);
-  const RunDesc& R = sR;
-  const int d = R.d, dp = R.dp, obj = R.obj;
-  double* Y = reinterpret_cast<double*>(smem_tc + slice_smem(kpad));
+// f of rows r0 .. r1 - 1 of x (row stride ld) with a sliced run; a warp per row
+// of the 8-row tiles.  Y, Z: 8 x dp doubles.
+__device__ __forceinline__ void eval_sliced(const RunDesc& R, SliceCtx& sc, const double* __restrict__ x, int64_t ld,
+                                            int r0, int r1, double* __restrict__ fout, uint8_t* __restrict__ fx_out,
+                                            double* Y, double* s_f, double (*s_comp)[10]) {
+  const int d = R.d, dp = R.dp, obj = R.obj, kpad = R.sl_kpad;
   double* Z = Y + kSliceRows * dp;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool suite = suite_objective(obj);
-  // this CTA's rows: a contiguous share in whole tiles
-  const int tiles = (n + kSliceRows - 1) / kSliceRows;
-  const int r0 = (int)((long long)tiles * blockIdx.x / gridDim.x) * kSliceRows;
-  const int r1 = min(n, (int)((long long)tiles * (blockIdx.x + 1) / gridDim.x) * kSliceRows);
   const int step = suite && obj >= kObjComposition1 ? kCompGroup : kSliceRows;
   for (int row0 = r0; row0 < r1; row0 += step) {
     const int nr = min(step, r1 - row0);
@@ -203,7 +190,7 @@ __global__ void __launch_bounds__(256, 1)
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
-    if (!sc.cur) slice_load_m(sc, R.sl, kpad);
+    if (sc.cur != R.sl) slice_load_m(sc, R.sl, kpad);
     const double f = slice_fitness(sc, R, Y, Z, nr);
     if (warp < nr) {
       if (lane == 0) {
@@ -214,9 +201,55 @@ __global__ void __launch_bounds__(256, 1)
   }
   // a wait that gave up (it should not on a healthy device) cannot be
   // returned by this launch: the rows come back as NaN, the run is marked
+  __syncthreads();
   if (*sc.s_fail) {
     for (int r = r0 + (int)threadIdx.x; r < r1; r += blockDim.x) fout[r] = CUDART_NAN;
     if (threadIdx.x == 0) atomicOr(&R.st->err, kErrTimeout);
+  }
+}
+
+// n rows of x with run `run`'s objective, in contiguous shares of whole tiles.
+__global__ void __launch_bounds__(256, 1)
+    k_eval_rows_tc(const RunDesc* __restrict__ runs, int run, const double* __restrict__ x, int64_t ld, int n,
+                   double* __restrict__ fout, uint8_t* __restrict__ fx_out, int kpad, uint32_t cols) {
+  extern __shared__ __align__(1024) uint8_t smem_tc[];
+  __shared__ SliceShared s_sl;
+  __shared__ RunDesc sR;
+  __shared__ double s_f[kCompGroup];
+  __shared__ double s_comp[kCompGroup][10];
+  load_desc(sR, runs + run);
+  SliceCtx sc;
+  slice_begin(sc, smem_tc, kpad, cols, s_sl);
+  double* Y = reinterpret_cast<double*>(smem_tc + slice_smem(kpad));
+  const int tiles = (n + kSliceRows - 1) / kSliceRows;
+  const int r0 = (int)((long long)tiles * blockIdx.x / gridDim.x) * kSliceRows;
+  const int r1 = min(n, (int)((long long)tiles * (blockIdx.x + 1) / gridDim.x) * kSliceRows);
+  eval_sliced(sR, sc, x, ld, r0, r1, fout, fx_out, Y, s_f, s_comp);
+  slice_end(sc);
+}
+
+// The populations X[0] of the sliced runs, in the shares of k_gen_fp64_tc.
+__global__ void __launch_bounds__(256, 1)
+    k_eval_pops_tc(const RunDesc* __restrict__ runs, const int4* __restrict__ items, const int2* __restrict__ shares,
+                   int kpad, uint32_t cols) {
+  extern __shared__ __align__(1024) uint8_t smem_tc[];
+  __shared__ SliceShared s_sl;
+  __shared__ RunDesc sR;
+  __shared__ double s_f[kCompGroup];
+  __shared__ double s_comp[kCompGroup][10];
+  SliceCtx sc;
+  slice_begin(sc, smem_tc, kpad, cols, s_sl);
+  double* Y = reinterpret_cast<double*>(smem_tc + slice_smem(kpad));
+  const int2 share = shares[blockIdx.x];
+  for (int i = share.x; i < share.y;) {
+    int e = i + 1;
+    while (e < share.y && items[e].x == items[i].x) ++e;
+    __syncthreads();
+    load_desc(sR, runs + items[i].x);
+    __syncthreads();
+    if (sR.sl)
+      eval_sliced(sR, sc, sR.X[0], sR.dp, items[i].z, items[e - 1].z + items[e - 1].w, sR.f[0], sR.fx[0], Y, s_f, s_comp);
+    i = e;
   }
   slice_end(sc);
 }
@@ -290,6 +323,13 @@ void k_tc_configure() {
   cudaFuncSetAttribute(k_gen_fp64_tc<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_gen_fp64_tc<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_eval_rows_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  cudaFuncSetAttribute(k_eval_pops_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+}
+
+void k_eval_pops_tc_launch(const RunDesc* runs, const int4* items, const int2* shares, int nct, const SlicePlan& p,
+                           int dp_max, cudaStream_t s) {
+  const size_t smem = p.smem_op + (size_t)2 * kSliceRows * dp_max * sizeof(double);
+  k_eval_pops_tc<<<nct, 256, smem, s>>>(runs, items, shares, p.kpad, p.cols);
 }
 
 void k_eval_rows_tc_launch(const RunDesc* runs, int run, const RunDesc& Rh, const double* x, int64_t ld, int n,

@@ -65,6 +65,9 @@ void k_gen_fp64_tc_launch(const RunDesc* runs, const int4* items, const int2* sh
                           bool var, bool suite, cudaStream_t s);
 void k_eval_rows_tc_launch(const RunDesc* runs, int run, const RunDesc& Rh, const double* x, int64_t ld, int n,
                            double* f, uint8_t* fx, cudaStream_t s);
+// the sliced runs' populations, in the shares of k_gen_fp64_tc_launch
+void k_eval_pops_tc_launch(const RunDesc* runs, const int4* items, const int2* shares, int nct, const SlicePlan& p,
+                           int dp_max, cudaStream_t s);
 void k_tc_configure();
 // Dynamic shared memory that gives a CTA of kernel k a whole SM (at least smem)
 size_t fp64_exclusive_smem(const void* k, size_t smem);
@@ -96,14 +99,23 @@ cudaError_t k_gen_fp64_cluster_launch(const RunDesc* runs, const int4* items, in
                                       bool var, bool suite, PersistCtl* ctl, long long gens, cudaStream_t s,
                                       const SlicePlan& sp);
 bool k_gen_fp64_cluster_fits(int nitems, int threads, size_t smem, bool var, bool suite, const SlicePlan& sp);
-void k_init_population_launch(const RunDesc* runs, int run, int np, int dp, cudaStream_t s);
+// the runs run0 .. run0 + n - 1 in one launch each: states after
+// (re)initialisation, populations from the INIT stream (which fill every row to
+// its stride), jDE parameters, FP64 evaluation of the populations that are
+// neither sliced nor ODE runs' (smem: what the largest tile takes, as
+// k_eval_rows_launch), best records
+void k_reset_states_launch(const RunDesc* runs, int run0, int n, cudaStream_t s);
+void k_init_population_launch(const RunDesc* runs, int run0, int n, int np_max, int dp_max, cudaStream_t s);
+void k_eval_pops_launch(const RunDesc* runs, int run0, int n, int np_max, size_t smem, cudaStream_t s);
+// split precisions: the best records made FP64
+void k_best_exact_launch(const RunDesc* runs, int run0, int n, int dp_max, cudaStream_t s);
 // f (and, when fx is not NULL, the FP64 flags) of n rows of x; Rh is the
 // host copy of run `run`'s descriptor
 void k_eval_rows_launch(const RunDesc* runs, int run, const RunDesc& Rh, const double* x, int64_t ld, int n,
                         double* f, uint8_t* fx, cudaStream_t s);
 inline int suite_comps(const RunDesc& R) { return R.obj >= DE_OBJ_COMPOSITION1 ? R.nc : 1; }
-void k_best_init_launch(const RunDesc* runs, int run, cudaStream_t s);
-void k_jde_init_launch(const RunDesc* runs, int run, int np, cudaStream_t s);
+void k_best_init_launch(const RunDesc* runs, int run0, int n, cudaStream_t s);
+void k_jde_init_launch(const RunDesc* runs, int run0, int n, int np_max, cudaStream_t s);
 void k_ode_reference_launch(const RunDesc* runs, int run, double* ref, cudaStream_t s);
 
 // island model (de_islands.cu)
@@ -220,6 +232,7 @@ de_status tc_set_geometry(TcPlan& p, std::vector<RunDesc>& runs, int trial_rows,
 void tc_generation_launch(const TcPlan& p, const RunDesc* runs, cudaStream_t s);
 // Split-precision evaluation of run `run`'s population X[0] into f[0] (fx = 0,
 // tau set): the initial evaluation of split-precision runs.
+void tc_init_eval_all_launch(const TcPlan& p, const RunDesc* runs, cudaStream_t s);  // every run's
 void tc_init_eval_launch(const TcPlan& p, const RunDesc* runs, int run, const RunDesc& R, cudaStream_t s);
 de_status tc_eval_launch(const TcPlan& p, const RunDesc* runs, int run, const RunDesc& R, const double* x, int64_t ld,
                          int n, double* f, cudaStream_t s, std::string& err);

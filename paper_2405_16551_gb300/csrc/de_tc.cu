@@ -173,14 +173,9 @@ __global__ void __launch_bounds__(256, OCC ? 3 : 2)
   else steps(std::false_type{});
 }
 
-// Rows of caller memory -> A operand tiles and |y| (evaluation mode).
+// One row of x -> A operand tile row and |y| (evaluation modes); a warp.
 template <int ESZ>
-__global__ void __launch_bounds__(256) k_prep_rows(const RunDesc* __restrict__ runs, int run,
-                                                   const double* __restrict__ x, int64_t ld, int n) {
-  const RunDesc& R = runs[run];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + warp;
-  if (i >= n) return;
+__device__ __forceinline__ void prep_row(const RunDesc& R, const double* __restrict__ xr, int i, int lane) {
   uint8_t* Ahi = R.A + (size_t)(i >> 7) * R.a_tile_bytes;
   const uint32_t a_part = (uint32_t)(R.a_tile_bytes / 2);
   float yn2 = 0.f;
@@ -189,7 +184,7 @@ __global__ void __launch_bounds__(256) k_prep_rows(const RunDesc* __restrict__ r
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int j = j0 + q;
-      y[q] = (j < R.d) ? to_f32_rn(shifted(x[(size_t)i * ld + j], R.o[j], R)) : 0.f;
+      y[q] = (j < R.d) ? to_f32_rn(shifted(xr[j], R.o[j], R)) : 0.f;
       yn2 += y[q] * y[q];
     }
     store_split4<ESZ>(Ahi, a_part, i & 127, j0, y);
@@ -199,10 +194,28 @@ __global__ void __launch_bounds__(256) k_prep_rows(const RunDesc* __restrict__ r
   if (lane == 0) R.ynorm[i] = sqrtf(yn2);
 }
 
+// Rows of caller memory.
+template <int ESZ>
+__global__ void __launch_bounds__(256) k_prep_rows(const RunDesc* __restrict__ runs, int run,
+                                                   const double* __restrict__ x, int64_t ld, int n) {
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (i < n) prep_row<ESZ>(runs[run], x + (size_t)i * ld, i, threadIdx.x & 31);
+}
+
+// The populations X[0] of every run (items: (run, 128-row tile)), 16 rows a CTA.
+template <int ESZ>
+__global__ void __launch_bounds__(256) k_prep_items(const RunDesc* __restrict__ runs, const int2* __restrict__ items) {
+  const int2 it = items[blockIdx.x >> 3];
+  const RunDesc& R = runs[it.x];
+  const int i0 = it.y * kTileM + 16 * (int)(blockIdx.x & 7);
+  for (int r = threadIdx.x >> 5; r < 16; r += 8)
+    if (i0 + r < R.np) prep_row<ESZ>(R, R.X[0] + (size_t)(i0 + r) * R.dp, i0 + r, threadIdx.x & 31);
+}
+
 // ------------------------------------------------------------------ fitness + selection kernel
 // mode 0: one generation (items = (run, 128-row tile)); mode 1: evaluation of
 // n_eval rows already converted by k_prep_rows, f written to fout; mode 2:
-// the same for the run's own population (n_eval = np), written as the
+// the same for the run's own population (n_eval = np, or -1 for each run's np), written as the
 // population's split fitness values with their error bounds (f, fx = 0, tau).
 //
 // MT = 2: a CTA takes two 128-row tiles (items = the run's tile pairs, 256
@@ -345,7 +358,7 @@ __global__ void __launch_bounds__(kFitThreads* MT, 1)
     return;
   }
   const int row0 = tile * kTileM;
-  const int nrows = max(0, min(kTileM, (mode == 0 ? R.np : n_eval) - row0));
+  const int nrows = max(0, min(kTileM, (mode == 0 || n_eval < 0 ? R.np : n_eval) - row0));
   const bool live = mt < ntile;  // a pair's second tile may be missing
 
   // per-thread epilogue state: row m (TMEM lane), column half h
@@ -1250,6 +1263,17 @@ void tc_init_eval_launch(const TcPlan& p, const RunDesc* runs, int run, const Ru
   } else {
     k_prep_rows<4><<<(R.np + 7) / 8, 256, 0, s>>>(runs, run, R.X[0], R.dp, R.np);
     k_fit_tc<4, 1><<<R.ntiles_tc, kFitThreads, p.smem_fit, s>>>(runs, items, 2, (double*)nullptr, R.np);
+  }
+}
+
+void tc_init_eval_all_launch(const TcPlan& p, const RunDesc* runs, cudaStream_t s) {
+  const int2* items = p.d_fit_items;
+  if (p.prec == DE_PREC_BF16X3) {
+    k_prep_items<2><<<8 * p.nitems_fit, 256, 0, s>>>(runs, items);
+    k_fit_tc<2, 1><<<p.nitems_fit, kFitThreads, p.smem_fit, s>>>(runs, items, 2, (double*)nullptr, -1);
+  } else {
+    k_prep_items<4><<<8 * p.nitems_fit, 256, 0, s>>>(runs, items);
+    k_fit_tc<4, 1><<<p.nitems_fit, kFitThreads, p.smem_fit, s>>>(runs, items, 2, (double*)nullptr, -1);
   }
 }
 
