@@ -11,9 +11,12 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <thread>
 #include <vector>
 
+#include <sys/mman.h>
 #include <sys/stat.h>
+#include <unistd.h>
 
 #include "de.h"
 #include "de_common.cuh"
@@ -51,6 +54,9 @@ struct de_handle {
   char* arena = nullptr;
   size_t arena_bytes = 0;
   RunState* h_state = nullptr;  // pinned mirror of the device states
+  bool state_fresh = false;     // nothing that changes the states was enqueued since the mirror was read
+  char* h_stage = nullptr;      // pinned staging of small populations (kStageBytes at most)
+  size_t stage_bytes = 0;
   cudaGraphExec_t graph = nullptr;
   int graph_gens = 0;
   Surrogate* surr = nullptr;  // surrogate-assisted generations (surrogate_k >= 2)
@@ -326,6 +332,7 @@ static void drop_graph(de_handle* h) {
 // (re)initialisation, a population change or a restore).
 static de_status islands_resync(de_handle* h) {
   if (!h->islands) return DE_OK;
+  h->state_fresh = false;
   h->isl.mig_gen = -1;
   h->isl.post_gen = -1;
   DE_CUDA(h, cudaMemcpyAsync(h->d_isl, &h->isl, sizeof(IslandCtl), cudaMemcpyHostToDevice, h->stream));
@@ -353,6 +360,11 @@ static de_status launch_generation(de_handle* h) { return launch_generation(h, h
 static de_status read_states(de_handle* h);
 
 static de_status enqueue_generations(de_handle* h, int64_t n) {
+  // whatever was read on the way, the mirror of the states is old at the end
+  struct Stale {
+    de_handle* h;
+    ~Stale() { h->state_fresh = false; }
+  } stale{h};
   if (h->surr) {
     // host-driven: each generation ends with the surrogate's screening decision
     for (int64_t k = 0; k < n; ++k) {
@@ -440,8 +452,13 @@ static de_status read_states(de_handle* h) {
   DE_CUDA(h, cudaMemcpyAsync(h->h_state, h->run[0].st, h->nruns * sizeof(RunState), cudaMemcpyDeviceToHost,
                              h->stream));
   DE_CUDA(h, cudaStreamSynchronize(h->stream));
+  h->state_fresh = true;
   return DE_OK;
 }
+
+// The mirror of the states, read only when something may have changed them
+// (a handle has one host thread at a time, and only its own calls change it).
+static de_status need_states(de_handle* h) { return h->state_fresh ? DE_OK : read_states(h); }
 
 static de_status check_device_errors(de_handle* h) {
   for (int r = 0; r < h->nruns; ++r) {
@@ -470,6 +487,7 @@ static size_t eval_smem(const de_handle* h, int run0, int n) {
 // stream and evaluate them, in one launch per step (a batch of 512 runs took
 // 3000 launches, 16 ms, run by run).
 static de_status init_runs(de_handle* h, int run0, int n) {
+  h->state_fresh = false;
   int np_max = 0, dp_max = 0;
   bool jde = false, plain = false;
   for (int r = run0; r < run0 + n; ++r) {
@@ -515,6 +533,7 @@ static de_status init_runs(de_handle* h, int run0, int n) {
 // FP64 when its stored value is not), and the mirror of the states read.
 static de_status exact_best(de_handle* h, int run0, int n) {
   if (h->prec == DE_PREC_FP64) return DE_OK;
+  h->state_fresh = false;
   int dp_max = 0;
   for (int r = run0; r < run0 + n; ++r) dp_max = std::max(dp_max, h->run[r].dp);
   k_best_exact_launch(h->d_run, run0, n, dp_max, h->stream);
@@ -1023,6 +1042,7 @@ de_status de_destroy(de_handle* h) {
   if (h->isl_mem) cudaFree(h->isl_mem);
   if (h->arena) cudaFree(h->arena);
   if (h->h_state) cudaFreeHost(h->h_state);
+  if (h->h_stage) cudaFreeHost(h->h_stage);
   delete h;
   return DE_OK;
 }
@@ -1580,19 +1600,77 @@ de_status de_get_shape(de_handle* h, int32_t run, int32_t* np, int32_t* d, int32
   return DE_OK;
 }
 
+// Host buffers up to this size come through pinned staging: two asynchronous
+// copies and one wait, where copies to pageable memory wait for each.
+static constexpr size_t kStageBytes = (size_t)2 << 20;
+
+// Large pageable destinations: map the pages first, on a few threads.  The
+// copy engine's faults on pages the caller has not touched yet (a fresh numpy
+// array) held a 65 MB copy to 1.2 GB/s; mapped, it runs at 40 GB/s.  Only whole
+// pages inside the buffer are touched, and their contents stay.
+static void map_pages(void* p, size_t bytes) {
+#ifndef MADV_POPULATE_WRITE
+#define MADV_POPULATE_WRITE 23
+#endif
+  const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+  const uintptr_t a = ((uintptr_t)p + page - 1) / page * page, e = ((uintptr_t)p + bytes) / page * page;
+  if (e <= a) return;
+  constexpr int kThreads = 8;
+  const size_t part = ((e - a) / kThreads + page - 1) / page * page;
+  auto touch = [=](int k) {
+    const uintptr_t x = a + (size_t)k * part, y = std::min(e, x + part);
+    if (x < y) madvise((void*)x, y - x, MADV_POPULATE_WRITE);  // on an error the copy faults as before
+  };
+  std::vector<std::thread> t;
+  try {
+    t.reserve(kThreads);
+    for (int k = 1; k < kThreads; ++k) t.emplace_back(touch, k);
+  } catch (...) {
+    // without (all) threads the remaining parts are mapped here
+    for (int k = (int)t.size() + 1; k < kThreads; ++k) touch(k);
+  }
+  touch(0);
+  for (auto& q : t) q.join();
+}
+
 de_status de_get_population(de_handle* h, int32_t run, double* x_host, double* f_host) {
   if (!h) return fail(nullptr, DE_ERR_INVALID_ARG, "handle is NULL");
   if (run < 0 || run >= h->nruns) return fail(h, DE_ERR_INVALID_ARG, "run out of range");
-  de_status s = read_states(h);
+  de_status s = need_states(h);
   if (s != DE_OK) return s;
   const RunDesc& R = h->run[run];
   const int cur = cur_buf(h, h->h_state[run].gen);
-  if (x_host)
-    DE_CUDA(h, cudaMemcpy2DAsync(x_host, R.d * sizeof(double), R.X[cur], R.dp * sizeof(double), R.d * sizeof(double),
-                                 R.np, cudaMemcpyDeviceToHost, h->stream));
-  if (f_host)
-    DE_CUDA(h, cudaMemcpyAsync(f_host, R.f[cur], R.np * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  const size_t row = (size_t)R.d * sizeof(double), xb = x_host ? row * R.np : 0;
+  const size_t fb = f_host ? (size_t)R.np * sizeof(double) : 0;
+  char* xd = (char*)x_host;
+  char* fd = (char*)f_host;
+  const bool staged = xb + fb <= kStageBytes;
+  if (staged && h->stage_bytes < xb + fb) {
+    if (h->h_stage) cudaFreeHost(h->h_stage);
+    h->h_stage = nullptr;
+    h->stage_bytes = 0;
+    size_t want = (size_t)64 << 10;
+    while (want < xb + fb) want *= 2;
+    DE_CUDA(h, cudaMallocHost((void**)&h->h_stage, want));
+    h->stage_bytes = want;
+  }
+  if (staged) {
+    xd = h->h_stage;
+    fd = h->h_stage + xb;
+  } else if (xb >= kStageBytes) {
+    map_pages(x_host, xb);
+  }
+  if (xb) {
+    if (R.d == R.dp)
+      DE_CUDA(h, cudaMemcpyAsync(xd, R.X[cur], xb, cudaMemcpyDeviceToHost, h->stream));
+    else
+      DE_CUDA(h, cudaMemcpy2DAsync(xd, row, R.X[cur], R.dp * sizeof(double), row, R.np, cudaMemcpyDeviceToHost,
+                                   h->stream));
+  }
+  if (fb) DE_CUDA(h, cudaMemcpyAsync(fd, R.f[cur], fb, cudaMemcpyDeviceToHost, h->stream));
   DE_CUDA(h, cudaStreamSynchronize(h->stream));
+  if (staged && xb) memcpy(x_host, xd, xb);
+  if (staged && fb) memcpy(f_host, fd, fb);
   return DE_OK;
 }
 
@@ -1615,6 +1693,7 @@ de_status de_set_population(de_handle* h, int32_t run, const double* x_host, con
   } else {
     k_eval_rows_launch(h->d_run, run, R, R.X[cur], R.dp, R.np, R.f[cur], R.fx[cur], h->stream);
   }
+  h->state_fresh = false;
   k_best_init_launch(h->d_run, run, 1, h->stream);
   DE_CUDA(h, cudaGetLastError());
   s = islands_resync(h);
@@ -1646,6 +1725,7 @@ de_status de_set_generation(de_handle* h, int32_t run, int64_t generation) {
   DE_CUDA(h, cudaMemcpyAsync(&R.st->gen, &generation, sizeof generation, cudaMemcpyHostToDevice, h->stream));
   int64_t ev = (int64_t)R.np * (1 + generation);
   DE_CUDA(h, cudaMemcpyAsync(&R.st->evals, &ev, sizeof ev, cudaMemcpyHostToDevice, h->stream));
+  h->state_fresh = false;
   k_best_init_launch(h->d_run, run, 1, h->stream);
   DE_CUDA(h, cudaGetLastError());
   s = islands_resync(h);
@@ -1914,6 +1994,7 @@ de_status de_load(de_handle* h, const char* path) {
     }
   }
   if (off != payload.size()) return fail(h, DE_ERR_IO, "checkpoint has trailing bytes");
+  h->state_fresh = false;
   for (int r = 0; r < h->nruns; ++r) {
     const RunDesc& R = h->run[r];
     RunCkpt& c = rc[r];
