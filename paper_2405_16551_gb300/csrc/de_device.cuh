@@ -393,6 +393,20 @@ struct Best {
   }
 };
 
+// The lowest key of the lanes and, among equals, the lowest index; a lane with
+// index -1 or a NaN key never wins.  Every lane returns the same (key, index).
+__device__ __forceinline__ void warp_best(long long& k, int& i) {
+  const bool on = i >= 0 && k != 0x7FFFFFFFFFFFFFFFLL;
+  const int hi = on ? (int)(k >> 32) : 0x7FFFFFFF;
+  const int mh = __reduce_min_sync(0xffffffffu, hi);
+  const unsigned lo = on && hi == mh ? (unsigned)k : 0xFFFFFFFFu;
+  const unsigned ml = __reduce_min_sync(0xffffffffu, lo);
+  const unsigned ix = on && hi == mh && (unsigned)k == ml ? (unsigned)i : 0xFFFFFFFFu;
+  const unsigned mi = __reduce_min_sync(0xffffffffu, ix);
+  k = ((long long)mh << 32) | (long long)ml;
+  i = (int)mi;  // -1 when no lane took part
+}
+
 // Finish a generation of a run: called by the last CTA to arrive.  Reduces
 // the tile partials in order (and, for the split precisions, the rows decided
 // in FP64 this generation, which carry no partial),
@@ -583,6 +597,31 @@ struct ChunkIn {
   U32x4 u;
 };
 
+// N consecutive coordinates of a row (N = 1, 2, 4; aligned to N doubles), read
+// at L2, and written.
+template <int N>
+__device__ __forceinline__ void ld_coords(const double* p, double (&v)[N]) {
+  if constexpr (N == 1) {
+    v[0] = __ldcg(p);
+  } else {
+#pragma unroll
+    for (int h = 0; h < N / 2; ++h) {
+      const double2 a = __ldcg(reinterpret_cast<const double2*>(p) + h);
+      v[2 * h] = a.x;
+      v[2 * h + 1] = a.y;
+    }
+  }
+}
+template <int N>
+__device__ __forceinline__ void st_coords(double* p, const double (&v)[N]) {
+  if constexpr (N == 1) {
+    *p = v[0];
+  } else {
+#pragma unroll
+    for (int h = 0; h < N / 2; ++h) reinterpret_cast<double2*>(p)[h] = make_double2(v[2 * h], v[2 * h + 1]);
+  }
+}
+
 // Issue the loads of chunk j0 (j0 < d, j0 % 4 == 0) and draw its block.
 // The rows are read at L2 (ld.global.cg): the persistent kernels read, in
 // generation g, population rows other CTAs wrote in generation g - 1, so the
@@ -604,15 +643,16 @@ __device__ __forceinline__ void trial_load(const RunDesc& R, const double* X, co
   }
 }
 
-// Coordinates j0 .. j0+3 of the trial from loaded inputs with weight F and
+// Coordinates j0 .. j0 + N - 1 of the trial from loaded inputs with weight F and
 // crossover threshold thr; entries at j >= d are 0.  L = 0: binomial
 // crossover (Eq. 3); L >= 1: exponential crossover of the cyclic block
 // j_rand .. j_rand + L - 1.  Returns the crossed-coordinate bits (bit m for
 // j0 + m).
-__device__ __forceinline__ uint32_t trial_compute(const RunDesc& R, const TrialSetup& s, int j0, const ChunkIn& c,
-                                                  double t[4], double F, uint64_t thr, int L) {
+template <int N>
+__device__ __forceinline__ uint32_t trial_coords(const RunDesc& R, uint32_t jr, int j0, const double (&xi)[N],
+                                                 const double (&x1)[N], const double (&x2)[N], const double (&x3)[N],
+                                                 const uint32_t (&u)[N], double* t, double F, uint64_t thr, int L) {
   const int d = R.d;
-  const uint32_t u[4] = {c.u.x, c.u.y, c.u.z, c.u.w};
   // u <= thr on 32 bits (thr = 2^32, CR = 1, crosses every coordinate, as
   // does the largest 32-bit value)
   const uint32_t thr32 = thr > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)thr;
@@ -620,21 +660,21 @@ __device__ __forceinline__ uint32_t trial_compute(const RunDesc& R, const TrialS
   // equal to a bound's (decided on all 64 bits below)
   uint32_t bits = 0, lowm = 0, highm = 0, eqm = 0;
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
+  for (int m = 0; m < N; ++m) {
     const int j = j0 + m;
     t[m] = 0.0;
     if (j < d) {
       bool crossed;
       if (L > 0) {
-        int off = j - (int)s.jr;
+        int off = j - (int)jr;
         if (off < 0) off += d;
         crossed = off < L;
       } else {
-        crossed = ((uint32_t)j == s.jr) || (u[m] <= thr32);
+        crossed = ((uint32_t)j == jr) || (u[m] <= thr32);
       }
       if (crossed) {
         // Eq. 2: y = x_r1 + F (x_r2 - x_r3), one rounding for the product-sum
-        const double v = __fma_rn(F, __dsub_rn(c.x2[m], c.x3[m]), c.x1[m]);
+        const double v = __fma_rn(F, __dsub_rn(x2[m], x3[m]), x1[m]);
         t[m] = v;
         bits |= 1u << m;
         // non-finite values land above hi (+NaN, +inf) or below lo
@@ -643,7 +683,7 @@ __device__ __forceinline__ uint32_t trial_compute(const RunDesc& R, const TrialS
         highm |= (uint32_t)(hk > R.hi_hk) << m;
         eqm |= (uint32_t)(hk == R.lo_hk || hk == R.hi_hk) << m;
       } else {
-        t[m] = c.xi[m];
+        t[m] = xi[m];
       }
     }
   }
@@ -659,7 +699,7 @@ __device__ __forceinline__ uint32_t trial_compute(const RunDesc& R, const TrialS
   if (__any_sync(__activemask(), (lowm | highm | eqm) != 0u)) {
     if (__any_sync(__activemask(), eqm != 0u)) {
 #pragma unroll
-      for (int m = 0; m < 4; ++m)
+      for (int m = 0; m < N; ++m)
         if ((eqm >> m) & 1u) {
           const long long kv = ordered_key(t[m]);
           lowm |= (uint32_t)(kv < R.lo_key) << m;
@@ -667,10 +707,17 @@ __device__ __forceinline__ uint32_t trial_compute(const RunDesc& R, const TrialS
         }
     }
 #pragma unroll
-    for (int m = 0; m < 4; ++m)
-      if (((lowm | highm) >> m) & 1u) t[m] = __fma_rn(0.5, c.xi[m], ((lowm >> m) & 1u) ? R.lo_half : R.hi_half);
+    for (int m = 0; m < N; ++m)
+      if (((lowm | highm) >> m) & 1u) t[m] = __fma_rn(0.5, xi[m], ((lowm >> m) & 1u) ? R.lo_half : R.hi_half);
   }
   return bits;
+}
+
+// A 4-coordinate chunk.
+__device__ __forceinline__ uint32_t trial_compute(const RunDesc& R, const TrialSetup& s, int j0, const ChunkIn& c,
+                                                  double t[4], double F, uint64_t thr, int L) {
+  const uint32_t u[4] = {c.u.x, c.u.y, c.u.z, c.u.w};
+  return trial_coords<4>(R, s.jr, j0, c.xi, c.x1, c.x2, c.x3, u, t, F, thr, L);
 }
 
 // DE/rand/1/bin with the run's F and CR.

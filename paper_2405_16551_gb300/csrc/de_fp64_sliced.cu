@@ -40,21 +40,10 @@ namespace de {
 
 constexpr long long kSlicedSpin = 1LL << 22;  // polls of the grid barrier (each a round trip to L2: seconds in all)
 
-// The lowest key of the lanes and, among equals, the lowest index; a lane with
-// index -1 or a NaN key never wins.  Every lane returns the same (key, index).
-__device__ __forceinline__ void warp_best(long long& k, int& i) {
-  const bool on = i >= 0 && k != 0x7FFFFFFFFFFFFFFFLL;
-  const int hi = on ? (int)(k >> 32) : 0x7FFFFFFF;
-  const int mh = __reduce_min_sync(0xffffffffu, hi);
-  const unsigned lo = on && hi == mh ? (unsigned)k : 0xFFFFFFFFu;
-  const unsigned ml = __reduce_min_sync(0xffffffffu, lo);
-  const unsigned ix = on && hi == mh && (unsigned)k == ml ? (unsigned)i : 0xFFFFFFFFu;
-  const unsigned mi = __reduce_min_sync(0xffffffffu, ix);
-  k = ((long long)mh << 32) | (long long)ml;
-  i = (int)mi;  // -1 when no lane took part
-}
-
-template <bool ISL, bool UNIT>
+// CPL: coordinates per lane (1, 2 or 4: d <= 32, 64, 128).  An FP64 instruction
+// costs its unit the same however few lanes are active, so short rows take one
+// coordinate a lane, not four on a quarter of the lanes.
+template <bool ISL, bool UNIT, int CPL>
 __global__ void __launch_bounds__(256, 1)
     k_gen_sliced(const RunDesc* __restrict__ runs, const int4* __restrict__ items, int nruns, PersistCtl* ctl,
                  long long gens, IslandCtl* isl, IslandStage stage, int kpad, uint32_t cols) {
@@ -96,31 +85,24 @@ __global__ void __launch_bounds__(256, 1)
   // ---- this warp's target: its row, fitness and the lane's part of the shift
   const bool mine = warp < nrows;
   const uint32_t i = (uint32_t)(it.z + warp);
-  const int j0 = 4 * lane;
+  const int j0 = CPL * lane;
   const bool in = mine && j0 < d;
-  double tx[4] = {0.0, 0.0, 0.0, 0.0}, tr[4] = {0.0, 0.0, 0.0, 0.0}, o4[4] = {0.0, 0.0, 0.0, 0.0}, fi = 0.0;
+  double tx[CPL] = {}, tr[CPL] = {}, ov[CPL] = {}, fi = 0.0;
   long long gen = *(volatile int64_t*)&st->gen;
   auto load_row = [&](int cur) {
-    if (in) {
-      const double2* p = reinterpret_cast<const double2*>(R.X[cur] + (size_t)i * dp + j0);
-      const double2 a = __ldcg(p), b = __ldcg(p + 1);
-      tx[0] = a.x;
-      tx[1] = a.y;
-      tx[2] = b.x;
-      tx[3] = b.y;
-    }
+    if (in) ld_coords(R.X[cur] + (size_t)i * dp + j0, tx);
     if (mine) fi = __ldcg(R.f[cur] + i);
   };
 #pragma unroll
-  for (int m = 0; m < 4; ++m)
-    if (in && j0 + m < d) o4[m] = R.o[j0 + m];
+  for (int m = 0; m < CPL; ++m)
+    if (in && j0 + m < d) ov[m] = R.o[j0 + m];
   load_row((int)(gen & 1));
   TrialSetup ts{};
   U32x4 ub{};
   auto draw = [&](long long g) {
     if (mine) {
       ts = trial_setup(R, i, g, lane, 0u, false);
-      if (in) ub = draw_block(R.seed, kPurposeStep, R.run_id, 0u, (uint32_t)g, i, 1u + (uint32_t)lane);
+      if (in) ub = draw_block(R.seed, kPurposeStep, R.run_id, 0u, (uint32_t)g, i, 1u + (uint32_t)(j0 >> 2));
     }
   };
   if (!s_stop) draw(gen + 1);
@@ -217,43 +199,26 @@ __global__ void __launch_bounds__(256, 1)
     const long long g = gen + 1;
     const bool more = itg < gens;
     // ---- the donors' loads, then (one warp) the last generation's decision
-    double x1[4], x2[4], x3[4];
+    double x1[CPL], x2[CPL], x3[CPL];
     if (live && more && in) {
       const double* X = R.X[gen & 1] + j0;
-      const double2* p1 = reinterpret_cast<const double2*>(X + (size_t)ts.r1 * dp);
-      const double2* p2 = reinterpret_cast<const double2*>(X + (size_t)ts.r2 * dp);
-      const double2* p3 = reinterpret_cast<const double2*>(X + (size_t)ts.r3 * dp);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const double2 a = __ldcg(p1 + h), b = __ldcg(p2 + h), c = __ldcg(p3 + h);
-        x1[2 * h] = a.x;
-        x1[2 * h + 1] = a.y;
-        x2[2 * h] = b.x;
-        x2[2 * h + 1] = b.y;
-        x3[2 * h] = c.x;
-        x3[2 * h + 1] = c.y;
-      }
+      ld_coords(X + (size_t)ts.r1 * dp, x1);
+      ld_coords(X + (size_t)ts.r2 * dp, x2);
+      ld_coords(X + (size_t)ts.r3 * dp, x3);
     }
     // (counted in the slot of the iteration that ran generation gen)
     if (pending && warp == rw) reduce_best(gen, (int)((itg + 2) % 3));
     // ---- trials: Eq. 2, Eq. 3, bound repair; y = (t - o) s as digits
     if (live && more && mine) {
-      double y[4] = {0.0, 0.0, 0.0, 0.0};
+      double y[CPL] = {};
       if (in) {
-        ChunkIn c;
-        c.u = ub;
+        uint32_t u[CPL];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          c.xi[m] = tx[m];
-          c.x1[m] = x1[m];
-          c.x2[m] = x2[m];
-          c.x3[m] = x3[m];
-        }
-        trial_compute(R, ts, j0, c, tr);
+        for (int m = 0; m < CPL; ++m) u[m] = word_of(ub, (j0 + m) & 3);
+        trial_coords<CPL>(R, ts.jr, j0, tx, x1, x2, x3, u, tr, R.F, R.cr_thr, 0);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) y[m] = j0 + m < d ? shifted_as<UNIT>(tr[m], o4[m], R.scale) : 0.0;
-        *reinterpret_cast<double2*>(Y + warp * dp + j0) = make_double2(y[0], y[1]);
-        *reinterpret_cast<double2*>(Y + warp * dp + j0 + 2) = make_double2(y[2], y[3]);
+        for (int m = 0; m < CPL; ++m) y[m] = j0 + m < d ? shifted_as<UNIT>(tr[m], ov[m], R.scale) : 0.0;
+        st_coords(Y + warp * dp + j0, y);
       }
       slice_digits(sc, warp, lane, R.sl_kpad, R.sl_qmin[0], y);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -274,13 +239,9 @@ __global__ void __launch_bounds__(256, 1)
         if (acc) {
           fi = ft;
 #pragma unroll
-          for (int m = 0; m < 4; ++m) tx[m] = tr[m];
+          for (int m = 0; m < CPL; ++m) tx[m] = tr[m];
         }
-        if (in) {
-          double2* q = reinterpret_cast<double2*>(R.X[g & 1] + (size_t)i * dp + j0);
-          q[0] = make_double2(tx[0], tx[1]);
-          q[1] = make_double2(tx[2], tx[3]);
-        }
+        if (in) st_coords(R.X[g & 1] + (size_t)i * dp + j0, tx);
         if (lane == 0) {
           R.f[g & 1][i] = fi;
           s_f[warp] = fi;
@@ -377,15 +338,18 @@ __global__ void __launch_bounds__(256, 1)
 }
 
 // ------------------------------------------------------------------ host side
-static const void* sliced_kernel(bool isl, bool unit) {
-  if (isl) return unit ? (const void*)k_gen_sliced<true, true> : (const void*)k_gen_sliced<true, false>;
-  return unit ? (const void*)k_gen_sliced<false, true> : (const void*)k_gen_sliced<false, false>;
+static const void* sliced_kernel(bool isl, bool unit, int kpad) {
+#define DE_SLICED(c)                                                                                       \
+  (isl ? (unit ? (const void*)k_gen_sliced<true, true, c> : (const void*)k_gen_sliced<true, false, c>)     \
+       : (unit ? (const void*)k_gen_sliced<false, true, c> : (const void*)k_gen_sliced<false, false, c>))
+  return kpad <= 32 ? DE_SLICED(1) : kpad <= 64 ? DE_SLICED(2) : DE_SLICED(4);
+#undef DE_SLICED
 }
 
 // All of an SM's shared memory, as the sliced instances of the general
 // cooperative kernel take (fp64_exclusive_smem).
-int k_gen_sliced_capacity(bool isl, bool unit, size_t smem) {
-  const void* k = sliced_kernel(isl, unit);
+int k_gen_sliced_capacity(bool isl, bool unit, const SlicePlan& p, size_t smem) {
+  const void* k = sliced_kernel(isl, unit, p.kpad);
   const size_t dyn = fp64_exclusive_smem(k, smem);
   int per_sm = 0, dev = 0, nsm = 0;
   cudaGetDevice(&dev);
@@ -413,7 +377,7 @@ cudaError_t k_gen_sliced_launch(const RunDesc* runs, const int4* items, int nite
   uint32_t cols = p.cols;
   void* args[] = {(void*)&runs, (void*)&items, (void*)&nruns, (void*)&ctl, (void*)&gens,
                   (void*)&isl,  (void*)&st,    (void*)&kpad,  (void*)&cols};
-  const void* k = sliced_kernel(isl != nullptr, unit);
+  const void* k = sliced_kernel(isl != nullptr, unit, p.kpad);
   return cudaLaunchCooperativeKernel(k, dim3((unsigned)nitems), dim3(256), args, fp64_exclusive_smem(k, smem), s);
 }
 

@@ -74,7 +74,7 @@ size_t fp64_exclusive_smem(const void* k, size_t smem);
 // the generation loop of plain DE/rand/1/bin runs that are all sliced
 // (de_fp64_sliced.cu); unit: every run's scale is 1
 size_t sliced_loop_smem(const SlicePlan& p, int dp_max);
-int k_gen_sliced_capacity(bool isl, bool unit, size_t smem);
+int k_gen_sliced_capacity(bool isl, bool unit, const SlicePlan& p, size_t smem);
 struct IslandCtl;
 struct IslandStage;
 cudaError_t k_gen_sliced_launch(const RunDesc* runs, const int4* items, int nitems, int nruns, PersistCtl* ctl,

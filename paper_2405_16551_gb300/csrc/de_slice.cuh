@@ -176,14 +176,16 @@ __device__ __forceinline__ void slice_end(SliceCtx& c) {
 }
 
 // Digits of one row of y into row r of the tile (one warp; lane L holds
-// coordinates 4 L .. 4 L + 3, zero past d).
+// coordinates N L .. N L + N - 1, zero past d; N = 1, 2 or 4, 32 N >= kpad).
+template <int N>
 __device__ __forceinline__ void slice_digits(const SliceCtx& c, int r, int lane, int kpad, int qmin,
-                                             const double (&y)[4]) {
-  uint32_t hw[4], mx = 0u;
+                                             const double (&y)[N]) {
+  uint32_t hw[N], mx = 0u, any = 0u;
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
+  for (int m = 0; m < N; ++m) {
     hw[m] = (uint32_t)__double2hiint(y[m]) & 0x7FFFFFFFu;
     mx = max(mx, hw[m]);
+    any |= (uint32_t)__double2loint(y[m]);
   }
   mx = __reduce_max_sync(0xffffffffu, mx);
   const int ex = (int)(mx >> 20);  // 2^(ex - 1022) exceeds every |y_k|
@@ -191,19 +193,18 @@ __device__ __forceinline__ void slice_digits(const SliceCtx& c, int r, int lane,
   const uint32_t thr = mx > (6u << 20) ? mx - (6u << 20) : 1u;
   int q = 0;
 #pragma unroll
-  for (int m = 0; m < 4; ++m) q += __popc(__ballot_sync(0xffffffffu, hw[m] >= thr));
+  for (int m = 0; m < N; ++m) q += __popc(__ballot_sync(0xffffffffu, hw[m] >= thr));
   // a row of zeros is exact; z stays in the normal range for e in [-800, 800]
-  const bool zero = mx == 0u && __all_sync(0xffffffffu, ((__double2loint(y[0]) | __double2loint(y[1]) |
-                                                         __double2loint(y[2]) | __double2loint(y[3])) == 0));
+  const bool zero = mx == 0u && __all_sync(0xffffffffu, any == 0u);
   const bool bad = !zero && (q < qmin || ex < 1022 - 800 || ex > 1022 + 800);
   if (lane == 0) {
     c.s_exp[r] = ex - 1022;
     if (bad) atomicOr(c.s_bad, 1u << r);
   }
-  if (4 * lane >= kpad) return;
-  uint32_t lo[4], hi[4];
+  if (N * lane >= kpad) return;
+  uint32_t lo[N], hi[N];
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
+  for (int m = 0; m < N; ++m) {
     const long long b = __double_as_longlong(y[m]);
     const int ek = (int)(hw[m] >> 20);
     // significand at bits 9 .. 61, shifted down to the row's exponent with
@@ -219,19 +220,26 @@ __device__ __forceinline__ void slice_digits(const SliceCtx& c, int r, int lane,
   // byte s of v (from the top) is digit s plus 128; in the low byte of
   // 2^23 + byte, minus 2^23 + 128, it is the digit in FP32, whose upper half
   // is its exact BF16 form
-  uint8_t* dst = c.sB + (uint32_t)(lane >> 1) * kSliceKg + (uint32_t)r * 16u + (uint32_t)(lane & 1) * 8u;
+  const uint32_t k0 = (uint32_t)(N * lane);
+  uint8_t* dst = c.sB + (k0 >> 3) * kSliceKg + (uint32_t)r * 16u + (k0 & 7u) * 2u;
 #pragma unroll
   for (int s = 0; s < kSlices; ++s) {
-    float f[4];
+    float f[N];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
+    for (int m = 0; m < N; ++m) {
       const uint32_t w = s < 4 ? hi[m] : lo[m];
       f[m] = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7550u | (uint32_t)(3 - (s & 3)))) - 8388736.0f;
     }
-    uint2 p;
-    p.x = __byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632u);
-    p.y = __byte_perm(__float_as_uint(f[2]), __float_as_uint(f[3]), 0x7632u);
-    *reinterpret_cast<uint2*>(dst + s * 128) = p;
+    if constexpr (N == 1) {
+      *reinterpret_cast<uint16_t*>(dst + s * 128) = (uint16_t)(__float_as_uint(f[0]) >> 16);
+    } else if constexpr (N == 2) {
+      *reinterpret_cast<uint32_t*>(dst + s * 128) = __byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632u);
+    } else {
+      uint2 p;
+      p.x = __byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632u);
+      p.y = __byte_perm(__float_as_uint(f[2]), __float_as_uint(f[3]), 0x7632u);
+      *reinterpret_cast<uint2*>(dst + s * 128) = p;
+    }
   }
 }
 
