@@ -591,12 +591,16 @@ DE_API de_status de_get_shape(de_handle* h, int32_t run, int32_t* np, int32_t* d
  *      stop run inside the loop, an extra grid barrier after each migration,
  *      except for the benchmark suite's objectives 5..20, whose islands run
  *      on path 0), or, for one run of at most 8
- *      tiles, the same loop as one thread-block cluster (cluster barrier);
+ *      tiles, the same loop as one thread-block cluster (cluster barrier), or,
+ *      for plain DE/rand/1/bin runs of objectives 0..3 with np <= 64 and
+ *      d <= 32 (d <= 64 with a rotation that runs as digit products), a
+ *      cluster per run with the population in shared memory;
  *      the FP64 autotuner chooses among path 0 and these when one times
- *      faster on the handle's problem; DE_GB300_FP64_PERSIST=0 / 1 / 2 forces
- *      path 0 / the cooperative launch / the cluster (where it applies)
+ *      faster on the handle's problem; DE_GB300_FP64_PERSIST=0 / 1 / 2 / 3 forces
+ *      path 0 / the cooperative launch / the cluster / the cluster per run
+ *      (where it applies)
  * cluster_size (may be NULL) receives the CTAs per cluster of path 2 or of
- * path 3 launched as one cluster, else 0;
+ * path 3 launched as clusters, else 0;
  * each cluster owns up to 128 targets (a multiple of the cluster size, timed
  * at de_init; DE_GB300_PERSIST_ROWS fixes it).
  * Paths 2 and 4 apply to a single run, path 2 of d <= 105 (its FP64 band

@@ -63,6 +63,9 @@ struct de_handle {
   bool variants = false;      // some run uses a strategy variant or jDE
   bool suite = false;         // some run uses an objective of the proposed benchmark (5..20)
   bool fp64_persist = false;  // FP64: every generation of a call in one cooperative launch
+  bool fp64_local = false;    // FP64: the same, a cluster per run with the population in shared memory
+  bool isl_even = true;       // the islands' generations and stop flags are known to agree
+  LocalPlan local;
   bool fp64_cluster = false;  // ... launched as one thread-block cluster (one run of at most 8 tiles)
   PersistCtl* d_ctl64 = nullptr;
   // island model (de_init_islands): the runs are islands on a migration ring
@@ -358,6 +361,28 @@ static de_status launch_generation(de_handle* h, cudaStream_t s) {
 static de_status launch_generation(de_handle* h) { return launch_generation(h, h->stream); }
 
 static de_status read_states(de_handle* h);
+static de_status need_states(de_handle* h);
+
+// Whether this call's generations run in the local form.  Its islands advance
+// together; islands whose states a call has set apart (one island reset or
+// given a generation of its own) run on the other forms, and so do islands
+// under the caller's stream capture (the graph may be replayed after such a call).
+static de_status use_local(de_handle* h, bool& use) {
+  use = true;
+  if (!h->islands) return DE_OK;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  DE_CUDA(h, cudaStreamIsCapturing(h->stream, &cap));
+  use = cap == cudaStreamCaptureStatusNone;
+  if (!use || h->isl_even) return DE_OK;
+  const de_status s = need_states(h);
+  if (s != DE_OK) return s;
+  h->isl_even = true;
+  for (int r = 1; r < h->nruns; ++r)
+    h->isl_even = h->isl_even && h->h_state[r].gen == h->h_state[0].gen && h->h_state[r].stop == h->h_state[0].stop &&
+                  h->h_state[r].evals == h->h_state[0].evals;
+  use = h->isl_even;
+  return DE_OK;
+}
 
 static de_status enqueue_generations(de_handle* h, int64_t n) {
   // whatever was read on the way, the mirror of the states is old at the end
@@ -376,12 +401,20 @@ static de_status enqueue_generations(de_handle* h, int64_t n) {
     }
     return DE_OK;
   }
-  if (h->fp64_persist) {
+  bool local = false;
+  if (h->fp64_local) {
+    const de_status s = use_local(h, local);
+    if (s != DE_OK) return s;
+  }
+  if (h->fp64_persist || local) {
     // one cooperative (or one-cluster) launch runs up to 2^20 generations (or
     // stops early)
     for (int64_t left = n; left > 0; left -= (int64_t)1 << 20) {
       const long long g = std::min<int64_t>(left, (int64_t)1 << 20);
-      if (h->fp64_cluster)
+      if (local)
+        DE_CUDA(h, k_gen_local_launch(h->d_run, h->nruns, h->local, h->d_ctl64, g, h->stream, h->test_grid_skip,
+                                      h->islands ? h->d_isl : nullptr, h->islands ? &h->stage : nullptr));
+      else if (h->fp64_cluster)
         DE_CUDA(h, k_gen_fp64_cluster_launch(h->d_run, h->d_items, h->nitems, h->threads, h->smem_gen, h->variants,
                                              h->suite, h->d_ctl64, g, h->stream, h->slices));
       else if (h->sliced_loop)
@@ -560,7 +593,7 @@ static std::string tune_key(const de_handle* h) {
     sum_d += (long long)R.np * R.d;
   }
   char b[256];
-  snprintf(b, sizeof b, "gen_fp64v5 runs=%d np0=%d d0=%d obj0=%d rot0=%d sumnp=%lld sumnd=%lld", h->nruns, h->run[0].np,
+  snprintf(b, sizeof b, "gen_fp64v6 runs=%d np0=%d d0=%d obj0=%d rot0=%d sumnp=%lld sumnd=%lld", h->nruns, h->run[0].np,
            h->run[0].d, h->run[0].obj, h->run[0].rotate, sum_np, sum_d);
   return b;
 }
@@ -662,6 +695,15 @@ static bool fp64_cluster_ok(const de_handle* h) {
          k_gen_fp64_cluster_fits(h->nitems, h->threads, h->smem_gen, h->variants, h->suite, h->slices);
 }
 
+// ... and as a cluster per run with the population in shared memory: small
+// runs of plain DE (local_plan).
+static bool fp64_local_ok(const de_handle* h) {
+  if (h->prec != DE_PREC_FP64 || h->surr || !h->d_ctl64 || h->local.csize == 0) return false;
+  if (const char* e = getenv("DE_GB300_FP64_PERSIST"))
+    if (e[0] != '3') return false;
+  return local_fits(h->local, h->nruns, h->islands);
+}
+
 static de_status autotune_fp64(de_handle* h, int nsm) {
   const char* env = getenv("DE_GB300_AUTOTUNE");
   const bool enabled = !(env && env[0] == '0');
@@ -671,10 +713,12 @@ static de_status autotune_fp64(de_handle* h, int nsm) {
   int cached = 0;
   if (tune_lookup(key, cached)) {
     // value: rows per tile, plus 100 x the mode that won (0: one kernel per
-    // generation, 1: cooperative persistent kernel, 2: the same as one cluster)
+    // generation, 1: cooperative persistent kernel, 2: the same as one cluster,
+    // 3: a cluster per run with the population in shared memory)
     h->rows = cached % 100;
     h->fp64_persist = cached >= 100;
-    h->fp64_cluster = cached >= 200;
+    h->fp64_cluster = cached >= 200 && cached < 300;
+    h->fp64_local = cached >= 300;
     return DE_OK;
   }
   // candidates are timed on the freshly initialised problem, which is then
@@ -714,15 +758,17 @@ static de_status autotune_fp64(de_handle* h, int nsm) {
       best_rows = rows;
       best_mode = 0;
     }
-    // the same tiles in one cooperative launch, and as one cluster
-    for (int mode = 1; mode <= 2 && st_all == DE_OK; ++mode) {
-      if (mode == 1 ? !fp64_persist_ok(h) : !fp64_cluster_ok(h)) continue;
+    // the same tiles in one cooperative launch, and as one cluster; the local
+    // form (which has no tiles) once
+    for (int mode = 1; mode <= 3 && st_all == DE_OK; ++mode) {
+      if (mode == 3 ? rows != 8 || !fp64_local_ok(h) : mode == 1 ? !fp64_persist_ok(h) : !fp64_cluster_ok(h)) continue;
       for (int r = 0; r < h->nruns; ++r) {
         int32_t zero = 0;
         DE_CUDA(h, cudaMemcpyAsync(&h->run[r].st->stop, &zero, sizeof zero, cudaMemcpyHostToDevice, h->stream));
       }
-      h->fp64_persist = true;
+      h->fp64_persist = mode <= 2;
       h->fp64_cluster = mode == 2;
+      h->fp64_local = mode == 3;
       st_all = enqueue_generations(h, 2);
       if (st_all == DE_OK) {
         DE_CUDA(h, cudaEventRecord(e0, h->stream));
@@ -733,9 +779,10 @@ static de_status autotune_fp64(de_handle* h, int nsm) {
       }
       h->fp64_persist = false;
       h->fp64_cluster = false;
+      h->fp64_local = false;
       if (st_all == DE_OK && ms < best_ms * 0.97f) {
         best_ms = ms;
-        best_rows = rows;
+        best_rows = mode == 3 ? heuristic_rows(h, nsm) : rows;
         best_mode = mode;
       }
     }
@@ -753,7 +800,9 @@ static de_status autotune_fp64(de_handle* h, int nsm) {
   h->rows = best_rows;
   h->fp64_persist = best_mode >= 1;
   h->fp64_cluster = best_mode == 2;
-  tune_store(key, best_rows + 100 * best_mode);
+  h->fp64_local = best_mode == 3;
+  // a choice among the forms that the environment left is not everyone's
+  if (!getenv("DE_GB300_FP64_PERSIST")) tune_store(key, best_rows + 100 * best_mode);
   return DE_OK;
 }
 
@@ -1368,6 +1417,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
     }
     h->smem_loop = sliced_loop_smem(h->slices, dp_max);
   }
+  if (h->prec == DE_PREC_FP64 && !h->variants && !h->suite) local_plan(h->local, h->run, h->slices);
   if (h->prec != DE_PREC_FP64) {
     TRY(tc_plan_build(h->tc, h->run, cfgs, h->prec, h->stream, h->err));
     h->dbuf = h->tc.persist.ok;
@@ -1385,10 +1435,13 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
     TRY(upload_desc(h));
     k_configure(h->smem_gen);
     if (const char* e = getenv("DE_GB300_FP64_PERSIST")) {
-      // forced on where it applies: 1 cooperative launch, 2 one cluster
-      if (e[0] == '1' || e[0] == '2') h->fp64_persist = true;
+      // forced on where it applies: 1 cooperative launch, 2 one cluster, 3 a
+      // cluster per run (else the cooperative launch)
+      if (e[0] >= '1' && e[0] <= '3') h->fp64_persist = true;
       h->fp64_cluster = e[0] == '2';
+      h->fp64_local = e[0] == '3';
     }
+    if (h->fp64_local && !fp64_local_ok(h)) h->fp64_local = false;
     if (h->fp64_cluster && !fp64_cluster_ok(h)) h->fp64_cluster = false;
     if (h->fp64_persist && !fp64_persist_ok(h)) h->fp64_persist = h->fp64_cluster = false;
     // the failure-detection test applies to the generations after set-up
@@ -1435,6 +1488,7 @@ de_status de_reset(de_handle* h, int32_t run) {
   h->err.clear();
   const de_status st = run < 0 ? init_runs(h, 0, h->nruns) : init_runs(h, run, 1);
   if (st != DE_OK) return st;
+  h->isl_even = run < 0;
   if (h->surr) {
     const de_status s = surr_reset(*h->surr, h->stream, h->err);
     if (s != DE_OK) return fail(h, s, h->err);
@@ -1498,6 +1552,7 @@ de_status de_init_islands_ex(const de_config* cfg, int32_t nislands, int32_t int
   // are at least two runs); otherwise migration runs between generations
   h->fp64_cluster = false;
   h->fp64_persist = h->fp64_persist && fp64_persist_ok(h);
+  h->fp64_local = h->fp64_local && fp64_local_ok(h);
   drop_graph(h);
   st = islands_resync(h);
   if (st == DE_OK) {
@@ -1538,7 +1593,8 @@ de_status de_run(de_handle* h, de_result* out) {
       }
     if (all) break;
     // the persistent kernels stop the run themselves: one launch
-    const bool persistent = h->fp64_persist || (h->prec != DE_PREC_FP64 && (h->tc.persist.ok || h->pbatch_on));
+    const bool persistent = h->fp64_persist || (h->fp64_local && !h->islands) ||
+                            (h->prec != DE_PREC_FP64 && (h->tc.persist.ok || h->pbatch_on));
     s = enqueue_generations(h, std::max<int64_t>(1, persistent ? left : std::min<int64_t>(chunk, left)));
     if (s != DE_OK) return s;
     s = read_states(h);
@@ -1693,7 +1749,7 @@ de_status de_set_population(de_handle* h, int32_t run, const double* x_host, con
   } else {
     k_eval_rows_launch(h->d_run, run, R, R.X[cur], R.dp, R.np, R.f[cur], R.fx[cur], h->stream);
   }
-  h->state_fresh = false;
+  h->state_fresh = h->isl_even = false;
   k_best_init_launch(h->d_run, run, 1, h->stream);
   DE_CUDA(h, cudaGetLastError());
   s = islands_resync(h);
@@ -1725,7 +1781,7 @@ de_status de_set_generation(de_handle* h, int32_t run, int64_t generation) {
   DE_CUDA(h, cudaMemcpyAsync(&R.st->gen, &generation, sizeof generation, cudaMemcpyHostToDevice, h->stream));
   int64_t ev = (int64_t)R.np * (1 + generation);
   DE_CUDA(h, cudaMemcpyAsync(&R.st->evals, &ev, sizeof ev, cudaMemcpyHostToDevice, h->stream));
-  h->state_fresh = false;
+  h->state_fresh = h->isl_even = false;
   k_best_init_launch(h->d_run, run, 1, h->stream);
   DE_CUDA(h, cudaGetLastError());
   s = islands_resync(h);
@@ -1833,12 +1889,14 @@ de_status de_get_plan(de_handle* h, int32_t* kernel_path, int32_t* cluster_size)
   if (!h) return fail(nullptr, DE_ERR_INVALID_ARG, "handle is NULL");
   const bool persist = h->prec != DE_PREC_FP64 && h->tc.persist.ok;
   if (kernel_path)
-    *kernel_path = h->prec == DE_PREC_FP64 ? (h->fp64_persist ? 3 : 0)
+    *kernel_path = h->prec == DE_PREC_FP64 ? (h->fp64_persist || h->fp64_local ? 3 : 0)
                    : h->pbatch_on         ? 5
                                            : (persist ? (h->tc.persist.mode == 1 ? 4 : 2) : 1);
   if (cluster_size)
     *cluster_size = persist ? (h->tc.persist.mode == 1 ? 0 : h->tc.persist.C)
-                            : (h->prec == DE_PREC_FP64 && h->fp64_cluster ? h->nitems : 0);
+                            : h->prec != DE_PREC_FP64 ? 0
+                            : h->fp64_local           ? h->local.csize
+                                                      : (h->fp64_cluster ? h->nitems : 0);
   return DE_OK;
 }
 
@@ -1994,7 +2052,7 @@ de_status de_load(de_handle* h, const char* path) {
     }
   }
   if (off != payload.size()) return fail(h, DE_ERR_IO, "checkpoint has trailing bytes");
-  h->state_fresh = false;
+  h->state_fresh = h->isl_even = false;
   for (int r = 0; r < h->nruns; ++r) {
     const RunDesc& R = h->run[r];
     RunCkpt& c = rc[r];

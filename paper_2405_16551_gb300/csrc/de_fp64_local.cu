@@ -1,0 +1,477 @@
+// de_fp64_local.cu -- the FP64 generation loop of small runs, a thread-block
+// cluster per run with the population in shared memory.
+//
+// A run of at most 64 targets of at most 64 coordinates is a chain of latencies:
+// NP = 64, D = 10 (sphere) took 6.35 us a generation in the general loop, for
+// 0.1 us of FP64 work, in trips to L2 (donors, partials, fitness), barriers, and
+// FP64 instructions on 3 of 32 lanes; here it takes 2.55 us.
+//   - every CTA of the run's cluster (at most 8, a warp per target) keeps a copy
+//     of the whole population in shared memory, double buffered: donors are
+//     local loads; a target's next row goes to every CTA's copy through
+//     distributed shared memory, with its fitness key;
+//   - the one synchronisation of a generation is the cluster barrier (the next
+//     generation's draws are made between arriving and waiting); after it every
+//     warp takes the best record and the stop decision from the keys itself;
+//   - a lane holds one coordinate (two for d > 32): an FP64 instruction costs
+//     the same however few lanes are active.
+// Populations, fitness and state go to global memory at the end of the launch
+// and at migrations.  The numbers are those of the general kernels: the same
+// trial, rotation (sliced, or the DFMA chain for the others) and term routines,
+// and the same order of every sum.
+//
+// ISL: the runs are islands.  The model stops as a whole at the first
+// generation in which some island's best is below the target; an island learns
+// of that one generation late (the counter it would have to wait for has had
+// a generation's time to fill), and then takes back its last one, whose
+// predecessor is still in the other buffer.  At migration points the islands
+// meet (bounded waits on global counters), and the exchange runs on the
+// populations in global memory as in the other kernels.
+#include <cooperative_groups.h>
+#include <cuda_runtime.h>
+#include <math_constants.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "de_common.cuh"
+#include "de_device.cuh"
+#include "de_gen_tile.cuh"
+#include "de_internal.cuh"
+#include "de_island_dev.cuh"
+#include "de_kernels.h"
+#include "de_slice.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace de {
+
+constexpr int kLocalNp = 64;                // targets of a run (8 CTAs of 8 warps)
+constexpr long long kLocalSpin = 1LL << 22;  // polls of an island counter (each a round trip to L2)
+
+// Byte offsets of a CTA's dynamic shared memory: operands of the sliced
+// rotation (SL), FP64 rows of y and of the rows that take the chain, the two
+// population buffers, M^T (not SL).
+struct LocalLayout {
+  uint32_t y, z, pop, mt, total;
+};
+__host__ __device__ inline LocalLayout local_layout(bool sl, int kpad, int dp, int d, bool rotate) {
+  LocalLayout L;
+  L.y = sl ? slice_smem(kpad) : 0u;
+  L.z = L.y + (uint32_t)(kSliceRows * dp) * 8u;
+  L.pop = L.z + (sl ? (uint32_t)(kSliceRows * dp) * 8u : 0u);
+  L.mt = L.pop + 2u * (uint32_t)(kLocalNp * dp) * 8u;
+  L.total = L.mt + (!sl && rotate ? (uint32_t)(d * d) * 8u : 0u);
+  return L;
+}
+
+template <int CPL, bool SL, bool ISL>
+__global__ void __launch_bounds__(256, 1)
+    k_gen_local(const RunDesc* __restrict__ runs, PersistCtl* ctl, long long gens, int csize, IslandCtl* isl,
+                IslandStage stage, int kpad, uint32_t cols, int dp_max) {
+  extern __shared__ __align__(1024) uint8_t smem_l[];
+  __shared__ SliceShared s_sl;
+  __shared__ RunDesc sR;
+  __shared__ long long s_key[2][kLocalNp];
+  // by generation parity: 1 the model had stopped before it, 2 a wait gave up;
+  // nonzero when a CTA's products did
+  __shared__ int s_flag[2], s_fail[2];
+  __shared__ int s_over;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int run = (int)blockIdx.x / csize, rank = (int)blockIdx.x % csize;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  load_desc(sR, runs + run);
+  if (tid < 2) s_flag[tid] = s_fail[tid] = 0;
+  if (tid < 2 * kLocalNp) s_key[tid / kLocalNp][tid % kLocalNp] = 0x7FFFFFFFFFFFFFFFLL;
+  __syncthreads();
+  const RunDesc& R = sR;
+  RunState* st = R.st;
+  const int np = R.np, d = R.d, dp = R.dp, obj = R.obj;
+  const bool stopped0 = *(volatile int32_t*)&st->stop != 0;
+  if (!ISL && stopped0) return;  // the whole cluster
+  const LocalLayout L = local_layout(SL, kpad, dp_max, 0, false);
+  double* Y = reinterpret_cast<double*>(smem_l + L.y);
+  double* Zf = reinterpret_cast<double*>(smem_l + L.z);
+  double* pop = reinterpret_cast<double*>(smem_l + L.pop);
+  double* mts = reinterpret_cast<double*>(smem_l + L.mt);
+  const int psz = kLocalNp * dp_max;  // doubles per population buffer
+  SliceCtx sc;
+  if constexpr (SL) {
+    slice_begin(sc, smem_l, kpad, cols, s_sl);
+    slice_load_m(sc, R.sl, R.sl_kpad);
+  } else if (R.rotate) {
+    for (int e = tid; e < d * d; e += blockDim.x) mts[e] = __ldg(R.MT + e);
+  }
+  long long gen = *(volatile int64_t*)&st->gen;
+  int64_t evals = *(volatile int64_t*)&st->evals;
+  double bestf = *(volatile double*)&st->best_f;
+  int best = *(volatile int32_t*)&st->best_idx;
+  int stop = stopped0 ? *(volatile int32_t*)&st->stop : 0;
+  int err = 0;
+
+  const int i = 8 * rank + warp;  // this warp's target
+  const bool mine = i < np;
+  const int nrows = max(0, min(8, np - 8 * rank));  // targets of this CTA
+  const int j0 = CPL * lane;
+  const bool in = mine && j0 < d;
+  double tx[CPL] = {}, tr[CPL] = {}, ov[CPL] = {}, fi = 0.0, fp = 0.0;
+#pragma unroll
+  for (int m = 0; m < CPL; ++m)
+    if (in && j0 + m < d) ov[m] = R.o[j0 + m];
+  // the population of generation g from global memory into the CTA's copy,
+  // this warp's row and fitness into registers
+  auto load_pop = [&](long long g) {
+    const double* X = R.X[g & 1];
+    double* p = pop + (size_t)(g & 1) * psz;
+    for (int e = tid; e < np * dp; e += blockDim.x) p[e] = __ldcg(X + e);
+    if (in) ld_coords(X + (size_t)i * dp + j0, tx);
+    if (mine) fi = __ldcg(R.f[g & 1] + i);
+  };
+  auto store_rows = [&](long long g) {
+    if (in) st_coords(R.X[g & 1] + (size_t)i * dp + j0, tx);
+    if (mine && lane == 0) R.f[g & 1][i] = fi;
+  };
+  load_pop(gen);
+  TrialSetup ts{};
+  U32x4 ub{};
+  auto draw = [&](long long g) {
+    if (mine) {
+      ts = trial_setup(R, (uint32_t)i, g, lane, 0u, false);
+      if (in) ub = draw_block(R.seed, kPurposeStep, R.run_id, 0u, (uint32_t)g, (uint32_t)i, 1u + (uint32_t)(j0 >> 2));
+    }
+  };
+  draw(gen + 1);
+  const bool common = ISL && R.target > 0.0;  // the islands' common stop applies
+  const unsigned m_isl = ISL ? (unsigned)isl->m : 1u;
+  const bool test_skip = ISL && ctl->test_skip == run + 1;
+  const long long spin = ISL && ctl->test_spin > 0 ? ctl->test_spin : kLocalSpin;
+  // rank 0's waits: until `want` arrivals on a counter (one lane polls)
+  auto wait_count = [&](unsigned* cnt, unsigned want) -> bool {
+    for (long long q = 0; q < spin; ++q) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
+      if (v >= want) return true;
+      if ((q & 15) == 15 && *(volatile int*)&ctl->abort) break;
+    }
+    atomicExch(&ctl->abort, 1);
+    return false;
+  };
+  auto arrive = [&](unsigned* cnt) { asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(cnt), "r"(1u) : "memory"); };
+  // the index (in this launch) of the first generation in which an island was
+  // below the target; large when none was
+  auto stop_index = [&]() { return (long long)(0xFFFFFFFFu - *(volatile unsigned*)&ctl->below[0]); };
+  // every CTA is running and has loaded before any peer writes its memory
+  cluster.sync();
+
+  long long it = 0;
+  for (; it < gens && !stop && !err; ++it) {
+    const long long g = gen + 1;
+    const double* P = pop + (size_t)(gen & 1) * psz;
+    double ft = 0.0;
+    double y[CPL] = {};
+    // ---- trial: Eq. 2, Eq. 3, bound repair; y = (t - o) s
+    if (in) {
+      double x1[CPL], x2[CPL], x3[CPL];
+      uint32_t u[CPL];
+#pragma unroll
+      for (int m = 0; m < CPL; ++m) {
+        x1[m] = P[ts.r1 * dp + j0 + m];
+        x2[m] = P[ts.r2 * dp + j0 + m];
+        x3[m] = P[ts.r3 * dp + j0 + m];
+        u[m] = word_of(ub, (j0 + m) & 3);
+      }
+      trial_coords<CPL>(R, ts.jr, j0, tx, x1, x2, x3, u, tr, R.F, R.cr_thr, 0);
+#pragma unroll
+      for (int m = 0; m < CPL; ++m) y[m] = j0 + m < d ? shifted(tr[m], ov[m], R) : 0.0;
+    }
+    // ---- fitness
+    if constexpr (SL) {
+      if (mine) {
+        if (in) st_coords(Y + warp * dp + j0, y);
+        slice_digits(sc, warp, lane, R.sl_kpad, R.sl_qmin[0], y);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      }
+      __syncthreads();
+      ft = slice_fitness(sc, R, Y, Zf, nrows);
+    } else if (mine) {
+      // one coordinate a lane (d <= 32): the sums of the general kernel, whose
+      // lane j holds coordinate j
+      double z = y[0];
+      if (R.rotate) {
+        double* yr = Y + warp * dp;
+        if (lane < d) yr[lane] = y[0];
+        __syncwarp();
+        z = 0.0;
+        if (lane < d)
+          for (int k = 0; k < d; ++k) z = fma(mts[k * d + lane], yr[k], z);
+        __syncwarp();
+      }
+      double t1 = 0.0, t2 = 0.0;
+      if (obj == kObjRosenbrock) {
+        const double zn = __shfl_down_sync(0xffffffffu, z, 1);
+        if (lane + 1 < d) {
+          const double t0 = z + 1.0, tn = zn + 1.0;
+          const double a = tn - t0 * t0, b = t0 - 1.0;
+          t1 = 100.0 * a * a + b * b;
+        }
+      } else if (lane < d) {
+        if (obj == kObjRastrigin) {
+          t1 = fma(z, z, rastrigin_w(z));
+        } else {
+          t1 = z * z;
+          if (obj == kObjAckley) t2 = cos2pi_fix(z);
+        }
+      }
+      const double s1 = warp_sum(t1);
+      ft = s1;
+      if (obj == kObjAckley) {
+        const double s2 = warp_sum(t2);
+        ft = 20.0 + 2.718281828459045 - 20.0 * exp(-0.2 * sqrt(s1 / d)) - exp(s2 / d);
+      }
+    }
+    // ---- selection; the row and its key to every CTA of the cluster
+    if (mine) {
+      fp = fi;
+      const long long kt = fit_key(ft);
+      const bool acc = kt <= fit_key(fi) && kt != 0x7FFFFFFFFFFFFFFFLL;  // ft <= fi, NaN never
+      if (acc) {
+        fi = ft;
+#pragma unroll
+        for (int m = 0; m < CPL; ++m) tx[m] = tr[m];
+      }
+      if (in) {
+        double* q = pop + (size_t)(g & 1) * psz + (size_t)i * dp + j0;
+        for (int c = 0; c < csize; ++c) st_coords(cluster.map_shared_rank(q, c), tx);
+      }
+      if (lane < csize) *cluster.map_shared_rank(&s_key[g & 1][i], lane) = fit_key(fi);
+    }
+    if (SL && tid == 0 && s_sl.fail)
+      for (int c = 0; c < csize; ++c) *cluster.map_shared_rank(&s_fail[g & 1], c) = 1;
+    if (common && rank == 0 && tid == 0 && it > 0) {
+      // whether the model stopped at an earlier generation: every island has
+      // counted the one before this
+      const bool ok = wait_count(&ctl->bar, m_isl * (unsigned)it);
+      const int f = !ok ? 2 : stop_index() < it ? 1 : 0;
+      if (f)
+        for (int c = 0; c < csize; ++c) *cluster.map_shared_rank(&s_flag[g & 1], c) = f;
+    }
+    cg::cluster_group::arrival_token tok = cluster.barrier_arrive();
+    draw(g + 1);
+    cluster.barrier_wait(std::move(tok));
+    const int flag = *(volatile int*)&s_flag[g & 1];
+    if (flag == 2 || *(volatile int*)&s_fail[g & 1]) {
+      err = kErrTimeout;
+      break;
+    }
+    if (ISL && flag == 1) {
+      // the model stopped at generation gen: back to it
+      if (in) {
+#pragma unroll
+        for (int m = 0; m < CPL; ++m) tx[m] = P[(size_t)i * dp + j0 + m];
+      }
+      fi = fp;
+      stop = 1;
+      break;
+    }
+    // ---- best record and stop rule, by every warp
+    gen = g;
+    evals += np;
+    {
+      long long bk = lane < np ? s_key[g & 1][lane] : 0x7FFFFFFFFFFFFFFFLL;
+      int bi = lane < np ? lane : -1;
+      const long long k2 = lane + 32 < np ? s_key[g & 1][lane + 32] : 0x7FFFFFFFFFFFFFFFLL;
+      if (k2 < bk) {
+        bk = k2;
+        bi = lane + 32;
+      }
+      warp_best(bk, bi);
+      if (bi >= 0) {
+        bestf = __longlong_as_double(bk >= 0 ? bk : (long long)(0x8000000000000000ULL | (unsigned long long)(-bk)));
+        best = bi;
+      } else if (rank == 0 && tid == 0) {
+        atomicOr(&st->err, kErrNonFinite);
+      }
+    }
+    const bool below = R.target > 0.0 && best >= 0 && bestf < R.target;
+    if (!ISL && below) stop = 1;
+    else if (R.max_evals > 0 && evals >= R.max_evals) stop = 2;
+    else if (gen >= R.max_gens) stop = 3;
+    if constexpr (ISL) {
+      if (rank == 0 && tid == 0 && (common || isl->interval > 0)) {
+        if (common && below) atomicMax(&ctl->below[0], 0xFFFFFFFFu - (unsigned)it);
+        if (!(test_skip && it == 0)) arrive(&ctl->bar);
+      }
+      const bool mig = isl->interval > 0 && gen % isl->interval == 0;
+      if (mig || stop || it + 1 >= gens) {
+        // the islands meet: the common stop at this generation, and migration
+        store_rows(gen);
+        if (rank == 0 && tid == 0) s_over = 0;
+        cluster.sync();
+        if (rank == 0) {
+          if (tid == 0) {
+            int f = 0;
+            if (common || mig) f = !wait_count(&ctl->bar, m_isl * (unsigned)(it + 1)) ? 2 : common && stop_index() <= it ? 1 : 0;
+            s_over = f;
+            const int sp = f == 1 ? 1 : stop;
+            if (f != 2) {
+              st->best_f = bestf;
+              st->best_idx = best;
+              st->gen = gen;
+              st->evals = evals;
+              st->stop = sp;
+            }
+          }
+          __syncthreads();
+          if (mig && s_over != 2) {
+            const int cur = (int)(gen & 1);
+            if (isl->async) {
+              // one interval late, through the mailbox (k_island_async's rule)
+              const int64_t ep = gen / isl->interval;
+              const long long pg = *(volatile long long*)&isl->post_gen;
+              const bool take = pg >= 0 && pg == gen - isl->interval;
+              island_exchange(R, run, isl->m, isl->nmig, cur, stage, true, (size_t)(ep & 1) * stage.slot, take,
+                              (size_t)((ep & 1) ^ 1) * stage.slot);
+            } else {
+              // every island posts before any island takes
+              island_exchange(R, run, isl->m, isl->nmig, cur, stage, true, 0, false, 0);
+            }
+            __syncthreads();
+            if (tid == 0) {
+              // (asynchronous: post_gen is written once every island has read it)
+              arrive(&ctl->sbar[0]);
+              const unsigned k = (unsigned)(gen / isl->interval - (gen - it - 1) / isl->interval);
+              if (!wait_count(&ctl->sbar[0], m_isl * k)) s_over = 2;
+            }
+            __syncthreads();
+            if (!isl->async && s_over != 2) island_exchange(R, run, isl->m, isl->nmig, cur, stage, false, 0, true, 0);
+            if (run == 0 && tid == 0 && s_over != 2) {
+              isl->mig_gen = gen;
+              if (isl->async) isl->post_gen = gen;
+            }
+          }
+          __syncthreads();
+          if (tid == 0)
+            for (int c = 1; c < csize; ++c) *cluster.map_shared_rank(&s_over, c) = s_over;
+        }
+        cluster.sync();
+        const int over = *(volatile int*)&s_over;
+        if (over == 2) {
+          err = kErrTimeout;
+          break;
+        }
+        if (over == 1) stop = 1;
+        if (mig) {
+          load_pop(gen);
+          best = *(volatile int32_t*)&st->best_idx;
+          bestf = *(volatile double*)&st->best_f;
+          __syncthreads();
+        }
+      }
+    }
+  }
+  // ---- what the caller reads
+  if (!err) {
+    store_rows(gen);
+    if (rank == 0 && tid == 0) {
+      st->best_f = bestf;
+      st->best_idx = best;
+      st->gen = gen;
+      st->evals = evals;
+      st->stop = stop;
+    }
+  } else if (rank == 0 && tid == 0) {
+    atomicOr(&st->err, err);
+  }
+  cluster.sync();  // no peer writes this CTA's memory any more
+  if constexpr (SL) slice_end(sc);
+}
+
+// ------------------------------------------------------------------ host side
+static const void* local_kernel(bool sl, bool isl, int kpad) {
+  if (!sl) return isl ? (const void*)k_gen_local<1, false, true> : (const void*)k_gen_local<1, false, false>;
+  if (kpad <= 32) return isl ? (const void*)k_gen_local<1, true, true> : (const void*)k_gen_local<1, true, false>;
+  return isl ? (const void*)k_gen_local<2, true, true> : (const void*)k_gen_local<2, true, false>;
+}
+
+static size_t local_smem(const LocalPlan& p, const void* k) {
+  const size_t need = local_layout(p.sl, p.kpad, p.dp_max, p.d_max, p.rotate).total;
+  // sliced: a whole SM (fp64_exclusive_smem: the cluster's CTAs wait for one
+  // another while they hold tensor memory)
+  return p.sl ? fp64_exclusive_smem(k, need) : need;
+}
+
+static cudaLaunchConfig_t local_config(const LocalPlan& p, const void* k, int nruns, bool isl, cudaStream_t s,
+                                       cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(nruns * p.csize));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = local_smem(p, k);
+  cfg.stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)p.csize;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  // the islands wait for one another: every cluster resident, or no launch
+  attr[1].id = cudaLaunchAttributeCooperative;
+  attr[1].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = isl ? 2 : 1;
+  return cfg;
+}
+
+// Whether the runs fit the form (np <= 64; sliced runs of d <= 64, or none
+// sliced and d <= 32), and its launch.
+bool local_plan(LocalPlan& p, const std::vector<RunDesc>& runs, const SlicePlan& sp) {
+  p = LocalPlan{};
+  int np_max = 0;
+  p.sl = sp.on;
+  for (const RunDesc& R : runs) {
+    p.csize = 0;  // does not fit, unless it gets to the end
+    if (R.np > kLocalNp || R.obj > kObjAckley || R.strategy != 0 || R.jde || R.dbg_trial) return false;
+    if (sp.on != (R.sl != nullptr)) return false;
+    if (R.d > (sp.on ? 64 : 32)) return false;
+    np_max = std::max(np_max, R.np);
+    p.d_max = std::max(p.d_max, R.d);
+    p.dp_max = std::max(p.dp_max, R.dp);
+    p.rotate = p.rotate || R.rotate;
+  }
+  p.csize = (np_max + 7) / 8;
+  p.kpad = sp.kpad;
+  p.cols = sp.cols;
+  return true;
+}
+
+bool local_fits(const LocalPlan& p, int nruns, bool isl) {
+  const void* k = local_kernel(p.sl, isl, p.kpad);
+  const size_t smem = local_smem(p, k);
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const cudaLaunchConfig_t cfg = local_config(p, k, nruns, isl, 0, attr);
+  if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return n >= (isl ? nruns : 1);
+}
+
+cudaError_t k_gen_local_launch(const RunDesc* runs, int nruns, const LocalPlan& p, PersistCtl* ctl, long long gens,
+                               cudaStream_t s, int test_skip, IslandCtl* isl, const IslandStage* stage) {
+  cudaError_t e = persist_ctl_reset(ctl, test_skip, s);
+  if (e != cudaSuccess) return e;
+  IslandStage st{};
+  if (stage) st = *stage;
+  const void* k = local_kernel(p.sl, isl != nullptr, p.kpad);
+  cudaLaunchAttribute attr[2];
+  const cudaLaunchConfig_t cfg = local_config(p, k, nruns, isl != nullptr, s, attr);
+  int csize = p.csize, kpad = p.kpad, dp_max = p.dp_max;
+  uint32_t cols = p.cols;
+  void* args[] = {(void*)&runs, (void*)&ctl, (void*)&gens, (void*)&csize, (void*)&isl,
+                  (void*)&st,   (void*)&kpad, (void*)&cols, (void*)&dp_max};
+  return cudaLaunchKernelExC(&cfg, k, args);
+}
+
+}  // namespace de

@@ -80,6 +80,19 @@ struct IslandStage;
 cudaError_t k_gen_sliced_launch(const RunDesc* runs, const int4* items, int nitems, int nruns, PersistCtl* ctl,
                                 long long gens, const SlicePlan& p, bool unit, size_t smem, cudaStream_t s,
                                 int test_skip, IslandCtl* isl, const IslandStage* stage);
+// the generation loop of small plain DE runs, a cluster of csize CTAs per run
+// with the population in shared memory (de_fp64_local.cu)
+struct LocalPlan {
+  bool sl = false;      // every run's rotation is sliced (else none's)
+  bool rotate = false;  // some run has a rotation
+  int csize = 0, kpad = 0, d_max = 0, dp_max = 0;
+  uint32_t cols = 0;
+};
+bool local_plan(LocalPlan& p, const std::vector<RunDesc>& runs, const SlicePlan& sp);
+// whether a cluster fits on the device (isl: all of them at once)
+bool local_fits(const LocalPlan& p, int nruns, bool isl);
+cudaError_t k_gen_local_launch(const RunDesc* runs, int nruns, const LocalPlan& p, PersistCtl* ctl, long long gens,
+                               cudaStream_t s, int test_skip, IslandCtl* isl, const IslandStage* stage);
 // the generation loop of FP64 runs in one cooperative launch (every item
 // co-resident: nitems <= k_gen_fp64_persist_capacity; gens <= 2^20)
 // test_skip > 0: the grid-barrier failure test (PersistCtl::test_skip)
