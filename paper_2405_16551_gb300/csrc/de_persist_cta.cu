@@ -188,9 +188,9 @@ __global__ void __launch_bounds__(256, 1)
   }
 
   // Targets of this warp: local rows (warp - shift) + 8 q.  With at most 7
-  // targets per CTA (plain DE/rand/1/bin) warp 0 has none: it reduces the
-  // previous generation's best partials while the other warps build trials.
-  const int shift = (!VAR && rows <= 7) ? 1 : 0;
+  // targets per CTA warp 0 has none: it reduces the previous generation's best
+  // partials while the other warps build trials.
+  const int shift = rows <= 7 ? 1 : 0;
   // per-warp registers: trial and current rows of this warp's targets, and the
   // lane's coordinates of the shift
   double tr[2][4], tx[2][4], osh[4];
@@ -204,8 +204,52 @@ __global__ void __launch_bounds__(256, 1)
   bool reduce_pending = false;  // partials of generation gen still to reduce
   bool rows_in_regs = false;    // tx holds the current rows (after the first generation of a launch)
   bool have_next = false;       // nts / nu hold the draws of generation gen + 1
-  TrialSetup nts[2];            // plain DE: r1, r2, r3, j_rand of the next generation
+  TrialSetup nts[2];            // r1, r2, r3, j_rand of the next generation
   U32x4 nu[2];                  // ... and the lane's crossover block
+  TrialVar ntv[2];              // variants: the trial's F, CR, threshold and exponential length
+  // jDE: the targets' F_i and CR_i (and the threshold of CR_i), as their rows
+  // in registers for the launch
+  double jFi[2] = {0.0, 0.0}, jCRi[2] = {0.0, 0.0};
+  uint64_t jthr[2] = {0, 0};
+  if (VAR && R.jde) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int lr = warp - shift + 8 * q, i = row0 + lr;
+      if (warp < shift || lr >= rows || i >= np) continue;
+      jFi[q] = __ldcg(R.jF[s_gen & 1] + i);
+      jCRi[q] = __ldcg(R.jCR[s_gen & 1] + i);
+      jthr[q] = (uint64_t)floor(__dmul_rn(jCRi[q], 4294967296.0));
+    }
+  }
+  // What generation g's trial of a target draws: it depends on (seed, g, target)
+  // and the target's own parameters only, so it is made while the CTA waits at
+  // the barrier before g (trial_setup_var's values; DE/best/1 puts the best
+  // row in where the trial is built).  Under jDE this and the trials built
+  // before the stop decision took 8.58 -> 6.36 us a generation at NP = 501, D = 50
+  // (TF32x3).
+  auto draws = [&](int64_t gd, int i, int q) {
+    nts[q] = trial_setup(R, (uint32_t)i, gd, lane, 0u, false);
+    nu[q] = draw_block(R.seed, kPurposeStep, R.run_id, 0u, (uint32_t)gd, (uint32_t)i, 1u + lane);
+    if constexpr (VAR) {
+      ntv[q].F = R.F;
+      ntv[q].CR = R.CR;
+      ntv[q].thr = R.cr_thr;
+      if (R.jde) {
+        // jde_params, from the registers; the threshold of a drawn CR_i = a2 / 2^32 is a2
+        const uint32_t tau = 429496729u;  // floor(0.1 * 2^32)
+        const U32x4 a = draw_block(R.seed, kPurposeJde, R.run_id, 0u, (uint32_t)gd, (uint32_t)i, 0u);
+        ntv[q].F = jFi[q];
+        ntv[q].CR = jCRi[q];
+        ntv[q].thr = jthr[q];
+        if (a.y < tau) ntv[q].F = __fma_rn(0.9, (double)a.x * 0x1p-32, 0.1);
+        if (a.w < tau) {
+          ntv[q].CR = (double)a.z * 0x1p-32;
+          ntv[q].thr = a.z;
+        }
+      }
+      ntv[q].L = R.strategy == 2 ? exp_length(R, (uint32_t)i, gd, lane, ntv[q].thr) : 0;
+    }
+  };
   unsigned nbar = 0;            // grid barriers passed in this launch
   uint32_t mma_phase = 0;
 
@@ -214,8 +258,6 @@ __global__ void __launch_bounds__(256, 1)
     const int cur = (int)(gen & 1), nxt = cur ^ 1;
     const double* __restrict__ X = R.X[cur];
     double* __restrict__ Xn = R.X[nxt];
-    const double* jFc = VAR && R.jde ? R.jF[cur] : nullptr;
-    const double* jCRc = VAR && R.jde ? R.jCR[cur] : nullptr;
     const bool more = itg < gens && !abort;
 
     // ---- 0. best record and stop rule of generation gen, whose partials are
@@ -250,10 +292,10 @@ __global__ void __launch_bounds__(256, 1)
       }
     }
     reduce_pending = false;
-    // the variants need the best record before their trials (DE/best/1
-    // base), and a debug capture must not record trials of a generation that
-    // the stop rule cancels: both take the stop decision first
-    const bool ordered = VAR || R.dbg_trial != nullptr;
+    // DE/best/1 needs the best record before its trials, and a debug capture
+    // must not record trials of a generation that the stop rule cancels: both
+    // take the stop decision first
+    const bool ordered = (VAR && R.strategy == 1) || R.dbg_trial != nullptr;
     if (ordered || !more) __syncthreads();
     if (!more) break;
     if (ordered && s_stop) break;
@@ -276,45 +318,47 @@ __global__ void __launch_bounds__(256, 1)
         const int i = row0 + lr;
         valid[q] = warp >= shift && lr < rows && i < np;
         if (!valid[q]) continue;
+        if (!have_next) draws(g, i, q);  // else made while this CTA waited at the last grid barrier
+        ts[q] = nts[q];
+        if (R.dbg_idx && lane == 0) {
+          R.dbg_idx[3 * i + 0] = (int32_t)ts[q].r1;
+          R.dbg_idx[3 * i + 1] = (int32_t)ts[q].r2;
+          R.dbg_idx[3 * i + 2] = (int32_t)ts[q].r3;
+          R.dbg_jrand[i] = (int32_t)ts[q].jr;
+        }
         if constexpr (VAR) {
-          ts[q] = trial_setup_var(R, (uint32_t)i, g, lane, s_bidx, jFc, jCRc, tv[q]);
-          if (j0 < d) trial_load(R, X, ts[q], (uint32_t)i, g, j0, cin[q]);
-        } else {
-          // the draws were made while this CTA waited at the last grid barrier
-          ts[q] = have_next ? nts[q] : trial_setup(R, (uint32_t)i, g, lane, 0u, false);
-          if (R.dbg_idx && lane == 0) {
-            R.dbg_idx[3 * i + 0] = (int32_t)ts[q].r1;
-            R.dbg_idx[3 * i + 1] = (int32_t)ts[q].r2;
-            R.dbg_idx[3 * i + 2] = (int32_t)ts[q].r3;
-            R.dbg_jrand[i] = (int32_t)ts[q].jr;
+          tv[q] = ntv[q];
+          if (R.strategy == 1) {
+            ts[q].r3 = ts[q].r2;
+            ts[q].r2 = ts[q].r1;
+            ts[q].r1 = (uint32_t)s_bidx;
           }
-          if (j0 < d) {
-            cin[q].u = have_next ? nu[q]
-                                 : draw_block(R.seed, kPurposeStep, R.run_id, 0u, (uint32_t)g, (uint32_t)i, 1u + lane);
-            const double* rows3[3] = {X + (size_t)ts[q].r1 * dp + j0, X + (size_t)ts[q].r2 * dp + j0,
-                                      X + (size_t)ts[q].r3 * dp + j0};
-            double* dst[3] = {cin[q].x1, cin[q].x2, cin[q].x3};
+        }
+        if (j0 < d) {
+          cin[q].u = nu[q];
+          const double* rows3[3] = {X + (size_t)ts[q].r1 * dp + j0, X + (size_t)ts[q].r2 * dp + j0,
+                                    X + (size_t)ts[q].r3 * dp + j0};
+          double* dst[3] = {cin[q].x1, cin[q].x2, cin[q].x3};
 #pragma unroll
-            for (int r = 0; r < 3; ++r) {
-              const double2 a = __ldcg(reinterpret_cast<const double2*>(rows3[r]));
-              const double2 b2 = __ldcg(reinterpret_cast<const double2*>(rows3[r] + 2));
-              dst[r][0] = a.x;
-              dst[r][1] = a.y;
-              dst[r][2] = b2.x;
-              dst[r][3] = b2.y;
-            }
-            if (rows_in_regs) {
-              // the target is the row this warp wrote in the last generation
+          for (int r = 0; r < 3; ++r) {
+            const double2 a = __ldcg(reinterpret_cast<const double2*>(rows3[r]));
+            const double2 b2 = __ldcg(reinterpret_cast<const double2*>(rows3[r] + 2));
+            dst[r][0] = a.x;
+            dst[r][1] = a.y;
+            dst[r][2] = b2.x;
+            dst[r][3] = b2.y;
+          }
+          if (rows_in_regs) {
+            // the target is the row this warp wrote in the last generation
 #pragma unroll
-              for (int e = 0; e < 4; ++e) cin[q].xi[e] = tx[q][e];
-            } else {
-              const double2 a = __ldcg(reinterpret_cast<const double2*>(X + (size_t)i * dp + j0));
-              const double2 b2 = __ldcg(reinterpret_cast<const double2*>(X + (size_t)i * dp + j0 + 2));
-              cin[q].xi[0] = a.x;
-              cin[q].xi[1] = a.y;
-              cin[q].xi[2] = b2.x;
-              cin[q].xi[3] = b2.y;
-            }
+            for (int e = 0; e < 4; ++e) cin[q].xi[e] = tx[q][e];
+          } else {
+            const double2 a = __ldcg(reinterpret_cast<const double2*>(X + (size_t)i * dp + j0));
+            const double2 b2 = __ldcg(reinterpret_cast<const double2*>(X + (size_t)i * dp + j0 + 2));
+            cin[q].xi[0] = a.x;
+            cin[q].xi[1] = a.y;
+            cin[q].xi[2] = b2.x;
+            cin[q].xi[3] = b2.y;
           }
         }
       }
@@ -527,12 +571,17 @@ __global__ void __launch_bounds__(256, 1)
       const int i = row0 + lr;
       if (warp < shift || lr >= rows || i >= np) continue;
       const bool acc = s_flag[lr] & 1;
-      if (VAR && R.jde && lane == 0) {
+      if (VAR && R.jde) {
         // jDE: an accepted trial passes its F_i and CR_i on
-        double Fi = __ldcg(jFc + i), CRi = __ldcg(jCRc + i);
-        if (acc) jde_params(R, (uint32_t)i, g, jFc, jCRc, Fi, CRi);
-        R.jF[nxt][i] = Fi;
-        R.jCR[nxt][i] = CRi;
+        if (acc) {
+          jFi[q] = ntv[q].F;
+          jCRi[q] = ntv[q].CR;
+          jthr[q] = ntv[q].thr;
+        }
+        if (lane == 0) {
+          R.jF[nxt][i] = jFi[q];
+          R.jCR[nxt][i] = jCRi[q];
+        }
       }
       if (acc) {
 #pragma unroll
@@ -601,17 +650,16 @@ __global__ void __launch_bounds__(256, 1)
         s_abort = 1;
       }
     }
-    if (!VAR) {
+    {
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const int lr = warp - shift + 8 * q;
         const int i = row0 + lr;
         if (warp < shift || lr >= rows || i >= np) continue;
-        nts[q] = trial_setup(R, (uint32_t)i, g + 1, lane, 0u, false);
-        nu[q] = draw_block(R.seed, kPurposeStep, R.run_id, 0u, (uint32_t)(g + 1), (uint32_t)i, 1u + lane);
+        draws(g + 1, i, q);
       }
     }
-    have_next = !VAR;
+    have_next = true;
     ++nbar;
     __syncthreads();
     abort = s_abort != 0;
