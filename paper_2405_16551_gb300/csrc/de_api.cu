@@ -593,8 +593,10 @@ static std::string tune_key(const de_handle* h) {
     sum_d += (long long)R.np * R.d;
   }
   char b[256];
-  snprintf(b, sizeof b, "gen_fp64v6 runs=%d np0=%d d0=%d obj0=%d rot0=%d sumnp=%lld sumnd=%lld", h->nruns, h->run[0].np,
-           h->run[0].d, h->run[0].obj, h->run[0].rotate, sum_np, sum_d);
+  // (var, form: which of the kernels apply)
+  snprintf(b, sizeof b, "gen_fp64v6 runs=%d np0=%d d0=%d obj0=%d rot0=%d sumnp=%lld sumnd=%lld var=%d form=%d", h->nruns,
+           h->run[0].np, h->run[0].d, h->run[0].obj, h->run[0].rotate, sum_np, sum_d, h->variants ? 1 : 0,
+           (h->slices.on ? 1 : 0) + (h->sliced_loop ? 2 : 0) + 4 * h->local.csize);
   return b;
 }
 

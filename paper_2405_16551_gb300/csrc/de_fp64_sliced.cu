@@ -241,7 +241,11 @@ __global__ void __launch_bounds__(256, 1)
 #pragma unroll
           for (int m = 0; m < CPL; ++m) tx[m] = tr[m];
         }
-        if (in) st_coords(R.X[g & 1] + (size_t)i * dp + j0, tx);
+        if constexpr (CPL == 4) {
+          if (in) st_row4(R.X[g & 1] + (size_t)i * dp + j0, tx);
+        } else {
+          if (in) st_coords(R.X[g & 1] + (size_t)i * dp + j0, tx);
+        }
         if (lane == 0) {
           R.f[g & 1][i] = fi;
           s_f[warp] = fi;

@@ -643,13 +643,8 @@ __global__ void __launch_bounds__(256, 1)
         const int j0 = 128 * c + 4 * lane;
         if (j0 >= d) continue;
         double* dst = Xn + (size_t)i * dp + j0;
-        if (acc) {
-          *reinterpret_cast<double2*>(dst) = make_double2(tr[q][c][0], tr[q][c][1]);
-          *reinterpret_cast<double2*>(dst + 2) = make_double2(tr[q][c][2], tr[q][c][3]);
-        } else {
-          *reinterpret_cast<double2*>(dst) = make_double2(tx[q][c][0], tx[q][c][1]);
-          *reinterpret_cast<double2*>(dst + 2) = make_double2(tx[q][c][2], tx[q][c][3]);
-        }
+        if (acc) st_row4(dst, tr[q][c]);
+        else st_row4(dst, tx[q][c]);
       }
     }
     // every CTA arrives at the grid barrier once its rows are written; the

@@ -300,9 +300,7 @@ __global__ void __launch_bounds__(kPbThreads, 1)
           if (j0 < d) {
             bits = trial_compute(R, U.s, j0, U.c, t);
             if (U.v) {
-              double* row = Xn + (size_t)i * dp + j0;
-              *reinterpret_cast<double2*>(row) = make_double2(t[0], t[1]);
-              *reinterpret_cast<double2*>(row + 2) = make_double2(t[2], t[3]);
+              st_row4(Xn + (size_t)i * dp + j0, t);
             }
           }
           float yn2 = 0.f;

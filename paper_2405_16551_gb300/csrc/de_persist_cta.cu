@@ -70,7 +70,8 @@ __host__ __device__ inline CtaLayout cta_layout(const RunDesc& R) {
 template <int ESZ, bool VAR>
 __global__ void __launch_bounds__(256, 1)
     k_persist_cta(const RunDesc* __restrict__ runs, int run, PersistCtl* ctl, long long gens, int rows) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // known to be the warp's own: a uniform branch for the products
   const int cta = (int)blockIdx.x, nct = (int)gridDim.x;
   // failure-detection test (off unless set by the launcher): this CTA leaves
   // out its first grid-barrier arrival and the barrier gives up after test_spin polls
@@ -336,29 +337,15 @@ __global__ void __launch_bounds__(256, 1)
         }
         if (j0 < d) {
           cin[q].u = nu[q];
-          const double* rows3[3] = {X + (size_t)ts[q].r1 * dp + j0, X + (size_t)ts[q].r2 * dp + j0,
-                                    X + (size_t)ts[q].r3 * dp + j0};
-          double* dst[3] = {cin[q].x1, cin[q].x2, cin[q].x3};
-#pragma unroll
-          for (int r = 0; r < 3; ++r) {
-            const double2 a = __ldcg(reinterpret_cast<const double2*>(rows3[r]));
-            const double2 b2 = __ldcg(reinterpret_cast<const double2*>(rows3[r] + 2));
-            dst[r][0] = a.x;
-            dst[r][1] = a.y;
-            dst[r][2] = b2.x;
-            dst[r][3] = b2.y;
-          }
+          ld_row4(X + (size_t)ts[q].r1 * dp + j0, cin[q].x1);
+          ld_row4(X + (size_t)ts[q].r2 * dp + j0, cin[q].x2);
+          ld_row4(X + (size_t)ts[q].r3 * dp + j0, cin[q].x3);
           if (rows_in_regs) {
             // the target is the row this warp wrote in the last generation
 #pragma unroll
             for (int e = 0; e < 4; ++e) cin[q].xi[e] = tx[q][e];
           } else {
-            const double2 a = __ldcg(reinterpret_cast<const double2*>(X + (size_t)i * dp + j0));
-            const double2 b2 = __ldcg(reinterpret_cast<const double2*>(X + (size_t)i * dp + j0 + 2));
-            cin[q].xi[0] = a.x;
-            cin[q].xi[1] = a.y;
-            cin[q].xi[2] = b2.x;
-            cin[q].xi[3] = b2.y;
+            ld_row4(X + (size_t)i * dp + j0, cin[q].xi);
           }
         }
       }
@@ -410,7 +397,9 @@ __global__ void __launch_bounds__(256, 1)
 
     // ---- 2. split products on tcgen05: z = Mh yh + Ml yh + Mh yl, M as the
     // 128-row A operand and the targets' y as the 16-row B operand
-    if (warp < 3 && lane == 0) {
+    // (issued from warp-uniform code by an elected lane: 20 cycles a product, 60
+    // to 80 from a divergent branch)
+    if (warp < 3) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int ksteps = R.kpad * ESZ / 32;
       const int pass = warp;
@@ -419,10 +408,13 @@ __global__ void __launch_bounds__(256, 1)
       // A in tensor memory: a K step (two k-groups) is 8 columns
       const uint32_t ta = tmem + kColA + (pass == 1 ? kColPart : 0u);
       const uint64_t dy = smem_desc(smem_u32(sYop) + (pass == 2 ? y_part : 0u), 256u, 128u);
-      for (int ks = 0; ks < ksteps; ++ks)
-        mma_split_ta<ESZ>(tmem + 16u * (uint32_t)pass, ta + 8u * (uint32_t)ks, dy + (uint64_t)(ks * 32), idesc,
-                          ks > 0 ? 1u : 0u);
-      mma_commit(bar_mma);
+      if (elect_one()) {
+        for (int ks = 0; ks < ksteps; ++ks)
+          mma_split_ta<ESZ>(tmem + 16u * (uint32_t)pass, ta + 8u * (uint32_t)ks, dy + (uint64_t)(ks * 32), idesc,
+                            ks > 0 ? 1u : 0u);
+        mma_commit(bar_mma);
+      }
+      __syncwarp();
     }
     // ---- 3a. every warp copies one block of the accumulator (TMEM lanes
     // 32 (w mod 4) .. + 31 = coordinates j, columns 8 (w / 4) .. + 7 = targets)
@@ -589,9 +581,7 @@ __global__ void __launch_bounds__(256, 1)
       }
       const int j0 = 4 * lane;
       if (j0 < d) {
-        double* dst = Xn + (size_t)i * dp + j0;
-        *reinterpret_cast<double2*>(dst) = make_double2(tx[q][0], tx[q][1]);
-        *reinterpret_cast<double2*>(dst + 2) = make_double2(tx[q][2], tx[q][3]);
+        st_row4(Xn + (size_t)i * dp + j0, tx[q]);
       }
     }
     rows_in_regs = true;

@@ -71,12 +71,6 @@ __host__ __device__ inline uint32_t slice_tmem_cols(int kpad) {
 __host__ __device__ inline uint32_t slice_b_bytes(int kpad) { return ((uint32_t)(kpad / 8) * kSliceKg + 1023u) / 1024u * 1024u; }
 __host__ __device__ inline uint32_t slice_smem(int kpad) { return slice_b_bytes(kpad) + (uint32_t)slice_nsm(kpad) * slice_bytes(kpad); }
 
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n .reg .pred P;\n elect.sync _|P, 0xffffffff;\n selp.u32 %0, 1, 0, P;\n}\n" : "=r"(p));
-  return p != 0u;
-}
-
 // Its part in static shared memory.
 struct SliceShared {
   double sum[2][4][kSliceRows];  // per quarter of the outputs and tile row: term sums

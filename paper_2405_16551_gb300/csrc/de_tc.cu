@@ -147,9 +147,7 @@ __global__ void __launch_bounds__(256, OCC ? 3 : 2)
           if constexpr (VAR) bits = trial_compute(R, G.s, j0, cur, t, G.v.F, G.v.thr, G.v.L);
           else bits = trial_compute(R, G.s, j0, cur, t);
           if (G.valid) {
-            double* Trow = R.T + (size_t)G.i * R.dp + j0;
-            *reinterpret_cast<double2*>(Trow) = make_double2(t[0], t[1]);
-            *reinterpret_cast<double2*>(Trow + 2) = make_double2(t[2], t[3]);
+            st_row4(R.T + (size_t)G.i * R.dp + j0, t);
           }
         }
         if (j0 < kpad) {
