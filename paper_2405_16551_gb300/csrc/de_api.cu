@@ -1187,7 +1187,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
     size_t X0, X1, f0, f1, fx0, fx1, o, MT, Mr, sl, slx;
     bool sliced;
     int32_t qmin[5];
-    size_t st, part, T, ref, jF0, jF1, jC0, jC1, perm;
+    size_t st, part, T, ref, jF0, jF1, jC0, jC1, perm, ctab;
     size_t dbg_idx, dbg_jrand, dbg_mask, dbg_trial, dbg_ftrial, dbg_accept, dbg_fp64, dbg_cand;
   };
   std::vector<Offs> offs(nruns);
@@ -1223,6 +1223,14 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
       O.jF1 = take(c.np * sizeof(double));
       O.jC0 = take(c.np * sizeof(double));
       O.jC1 = take(c.np * sizeof(double));
+    }
+    O.ctab = 0;
+    {
+      // the functions with constants per coordinate
+      const SuiteSpec sp = suite_spec(c.objective);
+      for (int q = 0; q < sp.n; ++q)
+        if (sp.kind != 1 && (sp.fn[q] == DE_OBJ_ELLIPTIC || sp.fn[q] == DE_OBJ_GRIEWANK)) O.ctab = 1;
+      if (O.ctab) O.ctab = take((size_t)sp.n * ((c.d + 3) / 4 * 4) * sizeof(double));
     }
     if (c.debug_capture) {
       const int nw = (c.d + 31) / 32;
@@ -1334,6 +1342,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
         R.skex[q] = 10.0 / std::pow((double)n, 1.2);
       }
     }
+    if (O.ctab) R.ctab = (const double*)(A + O.ctab);
     if (c.jde) {
       R.jF[0] = (double*)(A + O.jF0);
       R.jF[1] = (double*)(A + O.jF1);
@@ -1428,6 +1437,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
   TRY(build_items(h));
   TRY(upload_desc(h));
   k_configure(h->smem_gen);
+  if (h->suite) k_suite_table_launch(h->d_run, nruns, h->stream);
   TRY(init_runs(h, 0, nruns));
   if (h->prec == DE_PREC_FP64 && cfgs[0].surrogate_k < 2) {
     ce = cudaMalloc(&h->d_ctl64, sizeof(PersistCtl));

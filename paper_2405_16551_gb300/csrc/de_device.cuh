@@ -80,20 +80,9 @@ __host__ __device__ constexpr unsigned long long cos_fix(int n) {
   return (unsigned long long)((a + ((unsigned __int128)1 << 60)) >> 61);
 }
 
-__device__ __forceinline__ unsigned long long omcos2pi_fix(double z, bool& ok) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(z);
-  const int ex = (int)((b >> 52) & 0x7FF);
-  ok = ex != 0x7FF;
-  // 2z = m 2^(ex - 1074): the bits below the point as a 64-bit fraction, and
-  // the lowest bit of the integer part
-  const unsigned long long m = (b & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL;
-  const int up = ex - 1074 + 64;  // the fraction is m 2^up modulo 2^64
-  // (no branches, so that independent calls interleave)
-  const unsigned long long fl = up < 64 ? m << (up & 63) : 0ULL, fs = up > -64 ? m >> (-up & 63) : 0ULL;
-  const unsigned long long fr = up >= 0 ? fl : fs;
-  const int ib = 64 - up;  // the integer part's lowest bit
-  unsigned int odd = ib >= 0 && ib < 53 ? (unsigned int)(m >> (ib & 63)) & 1u : 0u;
-  // the sign of z does not matter; r = fr or fr - 1 (then k is one more)
+// The same at 2z = (odd or an even number) + fr 2^-64.
+__device__ __forceinline__ unsigned long long omcospi_frac(unsigned long long fr, unsigned int odd) {
+  // r = fr or fr - 1 (then the integer part is one more)
   odd ^= (unsigned int)(fr >> 63);
   const unsigned long long r = (fr >> 63) ? 0ULL - fr : fr;  // |r| <= 2^63
   const unsigned long long u = __umul64hi(r, r);             // r^2 <= 2^62
@@ -116,6 +105,23 @@ __device__ __forceinline__ unsigned long long omcos2pi_fix(double z, bool& ok) {
   return odd ? (1ULL << 63) - x : x;
 }
 
+__device__ __forceinline__ unsigned long long omcos2pi_fix(double z, bool& ok) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(z);
+  const int ex = (int)((b >> 52) & 0x7FF);
+  ok = ex != 0x7FF;
+  // 2z = m 2^(ex - 1074): the bits below the point as a 64-bit fraction, and
+  // the lowest bit of the integer part
+  const unsigned long long m = (b & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL;
+  const int up = ex - 1074 + 64;  // the fraction is m 2^up modulo 2^64
+  // (no branches, so that independent calls interleave)
+  const unsigned long long fl = up < 64 ? m << (up & 63) : 0ULL, fs = up > -64 ? m >> (-up & 63) : 0ULL;
+  const unsigned long long fr = up >= 0 ? fl : fs;
+  const int ib = 64 - up;  // the integer part's lowest bit
+  const unsigned int odd = ib >= 0 && ib < 53 ? (unsigned int)(m >> (ib & 63)) & 1u : 0u;
+  // the sign of z does not matter
+  return omcospi_frac(fr, odd);
+}
+
 // w 2^e rounded to nearest even, on the integer pipe (the conversion
 // instruction occupies the FP64 pipe).
 __device__ __forceinline__ double f64_of_u64(unsigned long long w, int e) {
@@ -129,13 +135,33 @@ __device__ __forceinline__ double f64_of_u64(unsigned long long w, int e) {
   return w == 0ULL ? 0.0 : r;
 }
 
+// The cosine, rounded, of 1 - cos in units of 2^-62.
+__device__ __forceinline__ double cos_of_om(unsigned long long x) {
+  const bool neg = x > (1ULL << 62);
+  const double c = f64_of_u64(neg ? x - (1ULL << 62) : (1ULL << 62) - x, -62);
+  return neg ? -c : c;
+}
+
 // cos(2 pi z) rounded from the fixed-point form.
 __device__ __forceinline__ double cos2pi_fix(double z) {
   bool ok;
   const unsigned long long x = omcos2pi_fix(z, ok);
-  const bool neg = x > (1ULL << 62);
-  const double c = f64_of_u64(neg ? x - (1ULL << 62) : (1ULL << 62) - x, -62);
-  return ok ? (neg ? -c : c) : CUDART_NAN;
+  return ok ? cos_of_om(x) : CUDART_NAN;
+}
+
+// cos(pi w K 2^-65): the cosine of w times a constant that is known to 64 bits
+// as a number of turns (K 2^-66 < 1/4).  The 117-bit product keeps the argument
+// to |w| 2^-67 turns, more than the rounded FP64 argument holds.
+__device__ __forceinline__ double cos_turns_fix(double w, unsigned long long K) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(w);
+  const int ex = (int)((b >> 52) & 0x7FF);
+  const unsigned long long m = (b & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL;
+  // twice the turns = m K 2^(ex - 1140), in units of 2^-64
+  const unsigned __int128 p = ((unsigned __int128)__umul64hi(m, K) << 64) | (m * K);
+  const int s = 1076 - ex;
+  const unsigned __int128 q = s >= 0 ? (s < 128 ? p >> s : 0) : (s > -128 ? p << -s : 0);
+  const unsigned long long x = omcospi_frac((unsigned long long)q, (unsigned int)(q >> 64) & 1u);
+  return ex == 0x7FF ? CUDART_NAN : cos_of_om(x);
 }
 
 // 10 (1 - cos(2 pi z)), the periodic part of Rastrigin's term z^2 - 10 cos(2 pi

@@ -152,6 +152,18 @@ __global__ void k_reset_states(const RunDesc* __restrict__ runs, int run0, int n
   *R.st = st;
 }
 
+// Constants per coordinate of the basic functions (they took a power, or a
+// square root, a division and a cosine's range reduction, for every row).
+__global__ void k_suite_table(const RunDesc* __restrict__ runs) {
+  const RunDesc& R = runs[blockIdx.x];
+  if (!R.ctab) return;
+  double* tab = const_cast<double*>(R.ctab);
+  for (int e = threadIdx.x; e < R.nc * R.d; e += blockDim.x) {
+    const int c = e / R.d, l = e - c * R.d;
+    tab[(size_t)c * R.dp + l] = basic_constant(R.sfn[c], l, R.d);
+  }
+}
+
 // Split precisions: the best individual's fitness in FP64 where it is stored
 // as a split value (blockIdx.x: the run, from run0 on).
 __global__ void __launch_bounds__(256) k_best_exact(const RunDesc* __restrict__ runs, int run0) {
@@ -744,6 +756,8 @@ void k_eval_rows_launch(const RunDesc* runs, int run, const RunDesc& Rh, const d
 void k_best_init_launch(const RunDesc* runs, int run0, int n, cudaStream_t s) {
   k_best_init<<<n, 256, 0, s>>>(runs, run0);
 }
+
+void k_suite_table_launch(const RunDesc* runs, int n, cudaStream_t s) { k_suite_table<<<n, 256, 0, s>>>(runs); }
 
 void k_jde_init_launch(const RunDesc* runs, int run0, int n, int np_max, cudaStream_t s) {
   for (int r = 0; r < n; r += 65535)

@@ -83,6 +83,9 @@ struct RunDesc {
   double skex[5];          // Katsuura's exponent 10 / n^1.2 of each (n: its length)
   double slambda[5], ssigma[5], sbias[5];  // composition: height, coverage, bias
   const int32_t* perm;     // hybrid: d positions of the permutation
+  // composition functions and basic ones that need it, dp per component:
+  // Elliptic's weights, Griewank's 1 / (2 pi sqrt(i)) (k_suite_table)
+  const double* ctab;
   // buffers
   double* X[2];
   double* f[2];

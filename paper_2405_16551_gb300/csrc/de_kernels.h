@@ -128,6 +128,8 @@ void k_eval_rows_launch(const RunDesc* runs, int run, const RunDesc& Rh, const d
                         double* f, uint8_t* fx, cudaStream_t s);
 inline int suite_comps(const RunDesc& R) { return R.obj >= DE_OBJ_COMPOSITION1 ? R.nc : 1; }
 void k_best_init_launch(const RunDesc* runs, int run0, int n, cudaStream_t s);
+// the constants R.ctab of every run that has them, once
+void k_suite_table_launch(const RunDesc* runs, int n, cudaStream_t s);
 void k_jde_init_launch(const RunDesc* runs, int run0, int n, int np_max, cudaStream_t s);
 void k_ode_reference_launch(const RunDesc* runs, int run, double* ref, cudaStream_t s);
 

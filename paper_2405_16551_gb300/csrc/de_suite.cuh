@@ -51,8 +51,10 @@ __device__ __forceinline__ double schwefel_term(double t, int n) {
 // transcendental functions), at w = w_l and v = w_{next(l)} (the cyclic
 // neighbour, for the pair functions); 0 where fn has none.  The whole CTA
 // computes these for a tile before one warp per row sums the terms.  kex:
-// Katsuura's exponent 10 / n^1.2 for this n (computed once per part).
-__device__ __forceinline__ double basic_costly(int fn, double w, double v, int l, int n, double kex) {
+// Katsuura's exponent 10 / n^1.2 for this n (computed once per part); tab: the
+// function's constants per coordinate (basic_constant), where it has them.
+__device__ __forceinline__ double basic_costly(int fn, double w, double v, int l, int n, double kex,
+                                               const double* __restrict__ tab) {
   switch (fn) {
     case kObjRastrigin: return rastrigin_w(w);
     case kObjAckley: return cos2pi_fix(w);
@@ -66,11 +68,13 @@ __device__ __forceinline__ double basic_costly(int fn, double w, double v, int l
     case kObjKatsuura: {
       // 1 + i sum_{j=1}^{32} |2^j w - nearest integer| / 2^j, to the power 10 / n^1.2;
       // 2^j w, its rounding and the difference are exact
-      double s = 0.0, p2 = 1.0;
+      // (so is the division by 2^j as a product)
+      double s = 0.0, p2 = 1.0, q2 = 1.0;
       for (int j = 1; j <= 32; ++j) {
         p2 *= 2.0;
+        q2 *= 0.5;
         const double t = p2 * w;
-        s += fabs(t - rint(t)) / p2;
+        s += fabs(t - rint(t)) * q2;
       }
       return pow(1.0 + (double)(l + 1) * s, kex);
     }
@@ -81,25 +85,44 @@ __device__ __forceinline__ double basic_costly(int fn, double w, double v, int l
       const double r = 100.0 * a * a + b * b;
       return r * r / 4000.0 - cos(r) + 1.0;
     }
-    case kObjElliptic: return n > 1 ? pow(1e6, (double)l / (double)(n - 1)) : 1.0;
-    case kObjGriewank: return cos(w / sqrt((double)(l + 1)));
+    case kObjGriewank:  // cos(w / sqrt(l + 1))
+      return cos_turns_fix(w, (unsigned long long)__double_as_longlong(tab[l]));
     default: return 0.0;
   }
 }
 
-__device__ __forceinline__ bool basic_has_costly(int fn) {
-  return fn == kObjRastrigin || fn == kObjAckley || fn == kObjSchwefel || fn == kObjSchafferF6 ||
-         fn == kObjKatsuura || fn == kObjGriewankRosenbrock || fn == kObjElliptic || fn == kObjGriewank;
+// The constant of coordinate l of basic function fn on n coordinates:
+// Elliptic's weight 10^(6 l / (n - 1)); Griewank's 1 / (2 pi sqrt(l + 1)) in
+// units of 2^-66 as an integer (cos_turns_fix), from a square root and a
+// quotient with their remainders (2^-59 relative or better).
+__device__ inline double basic_constant(int fn, int l, int n) {
+  if (fn == kObjElliptic) return n > 1 ? pow(1e6, (double)l / (double)(n - 1)) : 1.0;
+  if (fn != kObjGriewank) return 0.0;
+  const double i = (double)(l + 1);
+  // 1 / (2 pi) = 0.15915494309189533576888376337251436203446... as a sum of two doubles
+  const double c_hi = 0x1.45f306dc9c883p-3, c_lo = -0x1.6b01ec5417056p-57;
+  const double s = sqrt(i), s_lo = __fma_rn(-s, s, i) / (2.0 * s);
+  const double q = c_hi / s, r = __fma_rn(-q, s, c_hi);
+  const double q_lo = (r + c_lo - q * s_lo) / s;
+  return __longlong_as_double((long long)((unsigned long long)(q * 0x1p66) +
+                                          (unsigned long long)__double2ll_rn(q_lo * 0x1p66)));
 }
 
-// g of basic function fn on the n-vector w_l = sc * z[src(l)], src(l) =
-// idx[base + l] (idx != NULL: a hybrid part) or base + l; position i = l + 1;
-// E[l] holds basic_costly of coordinate l.  Called by a whole warp: lane k
-// sums the terms of l = k, k + 32, ... in order, then a fixed xor tree; every
-// lane returns g.
-static __device__ __noinline__ double basic_fn_warp(int fn, const double* __restrict__ z,
-                                                    const int32_t* __restrict__ idx, int base, int n, double sc,
-                                                    const double* __restrict__ E, int lane) {
+__device__ __forceinline__ bool basic_has_costly(int fn) {
+  return fn == kObjRastrigin || fn == kObjAckley || fn == kObjSchwefel || fn == kObjSchafferF6 ||
+         fn == kObjKatsuura || fn == kObjGriewankRosenbrock || fn == kObjGriewank;
+}
+
+// The two sums (or a sum and a product) over the coordinates of which
+// basic_finish makes g of basic function fn on the n-vector w_l = sc * z[src(l)],
+// src(l) = idx[base + l] (idx != NULL: a hybrid part) or base + l; position
+// i = l + 1; E[l] holds basic_costly of coordinate l, tab the constants.  Called
+// by a whole warp: lane k sums the terms of l = k, k + 32, ... in order, then a
+// fixed xor tree; every lane gets them.
+static __device__ __noinline__ double2 basic_sums_warp(int fn, const double* __restrict__ z,
+                                                       const int32_t* __restrict__ idx, int base, int n, double sc,
+                                                       const double* __restrict__ E, const double* __restrict__ tab,
+                                                       int lane) {
   auto W = [&](int l) { return sc * z[idx ? idx[base + l] : base + l]; };
   double s1 = 0.0, s2 = 0.0, p = 1.0;
   for (int l = lane; l < n; l += 32) {
@@ -135,9 +158,9 @@ static __device__ __noinline__ double basic_fn_warp(int fn, const double* __rest
         break;
       }
       case kObjKatsuura: p *= E[l]; break;
-      case kObjElliptic: s1 += E[l] * (w * w); break;
+      case kObjElliptic: s1 += tab[l] * (w * w); break;
       case kObjGriewank:
-        s1 += w * w / 4000.0;
+        s1 += w * w;
         p *= E[l];
         break;
       default: s1 = CUDART_NAN;
@@ -145,37 +168,50 @@ static __device__ __noinline__ double basic_fn_warp(int fn, const double* __rest
   }
   s1 = warp_sum(s1);
   switch (fn) {
+    case kObjAckley:
+    case kObjZakharov:
+    case kObjHGBat:
+    case kObjHappyCat: return make_double2(s1, warp_sum(s2));
+    case kObjKatsuura:
+    case kObjGriewank: return make_double2(s1, warp_prod(p));
+    default: return make_double2(s1, 0.0);
+  }
+}
+
+// g of basic function fn on n coordinates from its sums.
+static __device__ __noinline__ double basic_finish(int fn, double s1, double s2, int n) {
+  switch (fn) {
     case kObjAckley: {
-      s2 = warp_sum(s2);
       return 20.0 + 2.718281828459045 - 20.0 * exp(-0.2 * sqrt(s1 / n)) - exp(s2 / n);
     }
     case kObjZakharov: {
-      s2 = warp_sum(s2);
       const double b2 = s2 * s2;
       return s1 + b2 + b2 * b2;
     }
     case kObjSchwefel: return 418.9828872724338 * n - s1;
     case kObjHGBat: {
       // |a^2 - b^2|^(1/2) + (0.5 a + b) / n + 0.5, a = sum x^2, b = sum x
-      s2 = warp_sum(s2);
       return sqrt(fabs(s1 * s1 - s2 * s2)) + (0.5 * s1 + s2) / n + 0.5;
     }
     case kObjHappyCat: {
       // |a - n|^(1/4) + (0.5 a + b) / n + 0.5
-      s2 = warp_sum(s2);
       return pow(fabs(s1 - n), 0.25) + (0.5 * s1 + s2) / n + 0.5;
     }
     case kObjKatsuura: {
-      p = warp_prod(p);
       const double c = 10.0 / ((double)n * n);
-      return c * p - c;
+      return c * s2 - c;
     }
     case kObjGriewank: {
-      p = warp_prod(p);
-      return s1 - p + 1.0;
+      return s1 / 4000.0 - s2 + 1.0;
     }
     default: return s1;
   }
+}
+
+__device__ __forceinline__ double basic_fn_warp(int fn, const double* z, const int32_t* idx, int base, int n, double sc,
+                                                const double* E, const double* tab, int lane) {
+  const double2 s = basic_sums_warp(fn, z, idx, base, n, sc, E, tab, lane);
+  return basic_finish(fn, s.x, s.y, n);
 }
 
 // Rotation of the tile's nrows rows with a given transposed matrix: thread
@@ -260,26 +296,46 @@ __device__ __forceinline__ double suite_digits(const RunDesc& R, const SliceCtx&
   return warp_sum(dd);
 }
 
-// Weights and mixture of a composition function from g_c (comp[0..4]) and
-// D_c (comp[5..9]) of one row.
-__device__ __forceinline__ double comp_mix(const RunDesc& R, const double* comp) {
+// f[r] of nrows rows of a composition function from g_c (comp[r][0..4]) and
+// D_c (comp[r][5..9]); the whole CTA, which has synchronised.  A thread takes
+// a (row, component) pair: the logarithms and exponentials of a row in one
+// thread were the longest chain of a small tile.
+__device__ __forceinline__ void comp_mix(const RunDesc& R, double (*comp)[10], double* f, int nrows) {
   const int nc = R.nc, d = R.d;
-  int hit = -1;
-  for (int c = 0; c < nc; ++c)
-    if (comp[5 + c] == 0.0 && hit < 0) hit = c;
-  double om[5], m = -CUDART_INF, sum = 0.0;
-  for (int c = 0; c < nc; ++c) {
-    const double D = comp[5 + c];
-    om[c] = -0.5 * log(D) - D / (2.0 * d * R.ssigma[c] * R.ssigma[c]);
-    m = fmax(m, om[c]);
+  for (int e = threadIdx.x; e < nc * nrows; e += blockDim.x) {
+    const int c = e / nrows, r = e - c * nrows;
+    const double D = comp[r][5 + c];
+    // +infinity exactly at x = o_c
+    comp[r][5 + c] = -0.5 * log(D) - D / (2.0 * d * R.ssigma[c] * R.ssigma[c]);
   }
-  for (int c = 0; c < nc; ++c) {
-    om[c] = hit >= 0 ? (c == hit ? 1.0 : 0.0) : exp(om[c] - m);
-    sum += om[c];
+  __syncthreads();
+  // (rounds of whole rows: a row is read by all its threads before they write it)
+  const int per = max(1, (int)blockDim.x / nc);
+  for (int r0 = 0; r0 < nrows; r0 += per) {
+    const int c = (int)threadIdx.x / per, r = r0 + (int)threadIdx.x - c * per;
+    const bool in = c < nc && r < nrows;
+    double v = 0.0;
+    if (in) {
+      int hit = -1;
+      double m = -CUDART_INF;
+      for (int q = 0; q < nc; ++q) {
+        const double om = comp[r][5 + q];
+        if (om == CUDART_INF && hit < 0) hit = q;
+        m = fmax(m, om);
+      }
+      v = hit >= 0 ? (c == hit ? 1.0 : 0.0) : exp(comp[r][5 + c] - m);
+    }
+    __syncthreads();
+    if (in) comp[r][5 + c] = v;
+    __syncthreads();
   }
-  double acc = 0.0;
-  for (int c = 0; c < nc; ++c) acc += om[c] / sum * (R.slambda[c] * comp[c] + R.sbias[c]);
-  return acc;
+  for (int r = threadIdx.x; r < nrows; r += blockDim.x) {
+    double sum = 0.0, acc = 0.0;
+    for (int c = 0; c < nc; ++c) sum += comp[r][5 + c];
+    for (int c = 0; c < nc; ++c) acc += comp[r][5 + c] / sum * (R.slambda[c] * comp[r][c] + R.sbias[c]);
+    f[r] = acc;
+  }
+  __syncthreads();
 }
 
 // Composition function of nrows rows of src with the sliced rotation: one
@@ -295,6 +351,7 @@ static __device__ __noinline__ void suite_comp_sliced(const RunDesc& R, const do
     slice_load_m(sc, R.sl + (size_t)c * kSlices * slice_bytes(kpad), kpad);
     const int fn = R.sfn[c];
     const bool costly = basic_has_costly(fn);
+    const double* tab = R.ctab + (size_t)c * dp;
     for (int t0 = 0; t0 < nrows; t0 += kSliceRows) {
       const int nr = min(kSliceRows, nrows - t0);
       if (warp < nr) {
@@ -311,19 +368,25 @@ static __device__ __noinline__ void suite_comp_sliced(const RunDesc& R, const do
           const int r = e / dp, j = e - r * dp;
           if (j >= d) continue;
           const double* zr = Z + r * dp;
-          Y[e] = basic_costly(fn, zr[j], zr[j + 1 < d ? j + 1 : 0], j, d, R.skex[c]);
+          Y[e] = basic_costly(fn, zr[j], zr[j + 1 < d ? j + 1 : 0], j, d, R.skex[c], tab);
         }
         __syncthreads();
       }
       if (warp < nr) {
-        const double g = basic_fn_warp(fn, Z + warp * dp, nullptr, 0, d, 1.0, Y + warp * dp, lane);
-        if (lane == 0) comp[t0 + warp][c] = g;
+        const double2 g = basic_sums_warp(fn, Z + warp * dp, nullptr, 0, d, 1.0, Y + warp * dp, tab, lane);
+        if (lane == 0) {
+          comp[t0 + warp][c] = g.x;
+          f[t0 + warp] = g.y;  // until the component is finished
+        }
       }
       __syncthreads();
     }
+    // a thread per row (as a warp per row, every lane took the same
+    // exponentials and roots, 8 rows at a time)
+    for (int r = tid; r < nrows; r += blockDim.x) comp[r][c] = basic_finish(fn, comp[r][c], f[r], d);
   }
-  for (int r = tid; r < nrows; r += blockDim.x) f[r] = comp_mix(R, comp[r]);
   __syncthreads();
+  comp_mix(R, comp, f, nrows);
 }
 
 // Objective of the suite for nrows rows of src (row stride ld, in shared or
@@ -387,13 +450,14 @@ static __device__ __noinline__ void suite_tile(const RunDesc& R, const double* s
       const int c = e / blk, rem = e - c * blk, r = rem / dp, j = rem - r * dp;
       if (j >= d || !basic_has_costly(R.sfn[c])) continue;
       const double* zr = Z + (size_t)c * blk + r * dp;
-      Y[e] = basic_costly(R.sfn[c], zr[j], zr[j + 1 < d ? j + 1 : 0], j, d, R.skex[c]);
+      Y[e] = basic_costly(R.sfn[c], zr[j], zr[j + 1 < d ? j + 1 : 0], j, d, R.skex[c], R.ctab + (size_t)c * dp);
     }
     __syncthreads();
     for (int p = warp; p < nc * nrows; p += nwarps) {
       const int c = p / nrows, r = p - c * nrows;
       const double g =
-          basic_fn_warp(R.sfn[c], Z + (size_t)c * blk + r * dp, nullptr, 0, d, 1.0, Y + (size_t)c * blk + r * dp, lane);
+          basic_fn_warp(R.sfn[c], Z + (size_t)c * blk + r * dp, nullptr, 0, d, 1.0, Y + (size_t)c * blk + r * dp,
+                        R.ctab + (size_t)c * dp, lane);
       const double* oc = R.o + (size_t)c * dp;
       double dd = 0.0;
       for (int j = lane; j < d; j += 32) {
@@ -407,8 +471,7 @@ static __device__ __noinline__ void suite_tile(const RunDesc& R, const double* s
       }
     }
     __syncthreads();
-    for (int r = threadIdx.x; r < nrows; r += blockDim.x) f[r] = comp_mix(R, comp[r]);
-    __syncthreads();
+    comp_mix(R, comp, f, nrows);
     return;
   }
   // basic and hybrid functions: one shift and one rotation
@@ -454,14 +517,14 @@ static __device__ __noinline__ void suite_tile(const RunDesc& R, const double* s
       const double* zr = Z + r * dp;
       const double sc = R.sscale[q];
       Y[r * dp + b0 + l] =
-          basic_costly(R.sfn[q], sc * zr[R.perm[b0 + l]], sc * zr[R.perm[b0 + (l + 1 < n ? l + 1 : 0)]], l, n, R.skex[q]);
+          basic_costly(R.sfn[q], sc * zr[R.perm[b0 + l]], sc * zr[R.perm[b0 + (l + 1 < n ? l + 1 : 0)]], l, n, R.skex[q], nullptr);
     }
   } else if (basic_has_costly(R.obj)) {
     for (int e = threadIdx.x; e < nrows * dp; e += blockDim.x) {
       const int r = e / dp, j = e - r * dp;
       if (j >= d) continue;
       const double* zr = Z + r * dp;
-      Y[e] = basic_costly(R.obj, zr[j], zr[j + 1 < d ? j + 1 : 0], j, d, R.skex[0]);
+      Y[e] = basic_costly(R.obj, zr[j], zr[j + 1 < d ? j + 1 : 0], j, d, R.skex[0], R.ctab);
     }
   }
   __syncthreads();
@@ -471,9 +534,10 @@ static __device__ __noinline__ void suite_tile(const RunDesc& R, const double* s
     double g = 0.0;
     if (is_hyb) {
       for (int q = 0; q < R.nc; ++q)
-        g += basic_fn_warp(R.sfn[q], zr, R.perm, R.seg[q], R.seg[q + 1] - R.seg[q], R.sscale[q], er + R.seg[q], lane);
+        g += basic_fn_warp(R.sfn[q], zr, R.perm, R.seg[q], R.seg[q + 1] - R.seg[q], R.sscale[q], er + R.seg[q], nullptr,
+                           lane);
     } else {
-      g = basic_fn_warp(R.obj, zr, nullptr, 0, d, 1.0, er, lane);
+      g = basic_fn_warp(R.obj, zr, nullptr, 0, d, 1.0, er, R.ctab, lane);
     }
     if (lane == 0) f[r] = g;
   }
