@@ -13,7 +13,11 @@
 //     generation's draws are made between arriving and waiting); after it every
 //     warp takes the best record and the stop decision from the keys itself;
 //   - a lane holds one coordinate (two for d > 32): an FP64 instruction costs
-//     the same however few lanes are active.
+//     the same however few lanes are active;
+//   - for d <= 32 the digit products of a rotation run on mma.sync: at 32 x 32
+//     the issue, commit and read-back of tcgen05 cost more than the products,
+//     and its tensor memory would need a whole SM per CTA (fp64_exclusive_smem),
+//     which 16 islands of 8 CTAs do not get (15 such clusters fit at once).
 // Populations, fitness and state go to global memory at the end of the launch
 // and at migrations.  The numbers are those of the general kernels: the same
 // trial, rotation (sliced, or the DFMA chain for the others) and term routines,
@@ -48,24 +52,86 @@ namespace de {
 constexpr int kLocalNp = 64;                // targets of a run (8 CTAs of 8 warps)
 constexpr long long kLocalSpin = 1LL << 22;  // polls of an island counter (each a round trip to L2)
 
-// Byte offsets of a CTA's dynamic shared memory: operands of the sliced
-// rotation (SL), FP64 rows of y and of the rows that take the chain, the two
-// population buffers, M^T (not SL).
+// How the rotation runs: not at all or as the DFMA chain; as digit products
+// on tcgen05; as digit products on mma.sync (d <= 32).
+enum LocalRot { kRotChain = 0, kRotTc = 1, kRotMma = 2 };
+
+// Operands of the mma.sync form: y's digits as slice_digits writes them (32
+// coordinates), M's digits [digit][8-coordinate group][output < 32] of 16 bytes,
+// the group sums [group][row][output].
+constexpr uint32_t kMmaB = 4u * kSliceKg, kMmaA = (uint32_t)kSlices * 4u * 32u * 16u;
+constexpr int kMmaPst = 36;  // floats per row of the sums (the accumulators' stores meet no bank twice)
+constexpr uint32_t kMmaP = 9u * kSliceRows * kMmaPst * 4u;
+
+// Byte offsets of a CTA's dynamic shared memory: operands of the digit
+// products, FP64 rows of y and of the rows that take the chain, the two
+// population buffers, M^T (chain).
 struct LocalLayout {
   uint32_t y, z, pop, mt, total;
 };
-__host__ __device__ inline LocalLayout local_layout(bool sl, int kpad, int dp, int d, bool rotate) {
+__host__ __device__ inline LocalLayout local_layout(int rot, int kpad, int dp, int d, bool rotate) {
   LocalLayout L;
-  L.y = sl ? slice_smem(kpad) : 0u;
+  L.y = rot == kRotTc ? slice_smem(kpad) : rot == kRotMma ? kMmaB + kMmaA + kMmaP : 0u;
   L.z = L.y + (uint32_t)(kSliceRows * dp) * 8u;
-  L.pop = L.z + (sl ? (uint32_t)(kSliceRows * dp) * 8u : 0u);
+  L.pop = L.z + (rot == kRotTc ? (uint32_t)(kSliceRows * dp) * 8u : 0u);
   L.mt = L.pop + 2u * (uint32_t)(kLocalNp * dp) * 8u;
-  L.total = L.mt + (!sl && rotate ? (uint32_t)(d * d) * 8u : 0u);
+  L.total = L.mt + (rot == kRotChain && rotate ? (uint32_t)(d * d) * 8u : 0u);
   return L;
 }
 
-template <int CPL, bool SL, bool ISL>
-__global__ void __launch_bounds__(256, 1)
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, "
+      "%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// The digit products of outputs 16 mt .. + 15 in groups G0 >= G1 >= G2 (the
+// pairs of digits s of y and t of M with s + t = g; -1: none), into the sums.
+// Integers below 2^23 in FP32: exact.
+template <int G0, int G1, int G2>
+__device__ __forceinline__ void local_products(uint32_t sB, uint32_t sA, float* P, int mt, int lane) {
+  const int i = lane >> 3, r = lane & 7;
+  uint32_t b[kSlices][4];  // per digit of y: the 8-coordinate groups 0 .. 3
+#pragma unroll
+  for (int s = 0; s < kSlices; ++s)
+    if (s <= G0) ldmatrix4(b[s], sB + (uint32_t)i * kSliceKg + (uint32_t)s * 128u + (uint32_t)r * 16u);
+  float c[3][4] = {};
+  const uint32_t a0 = sA + ((uint32_t)(i >> 1) * 32u + (uint32_t)(16 * mt + 8 * (i & 1) + r)) * 16u;
+#pragma unroll
+  for (int t = 0; t < kSlices; ++t) {
+    if (t > G0) continue;
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks) {
+      uint32_t a[4];
+      ldmatrix4(a, a0 + (uint32_t)(t * 4 + 2 * ks) * 512u);
+      if (G0 - t >= 0 && G0 - t < kSlices) mma_16816(c[0], a, b[(G0 - t) & 7][2 * ks], b[(G0 - t) & 7][2 * ks + 1]);
+      if (G1 - t >= 0 && G1 - t < kSlices) mma_16816(c[1], a, b[(G1 - t) & 7][2 * ks], b[(G1 - t) & 7][2 * ks + 1]);
+      if (G2 - t >= 0 && G2 - t < kSlices) mma_16816(c[2], a, b[(G2 - t) & 7][2 * ks], b[(G2 - t) & 7][2 * ks + 1]);
+    }
+  }
+  constexpr int G[3] = {G0, G1, G2};
+  const int n = 2 * (lane & 3), j = 16 * mt + (lane >> 2);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (G[q] < 0) continue;
+    float* p = P + (size_t)(G[q] * kSliceRows + n) * kMmaPst + j;
+    p[0] = c[q][0];
+    p[kMmaPst] = c[q][1];
+    p[8] = c[q][2];
+    p[kMmaPst + 8] = c[q][3];
+  }
+}
+
+template <int CPL, int ROT, bool ISL>
+__global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
     k_gen_local(const RunDesc* __restrict__ runs, PersistCtl* ctl, long long gens, int csize, IslandCtl* isl,
                 IslandStage stage, int kpad, uint32_t cols, int dp_max) {
   extern __shared__ __align__(1024) uint8_t smem_l[];
@@ -89,7 +155,8 @@ __global__ void __launch_bounds__(256, 1)
   const int np = R.np, d = R.d, dp = R.dp, obj = R.obj;
   const bool stopped0 = *(volatile int32_t*)&st->stop != 0;
   if (!ISL && stopped0) return;  // the whole cluster
-  const LocalLayout L = local_layout(SL, kpad, dp_max, 0, false);
+  constexpr bool SL = ROT == kRotTc, MM = ROT == kRotMma;
+  const LocalLayout L = local_layout(ROT, kpad, dp_max, 0, false);
   double* Y = reinterpret_cast<double*>(smem_l + L.y);
   double* Zf = reinterpret_cast<double*>(smem_l + L.z);
   double* pop = reinterpret_cast<double*>(smem_l + L.pop);
@@ -99,9 +166,25 @@ __global__ void __launch_bounds__(256, 1)
   if constexpr (SL) {
     slice_begin(sc, smem_l, kpad, cols, s_sl);
     slice_load_m(sc, R.sl, R.sl_kpad);
+  } else if constexpr (MM) {
+    sc.sB = smem_l;
+    sc.s_exp = s_sl.exp;
+    sc.s_bad = &s_sl.bad;
+    if (tid == 0) s_sl.bad = 0u;
+    for (uint32_t q = tid * 16u; q < kMmaB; q += blockDim.x * 16u)
+      *reinterpret_cast<uint4*>(smem_l + q) = make_uint4(0u, 0u, 0u, 0u);
+    const int nkg = R.sl_kpad / 8;
+    for (int e = tid; e < kSlices * 4 * 32; e += blockDim.x) {
+      const int t = e >> 7, kg = (e >> 5) & 3, r = e & 31;
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+      if (kg < nkg)
+        v = __ldg(reinterpret_cast<const uint4*>(R.sl + (size_t)t * slice_bytes(R.sl_kpad) + (size_t)kg * 2048u + r * 16));
+      *reinterpret_cast<uint4*>(smem_l + kMmaB + (size_t)e * 16u) = v;
+    }
   } else if (R.rotate) {
     for (int e = tid; e < d * d; e += blockDim.x) mts[e] = __ldg(R.MT + e);
   }
+  const int fj = MM && lane < d ? __ldg(R.slx + lane) : 0;
   long long gen = *(volatile int64_t*)&st->gen;
   int64_t evals = *(volatile int64_t*)&st->evals;
   double bestf = *(volatile double*)&st->best_f;
@@ -193,11 +276,44 @@ __global__ void __launch_bounds__(256, 1)
       }
       __syncthreads();
       ft = slice_fitness(sc, R, Y, Zf, nrows);
-    } else if (mine) {
-      // one coordinate a lane (d <= 32): the sums of the general kernel, whose
+    } else {
+      // one coordinate a lane (d <= 32): the sums of the general kernels, whose
       // lane j holds coordinate j
       double z = y[0];
-      if (R.rotate) {
+      if constexpr (MM) {
+        if (mine) slice_digits(sc, warp, lane, R.sl_kpad, R.sl_qmin[0], y);
+        __syncthreads();
+        float* sP = reinterpret_cast<float*>(smem_l + kMmaB + kMmaA);
+        const uint32_t sB = smem_u32(smem_l), sA = sB + kMmaB;
+        // a warp takes 16 outputs and 10 to 12 of the 43 pairs of digits
+        if (16 * (warp & 1) < d) {
+          switch (warp >> 1) {
+            case 0: local_products<8, 3, -1>(sB, sA, sP, warp & 1, lane); break;
+            case 1: local_products<7, 2, -1>(sB, sA, sP, warp & 1, lane); break;
+            case 2: local_products<6, 1, 0>(sB, sA, sP, warp & 1, lane); break;
+            default: local_products<5, 4, -1>(sB, sA, sP, warp & 1, lane); break;
+          }
+        }
+        __syncthreads();
+        if (mine) {
+          float p[9];
+#pragma unroll
+          for (int q = 0; q < 9; ++q) p[q] = sP[(q * kSliceRows + warp) * kMmaPst + lane];
+          const double zj = slice_combine(p, s_sl.exp[warp] + fj - 76);
+          z = lane < d ? zj : 0.0;
+          if ((*(volatile uint32_t*)&s_sl.bad >> warp) & 1u) {
+            // outside the splitting's comparison: the DFMA chain
+            double* yr = Y + warp * dp;
+            if (lane < d) yr[lane] = y[0];
+            __syncwarp();
+            if (lane == 0) atomicAnd(&s_sl.bad, ~(1u << warp));
+            z = 0.0;
+            if (lane < d)
+              for (int k = 0; k < d; ++k) z = fma(__ldg(R.MT + (size_t)k * d + lane), yr[k], z);
+            __syncwarp();
+          }
+        }
+      } else if (mine && R.rotate) {
         double* yr = Y + warp * dp;
         if (lane < d) yr[lane] = y[0];
         __syncwarp();
@@ -206,27 +322,29 @@ __global__ void __launch_bounds__(256, 1)
           for (int k = 0; k < d; ++k) z = fma(mts[k * d + lane], yr[k], z);
         __syncwarp();
       }
-      double t1 = 0.0, t2 = 0.0;
-      if (obj == kObjRosenbrock) {
-        const double zn = __shfl_down_sync(0xffffffffu, z, 1);
-        if (lane + 1 < d) {
-          const double t0 = z + 1.0, tn = zn + 1.0;
-          const double a = tn - t0 * t0, b = t0 - 1.0;
-          t1 = 100.0 * a * a + b * b;
+      if (mine) {
+        double t1 = 0.0, t2 = 0.0;
+        if (obj == kObjRosenbrock) {
+          const double zn = __shfl_down_sync(0xffffffffu, z, 1);
+          if (lane + 1 < d) {
+            const double t0 = z + 1.0, tn = zn + 1.0;
+            const double a = tn - t0 * t0, b = t0 - 1.0;
+            t1 = 100.0 * a * a + b * b;
+          }
+        } else if (lane < d) {
+          if (obj == kObjRastrigin) {
+            t1 = fma(z, z, rastrigin_w(z));
+          } else {
+            t1 = z * z;
+            if (obj == kObjAckley) t2 = cos2pi_fix(z);
+          }
         }
-      } else if (lane < d) {
-        if (obj == kObjRastrigin) {
-          t1 = fma(z, z, rastrigin_w(z));
-        } else {
-          t1 = z * z;
-          if (obj == kObjAckley) t2 = cos2pi_fix(z);
+        const double s1 = warp_sum(t1);
+        ft = s1;
+        if (obj == kObjAckley) {
+          const double s2 = warp_sum(t2);
+          ft = 20.0 + 2.718281828459045 - 20.0 * exp(-0.2 * sqrt(s1 / d)) - exp(s2 / d);
         }
-      }
-      const double s1 = warp_sum(t1);
-      ft = s1;
-      if (obj == kObjAckley) {
-        const double s2 = warp_sum(t2);
-        ft = 20.0 + 2.718281828459045 - 20.0 * exp(-0.2 * sqrt(s1 / d)) - exp(s2 / d);
       }
     }
     // ---- selection; the row and its key to every CTA of the cluster
@@ -387,17 +505,21 @@ __global__ void __launch_bounds__(256, 1)
 }
 
 // ------------------------------------------------------------------ host side
-static const void* local_kernel(bool sl, bool isl, int kpad) {
-  if (!sl) return isl ? (const void*)k_gen_local<1, false, true> : (const void*)k_gen_local<1, false, false>;
-  if (kpad <= 32) return isl ? (const void*)k_gen_local<1, true, true> : (const void*)k_gen_local<1, true, false>;
-  return isl ? (const void*)k_gen_local<2, true, true> : (const void*)k_gen_local<2, true, false>;
+static int local_rot(const LocalPlan& p) { return !p.sl ? kRotChain : p.kpad <= 32 ? kRotMma : kRotTc; }
+
+static const void* local_kernel(const LocalPlan& p, bool isl) {
+  switch (local_rot(p)) {
+    case kRotChain: return isl ? (const void*)k_gen_local<1, kRotChain, true> : (const void*)k_gen_local<1, kRotChain, false>;
+    case kRotMma: return isl ? (const void*)k_gen_local<1, kRotMma, true> : (const void*)k_gen_local<1, kRotMma, false>;
+    default: return isl ? (const void*)k_gen_local<2, kRotTc, true> : (const void*)k_gen_local<2, kRotTc, false>;
+  }
 }
 
 static size_t local_smem(const LocalPlan& p, const void* k) {
-  const size_t need = local_layout(p.sl, p.kpad, p.dp_max, p.d_max, p.rotate).total;
-  // sliced: a whole SM (fp64_exclusive_smem: the cluster's CTAs wait for one
-  // another while they hold tensor memory)
-  return p.sl ? fp64_exclusive_smem(k, need) : need;
+  const size_t need = local_layout(local_rot(p), p.kpad, p.dp_max, p.d_max, p.rotate).total;
+  // with tensor memory: a whole SM (fp64_exclusive_smem: the cluster's CTAs
+  // wait for one another while they hold it)
+  return local_rot(p) == kRotTc ? fp64_exclusive_smem(k, need) : need;
 }
 
 static cudaLaunchConfig_t local_config(const LocalPlan& p, const void* k, int nruns, bool isl, cudaStream_t s,
@@ -442,7 +564,7 @@ bool local_plan(LocalPlan& p, const std::vector<RunDesc>& runs, const SlicePlan&
 }
 
 bool local_fits(const LocalPlan& p, int nruns, bool isl) {
-  const void* k = local_kernel(p.sl, isl, p.kpad);
+  const void* k = local_kernel(p, isl);
   const size_t smem = local_smem(p, k);
   cudaLaunchAttribute attr[2];
   int n = 0;
@@ -464,7 +586,7 @@ cudaError_t k_gen_local_launch(const RunDesc* runs, int nruns, const LocalPlan& 
   if (e != cudaSuccess) return e;
   IslandStage st{};
   if (stage) st = *stage;
-  const void* k = local_kernel(p.sl, isl != nullptr, p.kpad);
+  const void* k = local_kernel(p, isl != nullptr);
   cudaLaunchAttribute attr[2];
   const cudaLaunchConfig_t cfg = local_config(p, k, nruns, isl != nullptr, s, attr);
   int csize = p.csize, kpad = p.kpad, dp_max = p.dp_max;
