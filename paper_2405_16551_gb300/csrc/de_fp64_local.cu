@@ -228,21 +228,44 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
   const unsigned m_isl = ISL ? (unsigned)isl->m : 1u;
   const bool test_skip = ISL && ctl->test_skip == run + 1;
   const long long spin = ISL && ctl->test_spin > 0 ? ctl->test_spin : kLocalSpin;
-  // rank 0's waits: until `want` arrivals on a counter (one lane polls)
-  auto wait_count = [&](unsigned* cnt, unsigned want) -> bool {
+  // One island's arrival at iteration k is one relaxed addition to the counter
+  // of k's parity: 1, plus 2^32 when its best is below the target.  No other
+  // memory hangs on it, so nothing waits for a fence (an island is at most one
+  // iteration ahead of another that it waits for, and none passes a point where
+  // they meet, so a counter that reads complete holds no later arrival).
+  auto count_of = [&](long long k) -> unsigned long long* { return &ctl->isl_cnt[k & 1]; };
+  auto count_want = [&](long long k) { return m_isl * (unsigned)(k / 2 + 1); };
+  auto read_count = [&](long long k) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count_of(k)) : "memory");
+    return v;
+  };
+  auto arrive = [&](long long k, bool below) {
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(count_of(k)), "l"(1ULL + (below ? 1ULL << 32 : 0ULL))
+                 : "memory");
+  };
+  // until every island has arrived at iteration k (v: the counter as read
+  // before; one lane polls): 0, 1 when some island is below the target, 2 gave up
+  auto wait_islands = [&](long long k, unsigned long long v) -> int {
+    for (long long q = 0; q < spin; ++q) {
+      if ((unsigned)v >= count_want(k)) return v >> 32 ? 1 : 0;
+      if ((q & 15) == 15 && *(volatile int*)&ctl->abort) break;
+      v = read_count(k);
+    }
+    atomicExch(&ctl->abort, 1);
+    return 2;
+  };
+  // the migrations' own counter: orders the mailbox's writes before its reads
+  auto wait_posted = [&](unsigned want) -> bool {
     for (long long q = 0; q < spin; ++q) {
       unsigned v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&ctl->sbar[0]) : "memory");
       if (v >= want) return true;
       if ((q & 15) == 15 && *(volatile int*)&ctl->abort) break;
     }
     atomicExch(&ctl->abort, 1);
     return false;
   };
-  auto arrive = [&](unsigned* cnt) { asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(cnt), "r"(1u) : "memory"); };
-  // the index (in this launch) of the first generation in which an island was
-  // below the target; large when none was
-  auto stop_index = [&]() { return (long long)(0xFFFFFFFFu - *(volatile unsigned*)&ctl->below[0]); };
   // every CTA is running and has loaded before any peer writes its memory
   cluster.sync();
 
@@ -251,6 +274,7 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
     const long long g = gen + 1;
     const double* P = pop + (size_t)(gen & 1) * psz;
     double ft = 0.0;
+    unsigned long long early = 0ULL;  // rank 0, thread 0: the islands' last counter, read ahead of its use
     double y[CPL] = {};
     // ---- trial: Eq. 2, Eq. 3, bound repair; y = (t - o) s
     if (in) {
@@ -322,6 +346,7 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
           for (int k = 0; k < d; ++k) z = fma(mts[k * d + lane], yr[k], z);
         __syncwarp();
       }
+      if (common && rank == 0 && tid == 0 && it > 0) early = read_count(it - 1);
       if (mine) {
         double t1 = 0.0, t2 = 0.0;
         if (obj == kObjRosenbrock) {
@@ -366,10 +391,8 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
     if (SL && tid == 0 && s_sl.fail)
       for (int c = 0; c < csize; ++c) *cluster.map_shared_rank(&s_fail[g & 1], c) = 1;
     if (common && rank == 0 && tid == 0 && it > 0) {
-      // whether the model stopped at an earlier generation: every island has
-      // counted the one before this
-      const bool ok = wait_count(&ctl->bar, m_isl * (unsigned)it);
-      const int f = !ok ? 2 : stop_index() < it ? 1 : 0;
+      // whether the model stopped at the generation before this
+      const int f = wait_islands(it - 1, early);
       if (f)
         for (int c = 0; c < csize; ++c) *cluster.map_shared_rank(&s_flag[g & 1], c) = f;
     }
@@ -416,8 +439,7 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
     else if (gen >= R.max_gens) stop = 3;
     if constexpr (ISL) {
       if (rank == 0 && tid == 0 && (common || isl->interval > 0)) {
-        if (common && below) atomicMax(&ctl->below[0], 0xFFFFFFFFu - (unsigned)it);
-        if (!(test_skip && it == 0)) arrive(&ctl->bar);
+        if (!(test_skip && it == 0)) arrive(it, common && below);
       }
       const bool mig = isl->interval > 0 && gen % isl->interval == 0;
       if (mig || stop || it + 1 >= gens) {
@@ -428,7 +450,10 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
         if (rank == 0) {
           if (tid == 0) {
             int f = 0;
-            if (common || mig) f = !wait_count(&ctl->bar, m_isl * (unsigned)(it + 1)) ? 2 : common && stop_index() <= it ? 1 : 0;
+            if (common || mig) f = wait_islands(it, read_count(it));
+            // with the fence after the last exchange: what it read is read, and
+            // its mailbox may be written again
+            if (mig) __threadfence();
             s_over = f;
             const int sp = f == 1 ? 1 : stop;
             if (f != 2) {
@@ -456,9 +481,9 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
             __syncthreads();
             if (tid == 0) {
               // (asynchronous: post_gen is written once every island has read it)
-              arrive(&ctl->sbar[0]);
+              asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&ctl->sbar[0]), "r"(1u) : "memory");
               const unsigned k = (unsigned)(gen / isl->interval - (gen - it - 1) / isl->interval);
-              if (!wait_count(&ctl->sbar[0], m_isl * k)) s_over = 2;
+              if (!wait_posted(m_isl * k)) s_over = 2;
             }
             __syncthreads();
             if (!isl->async && s_over != 2) island_exchange(R, run, isl->m, isl->nmig, cur, stage, false, 0, true, 0);
@@ -468,8 +493,10 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
             }
           }
           __syncthreads();
-          if (tid == 0)
+          if (tid == 0) {
+            if (mig) __threadfence();
             for (int c = 1; c < csize; ++c) *cluster.map_shared_rank(&s_over, c) = s_over;
+          }
         }
         cluster.sync();
         const int over = *(volatile int*)&s_over;

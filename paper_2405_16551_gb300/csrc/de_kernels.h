@@ -26,6 +26,9 @@ struct PersistCtl {
   // island model in the cooperative FP64 kernel: tiles whose best is below
   // the target, per iteration mod 3 (the model's common stop)
   unsigned int below[3];
+  // ... in the local form: arrivals (low half) and islands below the target
+  // (high half) per iteration parity
+  unsigned long long isl_cnt[2];
   // grid-barrier arrivals of the CTA-local split kernel in sbar[0] (the rest
   // of the 128 bytes keeps other fields off its line)
   unsigned int sbar[32];
