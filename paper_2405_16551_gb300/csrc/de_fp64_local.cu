@@ -18,8 +18,8 @@
 //     the issue, commit and read-back of tcgen05 cost more than the products,
 //     and its tensor memory would need a whole SM per CTA (fp64_exclusive_smem),
 //     which 16 islands of 8 CTAs do not get (15 such clusters fit at once).
-// Populations, fitness and state go to global memory at the end of the launch
-// and at migrations.  The numbers are those of the general kernels: the same
+// Populations, fitness and state go to global memory at the end of the launch.
+// The numbers are those of the general kernels: the same
 // trial, rotation (sliced, or the DFMA chain for the others) and term routines,
 // and the same order of every sum.
 //
@@ -28,8 +28,9 @@
 // of that one generation late (the counter it would have to wait for has had
 // a generation's time to fill), and then takes back its last one, whose
 // predecessor is still in the other buffer.  At migration points the islands
-// meet (bounded waits on global counters), and the exchange runs on the
-// populations in global memory as in the other kernels.
+// meet (bounded waits on global counters); a warp picks the migrants from the
+// keys and passes them through the mailbox, in island_exchange's order (that
+// routine, a CTA on the populations in global memory, took 35 us a point).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math_constants.h>
@@ -41,7 +42,6 @@
 #include "de_device.cuh"
 #include "de_gen_tile.cuh"
 #include "de_internal.cuh"
-#include "de_island_dev.cuh"
 #include "de_kernels.h"
 #include "de_slice.cuh"
 
@@ -128,6 +128,44 @@ __device__ __forceinline__ void local_products(uint32_t sB, uint32_t sA, float* 
     p[8] = c[q][2];
     p[kMmaPst + 8] = c[q][3];
   }
+}
+
+// The fitness of a key (NaN for the largest).
+__device__ __forceinline__ double key_value(long long k) {
+  if (k == 0x7FFFFFFFFFFFFFFFLL) return CUDART_NAN;
+  return __longlong_as_double(k >= 0 ? k : (long long)(0x8000000000000000ULL | (unsigned long long)(-k)));
+}
+
+// island_pick over at most 64 keys in shared memory, n <= 32 times without
+// repetition, by one warp: lane q returns the index of the q-th smallest
+// (key, index), or largest.
+__device__ __forceinline__ int local_pick(const long long* keys, int np, int n, bool worst, int lane) {
+  // the largest as the smallest of the complements; idle entries come last
+  long long k[2];
+  int x[2], sel = 0;
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const int i = lane + 32 * e;
+    const bool in = i < np;
+    k[e] = in ? (worst ? ~keys[i] : keys[i]) : 0x7FFFFFFFFFFFFFFFLL;
+    x[e] = in ? (worst ? kLocalNp - 1 - i : i) : 2 * kLocalNp;
+  }
+  for (int q = 0; q < n; ++q) {
+    const int a = k[1] < k[0] || (k[1] == k[0] && x[1] < x[0]) ? 1 : 0;
+    const long long v = a ? k[1] : k[0];
+    const int hi = __reduce_min_sync(0xffffffffu, (int)(v >> 32));
+    const unsigned lo = __reduce_min_sync(0xffffffffu, (int)(v >> 32) == hi ? (unsigned)v : 0xffffffffu);
+    const bool cand = (int)(v >> 32) == hi && (unsigned)v == lo;
+    const int w = __reduce_min_sync(0xffffffffu, cand ? (a ? x[1] : x[0]) : 4 * kLocalNp);
+    if (lane == q) sel = worst ? kLocalNp - 1 - w : w;
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      if (x[e] == w) {
+        k[e] = 0x7FFFFFFFFFFFFFFFLL;
+        x[e] = 2 * kLocalNp;
+      }
+  }
+  return sel;
 }
 
 template <int CPL, int ROT, bool ISL>
@@ -269,6 +307,23 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
   // every CTA is running and has loaded before any peer writes its memory
   cluster.sync();
 
+  bool changed = true;  // the row in the other buffer is not the one before this
+  // the best of the keys of generation gen (every warp)
+  auto reduce_best = [&]() {
+    long long bk = lane < np ? s_key[gen & 1][lane] : 0x7FFFFFFFFFFFFFFFLL;
+    int bi = lane < np ? lane : -1;
+    const long long k2 = lane + 32 < np ? s_key[gen & 1][lane + 32] : 0x7FFFFFFFFFFFFFFFLL;
+    if (k2 < bk) {
+      bk = k2;
+      bi = lane + 32;
+    }
+    warp_best(bk, bi);
+    if (bi >= 0) {
+      bestf = key_value(bk);
+      best = bi;
+    }
+    return bi >= 0;
+  };
   long long it = 0;
   for (; it < gens && !stop && !err; ++it) {
     const long long g = gen + 1;
@@ -382,7 +437,11 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
 #pragma unroll
         for (int m = 0; m < CPL; ++m) tx[m] = tr[m];
       }
-      if (in) {
+      // the buffer holds the row of two generations ago: nothing to write for a
+      // row that neither this generation nor the last one changed
+      const bool write = acc || changed;
+      changed = acc;
+      if (in && write) {
         double* q = pop + (size_t)(g & 1) * psz + (size_t)i * dp + j0;
         for (int c = 0; c < csize; ++c) st_coords(cluster.map_shared_rank(q, c), tx);
       }
@@ -417,22 +476,7 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
     // ---- best record and stop rule, by every warp
     gen = g;
     evals += np;
-    {
-      long long bk = lane < np ? s_key[g & 1][lane] : 0x7FFFFFFFFFFFFFFFLL;
-      int bi = lane < np ? lane : -1;
-      const long long k2 = lane + 32 < np ? s_key[g & 1][lane + 32] : 0x7FFFFFFFFFFFFFFFLL;
-      if (k2 < bk) {
-        bk = k2;
-        bi = lane + 32;
-      }
-      warp_best(bk, bi);
-      if (bi >= 0) {
-        bestf = __longlong_as_double(bk >= 0 ? bk : (long long)(0x8000000000000000ULL | (unsigned long long)(-bk)));
-        best = bi;
-      } else if (rank == 0 && tid == 0) {
-        atomicOr(&st->err, kErrNonFinite);
-      }
-    }
+    if (!reduce_best() && rank == 0 && tid == 0) atomicOr(&st->err, kErrNonFinite);
     const bool below = R.target > 0.0 && best >= 0 && bestf < R.target;
     if (!ISL && below) stop = 1;
     else if (R.max_evals > 0 && evals >= R.max_evals) stop = 2;
@@ -443,60 +487,72 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
       }
       const bool mig = isl->interval > 0 && gen % isl->interval == 0;
       if (mig || stop || it + 1 >= gens) {
-        // the islands meet: the common stop at this generation, and migration
-        store_rows(gen);
-        if (rank == 0 && tid == 0) s_over = 0;
-        cluster.sync();
-        if (rank == 0) {
-          if (tid == 0) {
-            int f = 0;
-            if (common || mig) f = wait_islands(it, read_count(it));
+        // the islands meet: the common stop at this generation, and migration,
+        // by the first warp of rank 0, which holds the whole population
+        if (mig) cluster.sync();  // every warp has taken the best of the keys that migration changes
+        if (rank == 0 && warp == 0) {
+          int f = 0;
+          if (lane == 0 && (common || mig)) f = wait_islands(it, read_count(it));
+          f = __shfl_sync(0xffffffffu, f, 0);
+          if (mig && f != 2) {
             // with the fence after the last exchange: what it read is read, and
             // its mailbox may be written again
-            if (mig) __threadfence();
-            s_over = f;
-            const int sp = f == 1 ? 1 : stop;
-            if (f != 2) {
-              st->best_f = bestf;
-              st->best_idx = best;
-              st->gen = gen;
-              st->evals = evals;
-              st->stop = sp;
+            __threadfence();
+            double* p = pop + (size_t)(gen & 1) * psz;
+            long long* keys = s_key[gen & 1];
+            const int m = isl->m, nmig = isl->nmig;
+            const int64_t ep = gen / isl->interval;
+            // asynchronous: one interval late, from the slot of the last point
+            // (k_island_async's rule)
+            const bool late = isl->async != 0;
+            const long long pg = *(volatile long long*)&isl->post_gen;
+            const bool take = !late || (pg >= 0 && pg == gen - isl->interval);
+            const size_t wslot = late ? (size_t)(ep & 1) * stage.slot : 0;
+            const size_t rslot = late ? (size_t)((ep & 1) ^ 1) * stage.slot : 0;
+            const int good = local_pick(keys, np, nmig, false, lane);
+            const int poor = take ? local_pick(keys, np, nmig, true, lane) : 0;
+            for (int q = 0; q < nmig; ++q) {
+              const int i1 = __shfl_sync(0xffffffffu, good, q);
+              const size_t e = wslot + (size_t)run * nmig + q;
+              for (int j = lane; j < dp; j += 32) stage.x[e * stage.dp + j] = p[(size_t)i1 * dp + j];
+              if (lane == 0) {
+                stage.f[e] = key_value(keys[i1]);
+                stage.fx[e] = 1;
+              }
             }
-          }
-          __syncthreads();
-          if (mig && s_over != 2) {
-            const int cur = (int)(gen & 1);
-            if (isl->async) {
-              // one interval late, through the mailbox (k_island_async's rule)
-              const int64_t ep = gen / isl->interval;
-              const long long pg = *(volatile long long*)&isl->post_gen;
-              const bool take = pg >= 0 && pg == gen - isl->interval;
-              island_exchange(R, run, isl->m, isl->nmig, cur, stage, true, (size_t)(ep & 1) * stage.slot, take,
-                              (size_t)((ep & 1) ^ 1) * stage.slot);
-            } else {
-              // every island posts before any island takes
-              island_exchange(R, run, isl->m, isl->nmig, cur, stage, true, 0, false, 0);
+            __syncwarp();
+            // every island has posted (asynchronous: and read post_gen)
+            auto posted = [&]() {
+              int ok = 1;
+              if (lane == 0) {
+                asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&ctl->sbar[0]), "r"(1u) : "memory");
+                ok = wait_posted(m_isl * (unsigned)(ep - (gen - it - 1) / isl->interval)) ? 1 : 0;
+              }
+              ok = __shfl_sync(0xffffffffu, ok, 0);
+              __syncwarp();
+              if (!ok) f = 2;
+            };
+            if (!late) posted();
+            const int from = (run + m - 1) % m;
+            for (int q = 0; take && f != 2 && q < nmig; ++q) {
+              const int i1 = __shfl_sync(0xffffffffu, poor, q);
+              const size_t e = rslot + (size_t)from * nmig + q;
+              for (int j = lane; j < dp; j += 32) {
+                const double v = __ldcg(stage.x + e * stage.dp + j);
+                for (int c = 0; c < csize; ++c) *cluster.map_shared_rank(p + (size_t)i1 * dp + j, c) = v;
+              }
+              const long long k = fit_key(__ldcg(stage.f + e));
+              if (lane < csize) *cluster.map_shared_rank(keys + i1, lane) = k;
             }
-            __syncthreads();
-            if (tid == 0) {
-              // (asynchronous: post_gen is written once every island has read it)
-              asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&ctl->sbar[0]), "r"(1u) : "memory");
-              const unsigned k = (unsigned)(gen / isl->interval - (gen - it - 1) / isl->interval);
-              if (!wait_posted(m_isl * k)) s_over = 2;
-            }
-            __syncthreads();
-            if (!isl->async && s_over != 2) island_exchange(R, run, isl->m, isl->nmig, cur, stage, false, 0, true, 0);
-            if (run == 0 && tid == 0 && s_over != 2) {
+            __syncwarp();
+            if (late) posted();
+            if (run == 0 && lane == 0 && f != 2) {
               isl->mig_gen = gen;
-              if (isl->async) isl->post_gen = gen;
+              if (late) isl->post_gen = gen;
             }
+            __threadfence();
           }
-          __syncthreads();
-          if (tid == 0) {
-            if (mig) __threadfence();
-            for (int c = 1; c < csize; ++c) *cluster.map_shared_rank(&s_over, c) = s_over;
-          }
+          if (lane < csize) *cluster.map_shared_rank(&s_over, lane) = f;
         }
         cluster.sync();
         const int over = *(volatile int*)&s_over;
@@ -506,10 +562,13 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
         }
         if (over == 1) stop = 1;
         if (mig) {
-          load_pop(gen);
-          best = *(volatile int32_t*)&st->best_idx;
-          bestf = *(volatile double*)&st->best_f;
-          __syncthreads();
+          if (in) {
+#pragma unroll
+            for (int e = 0; e < CPL; ++e) tx[e] = pop[(size_t)(gen & 1) * psz + (size_t)i * dp + j0 + e];
+          }
+          if (mine) fi = key_value(s_key[gen & 1][i]);
+          changed = true;
+          reduce_best();
         }
       }
     }
