@@ -201,6 +201,16 @@ __device__ __forceinline__ long long fit_key(double f) {
 }
 
 // ------------------------------------------------------------------ objective
+// Ackley's value from the means m of the squares (even lanes) and of the
+// cosines (odd lanes): a lane takes one of the two exponentials (each some 20
+// FP64 instructions).  The whole warp; every lane gets the value.
+__device__ __forceinline__ double ackley_value(double m, int lane) {
+  const double r = sqrt(fabs(m));
+  const double e = exp(lane & 1 ? m : -0.2 * r);
+  const double e1 = __shfl_sync(0xffffffffu, e, 0), e2 = __shfl_sync(0xffffffffu, e, 1);
+  return 20.0 + 2.718281828459045 - 20.0 * e1 - e2;
+}
+
 // Objective of one row held in shared memory (z, length d); the calling warp
 // returns the same value in every lane.  Terms are summed per lane in
 // coordinate order, then across lanes by a fixed xor tree.
@@ -338,7 +348,7 @@ __device__ __forceinline__ double row_objective_fp64(int obj, const double* __re
   if (obj == kObjAckley) {
     s2 = warp_sum(s2);
     const double inv_d = 1.0 / (double)d;
-    return 20.0 + 2.718281828459045 - 20.0 * exp(-0.2 * sqrt(s1 * inv_d)) - exp(s2 * inv_d);
+    return ackley_value((lane & 1 ? s2 : s1) * inv_d, lane);
   }
   return s1;
 }

@@ -732,6 +732,7 @@ void k_best_exact_launch(const RunDesc* runs, int run0, int n, int dp_max, cudaS
 void k_eval_rows_launch(const RunDesc* runs, int run, const RunDesc& Rh, const double* x, int64_t ld, int n,
                         double* f, uint8_t* fx, cudaStream_t s) {
   if (n <= 0) return;
+  if (k_eval_few_launch(Rh, x, ld, n, f, fx, s)) return;
   if (Rh.sl) {
     k_eval_rows_tc_launch(runs, run, Rh, x, ld, n, f, fx, s);
     return;

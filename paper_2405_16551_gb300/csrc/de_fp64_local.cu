@@ -130,6 +130,82 @@ __device__ __forceinline__ void local_products(uint32_t sB, uint32_t sA, float* 
   }
 }
 
+// M's digits and the zeroed operand of y's, by the whole CTA (which
+// synchronises before the first product).
+__device__ __forceinline__ void local_load_m(const RunDesc& R, uint8_t* smem) {
+  const int tid = threadIdx.x, nkg = R.sl_kpad / 8;
+  for (uint32_t q = tid * 16u; q < kMmaB; q += blockDim.x * 16u)
+    *reinterpret_cast<uint4*>(smem + q) = make_uint4(0u, 0u, 0u, 0u);
+  for (int e = tid; e < kSlices * 4 * 32; e += blockDim.x) {
+    const int t = e >> 7, kg = (e >> 5) & 3, r = e & 31;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (kg < nkg)
+      v = __ldg(reinterpret_cast<const uint4*>(R.sl + (size_t)t * slice_bytes(R.sl_kpad) + (size_t)kg * 2048u + r * 16));
+    *reinterpret_cast<uint4*>(smem + kMmaB + (size_t)e * 16u) = v;
+  }
+}
+
+// z_j (lane j) of the row of y (lane k: y_k) whose digits this warp has
+// written; the whole CTA calls it (a warp without a row: mine = false).  fj: the
+// exponent of M's row j; Yr: room for the row where it takes the DFMA chain.
+__device__ __forceinline__ double local_rotate(const RunDesc& R, uint8_t* smem, SliceShared& sh, int fj, double* Yr,
+                                               double y, bool mine, int warp, int lane) {
+  const int d = R.d;
+  __syncthreads();
+  float* sP = reinterpret_cast<float*>(smem + kMmaB + kMmaA);
+  const uint32_t sB = smem_u32(smem), sA = sB + kMmaB;
+  // a warp takes 16 outputs and 10 to 12 of the 43 pairs of digits
+  if (16 * (warp & 1) < d) {
+    switch (warp >> 1) {
+      case 0: local_products<8, 3, -1>(sB, sA, sP, warp & 1, lane); break;
+      case 1: local_products<7, 2, -1>(sB, sA, sP, warp & 1, lane); break;
+      case 2: local_products<6, 1, 0>(sB, sA, sP, warp & 1, lane); break;
+      default: local_products<5, 4, -1>(sB, sA, sP, warp & 1, lane); break;
+    }
+  }
+  __syncthreads();
+  if (!mine) return 0.0;
+  float p[9];
+#pragma unroll
+  for (int q = 0; q < 9; ++q) p[q] = sP[(q * kSliceRows + warp) * kMmaPst + lane];
+  const double zj = slice_combine(p, sh.exp[warp] + fj - 76);
+  double z = lane < d ? zj : 0.0;
+  if ((*(volatile uint32_t*)&sh.bad >> warp) & 1u) {
+    // outside the splitting's comparison: the DFMA chain
+    if (lane < d) Yr[lane] = y;
+    __syncwarp();
+    if (lane == 0) atomicAnd(&sh.bad, ~(1u << warp));
+    z = 0.0;
+    if (lane < d)
+      for (int k = 0; k < d; ++k) z = fma(__ldg(R.MT + (size_t)k * d + lane), Yr[k], z);
+    __syncwarp();
+  }
+  return z;
+}
+
+// Objective of a row, lane j holding z_j (d <= 32); every lane returns it.
+__device__ __forceinline__ double local_objective(int obj, double z, int d, int lane) {
+  double t1 = 0.0, t2 = 0.0;
+  if (obj == kObjRosenbrock) {
+    const double zn = __shfl_down_sync(0xffffffffu, z, 1);
+    if (lane + 1 < d) {
+      const double t0 = z + 1.0, tn = zn + 1.0;
+      const double a = tn - t0 * t0, b = t0 - 1.0;
+      t1 = 100.0 * a * a + b * b;
+    }
+  } else if (lane < d) {
+    if (obj == kObjRastrigin) {
+      t1 = fma(z, z, rastrigin_w(z));
+    } else {
+      t1 = z * z;
+      if (obj == kObjAckley) t2 = cos2pi_fix(z);
+    }
+  }
+  if (obj != kObjAckley) return warp_sum(t1);
+  const double s1 = warp_sum(t1), s2 = warp_sum(t2);
+  return ackley_value((lane & 1 ? s2 : s1) / d, lane);
+}
+
 // The fitness of a key (NaN for the largest).
 __device__ __forceinline__ double key_value(long long k) {
   if (k == 0x7FFFFFFFFFFFFFFFLL) return CUDART_NAN;
@@ -209,16 +285,7 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
     sc.s_exp = s_sl.exp;
     sc.s_bad = &s_sl.bad;
     if (tid == 0) s_sl.bad = 0u;
-    for (uint32_t q = tid * 16u; q < kMmaB; q += blockDim.x * 16u)
-      *reinterpret_cast<uint4*>(smem_l + q) = make_uint4(0u, 0u, 0u, 0u);
-    const int nkg = R.sl_kpad / 8;
-    for (int e = tid; e < kSlices * 4 * 32; e += blockDim.x) {
-      const int t = e >> 7, kg = (e >> 5) & 3, r = e & 31;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (kg < nkg)
-        v = __ldg(reinterpret_cast<const uint4*>(R.sl + (size_t)t * slice_bytes(R.sl_kpad) + (size_t)kg * 2048u + r * 16));
-      *reinterpret_cast<uint4*>(smem_l + kMmaB + (size_t)e * 16u) = v;
-    }
+    local_load_m(R, smem_l);
   } else if (R.rotate) {
     for (int e = tid; e < d * d; e += blockDim.x) mts[e] = __ldg(R.MT + e);
   }
@@ -361,37 +428,8 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
       double z = y[0];
       if constexpr (MM) {
         if (mine) slice_digits(sc, warp, lane, R.sl_kpad, R.sl_qmin[0], y);
-        __syncthreads();
-        float* sP = reinterpret_cast<float*>(smem_l + kMmaB + kMmaA);
-        const uint32_t sB = smem_u32(smem_l), sA = sB + kMmaB;
-        // a warp takes 16 outputs and 10 to 12 of the 43 pairs of digits
-        if (16 * (warp & 1) < d) {
-          switch (warp >> 1) {
-            case 0: local_products<8, 3, -1>(sB, sA, sP, warp & 1, lane); break;
-            case 1: local_products<7, 2, -1>(sB, sA, sP, warp & 1, lane); break;
-            case 2: local_products<6, 1, 0>(sB, sA, sP, warp & 1, lane); break;
-            default: local_products<5, 4, -1>(sB, sA, sP, warp & 1, lane); break;
-          }
-        }
-        __syncthreads();
-        if (mine) {
-          float p[9];
-#pragma unroll
-          for (int q = 0; q < 9; ++q) p[q] = sP[(q * kSliceRows + warp) * kMmaPst + lane];
-          const double zj = slice_combine(p, s_sl.exp[warp] + fj - 76);
-          z = lane < d ? zj : 0.0;
-          if ((*(volatile uint32_t*)&s_sl.bad >> warp) & 1u) {
-            // outside the splitting's comparison: the DFMA chain
-            double* yr = Y + warp * dp;
-            if (lane < d) yr[lane] = y[0];
-            __syncwarp();
-            if (lane == 0) atomicAnd(&s_sl.bad, ~(1u << warp));
-            z = 0.0;
-            if (lane < d)
-              for (int k = 0; k < d; ++k) z = fma(__ldg(R.MT + (size_t)k * d + lane), yr[k], z);
-            __syncwarp();
-          }
-        }
+        const double zj = local_rotate(R, smem_l, s_sl, fj, Y + warp * dp, y[0], mine, warp, lane);
+        if (mine) z = zj;
       } else if (mine && R.rotate) {
         double* yr = Y + warp * dp;
         if (lane < d) yr[lane] = y[0];
@@ -402,30 +440,7 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
         __syncwarp();
       }
       if (common && rank == 0 && tid == 0 && it > 0) early = read_count(it - 1);
-      if (mine) {
-        double t1 = 0.0, t2 = 0.0;
-        if (obj == kObjRosenbrock) {
-          const double zn = __shfl_down_sync(0xffffffffu, z, 1);
-          if (lane + 1 < d) {
-            const double t0 = z + 1.0, tn = zn + 1.0;
-            const double a = tn - t0 * t0, b = t0 - 1.0;
-            t1 = 100.0 * a * a + b * b;
-          }
-        } else if (lane < d) {
-          if (obj == kObjRastrigin) {
-            t1 = fma(z, z, rastrigin_w(z));
-          } else {
-            t1 = z * z;
-            if (obj == kObjAckley) t2 = cos2pi_fix(z);
-          }
-        }
-        const double s1 = warp_sum(t1);
-        ft = s1;
-        if (obj == kObjAckley) {
-          const double s2 = warp_sum(t2);
-          ft = 20.0 + 2.718281828459045 - 20.0 * exp(-0.2 * sqrt(s1 / d)) - exp(s2 / d);
-        }
-      }
+      if (mine) ft = local_objective(obj, z, d, lane);
     }
     // ---- selection; the row and its key to every CTA of the cluster
     if (mine) {
@@ -590,7 +605,60 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
   if constexpr (SL) slice_end(sc);
 }
 
+// ------------------------------------------------------------------ evaluation
+// f of n rows of x (row stride ld) of a sliced run with d <= 32, a warp per
+// row, `rows` <= 8 rows a tile, CTA b taking tiles b, b + gridDim.x, ...  Bound
+// by its latencies: the descriptor is a parameter, M's digits are loaded while
+// the rows are, and few rows are spread over every SM (a row's FP64
+// instructions do not wait for another's).
+__global__ void __launch_bounds__(256, 2)
+    k_eval_few(const __grid_constant__ RunDesc R, const double* __restrict__ x, int64_t ld, int n, int rows,
+               double* __restrict__ fout, uint8_t* __restrict__ fx_out) {
+  __shared__ __align__(16) uint8_t smem[kMmaB + kMmaA + kMmaP];
+  __shared__ SliceShared sh;
+  __shared__ double sY[kSliceRows][32];
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
+  const int d = R.d;
+  SliceCtx sc;
+  sc.sB = smem;
+  sc.s_exp = sh.exp;
+  sc.s_bad = &sh.bad;
+  const double o = lane < d ? __ldg(R.o + lane) : 0.0;
+  const int fj = lane < d ? __ldg(R.slx + lane) : 0;
+  int row = blockIdx.x * rows + warp;
+  double xv = warp < rows && row < n && lane < d ? __ldg(x + (size_t)row * ld + lane) : 0.0;
+  if (threadIdx.x == 0) sh.bad = 0u;
+  local_load_m(R, smem);
+  __syncthreads();
+  for (int t0 = blockIdx.x * rows; t0 < n; t0 += gridDim.x * rows) {
+    row = t0 + warp;
+    const bool mine = warp < rows && row < n;
+    const double y[1] = {mine && lane < d ? shifted(xv, o, R) : 0.0};
+    const int nx = row + (int)gridDim.x * rows;
+    xv = warp < rows && nx < n && lane < d ? __ldg(x + (size_t)nx * ld + lane) : 0.0;
+    if (mine) slice_digits(sc, warp, lane, R.sl_kpad, R.sl_qmin[0], y);
+    const double z = local_rotate(R, smem, sh, fj, sY[warp], y[0], mine, warp, lane);
+    if (!mine) continue;
+    const double f = local_objective(R.obj, z, d, lane);
+    if (lane == 0) {
+      fout[row] = f;
+      if (fx_out) fx_out[row] = 1;
+    }
+  }
+}
+
 // ------------------------------------------------------------------ host side
+bool k_eval_few_launch(const RunDesc& Rh, const double* x, int64_t ld, int n, double* f, uint8_t* fx, cudaStream_t s) {
+  if (!Rh.sl || Rh.d > 32 || Rh.obj > kObjAckley) return false;
+  int dev = 0, nsm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int rows = std::max(1, std::min(kSliceRows, (n + nsm - 1) / nsm));
+  const int tiles = (n + rows - 1) / rows;
+  k_eval_few<<<std::min(tiles, 2 * nsm), 256, 0, s>>>(Rh, x, ld, n, rows, f, fx);
+  return true;
+}
+
 static int local_rot(const LocalPlan& p) { return !p.sl ? kRotChain : p.kpad <= 32 ? kRotMma : kRotTc; }
 
 static const void* local_kernel(const LocalPlan& p, bool isl) {

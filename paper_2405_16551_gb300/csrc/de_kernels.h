@@ -130,6 +130,8 @@ void k_best_exact_launch(const RunDesc* runs, int run0, int n, int dp_max, cudaS
 void k_eval_rows_launch(const RunDesc* runs, int run, const RunDesc& Rh, const double* x, int64_t ld, int n,
                         double* f, uint8_t* fx, cudaStream_t s);
 inline int suite_comps(const RunDesc& R) { return R.obj >= DE_OBJ_COMPOSITION1 ? R.nc : 1; }
+// the same for runs it takes (sliced, d <= 32); false: not launched
+bool k_eval_few_launch(const RunDesc& Rh, const double* x, int64_t ld, int n, double* f, uint8_t* fx, cudaStream_t s);
 void k_best_init_launch(const RunDesc* runs, int run0, int n, cudaStream_t s);
 // the constants R.ctab of every run that has them, once
 void k_suite_table_launch(const RunDesc* runs, int n, cudaStream_t s);

@@ -478,7 +478,7 @@ __device__ __forceinline__ double slice_fitness(SliceCtx& c, const RunDesc& R, c
   if (obj != kObjAckley) return s1;
   double s2 = c.sh->sum[1][0][warp];
   for (int q = 1; 32 * q < d; ++q) s2 += c.sh->sum[1][q][warp];
-  return 20.0 + 2.718281828459045 - 20.0 * exp(-0.2 * sqrt(s1 / d)) - exp(s2 / d);
+  return ackley_value((lane & 1 ? s2 : s1) / d, lane);
 }
 
 }  // namespace de

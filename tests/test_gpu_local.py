@@ -133,3 +133,48 @@ def test_matches_the_oracle(monkeypatch):
         assert np.array_equal(capi.de_get_population(h)[0], Xo)
     finally:
         capi.de_destroy(h)
+
+
+@pytest.mark.parametrize("obj", [0, 1, 2, 3])
+@pytest.mark.parametrize("d,n,ld", [(16, 1, 16), (17, 9, 20), (30, 153, 30), (31, 1217, 31), (32, 5000, 33)])
+def test_evaluation_of_rows(obj, d, n, ld):
+    """Rows of every kind (ordinary, one coordinate far above the rest, zero,
+    huge, not finite) at the edges of a tile and of a round over the device,
+    against the oracle, and against the fitness of the generation loop."""
+    import torch
+
+    o, M = problems.shift(d, seed=d), problems.rotation(d, seed=d)
+    x = problems.population(n, d, seed=n)
+    for r in range(0, n, 7):
+        x[r, r % d] *= 1e9
+    if n > 8:
+        x[3] = o
+        x[5] *= 1e-300
+        x[6, 1] = np.nan
+        x[8, 0] = np.inf
+    buf = np.full((n, ld), 1e30)
+    buf[:, :d] = x
+    xd = torch.from_numpy(buf).cuda()
+    f = torch.full((n + 2,), -7.0, dtype=torch.float64, device="cuda")
+    h = capi.de_init(capi.make_config(16, d, objective=obj, shift=o, rot=M, seed=3, max_generations=10**6,
+                                      target_error=0.0))
+    try:
+        capi.de_eval(h, 0, xd.data_ptr(), ld, n, f.data_ptr())
+        capi.de_step(h, 5)
+        xp, fp = capi.de_get_population(h)
+        xg = torch.from_numpy(xp).cuda()
+        g = torch.zeros(16, dtype=torch.float64, device="cuda")
+        capi.de_eval(h, 0, xg.data_ptr(), d, 16, g.data_ptr())
+        torch.cuda.synchronize()
+    finally:
+        capi.de_destroy(h)
+    assert np.array_equal(g.cpu().numpy(), fp)
+    f = f.cpu().numpy()
+    assert np.all(f[n:] == -7.0)
+    ok = np.isfinite(x).all(1)
+    assert not np.isfinite(f[:n][~ok]).any()
+    fo, S = oracle.evaluate(obj, x[ok], o, M)
+    # the oracle's own bound (its rows' rounding enters the cosines of z = 2^30 as well)
+    big = np.abs(x[ok]).max(1) > 1e6
+    assert np.all((np.abs(f[:n][ok] - fo) <= 1e-12 * (np.abs(fo) + S))[~big])
+    assert np.all((np.abs(f[:n][ok] - fo) <= (1e-12 if obj in (0, 2) else 1e-9) * (np.abs(fo) + S) + 100 * d)[big])
