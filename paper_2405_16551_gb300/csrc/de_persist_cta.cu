@@ -264,14 +264,28 @@ __global__ void __launch_bounds__(256, 1)
     // ---- 0. best record and stop rule of generation gen, whose partials are
     // complete (the grid barrier passed): warp 0, the same order in every CTA
     if (reduce_pending && warp == 0) {
-      Best b;
-      b.init();
-      const BestPartial* pp = R.part + (size_t)(gen & 1) * nct;
-      for (int t = lane; t < nct; t += 32) b.offer(__ldcg(&pp[t].f), __ldcg(&pp[t].idx));
-      b.warp_reduce();
+      // (one load per partial, four in flight; the key is the value's integer image)
+      long long bk = 0x7FFFFFFFFFFFFFFFLL;
+      int bi = -1;
+      const int4* pp = reinterpret_cast<const int4*>(R.part + (size_t)(gen & 1) * nct);
+      for (int t0 = lane; t0 < nct; t0 += 128) {
+        int4 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = t0 + 32 * q < nct ? __ldcg(pp + t0 + 32 * q) : make_int4(0, 0, -1, 0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const long long k = fit_key(__hiloint2double(v[q].y, v[q].x));
+          if (v[q].z >= 0 && (bi < 0 || k < bk || (k == bk && v[q].z < bi))) {
+            bk = k;
+            bi = v[q].z;
+          }
+        }
+      }
+      warp_best(bk, bi);
       if (lane == 0) {
-        const double bf = b.f;
-        const int bi = b.i;
+        const double bf =
+            bi < 0 ? CUDART_INF
+                   : __longlong_as_double(bk >= 0 ? bk : (long long)(0x8000000000000000ULL | (unsigned long long)(-bk)));
         const int64_t evals = (int64_t)np * (1 + gen);  // the initial population counts as NP evaluations
         int sp = 0;
         if (R.target > 0.0 && bi >= 0 && bf < R.target) sp = 1;
@@ -585,19 +599,17 @@ __global__ void __launch_bounds__(256, 1)
       }
     }
     rows_in_regs = true;
-    if (tid == 0) {
-      // the CTA's best (lowest key, then lowest index; NaN never): a scan of
-      // at most 16 precomputed keys
-      long long bk = 0x7FFFFFFFFFFFFFFFLL;
-      int bi = -1;
-      for (int r = 0; r < rows && row0 + r < np; ++r)
-        if (s_key[r] != 0x7FFFFFFFFFFFFFFFLL && (bi < 0 || s_key[r] < bk)) {
-          bk = s_key[r];
-          bi = r;
-        }
-      BestPartial* pp = R.part + (size_t)(g & 1) * nct + cta;
-      pp->f = bi >= 0 ? s_f[bi] : CUDART_INF;
-      pp->idx = bi >= 0 ? row0 + bi : -1;
+    if (warp == 0) {
+      // the CTA's best (lowest key, then lowest index; NaN never) of at most 16
+      // precomputed keys
+      int bi = lane < rows && row0 + lane < np ? lane : -1;
+      long long bk = bi >= 0 ? s_key[lane] : 0x7FFFFFFFFFFFFFFFLL;
+      warp_best(bk, bi);
+      if (lane == 0) {
+        BestPartial* pp = R.part + (size_t)(g & 1) * nct + cta;
+        pp->f = bi >= 0 ? s_f[bi] : CUDART_INF;
+        pp->idx = bi >= 0 ? row0 + bi : -1;
+      }
     }
     if (R.dbg_ftrial && warp == 0 && lane < rows && row0 + lane < np) {
       const int i = row0 + lane;

@@ -252,31 +252,46 @@ __device__ __forceinline__ void epi_dispatch(int obj, const float* v, int w, int
 
 // The same terms over one accumulator row held in shared memory, the
 // columns j = sub, sub + 16, ... of one of 16 threads (each term in the order
-// of epi_cols; Rosenbrock's term of coordinate j pairs z_j with z_{j+1}).
+// of epi_cols; Rosenbrock's term of coordinate j pairs z_j with z_{j+1}).  Four
+// columns at a time: their loads and cosines overlap, the sums stay in order.
 template <int OBJ>
 __device__ __forceinline__ void epi_strided(const float* z, int sub, int d, EpiAcc& A) {
-  for (int j = sub; j < d; j += 16) {
-    const float zj = z[j];
-    if constexpr (OBJ == kObjSphere) {
-      A.a1 = fmaf(zj, zj, A.a1);
-      A.aG += 2.f * fabsf(zj);
-    } else if constexpr (OBJ == kObjRastrigin) {
-      const float cz = cos2pi_f32(zj);
-      A.a1 += fmaf(zj, zj, fmaf(-10.f, cz, 10.f));
-      A.aS += fmaf(zj, zj, fmaf(10.f, fabsf(cz), 10.f));
-      A.aG += fmaf(2.f, fabsf(zj), 62.83185307f);
-    } else if constexpr (OBJ == kObjAckley) {
-      const float cz = cos2pi_f32(zj);
-      A.a1 = fmaf(zj, zj, A.a1);
-      A.a2 += cz;
-      A.a3 += fabsf(zj);
-      A.aS += fabsf(cz);
-    } else {  // Rosenbrock at t = z + 1
-      if (j + 1 < d) {
-        const float t = zj + 1.f, tn = z[j + 1] + 1.f;
-        const float aa = tn - t * t, bb = t - 1.f;
-        A.a1 += fmaf(100.f * aa, aa, bb * bb);
-        A.aG += 400.f * fabsf(t) * fabsf(aa) + 2.f * fabsf(bb) + 200.f * fabsf(aa);
+  for (int j0 = sub; j0 < d; j0 += 64) {
+    float zq[4], zn[4], cz[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = j0 + 16 * q;
+      zq[q] = j < d ? z[j] : 0.f;
+      if constexpr (OBJ == kObjRosenbrock) zn[q] = j + 1 < d ? z[j + 1] : 0.f;
+    }
+    if constexpr (OBJ == kObjRastrigin || OBJ == kObjAckley) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) cz[q] = cos2pi_f32(zq[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = j0 + 16 * q;
+      const float zj = zq[q];
+      if (j >= d) continue;
+      if constexpr (OBJ == kObjSphere) {
+        A.a1 = fmaf(zj, zj, A.a1);
+        A.aG += 2.f * fabsf(zj);
+      } else if constexpr (OBJ == kObjRastrigin) {
+        A.a1 += fmaf(zj, zj, fmaf(-10.f, cz[q], 10.f));
+        A.aS += fmaf(zj, zj, fmaf(10.f, fabsf(cz[q]), 10.f));
+        A.aG += fmaf(2.f, fabsf(zj), 62.83185307f);
+      } else if constexpr (OBJ == kObjAckley) {
+        A.a1 = fmaf(zj, zj, A.a1);
+        A.a2 += cz[q];
+        A.a3 += fabsf(zj);
+        A.aS += fabsf(cz[q]);
+      } else {  // Rosenbrock at t = z + 1
+        if (j + 1 < d) {
+          const float t = zj + 1.f, tn = zn[q] + 1.f;
+          const float aa = tn - t * t, bb = t - 1.f;
+          A.a1 += fmaf(100.f * aa, aa, bb * bb);
+          A.aG += 400.f * fabsf(t) * fabsf(aa) + 2.f * fabsf(bb) + 200.f * fabsf(aa);
+        }
       }
     }
   }
