@@ -354,20 +354,26 @@ struct AdamArgs {
   float omb1, omb2;                     // 1 - beta1, 1 - beta2 (rounded once from FP64)
 };
 
-__device__ __forceinline__ float adam_step(float w, float g, float* m, float* v, const AdamArgs& A) {
-  const float mn = fmaf(A.beta1, *m, A.omb1 * g);
-  const float vn = fmaf(A.beta2, *v, A.omb2 * g * g);
-  *m = mn;
-  *v = vn;
+__device__ __forceinline__ float adam_step(float w, float g, float& m, float& v, const AdamArgs& A) {
+  const float mn = fmaf(A.beta1, m, A.omb1 * g);
+  const float vn = fmaf(A.beta2, v, A.omb2 * g * g);
+  m = mn;
+  v = vn;
   return w - A.lr * (mn / A.c1) / (sqrtf(vn / A.c2) + A.eps);
 }
 
 // Weight gradients of one step and their Adam update (apply = 0: into P.grad
-// only).  Blocks 0 .. 15: rows 128 (b / 8) .. + 127 of W2, columns 32 (b mod 8)
-// .. + 31 (the first column block also b2); blocks 16, 17: 128 rows of W1 and b1
-// (block 16 also w3, b3 and the loss).  The products leave a tile of 128 x 32
-// gradients in shared memory, from which each thread updates 8 consecutive
-// parameters at a time: coalesced masters and moments, 16-byte operand stores.
+// only).  Blocks 0 .. 31: rows 128 (b / 16) .. + 127 of W2, columns 16 (b mod 16)
+// .. + 15 (the first column block also b2); blocks 32, 33: 128 rows of W1 and b1
+// (block 32 also w3, b3 and the loss).  The products leave a tile of gradients
+// in shared memory, from which each thread updates 8 consecutive parameters:
+// coalesced masters and moments, 16-byte operand stores.
+//
+// Masters and moments are read before the wait for the step's pass: only the
+// update before wrote them, and that one had finished when the pass released
+// this launch.  (Read where they are used, a few at a time, they took 10.4 k
+// cycles in the blocks of W2, then 32 columns wide, and 17 k in those of W1.)
+constexpr int kUpW2 = 32;  // blocks of W2
 constexpr uint32_t kUpA = 0, kUpB = 65536, kUpOnes = kUpB + 16384, kUpG = kUpOnes + 8192;
 constexpr int kUpStride = 36;  // floats per row of the gradient tile (16-byte rows, spread over the banks)
 constexpr uint32_t kUpSmem = kUpG + 128u * kUpStride * 4u;
@@ -381,8 +387,8 @@ __global__ void __launch_bounds__(256, 1) k_mlp_update(MlpDev P, AdamArgs A, int
   const int q = warp & 3, h = warp >> 2;
   const uint32_t sb = smem_u32(smem);
   const uint32_t b_ld = smem_u32(&bars[0]), b_mma = smem_u32(&bars[1]);
-  const bool w2 = blockIdx.x < 16;
-  const int ob = w2 ? blockIdx.x >> 3 : blockIdx.x - 16, ig = w2 ? blockIdx.x & 7 : 0;
+  const bool w2 = blockIdx.x < kUpW2;
+  const int ob = w2 ? blockIdx.x >> 4 : blockIdx.x - kUpW2, ig = w2 ? blockIdx.x & 15 : 0;
   const bool bias = w2 && ig == 0;
   float* gt = reinterpret_cast<float*>(smem + kUpG);
   if (tid == 0) {
@@ -403,15 +409,46 @@ __global__ void __launch_bounds__(256, 1) k_mlp_update(MlpDev P, AdamArgs A, int
   }
   // the next step's kernel may start (its inputs do not depend on this one)
   pdl_launch_dependents();
+  // ---- this thread's parameters
+  struct Par {
+    float w, m, v;
+  };
+  auto fetch = [&](int k) { return Par{__ldcg(P.W1 + k), __ldcg(P.mW1 + k), __ldcg(P.vW1 + k)}; };
+  // W2: row r2, 8 columns from c2 on
+  const int r2 = tid >> 1, c2 = 8 * (tid & 1), k2 = kMlpOffW2 + (128 * ob + r2) * kMlpH + 16 * ig + c2;
+  const int kb = kMlpOffB2 + 128 * ob + 32 * q + lane;  // b2 (bias, h = 0)
+  // W1 (256 x 20) and, in column 20, b1: elements tid + 256 u of 128 x 21
+  constexpr int kN1 = 128 * (kMlpIn + 1), kU1 = (kN1 + 255) / 256;
+  auto k1 = [&](int e) {
+    const int r = e / (kMlpIn + 1), c = e - r * (kMlpIn + 1), o = 128 * ob + r;
+    return c < kMlpIn ? kMlpOffW1 + o * kMlpIn + c : kMlpOffB1 + o;
+  };
+  float w8[8], m8[8], v8[8];
+  Par p1[kU1], px{};
+  if (apply && w2) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      *reinterpret_cast<float4*>(w8 + 4 * e) = __ldcg(reinterpret_cast<const float4*>(P.W1 + k2) + e);
+      *reinterpret_cast<float4*>(m8 + 4 * e) = __ldcg(reinterpret_cast<const float4*>(P.mW1 + k2) + e);
+      *reinterpret_cast<float4*>(v8 + 4 * e) = __ldcg(reinterpret_cast<const float4*>(P.vW1 + k2) + e);
+    }
+    if (bias && h == 0) px = fetch(kb);
+  } else if (apply) {
+#pragma unroll
+    for (int u = 0; u < kU1; ++u)
+      if (tid + 256 * u < kN1) p1[u] = fetch(k1(tid + 256 * u));
+    if (ob == 0) px = fetch(kMlpOffW3 + tid);
+  }
   pdl_wait();
   if (tid == 0) {
     const uint8_t *sa = w2 ? P.dz2 : P.dz1, *sbm = w2 ? P.h1 : P.a1;
     const size_t bh = w2 ? kMlpActBytes : kMlpA1Bytes;  // bytes of one half of the batch
     asm volatile("fence.proxy.async.global;" ::: "memory");
-    mbar_expect_tx(b_ld, 65536u + 16384u);
+    const uint32_t bb = w2 ? 4096u : 8192u;  // 16 or 32 columns of one half
+    mbar_expect_tx(b_ld, 65536u + 2u * bb);
     for (int f = 0; f < 2; ++f) {
       bulk_g2s(sb + kUpA + 32768u * f, sa + (size_t)f * kMlpActBytes + (size_t)ob * 32768u, 32768u, b_ld);
-      bulk_g2s(sb + kUpB + 8192u * f, sbm + f * bh + (size_t)ig * 8192u, 8192u, b_ld);
+      bulk_g2s(sb + kUpB + 8192u * f, sbm + f * bh + (size_t)ig * 4096u, bb, b_ld);
     }
   }
   fence_async_smem();
@@ -423,10 +460,11 @@ __global__ void __launch_bounds__(256, 1) k_mlp_update(MlpDev P, AdamArgs A, int
     if (!mbar_wait(b_ld, 0)) s_err = 1;
     else {
       tc_after_sync();
+      const uint32_t id = idesc_bf16(w2 ? 16 : 32) | kAMn | kBMn;
       for (int ks = 0; ks < 16; ++ks) {
         const uint32_t f = ks >> 3, kk = (uint32_t)(ks & 7) * 256u;
         const uint64_t da = desc_mn(sb + kUpA + 32768u * f + kk, 16);
-        mma_split<2>(tmem, da, desc_mn(sb + kUpB + 8192u * f + kk, 16), idesc_bf16(32) | kAMn | kBMn, ks > 0 ? 1u : 0u);
+        mma_split<2>(tmem, da, desc_mn(sb + kUpB + 8192u * f + kk, 16), id, ks > 0 ? 1u : 0u);
         if (bias)
           mma_split<2>(tmem + 32, da, smem_desc(sb + kUpOnes + (uint32_t)ks * 512u, 256u, 128u), idesc_bf16(16) | kAMn,
                        ks > 0 ? 1u : 0u);
@@ -437,8 +475,14 @@ __global__ void __launch_bounds__(256, 1) k_mlp_update(MlpDev P, AdamArgs A, int
   if (!mbar_wait(b_mma, 0)) s_err = 1;
   tc_after_sync();
   const uint32_t lane_base = (uint32_t)(32 * q) << 16;
-  // gradient tile: row 32 q + lane, 16 columns per half of the warps
-  {
+  // gradient tile: row 32 q + lane, half of the columns per half of the warps
+  if (w2) {
+    float g[8];
+    tmem_ld8(tmem + lane_base + 8u * (uint32_t)h, g);
+    float4* dst = reinterpret_cast<float4*>(gt + (32 * q + lane) * kUpStride + 8 * h);
+    dst[0] = make_float4(g[0], g[1], g[2], g[3]);
+    dst[1] = make_float4(g[4], g[5], g[6], g[7]);
+  } else {
     float g[16];
     tmem_ld_cols16(tmem + lane_base + 16u * (uint32_t)h, g);
     float4* dst = reinterpret_cast<float4*>(gt + (32 * q + lane) * kUpStride + 16 * h);
@@ -449,62 +493,51 @@ __global__ void __launch_bounds__(256, 1) k_mlp_update(MlpDev P, AdamArgs A, int
   tc_before_sync();
   __syncthreads();
   // one parameter of the vector: its gradient, or its update
-  auto one = [&](int k, float g) -> float {
+  auto one = [&](int k, float g, Par p) -> float {
     if (!apply) {
       P.grad[k] = g;
       return 0.f;
     }
-    const float w = adam_step(P.W1[k], g, P.mW1 + k, P.vW1 + k, A);
+    const float w = adam_step(p.w, g, p.m, p.v, A);
     P.W1[k] = w;
+    P.mW1[k] = p.m;
+    P.vW1[k] = p.v;
     return w;
   };
-  if (bias && h == 0) one(kMlpOffB2 + 128 * ob + 32 * q + lane, gb);
+  if (bias && h == 0) one(kb, gb, px);
   if (w2) {
-    // 128 x 32 parameters, 8 consecutive per thread and turn: 4 threads a row
+    float g[8];
+    const float4* gs = reinterpret_cast<const float4*>(gt + r2 * kUpStride + c2);
+    *reinterpret_cast<float4*>(g) = gs[0];
+    *reinterpret_cast<float4*>(g + 4) = gs[1];
+    if (!apply) {
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int r = (tid >> 2) + 64 * u, c = 8 * (tid & 3);
-      const int o = 128 * ob + r, i = 32 * ig + c, k = kMlpOffW2 + o * kMlpH + i;
-      float g[8], w[8];
-      const float4* gs = reinterpret_cast<const float4*>(gt + r * kUpStride + c);
-      *reinterpret_cast<float4*>(g) = gs[0];
-      *reinterpret_cast<float4*>(g + 4) = gs[1];
-      if (!apply) {
+      for (int e = 0; e < 8; ++e) P.grad[k2 + e] = g[e];
+    } else {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) P.grad[k + e] = g[e];
-        continue;
-      }
-      float mm[8], vv[8];
-      float4 *pw = reinterpret_cast<float4*>(P.W1 + k), *pm = reinterpret_cast<float4*>(P.mW1 + k),
-             *pv = reinterpret_cast<float4*>(P.vW1 + k);
+      for (int e = 0; e < 8; ++e) w8[e] = adam_step(w8[e], g[e], m8[e], v8[e], A);
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        *reinterpret_cast<float4*>(w + 4 * e) = pw[e];
-        *reinterpret_cast<float4*>(mm + 4 * e) = pm[e];
-        *reinterpret_cast<float4*>(vv + 4 * e) = pv[e];
+        reinterpret_cast<float4*>(P.W1 + k2)[e] = *reinterpret_cast<const float4*>(w8 + 4 * e);
+        reinterpret_cast<float4*>(P.mW1 + k2)[e] = *reinterpret_cast<const float4*>(m8 + 4 * e);
+        reinterpret_cast<float4*>(P.vW1 + k2)[e] = *reinterpret_cast<const float4*>(v8 + 4 * e);
       }
-#pragma unroll
-      for (int e = 0; e < 8; ++e) w[e] = adam_step(w[e], g[e], mm + e, vv + e, A);
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        pw[e] = *reinterpret_cast<const float4*>(w + 4 * e);
-        pm[e] = *reinterpret_cast<const float4*>(mm + 4 * e);
-        pv[e] = *reinterpret_cast<const float4*>(vv + 4 * e);
-      }
-      st_bf16x8(P.w2k, o, i, 32, w);
+      st_bf16x8(P.w2k, 128 * ob + r2, 16 * ig + c2, 32, w8);
     }
   } else {
-    // W1 (256 x 20) and, in column 20, b1
-    for (int e = tid; e < 128 * (kMlpIn + 1); e += blockDim.x) {
-      const int r = e / (kMlpIn + 1), c = e - r * (kMlpIn + 1), o = 128 * ob + r;
-      const float w = one(c < kMlpIn ? kMlpOffW1 + o * kMlpIn + c : kMlpOffB1 + o, gt[r * kUpStride + c]);
-      if (apply) st_bf16(P.w1k, toff(o, c, 32), w);
+#pragma unroll
+    for (int u = 0; u < kU1; ++u) {
+      const int e = tid + 256 * u;
+      if (e >= kN1) continue;
+      const int r = e / (kMlpIn + 1), c = e - r * (kMlpIn + 1);
+      const float w = one(k1(e), gt[r * kUpStride + c], p1[u]);
+      if (apply) st_bf16(P.w1k, toff(128 * ob + r, c, 32), w);
     }
     if (ob == 0) {
       // w3 and b3 from the two halves' partial sums, in a fixed order
-      one(kMlpOffW3 + tid, P.part[tid] + P.part[kMlpPart + tid]);
+      one(kMlpOffW3 + tid, P.part[tid] + P.part[kMlpPart + tid], px);
       if (tid == 0) {
-        one(kMlpOffB3, P.part[kMlpH] + P.part[kMlpPart + kMlpH]);
+        one(kMlpOffB3, P.part[kMlpH] + P.part[kMlpPart + kMlpH], apply ? fetch(kMlpOffB3) : Par{});
         P.loss[0] = (P.part[kMlpH + 1] + P.part[kMlpPart + kMlpH + 1]) / (float)kMlpBatch;
       }
     }
@@ -569,7 +602,7 @@ void mlp_step_launch(const MlpDev& P, const MlpStepArgs& a, const double* x, int
   cfg.dynamicSmemBytes = kMlpSmem;
   cfg.numAttrs = chained ? 1 : 0;
   cudaLaunchKernelEx(&cfg, k_mlp_pass<true>, P, a, x, ld, 0, t, (float*)nullptr);
-  cfg.gridDim = dim3(18);
+  cfg.gridDim = dim3(kUpW2 + 2);
   cfg.dynamicSmemBytes = kUpSmem;
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, k_mlp_update, P, A, apply ? 1 : 0);
