@@ -78,8 +78,10 @@ __device__ __forceinline__ void mma_bf16(uint32_t d, uint32_t a, int rga, uint32
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
-  const __nv_bfloat16 lo = __float2bfloat16_rn(a), hi = __float2bfloat16_rn(b);
-  return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+  // one conversion for two values: conversions bound the epilogues (16 lanes a
+  // clock and SM)
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
 }
 
 __device__ __forceinline__ void st_bf16(uint8_t* base, uint32_t off, float v) {
@@ -124,8 +126,12 @@ constexpr uint32_t kMlpSmem = 221184;
 
 // TRAIN = false: forward of n rows of x (row stride ld) to y.
 // TRAIN = true : forward + backward of minibatch half blockIdx.x.
+// 16 warps: warp w has tile rows 32 (w mod 4) .. + 31 and columns 64 (w / 4) ..
+// + 63.  The epilogues are a thread's walk along its columns, so they take half
+// the time that 8 warps of 128 columns took (12.2 us a pass).
+constexpr int kPassThreads = 512;
 template <bool TRAIN>
-__global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, const double* __restrict__ x,
+__global__ void __launch_bounds__(kPassThreads, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, const double* __restrict__ x,
                                                      int64_t ld, int n, const float* __restrict__ t,
                                                      float* __restrict__ yout) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -133,9 +139,9 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
   __shared__ uint32_t s_tmem;
   __shared__ float s_y[2][kTileM];
   __shared__ float s_t[kTileM];
-  __shared__ float s_b2[kMlpH], s_w3[kMlpH];
+  __shared__ __align__(16) float s_b2[kMlpH], s_w3[kMlpH];
   __shared__ float s_dw3[4][kMlpH];
-  __shared__ float s_red[8][2];
+  __shared__ float s_red[kPassThreads / 32][2];
   __shared__ int s_err;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int q = warp & 3, h = warp >> 2;
@@ -151,19 +157,19 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
   }
   if (warp == 0) tmem_alloc(&s_tmem, 512);
 
-  // ---- inputs: A1 row = (x / 100, 1, 0 ...) in bf16; two threads per row.
+  // ---- inputs: A1 row = (x / 100, 1, 0 ...) in bf16; four threads per row.
   // They do not depend on the weights: a training step reads them before it
   // waits for the step before.
   {
-    const int r = tid >> 1, half = tid & 1;
+    const int r = tid >> 2, part = tid & 3;
     const int grow = row0 + r;
     int src = -1;
     if (TRAIN) src = batch_row(a, grow);
     else if (grow < n) src = grow;
-    float v[16];
+    float v[8];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const int col = 16 * half + c;
+    for (int c = 0; c < 8; ++c) {
+      const int col = 8 * part + c;
       float val = 0.f;
       if (src >= 0) {
         if (col < kMlpIn) val = to_f32_rn(x[(size_t)src * ld + col] * 0.01);
@@ -171,14 +177,12 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
       }
       v[c] = val;
     }
-    st_bf16x8(smem + kSA1, r, 16 * half, 16, v);
-    st_bf16x8(smem + kSA1, r, 16 * half + 8, 16, v + 8);
-    if (TRAIN && half == 0) s_t[r] = src >= 0 ? t[src] : 0.f;
+    st_bf16x8(smem + kSA1, r, 8 * part, 16, v);
+    if (TRAIN && part == 0) s_t[r] = src >= 0 ? t[src] : 0.f;
     if (TRAIN) {
       pdl_wait();
       // (after the wait: the update before this step no longer reads it)
-      st_bf16x8(P.a1 + (size_t)blockIdx.x * kMlpA1Bytes, r, 16 * half, 16, v);
-      st_bf16x8(P.a1 + (size_t)blockIdx.x * kMlpA1Bytes, r, 16 * half + 8, 16, v + 8);
+      st_bf16x8(P.a1 + (size_t)blockIdx.x * kMlpA1Bytes, r, 8 * part, 16, v);
       pdl_launch_dependents();
     }
   }
@@ -189,8 +193,10 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
     bulk_g2s(sb + kSW1, P.w1k, kMlpW1Bytes, b_w);
     bulk_g2s(sb + kSBig, P.w2k, kMlpW2Bytes, b_w);
   }
-  s_b2[tid] = P.b2[tid];
-  s_w3[tid] = P.w3[tid];
+  if (tid < kMlpH) {
+    s_b2[tid] = P.b2[tid];
+    s_w3[tid] = P.w3[tid];
+  }
   fence_async_smem();
   tc_before_sync();
   __syncthreads();
@@ -211,20 +217,14 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
   tc_after_sync();
 
   // ---- epilogue 1: H1 = relu(Z1) to shared memory (A operand of layer 2);
-  // training: also to global memory, and the ReLU mask in registers
-  uint32_t mask[4];
+  // training: also to global memory
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int c0 = 128 * h + 32 * j;
+  for (int j = 0; j < 2; ++j) {
+    const int c0 = 64 * h + 32 * j;
     float v[32];
     tmem_ld_cols32(tmem + lane_base + (uint32_t)c0, v);
-    uint32_t mk = 0;
 #pragma unroll
-    for (int e = 0; e < 32; ++e) {
-      v[e] = fmaxf(v[e], 0.f);
-      mk |= (v[e] > 0.f ? 1u : 0u) << e;
-    }
-    mask[j] = mk;
+    for (int e = 0; e < 32; ++e) v[e] = fmaxf(v[e], 0.f);
 #pragma unroll
     for (int e = 0; e < 32; e += 8) {
       st_bf16x8(smem + kSH1, m, c0 + e, 16, v + e);
@@ -243,17 +243,38 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
   }
   if (!mbar_wait(b_mma, 1)) s_err = 1;
   tc_after_sync();
-  // ---- epilogue 2: y = w3 . relu(Z2 + b2) + b3
-  float yp = 0.f;
+  // ---- epilogue 2: y = w3 . relu(Z2 + b2) + b3, H2 = relu(Z2 + b2) in registers.
+  // A chain of additions covers 128 columns, i.e. two threads' in turn.
+  float h2[2][32];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int c0 = 128 * h + 32 * j;
-    float v[32];
-    tmem_ld_cols32(tmem + lane_base + 256u + (uint32_t)c0, v);
+  for (int j = 0; j < 2; ++j) {
+    const int c0 = 64 * h + 32 * j;
+    tmem_ld_cols32(tmem + lane_base + 256u + (uint32_t)c0, h2[j]);
 #pragma unroll
-    for (int e = 0; e < 32; ++e) yp = fmaf(fmaxf(v[e] + s_b2[c0 + e], 0.f), s_w3[c0 + e], yp);
+    for (int e = 0; e < 32; e += 4) {
+      const float4 b = *reinterpret_cast<const float4*>(s_b2 + c0 + e);
+      h2[j][e] = fmaxf(h2[j][e] + b.x, 0.f);
+      h2[j][e + 1] = fmaxf(h2[j][e + 1] + b.y, 0.f);
+      h2[j][e + 2] = fmaxf(h2[j][e + 2] + b.z, 0.f);
+      h2[j][e + 3] = fmaxf(h2[j][e + 3] + b.w, 0.f);
+    }
   }
-  s_y[h][m] = yp;
+  auto dot = [&](float yp) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int e = 0; e < 32; e += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(s_w3 + 64 * h + 32 * j + e);
+        yp = fmaf(h2[j][e], w.x, yp);
+        yp = fmaf(h2[j][e + 1], w.y, yp);
+        yp = fmaf(h2[j][e + 2], w.z, yp);
+        yp = fmaf(h2[j][e + 3], w.w, yp);
+      }
+    return yp;
+  };
+  if (!(h & 1)) s_y[h >> 1][m] = dot(0.f);
+  __syncthreads();
+  if (h & 1) s_y[h >> 1][m] = dot(s_y[h >> 1][m]);
   __syncthreads();
   const float y = s_y[0][m] + s_y[1][m] + P.b3[0];
   if (!TRAIN) {
@@ -264,21 +285,22 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
     const float dy = 2.f * r / (float)kMlpBatch;
     // dZ2 = dy w3 relu'(Z2 + b2): A operand of dH1 (in H1's place, which
     // layer 2 has consumed) and of dW2 (global); dw3 = sum over rows of H2 dy
-#pragma unroll 1
-    for (int j = 0; j < 4; ++j) {
-      const int c0 = 128 * h + 32 * j;
-      float v[32], dz[32];
-      tmem_ld_cols32(tmem + lane_base + 256u + (uint32_t)c0, v);
 #pragma unroll
-      for (int e = 0; e < 32; ++e) {
-        const float zb = v[e] + s_b2[c0 + e];
-        dz[e] = zb > 0.f ? dy * s_w3[c0 + e] : 0.f;
-        v[e] = fmaxf(zb, 0.f) * dy;  // row contribution to dw3[c0 + e]
-      }
+    for (int j = 0; j < 2; ++j) {
+      const int c0 = 64 * h + 32 * j;
+      float(&v)[32] = h2[j];
 #pragma unroll
       for (int e = 0; e < 32; e += 8) {
-        st_bf16x8(smem + kSH1, m, c0 + e, 16, dz + e);
-        st_bf16x8(P.dz2 + (size_t)blockIdx.x * kMlpActBytes, m, c0 + e, 16, dz + e);
+        float dz[8], w[8];
+        *reinterpret_cast<float4*>(w) = *reinterpret_cast<const float4*>(s_w3 + c0 + e);
+        *reinterpret_cast<float4*>(w + 4) = *reinterpret_cast<const float4*>(s_w3 + c0 + e + 4);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          dz[u] = v[e + u] > 0.f ? dy * w[u] : 0.f;
+          v[e + u] *= dy;  // row contribution to dw3[c0 + e + u]
+        }
+        st_bf16x8(smem + kSH1, m, c0 + e, 16, dz);
+        st_bf16x8(P.dz2 + (size_t)blockIdx.x * kMlpActBytes, m, c0 + e, 16, dz);
       }
       // sums over the 32 rows of all 32 columns: at each step a lane keeps the
       // columns whose index agrees with it in one bit, so 31 additions do
@@ -319,11 +341,12 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
       P.part[blockIdx.x * kMlpPart + kMlpH + 1] = ((s_red[0][0] + s_red[1][0]) + s_red[2][0]) + s_red[3][0];
     }
 
-    // ---- dH1 = dZ2 W2: A = dZ2 (shared), B = W2 read MN-major -> TMEM [0, 256)
+    // ---- dH1 = dZ2 W2: A = dZ2 (shared), B = W2 read MN-major -> TMEM [256, 512)
+    // (H2 is in registers; Z1 stays for the last epilogue)
     if (tid == 0) {
       const uint32_t id = idesc_bf16(kMlpH) | kBMn;
       for (int ks = 0; ks < 16; ++ks)
-        mma_split<2>(tmem, smem_desc(sb + kSH1 + (uint32_t)ks * 4096u, 2048u, 128u),
+        mma_split<2>(tmem + 256, smem_desc(sb + kSH1 + (uint32_t)ks * 4096u, 2048u, 128u),
                      desc_mn(sb + kSBig + (uint32_t)ks * 256u, 32), id, ks > 0 ? 1u : 0u);
       mma_commit(b_mma);
     }
@@ -332,12 +355,13 @@ __global__ void __launch_bounds__(256, 1) k_mlp_pass(MlpDev P, MlpStepArgs a, co
 
     // ---- epilogue 3: dZ1 = dH1 relu'(Z1) to global memory
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c0 = 128 * h + 32 * j;
-      float v[32];
-      tmem_ld_cols32(tmem + lane_base + (uint32_t)c0, v);
+    for (int j = 0; j < 2; ++j) {
+      const int c0 = 64 * h + 32 * j;
+      float v[32], z[32];
+      tmem_ld_cols32(tmem + lane_base + (uint32_t)c0, z);
+      tmem_ld_cols32(tmem + lane_base + 256u + (uint32_t)c0, v);
 #pragma unroll
-      for (int e = 0; e < 32; ++e) v[e] = ((mask[j] >> e) & 1u) ? v[e] : 0.f;
+      for (int e = 0; e < 32; ++e) v[e] = z[e] > 0.f ? v[e] : 0.f;
 #pragma unroll
       for (int e = 0; e < 32; e += 8) st_bf16x8(P.dz1 + (size_t)blockIdx.x * kMlpActBytes, m, c0 + e, 16, v + e);
     }
@@ -364,8 +388,8 @@ __device__ __forceinline__ float adam_step(float w, float g, float& m, float& v,
 
 // Weight gradients of one step and their Adam update (apply = 0: into P.grad
 // only).  Blocks 0 .. 31: rows 128 (b / 16) .. + 127 of W2, columns 16 (b mod 16)
-// .. + 15 (the first column block also b2); blocks 32, 33: 128 rows of W1 and b1
-// (block 32 also w3, b3 and the loss).  The products leave a tile of gradients
+// .. + 15 (the first column block also b2); blocks 32 .. 39: a quarter of the
+// parameters of 128 rows of W1 and b1 (block 32 also w3, b3 and the loss).  The products leave a tile of gradients
 // in shared memory, from which each thread updates 8 consecutive parameters:
 // coalesced masters and moments, 16-byte operand stores.
 //
@@ -373,7 +397,7 @@ __device__ __forceinline__ float adam_step(float w, float g, float& m, float& v,
 // update before wrote them, and that one had finished when the pass released
 // this launch.  (Read where they are used, a few at a time, they took 10.4 k
 // cycles in the blocks of W2, then 32 columns wide, and 17 k in those of W1.)
-constexpr int kUpW2 = 32;  // blocks of W2
+constexpr int kUpW2 = 32, kUpW1 = 8;  // blocks of W2, of W1
 constexpr uint32_t kUpA = 0, kUpB = 65536, kUpOnes = kUpB + 16384, kUpG = kUpOnes + 8192;
 constexpr int kUpStride = 36;  // floats per row of the gradient tile (16-byte rows, spread over the banks)
 constexpr uint32_t kUpSmem = kUpG + 128u * kUpStride * 4u;
@@ -388,7 +412,8 @@ __global__ void __launch_bounds__(256, 1) k_mlp_update(MlpDev P, AdamArgs A, int
   const uint32_t sb = smem_u32(smem);
   const uint32_t b_ld = smem_u32(&bars[0]), b_mma = smem_u32(&bars[1]);
   const bool w2 = blockIdx.x < kUpW2;
-  const int ob = w2 ? blockIdx.x >> 4 : blockIdx.x - kUpW2, ig = w2 ? blockIdx.x & 15 : 0;
+  const int ob = w2 ? blockIdx.x >> 4 : (blockIdx.x - kUpW2) >> 2, ig = w2 ? blockIdx.x & 15 : 0;
+  const int part1 = (blockIdx.x - kUpW2) & 3;  // quarter of W1's rows' parameters
   const bool bias = w2 && ig == 0;
   float* gt = reinterpret_cast<float*>(smem + kUpG);
   if (tid == 0) {
@@ -417,8 +442,10 @@ __global__ void __launch_bounds__(256, 1) k_mlp_update(MlpDev P, AdamArgs A, int
   // W2: row r2, 8 columns from c2 on
   const int r2 = tid >> 1, c2 = 8 * (tid & 1), k2 = kMlpOffW2 + (128 * ob + r2) * kMlpH + 16 * ig + c2;
   const int kb = kMlpOffB2 + 128 * ob + 32 * q + lane;  // b2 (bias, h = 0)
-  // W1 (256 x 20) and, in column 20, b1: elements tid + 256 u of 128 x 21
-  constexpr int kN1 = 128 * (kMlpIn + 1), kU1 = (kN1 + 255) / 256;
+  // W1 (256 x 20) and, in column 20, b1: elements of 128 x 21, this quarter's
+  // from e1 on
+  constexpr int kN1 = 128 * (kMlpIn + 1) / 4, kU1 = (kN1 + 255) / 256;
+  const int e1 = part1 * kN1;
   auto k1 = [&](int e) {
     const int r = e / (kMlpIn + 1), c = e - r * (kMlpIn + 1), o = 128 * ob + r;
     return c < kMlpIn ? kMlpOffW1 + o * kMlpIn + c : kMlpOffB1 + o;
@@ -436,8 +463,8 @@ __global__ void __launch_bounds__(256, 1) k_mlp_update(MlpDev P, AdamArgs A, int
   } else if (apply) {
 #pragma unroll
     for (int u = 0; u < kU1; ++u)
-      if (tid + 256 * u < kN1) p1[u] = fetch(k1(tid + 256 * u));
-    if (ob == 0) px = fetch(kMlpOffW3 + tid);
+      if (tid + 256 * u < kN1) p1[u] = fetch(k1(e1 + tid + 256 * u));
+    if (blockIdx.x == kUpW2) px = fetch(kMlpOffW3 + tid);
   }
   pdl_wait();
   if (tid == 0) {
@@ -527,13 +554,13 @@ __global__ void __launch_bounds__(256, 1) k_mlp_update(MlpDev P, AdamArgs A, int
   } else {
 #pragma unroll
     for (int u = 0; u < kU1; ++u) {
-      const int e = tid + 256 * u;
-      if (e >= kN1) continue;
+      if (tid + 256 * u >= kN1) continue;
+      const int e = e1 + tid + 256 * u;
       const int r = e / (kMlpIn + 1), c = e - r * (kMlpIn + 1);
       const float w = one(k1(e), gt[r * kUpStride + c], p1[u]);
       if (apply) st_bf16(P.w1k, toff(128 * ob + r, c, 32), w);
     }
-    if (ob == 0) {
+    if (blockIdx.x == kUpW2) {
       // w3 and b3 from the two halves' partial sums, in a fixed order
       one(kMlpOffW3 + tid, P.part[tid] + P.part[kMlpPart + tid], px);
       if (tid == 0) {
@@ -574,7 +601,7 @@ void mlp_pack_launch(const MlpDev& P, cudaStream_t s) { k_mlp_pack<<<64, 256, 0,
 void mlp_forward_launch(const MlpDev& P, const double* x, int64_t ld, int n, float* y, cudaStream_t s) {
   if (n <= 0) return;
   MlpStepArgs a{};
-  k_mlp_pass<false><<<(n + kTileM - 1) / kTileM, 256, kMlpSmem, s>>>(P, a, x, ld, n, nullptr, y);
+  k_mlp_pass<false><<<(n + kTileM - 1) / kTileM, kPassThreads, kMlpSmem, s>>>(P, a, x, ld, n, nullptr, y);
 }
 
 // chained: the launch before this one on the stream is a step's k_mlp_update,
@@ -592,7 +619,7 @@ void mlp_step_launch(const MlpDev& P, const MlpStepArgs& a, const double* x, int
   A.omb1 = (float)(1.0 - b1);
   A.omb2 = (float)(1.0 - b2);
   cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(kPassThreads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -602,7 +629,8 @@ void mlp_step_launch(const MlpDev& P, const MlpStepArgs& a, const double* x, int
   cfg.dynamicSmemBytes = kMlpSmem;
   cfg.numAttrs = chained ? 1 : 0;
   cudaLaunchKernelEx(&cfg, k_mlp_pass<true>, P, a, x, ld, 0, t, (float*)nullptr);
-  cfg.gridDim = dim3(kUpW2 + 2);
+  cfg.gridDim = dim3(kUpW2 + kUpW1);
+  cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = kUpSmem;
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, k_mlp_update, P, A, apply ? 1 : 0);
