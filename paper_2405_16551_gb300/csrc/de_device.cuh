@@ -732,13 +732,15 @@ __device__ __forceinline__ uint32_t trial_coords(const RunDesc& R, uint32_t jr, 
   // the target's coordinate to the violated bound (the paper leaves bounds
   // handling open).  (x_i + b) / 2 rounded once equals fma(0.5, x_i, b / 2):
   // halving commutes with rounding away from the subnormal range, and b / 2 is
-  // exact, so the repair is one FP64 instruction per slot.  It runs only when
-  // some lane of the warp needs it (one vote per chunk: a vote per slot cost
-  // the FP64 generation kernel more than the instructions it saved), and the
-  // 64-bit keys only when some lane has a high word equal to a bound's (their
-  // compare costs an FP64-pipe instruction per slot).
-  if (__any_sync(__activemask(), (lowm | highm | eqm) != 0u)) {
-    if (__any_sync(__activemask(), eqm != 0u)) {
+  // exact, so the repair is one FP64 instruction.  Each lane repairs its first
+  // offending coordinate, then its second, ..., until no lane has one left: few
+  // lanes have two, while an instruction per slot runs for every slot that any
+  // lane of the warp needs (all four, in most warps of a wide population).  The
+  // 64-bit keys are compared only when some lane has a high word equal to a
+  // bound's (an FP64-pipe instruction per slot).
+  const unsigned act = __activemask();
+  if (__any_sync(act, (lowm | highm | eqm) != 0u)) {
+    if (__any_sync(act, eqm != 0u)) {
 #pragma unroll
       for (int m = 0; m < N; ++m)
         if ((eqm >> m) & 1u) {
@@ -747,9 +749,18 @@ __device__ __forceinline__ uint32_t trial_coords(const RunDesc& R, uint32_t jr, 
           highm |= (uint32_t)(kv > R.hi_key) << m;
         }
     }
+    uint32_t need = lowm | highm;
+    do {
+      const uint32_t first = need & (0u - need);
+      double x = xi[0];
 #pragma unroll
-    for (int m = 0; m < N; ++m)
-      if (((lowm | highm) >> m) & 1u) t[m] = __fma_rn(0.5, xi[m], ((lowm >> m) & 1u) ? R.lo_half : R.hi_half);
+      for (int m = 1; m < N; ++m) x = first >> m & 1u ? xi[m] : x;
+      const double v = __fma_rn(0.5, x, lowm & first ? R.lo_half : R.hi_half);
+#pragma unroll
+      for (int m = 0; m < N; ++m)
+        if (first >> m & 1u) t[m] = v;
+      need ^= first;
+    } while (N > 1 && __any_sync(act, need != 0u));
   }
   return bits;
 }
