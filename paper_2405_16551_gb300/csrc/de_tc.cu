@@ -1039,7 +1039,7 @@ de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* 
   p.nruns = (int)runs.size();
   // two row tiles per fitness CTA where every run has several N tiles and
   // one-tile CTAs need a second wave: NP = 8192, D = 1000 (256 one-tile CTAs on
-  // 152 SMs) 150 -> 45 us; in one wave the pairs would only leave SMs idle
+  // 152 SMs) 150 -> 59 us; in one wave the pairs would only leave SMs idle
   int dev = 0, nsm = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
