@@ -919,14 +919,10 @@ def accuracy_workload(capi, torch, stream, problems):
                 forms=out, gpu_launches=None)
 
 
-# DRAM traffic of one launch of the dominant kernel, from an ncu capture
-# (dram__bytes_read.sum + dram__bytes_write.sum) of a 200-generation launch of
-# the BF16x3 persistent kernel on this workload, scaled to a launch of 3000
-# generations (traffic grows with generations); a kernel changed since its
-# last capture has no entry
-TRAFFIC_PER_LAUNCH = {
-    # k_persist_cta, 7 targets per CTA: 986,112 + 448,000 bytes per 200 generations
-    ("k_persist_cta", 3000): (986112 + 448000) * 3000 // 200}
+# DRAM traffic of one launch of the dominant kernel by (kernel, generations), from
+# an ncu capture (dram__bytes_read.sum + dram__bytes_write.sum); a kernel changed
+# since its last capture has no entry
+TRAFFIC_PER_LAUNCH = {}
 
 
 if __name__ == "__main__":

@@ -258,6 +258,12 @@ __global__ void __launch_bounds__(256, ROT == kRotTc ? 1 : 2)
   __shared__ int s_over;
   cg::cluster_group cluster = cg::this_cluster();
   const int run = (int)blockIdx.x / csize, rank = (int)blockIdx.x % csize;
+  // a launch without its cluster dimension (a tool that launches the kernel
+  // again by itself) has no peers to write to: an error, not a fault
+  if ((int)cluster.num_blocks() != csize) {
+    if (threadIdx.x == 0) atomicOr(&runs[run].st->err, kErrTimeout);
+    return;
+  }
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   load_desc(sR, runs + run);
