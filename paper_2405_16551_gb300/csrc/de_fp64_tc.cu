@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(256, 1)
 // coordinates a row needs per matrix (de_slice.cuh).  M: nc row-major d x d
 // matrices.
 bool slice_plan(const double* M, int nc, int d, int32_t qmin[5]) {
-  // below 24 coordinates the chain of d DFMAs is shorter than the products' latency
+  // below 16 coordinates the chain of d DFMAs is shorter than the products' latency
   if (d < kSliceDMin || d > kSliceDMax) return false;
   for (int c = 0; c < nc; ++c) {
     int cm = 0;
