@@ -55,6 +55,7 @@ struct de_handle {
   size_t arena_bytes = 0;
   RunState* h_state = nullptr;  // pinned mirror of the device states
   bool state_fresh = false;     // nothing that changes the states was enqueued since the mirror was read
+  bool captured = false;        // a call was captured by the caller: its graph changes the states without a call
   char* h_stage = nullptr;      // pinned staging of small populations (kStageBytes at most)
   size_t stage_bytes = 0;
   cudaGraphExec_t graph = nullptr;
@@ -384,6 +385,16 @@ static de_status use_local(de_handle* h, bool& use) {
   return DE_OK;
 }
 
+// Whether the caller is capturing the handle's stream.  What a call enqueues
+// then runs whenever the caller launches the graph, at a time unknown here, so
+// from then on the mirror of the states is never taken for current.
+static de_status note_capture(de_handle* h) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  DE_CUDA(h, cudaStreamIsCapturing(h->stream, &cap));
+  h->captured = h->captured || cap != cudaStreamCaptureStatusNone;
+  return DE_OK;
+}
+
 static de_status enqueue_generations(de_handle* h, int64_t n) {
   // whatever was read on the way, the mirror of the states is old at the end
   struct Stale {
@@ -489,9 +500,10 @@ static de_status read_states(de_handle* h) {
   return DE_OK;
 }
 
-// The mirror of the states, read only when something may have changed them
-// (a handle has one host thread at a time, and only its own calls change it).
-static de_status need_states(de_handle* h) { return h->state_fresh ? DE_OK : read_states(h); }
+// The mirror of the states, read only when something may have changed them: a
+// call of the handle (one host thread at a time) or the launch of a graph that
+// captured one.
+static de_status need_states(de_handle* h) { return h->state_fresh && !h->captured ? DE_OK : read_states(h); }
 
 static de_status check_device_errors(de_handle* h) {
   for (int r = 0; r < h->nruns; ++r) {
@@ -1498,6 +1510,8 @@ de_status de_reset(de_handle* h, int32_t run) {
   if (!h) return fail(nullptr, DE_ERR_INVALID_ARG, "handle is NULL");
   if (run < -1 || run >= h->nruns) return fail(h, DE_ERR_INVALID_ARG, "run out of range");
   h->err.clear();
+  const de_status cap = note_capture(h);
+  if (cap != DE_OK) return cap;
   const de_status st = run < 0 ? init_runs(h, 0, h->nruns) : init_runs(h, run, 1);
   if (st != DE_OK) return st;
   h->isl_even = run < 0;
@@ -1585,7 +1599,8 @@ de_status de_step(de_handle* h, int64_t generations) {
   if (!h) return fail(nullptr, DE_ERR_INVALID_ARG, "handle is NULL");
   if (generations < 0) return fail(h, DE_ERR_INVALID_ARG, "generations must be >= 0");
   h->err.clear();
-  return enqueue_generations(h, generations);
+  const de_status s = note_capture(h);
+  return s == DE_OK ? enqueue_generations(h, generations) : s;
 }
 
 de_status de_run(de_handle* h, de_result* out) {
