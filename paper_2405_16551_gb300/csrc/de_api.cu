@@ -533,12 +533,13 @@ static size_t eval_smem(const de_handle* h, int run0, int n) {
 // 3000 launches, 16 ms, run by run).
 static de_status init_runs(de_handle* h, int run0, int n) {
   h->state_fresh = false;
-  int np_max = 0, dp_max = 0;
+  int np_max = 0, dp_max = 0, dp_sliced = 0;
   bool jde = false, plain = false;
   for (int r = run0; r < run0 + n; ++r) {
     const RunDesc& R = h->run[r];
     np_max = std::max(np_max, R.np);
     dp_max = std::max(dp_max, R.dp);
+    if (R.sl) dp_sliced = std::max(dp_sliced, R.dp);
     jde = jde || R.jde;
     plain = plain || (!R.sl && R.obj != DE_OBJ_ODE);
     if (R.obj == DE_OBJ_ODE && !h->ode_ref_done[r]) {
@@ -560,7 +561,7 @@ static de_status init_runs(de_handle* h, int run0, int n) {
       for (int r = run0; r < run0 + n; ++r) tc_init_eval_launch(h->tc, h->d_run, r, h->run[r], h->stream);
   } else {
     if (all && h->slices.on)
-      k_eval_pops_tc_launch(h->d_run, h->d_items, h->d_shares, h->nshares, h->slices, dp_max, h->stream);
+      k_eval_pops_tc_launch(h->d_run, h->d_items, h->d_shares, h->nshares, h->slices, dp_sliced, h->stream);
     if (all && plain) k_eval_pops_launch(h->d_run, run0, n, np_max, eval_smem(h, run0, n), h->stream);
     for (int r = run0; r < run0 + n; ++r) {
       const RunDesc& R = h->run[r];

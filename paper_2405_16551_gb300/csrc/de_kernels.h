@@ -68,7 +68,8 @@ void k_gen_fp64_tc_launch(const RunDesc* runs, const int4* items, const int2* sh
                           bool var, bool suite, cudaStream_t s);
 void k_eval_rows_tc_launch(const RunDesc* runs, int run, const RunDesc& Rh, const double* x, int64_t ld, int n,
                            double* f, uint8_t* fx, cudaStream_t s);
-// the sliced runs' populations, in the shares of k_gen_fp64_tc_launch
+// the sliced runs' populations, in the shares of k_gen_fp64_tc_launch (dp_max:
+// the largest stride among the sliced runs)
 void k_eval_pops_tc_launch(const RunDesc* runs, const int4* items, const int2* shares, int nct, const SlicePlan& p,
                            int dp_max, cudaStream_t s);
 void k_tc_configure();
