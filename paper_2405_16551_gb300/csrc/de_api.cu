@@ -105,7 +105,14 @@ void set_last_error(const std::string& m) { g_err = m; }
 static const char* kVersion = "de_gb300 1.0 sm_103a";
 
 // ---------------------------------------------------------------- helpers
+// The runtime's last error goes with the status that reports it: left behind it
+// would be taken for that of the next call's launches (of any handle).
+static void clear_error(de_status s) {
+  if (s == DE_ERR_CUDA || s == DE_ERR_OOM) cudaGetLastError();
+}
+
 static de_status fail(de_handle* h, de_status s, const std::string& msg) {
+  clear_error(s);
   if (h) h->err = msg;
   g_err = msg;
   return s;
@@ -1266,6 +1273,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
   }
   auto fin = [&](de_status s) {
     if (s != DE_OK) {
+      clear_error(s);
       std::string m = h->err;
       de_destroy(h);
       g_err = m;

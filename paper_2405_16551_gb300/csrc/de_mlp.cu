@@ -651,6 +651,7 @@ struct de_mlp {
 namespace de {
 
 static de_status mlp_fail(de_mlp* m, de_status s, const std::string& msg) {
+  if (s == DE_ERR_CUDA || s == DE_ERR_OOM) cudaGetLastError();  // reported here, not by the next call
   if (m) m->err = msg;
   set_last_error(msg);
   return s;
