@@ -762,7 +762,6 @@ static de_status autotune_fp64(de_handle* h, int nsm) {
     st_all = build_items(h);
     if (st_all == DE_OK) st_all = upload_desc(h);
     if (st_all != DE_OK) break;
-    k_configure(h->smem_gen);
     for (int r = 0; r < h->nruns; ++r) {
       int32_t zero = 0;
       DE_CUDA(h, cudaMemcpyAsync(&h->run[r].st->stop, &zero, sizeof zero, cudaMemcpyHostToDevice, h->stream));
@@ -1457,7 +1456,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
   for (auto& R : h->run) R.dbuf = h->dbuf ? 1 : 0;
   TRY(build_items(h));
   TRY(upload_desc(h));
-  k_configure(h->smem_gen);
+  k_configure();
   if (h->suite) k_suite_table_launch(h->d_run, nruns, h->stream);
   TRY(init_runs(h, 0, nruns));
   if (h->prec == DE_PREC_FP64 && cfgs[0].surrogate_k < 2) {
@@ -1466,7 +1465,6 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
     TRY(autotune_fp64(h, nsm));
     TRY(build_items(h));
     TRY(upload_desc(h));
-    k_configure(h->smem_gen);
     if (const char* e = getenv("DE_GB300_FP64_PERSIST")) {
       // forced on where it applies: 1 cooperative launch, 2 one cluster, 3 a
       // cluster per run (else the cooperative launch)

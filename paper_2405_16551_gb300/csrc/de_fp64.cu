@@ -591,21 +591,27 @@ size_t fp64_exclusive_smem(const void* k, size_t smem) {
 
 static size_t persist_smem(const void* k, size_t smem, bool tc) { return tc ? fp64_exclusive_smem(k, smem) : smem; }
 
-void k_configure(size_t smem_gen) {
-  const int smem = (int)std::max<size_t>(smem_gen, 1);
-  cudaFuncSetAttribute(k_gen_fp64<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_gen_fp64<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_gen_fp64<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_gen_fp64<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  for (int q = 0; q < 12; ++q) {
-    const bool tc = (q & 1) != 0, var = (q & 2) != 0, suite = q / 4 == 1, isl = q / 4 == 2;
-    const void* k = persist_kernel(var, suite, isl, tc);
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)persist_smem(k, smem, tc));
-  }
+cudaError_t allow_dynamic_smem(const void* k) {
+  cudaFuncAttributes a{};
+  int dev = 0, most = 0;
+  cudaError_t e = cudaFuncGetAttributes(&a, k);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  const int limit = most - (int)a.sharedSizeBytes;
+  return a.maxDynamicSharedSizeBytes == limit
+             ? cudaSuccess
+             : cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
+}
+
+void k_configure() {
+  for (const void* k : {(const void*)k_gen_fp64<false, false>, (const void*)k_gen_fp64<true, false>,
+                        (const void*)k_gen_fp64<false, true>, (const void*)k_gen_fp64<true, true>,
+                        (const void*)k_eval_rows, (const void*)k_eval_pops, (const void*)k_best_exact})
+    allow_dynamic_smem(k);
+  for (int q = 0; q < 12; ++q)
+    allow_dynamic_smem(persist_kernel((q & 2) != 0, q / 4 == 1, q / 4 == 2, (q & 1) != 0));
   k_tc_configure();
-  cudaFuncSetAttribute(k_eval_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  cudaFuncSetAttribute(k_eval_pops, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  cudaFuncSetAttribute(k_best_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
 cudaError_t k_gen_fp64_persist_launch(const RunDesc* runs, const int4* items, int nitems, int nruns, int threads,

@@ -725,15 +725,10 @@ bool local_plan(LocalPlan& p, const std::vector<RunDesc>& runs, const SlicePlan&
 
 bool local_fits(const LocalPlan& p, int nruns, bool isl) {
   const void* k = local_kernel(p, isl);
-  const size_t smem = local_smem(p, k);
   cudaLaunchAttribute attr[2];
   int n = 0;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
   const cudaLaunchConfig_t cfg = local_config(p, k, nruns, isl, 0, attr);
-  if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
+  if (allow_dynamic_smem(k) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }

@@ -358,7 +358,7 @@ int k_gen_sliced_capacity(bool isl, bool unit, const SlicePlan& p, size_t smem) 
   int per_sm = 0, dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess ||
+  if (allow_dynamic_smem(k) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, dyn) != cudaSuccess) {
     cudaGetLastError();
     return 0;

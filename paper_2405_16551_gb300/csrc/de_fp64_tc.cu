@@ -317,13 +317,10 @@ void k_gen_fp64_tc_launch(const RunDesc* runs, const int4* items, const int2* sh
 }
 
 void k_tc_configure() {
-  const int mx = 208 * 1024;  // beside up to 9 KB of static shared memory
-  cudaFuncSetAttribute(k_gen_fp64_tc<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_gen_fp64_tc<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_gen_fp64_tc<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_gen_fp64_tc<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_eval_rows_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_eval_pops_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  for (const void* k : {(const void*)k_gen_fp64_tc<false, false>, (const void*)k_gen_fp64_tc<true, false>,
+                        (const void*)k_gen_fp64_tc<false, true>, (const void*)k_gen_fp64_tc<true, true>,
+                        (const void*)k_eval_rows_tc, (const void*)k_eval_pops_tc})
+    allow_dynamic_smem(k);
 }
 
 void k_eval_pops_tc_launch(const RunDesc* runs, const int4* items, const int2* shares, int nct, const SlicePlan& p,

@@ -37,7 +37,12 @@ struct PersistCtl {
 // failure-detection test (test_skip, and test_spin = 4096 polls)
 cudaError_t persist_ctl_reset(PersistCtl* ctl, int test_skip, cudaStream_t s);
 // FP64 path (de_fp64.cu)
-void k_configure(size_t smem_gen);
+void k_configure();
+// Lets kernel k be launched with whatever dynamic shared memory the device
+// allows beside its static part.  The limit belongs to the function, not to a
+// handle: set to one handle's need it would refuse the launches of another,
+// larger one, so every kernel gets the same limit from every handle.
+cudaError_t allow_dynamic_smem(const void* k);
 // var: some run uses a strategy variant or jDE; suite: some run uses an
 // objective of the proposed benchmark (5..20)
 void k_gen_fp64_launch(const RunDesc* runs, const int4* items, int nitems, int threads, size_t smem, bool var,

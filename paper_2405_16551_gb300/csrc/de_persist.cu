@@ -788,7 +788,7 @@ static bool persist_cluster_plan(PersistPlan& pp, const RunDesc& R, int nruns, i
   cfg.numAttrs = 1;
   int nclusters = 0;
   auto query = [&](auto kern) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_dynamic_smem((const void*)kern);
     return cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg);
   };
   const bool var = R.strategy != 0 || R.jde;

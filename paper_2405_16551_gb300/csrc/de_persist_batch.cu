@@ -626,7 +626,7 @@ bool pbatch_plan(PbPlan& pp, const std::vector<RunDesc>& runs, int prec) {
     return false;
   }
   if (smem + fa.sharedSizeBytes > (size_t)optin) return false;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+  if (allow_dynamic_smem(k) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kPbThreads, smem) != cudaSuccess || per_sm < 1) {
     cudaGetLastError();
     return false;

@@ -711,7 +711,7 @@ bool persist_cta_plan(PersistPlan& pp, const RunDesc& R, int nruns, int prec) {
   const bool var = R.strategy != 0 || R.jde;
   const void* k = cta_kernel(prec, var);
   int per_sm = 0, dev = 0, nsm = 0;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+  if (allow_dynamic_smem(k) != cudaSuccess ||
       cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem) != cudaSuccess || per_sm < 1) {

@@ -949,6 +949,8 @@ static void pack_b(const de_config& c, const RunDesc& R, std::vector<uint8_t>& o
     }
 }
 
+static const void* fit_kernel(int esz) { return esz == 2 ? (const void*)k_fit_tc<2, 1> : (const void*)k_fit_tc<4, 1>; }
+
 de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* cfgs, int prec, cudaStream_t s,
                         std::string& err) {
   p.prec = prec;
@@ -1119,8 +1121,7 @@ de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* 
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(p.d_pair_items, pair_items.data(), pair_items.size() * sizeof(int2), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
-      e = esz == 2 ? cudaFuncSetAttribute(k_fit_tc<2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem)
-                   : cudaFuncSetAttribute(k_fit_tc<4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
+      e = allow_dynamic_smem(esz == 2 ? (const void*)k_fit_tc<2, 2> : (const void*)k_fit_tc<4, 2>);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   p.nitems_trial = (int)trial_items.size();
@@ -1139,15 +1140,8 @@ de_status tc_plan_build(TcPlan& p, std::vector<RunDesc>& runs, const de_config* 
     cudaGetLastError();
   }
   p.d_band_cnt = (uint32_t*)((uint8_t*)p.arena + off_bcnt);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_band_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(p.smem_band, 1));
-  if (e == cudaSuccess) {
-    if (esz == 2) {
-      e = cudaFuncSetAttribute(k_fit_tc<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    } else {
-      e = cudaFuncSetAttribute(k_fit_tc<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    }
-  }
+  if (e == cudaSuccess) e = allow_dynamic_smem((const void*)k_band_fp64);
+  if (e == cudaSuccess) e = allow_dynamic_smem(fit_kernel(esz));
   if (e != cudaSuccess) {
     err = std::string("split-precision plan: ") + cudaGetErrorString(e);
     return DE_ERR_CUDA;
@@ -1176,10 +1170,6 @@ de_status tc_set_geometry(TcPlan& p, std::vector<RunDesc>& runs, int trial_rows,
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(p.d_trial_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e == cudaSuccess) {
-    e = esz == 2 ? cudaFuncSetAttribute(k_fit_tc<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                 : cudaFuncSetAttribute(k_fit_tc<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  }
   if (e != cudaSuccess) {
     err = std::string("split-precision geometry: ") + cudaGetErrorString(e);
     return DE_ERR_CUDA;
@@ -1301,12 +1291,7 @@ de_status tc_eval_launch(const TcPlan& p, const RunDesc* runs, int run, const Ru
 
 de_status tc_eval_rows(const RunDesc* desc, const int2* items, int tiles, int esz, size_t smem, const double* x,
                        int64_t ld, int n, double* f, cudaStream_t s, std::string& err) {
-  cudaFuncAttributes fa{};
-  cudaError_t e = esz == 2 ? cudaFuncGetAttributes(&fa, k_fit_tc<2, 1>) : cudaFuncGetAttributes(&fa, k_fit_tc<4, 1>);
-  if (e == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes < smem) {
-    e = esz == 2 ? cudaFuncSetAttribute(k_fit_tc<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                 : cudaFuncSetAttribute(k_fit_tc<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  }
+  cudaError_t e = allow_dynamic_smem(fit_kernel(esz));
   if (e == cudaSuccess) {
     if (esz == 2) {
       k_prep_rows<2><<<(n + 7) / 8, 256, 0, s>>>(desc, 0, x, ld, n);
