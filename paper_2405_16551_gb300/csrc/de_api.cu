@@ -1734,15 +1734,21 @@ de_status de_get_population(de_handle* h, int32_t run, double* x_host, double* f
   const size_t fb = f_host ? (size_t)R.np * sizeof(double) : 0;
   char* xd = (char*)x_host;
   char* fd = (char*)f_host;
-  const bool staged = xb + fb <= kStageBytes;
+  bool staged = xb + fb <= kStageBytes;
   if (staged && h->stage_bytes < xb + fb) {
     if (h->h_stage) cudaFreeHost(h->h_stage);
     h->h_stage = nullptr;
     h->stage_bytes = 0;
     size_t want = (size_t)64 << 10;
     while (want < xb + fb) want *= 2;
-    DE_CUDA(h, cudaMallocHost((void**)&h->h_stage, want));
-    h->stage_bytes = want;
+    if (cudaMallocHost((void**)&h->h_stage, want) == cudaSuccess) {
+      h->stage_bytes = want;
+    } else {
+      // no pinned memory to be had: straight into the caller's buffers
+      cudaGetLastError();
+      h->h_stage = nullptr;
+      staged = false;
+    }
   }
   if (staged) {
     xd = h->h_stage;
