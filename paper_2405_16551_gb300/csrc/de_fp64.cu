@@ -358,6 +358,8 @@ __global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restr
   __syncthreads();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = blockDim.x >> 5;
   if (nruns == 1 && s_stop) return;
+  // (read before the first barrier: no island has advanced)
+  const int interval = ISL && islands_together(runs, nruns, true) ? isl->interval : 0;
   SliceCtx sc;
   if constexpr (TC) slice_begin(sc, smem_p, kpad, cols, s_sl);
   unsigned nstopped = 0;  // runs known stopped (thread 0)
@@ -508,9 +510,9 @@ __global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restr
       if (nruns == 1 && s_stop) break;
     }
     if constexpr (ISL) {
-      if (!(live && isl->interval > 0 && g % isl->interval == 0)) continue;
-      // island model: migration after generation g (the islands advance
-      // together, so every CTA takes this branch).  The CTA of each island's
+      if (!(live && interval > 0 && g % interval == 0)) continue;
+      // island model: migration after generation g (islands that are together
+      // advance together, so every CTA takes this branch).  The CTA of each island's
       // tile 0 exchanges; a grid barrier then keeps every tile from building
       // generation g + 1 before the migrants are in place.
       const int cur = (int)(g & 1);

@@ -76,6 +76,8 @@ __global__ void __launch_bounds__(256, 1)
   }
   __syncthreads();
   if (nruns == 1 && s_stop) return;
+  // (read before the first barrier: no island has advanced)
+  const int interval = ISL && islands_together(runs, nruns, true) ? isl->interval : 0;
   SliceCtx sc;
   slice_begin(sc, smem_s, kpad, cols, s_sl);
   slice_load_m(sc, R.sl, R.sl_kpad);
@@ -301,9 +303,9 @@ __global__ void __launch_bounds__(256, 1)
     gen = g;
     pending = true;
     if constexpr (ISL) {
-      if (!(isl->interval > 0 && g % isl->interval == 0)) continue;
+      if (!(interval > 0 && g % interval == 0)) continue;
       // island model: the stop decision, then migration after generation g
-      // (the islands advance together, so every CTA takes this branch).  The CTA
+      // (islands that are together advance together, so every CTA takes this branch).  The CTA
       // of each island's tile 0 exchanges; a grid barrier then keeps every
       // tile from building generation g + 1 before the migrants are in place.
       if (warp == rw) reduce_best(g, (int)(itg % 3));

@@ -11,6 +11,23 @@
 
 namespace de {
 
+// Whether the m islands are at one generation (and none or all of them have
+// stopped, where `stops`), by the whole CTA.  Islands that a call has set apart
+// (one of them reset, or given a generation of its own) do not exchange
+// migrants: their points differ, so a mailbox would hold nobody's or old ones,
+// and a loop that meets at each point would meet at none.
+static __device__ bool islands_together(const RunDesc* __restrict__ runs, int m, bool stops) {
+  const RunState* a = runs[0].st;
+  const int64_t gen = *(volatile const int64_t*)&a->gen;
+  const bool stop = *(volatile const int32_t*)&a->stop != 0;
+  int apart = 0;
+  for (int k = threadIdx.x; k < m; k += blockDim.x) {
+    const RunState* b = runs[k].st;
+    apart |= *(volatile const int64_t*)&b->gen != gen || (stops && (*(volatile const int32_t*)&b->stop != 0) != stop);
+  }
+  return __syncthreads_or(apart) == 0;
+}
+
 // CTA-wide arg-extremum of (key, index) over i in [0, np) minus the `ntaken`
 // indices already chosen; worst = largest (key, index), else smallest.
 static __device__ int island_pick(const double* __restrict__ f, int np, const int* taken, int ntaken, bool worst) {

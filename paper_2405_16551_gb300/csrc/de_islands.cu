@@ -44,9 +44,10 @@
 
 namespace de {
 
-// a migration is due after generation gen
-__device__ __forceinline__ bool island_due(const IslandCtl* ctl, int64_t gen) {
-  return ctl->interval > 0 && gen > 0 && gen % ctl->interval == 0 && gen > ctl->mig_gen;
+// a migration is due after generation gen of some island (the whole CTA)
+__device__ __forceinline__ bool island_due(const RunDesc* runs, const IslandCtl* ctl, int64_t gen) {
+  return ctl->interval > 0 && gen > 0 && gen % ctl->interval == 0 && gen > ctl->mig_gen &&
+         islands_together(runs, ctl->m, false);
 }
 
 __global__ void __launch_bounds__(256) k_island_select(const RunDesc* __restrict__ runs, const IslandCtl* ctl,
@@ -54,7 +55,7 @@ __global__ void __launch_bounds__(256) k_island_select(const RunDesc* __restrict
   const int k = blockIdx.x;
   const RunDesc& R = runs[k];
   const int64_t gen = *(volatile int64_t*)&R.st->gen;
-  if (!island_due(ctl, gen)) return;
+  if (!island_due(runs, ctl, gen)) return;
   const int cur = (int)(gen & 1), nmig = ctl->nmig;
   const double* f = R.f[cur];
   __shared__ int best[kIslandMaxMigrants], worst[kIslandMaxMigrants];
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__(256) k_island_apply(const RunDesc* __restrict_
   const int k = blockIdx.x, m = ctl->m;
   const RunDesc& R = runs[k];
   const int64_t gen = *(volatile int64_t*)&R.st->gen;
-  if (!island_due(ctl, gen)) return;
+  if (!island_due(runs, ctl, gen)) return;
   const int cur = (int)(gen & 1), nmig = ctl->nmig;
   const int from = (k + m - 1) % m;
   for (int q = 0; q < nmig; ++q) {
@@ -115,7 +116,7 @@ __global__ void __launch_bounds__(256) k_island_async(const RunDesc* __restrict_
   const int k = blockIdx.x;
   const RunDesc& R = runs[k];
   const int64_t gen = *(volatile int64_t*)&R.st->gen;
-  if (!island_due(ctl, gen)) return;
+  if (!island_due(runs, ctl, gen)) return;
   const int64_t ep = gen / ctl->interval;
   const size_t wslot = (size_t)(ep & 1) * stage.slot, rslot = (size_t)((ep & 1) ^ 1) * stage.slot;
   // the previous migration point posted (not so after a reset or a population change)
@@ -137,12 +138,10 @@ __global__ void __launch_bounds__(256) k_island_group(const RunDesc* __restrict_
   __syncthreads();
   if (any)
     for (int k = threadIdx.x; k < m; k += blockDim.x) runs[k].st->stop = 1;
-  if (threadIdx.x == 0) {
-    const int64_t gen = runs[0].st->gen;
-    if (island_due(ctl, gen)) {
-      ctl->mig_gen = gen;
-      if (posted) ctl->post_gen = gen;
-    }
+  const int64_t gen = runs[0].st->gen;
+  if (island_due(runs, ctl, gen) && threadIdx.x == 0) {
+    ctl->mig_gen = gen;
+    if (posted) ctl->post_gen = gen;
   }
 }
 
