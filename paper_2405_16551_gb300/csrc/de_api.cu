@@ -66,6 +66,7 @@ struct de_handle {
   bool fp64_persist = false;  // FP64: every generation of a call in one cooperative launch
   bool fp64_local = false;    // FP64: the same, a cluster per run with the population in shared memory
   bool isl_even = true;       // the islands' generations and stop flags are known to agree
+  bool apart_captured = false;  // ... may cease to whenever the caller launches a graph (one island's captured reset)
   LocalPlan local;
   bool fp64_cluster = false;  // ... launched as one thread-block cluster (one run of at most 8 tiles)
   PersistCtl* d_ctl64 = nullptr;
@@ -369,36 +370,30 @@ static de_status launch_generation(de_handle* h, cudaStream_t s) {
 static de_status launch_generation(de_handle* h) { return launch_generation(h, h->stream); }
 
 static de_status read_states(de_handle* h);
-static de_status need_states(de_handle* h);
 
 // Whether this call's generations run in the local form.  Its islands advance
 // together; islands whose states a call has set apart (one island reset or
-// given a generation of its own) run on the other forms, and so do islands
-// under the caller's stream capture (the graph may be replayed after such a call).
+// given a generation of its own) run on the other forms until the states have
+// been read and agree again (a call that only enqueues does not wait to see),
+// and so do islands under the caller's stream capture (the graph may be launched
+// after such a call).
 static de_status use_local(de_handle* h, bool& use) {
   use = true;
   if (!h->islands) return DE_OK;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   DE_CUDA(h, cudaStreamIsCapturing(h->stream, &cap));
-  use = cap == cudaStreamCaptureStatusNone;
-  if (!use || h->isl_even) return DE_OK;
-  const de_status s = need_states(h);
-  if (s != DE_OK) return s;
-  h->isl_even = true;
-  for (int r = 1; r < h->nruns; ++r)
-    h->isl_even = h->isl_even && h->h_state[r].gen == h->h_state[0].gen && h->h_state[r].stop == h->h_state[0].stop &&
-                  h->h_state[r].evals == h->h_state[0].evals;
-  use = h->isl_even;
+  use = cap == cudaStreamCaptureStatusNone && h->isl_even && !h->apart_captured;
   return DE_OK;
 }
 
 // Whether the caller is capturing the handle's stream.  What a call enqueues
 // then runs whenever the caller launches the graph, at a time unknown here, so
 // from then on the mirror of the states is never taken for current.
-static de_status note_capture(de_handle* h) {
+static de_status note_capture(de_handle* h, bool& on) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   DE_CUDA(h, cudaStreamIsCapturing(h->stream, &cap));
-  h->captured = h->captured || cap != cudaStreamCaptureStatusNone;
+  on = cap != cudaStreamCaptureStatusNone;
+  h->captured = h->captured || on;
   return DE_OK;
 }
 
@@ -504,6 +499,12 @@ static de_status read_states(de_handle* h) {
                              h->stream));
   DE_CUDA(h, cudaStreamSynchronize(h->stream));
   h->state_fresh = true;
+  const RunState& a = h->h_state[0];
+  h->isl_even = true;
+  for (int r = 1; r < h->nruns && h->islands; ++r) {
+    const RunState& b = h->h_state[r];
+    h->isl_even = h->isl_even && a.gen == b.gen && a.stop == b.stop && a.evals == b.evals;
+  }
   return DE_OK;
 }
 
@@ -1517,11 +1518,13 @@ de_status de_reset(de_handle* h, int32_t run) {
   if (!h) return fail(nullptr, DE_ERR_INVALID_ARG, "handle is NULL");
   if (run < -1 || run >= h->nruns) return fail(h, DE_ERR_INVALID_ARG, "run out of range");
   h->err.clear();
-  const de_status cap = note_capture(h);
-  if (cap != DE_OK) return cap;
-  const de_status st = run < 0 ? init_runs(h, 0, h->nruns) : init_runs(h, run, 1);
+  bool cap = false;
+  de_status st = note_capture(h, cap);
+  if (st == DE_OK) st = run < 0 ? init_runs(h, 0, h->nruns) : init_runs(h, run, 1);
   if (st != DE_OK) return st;
-  h->isl_even = run < 0;
+  // (a captured call has reset nothing yet)
+  if (cap) h->apart_captured = h->apart_captured || run >= 0;
+  else h->isl_even = run < 0;
   if (h->surr) {
     const de_status s = surr_reset(*h->surr, h->stream, h->err);
     if (s != DE_OK) return fail(h, s, h->err);
@@ -1606,7 +1609,8 @@ de_status de_step(de_handle* h, int64_t generations) {
   if (!h) return fail(nullptr, DE_ERR_INVALID_ARG, "handle is NULL");
   if (generations < 0) return fail(h, DE_ERR_INVALID_ARG, "generations must be >= 0");
   h->err.clear();
-  const de_status s = note_capture(h);
+  bool cap = false;
+  const de_status s = note_capture(h, cap);
   return s == DE_OK ? enqueue_generations(h, generations) : s;
 }
 
@@ -1794,8 +1798,7 @@ de_status de_set_population(de_handle* h, int32_t run, const double* x_host, con
   DE_CUDA(h, cudaGetLastError());
   s = islands_resync(h);
   if (s != DE_OK) return s;
-  DE_CUDA(h, cudaStreamSynchronize(h->stream));
-  return DE_OK;
+  return read_states(h);
 }
 
 de_status de_set_generation(de_handle* h, int32_t run, int64_t generation) {
@@ -1826,8 +1829,7 @@ de_status de_set_generation(de_handle* h, int32_t run, int64_t generation) {
   DE_CUDA(h, cudaGetLastError());
   s = islands_resync(h);
   if (s != DE_OK) return s;
-  DE_CUDA(h, cudaStreamSynchronize(h->stream));
-  return DE_OK;
+  return read_states(h);
 }
 
 de_status de_get_adaptive(de_handle* h, int32_t run, double* f_host, double* cr_host) {
@@ -2115,8 +2117,7 @@ de_status de_load(de_handle* h, const char* path) {
   DE_CUDA(h, cudaStreamSynchronize(h->stream));
   const de_status s = islands_resync(h);
   if (s != DE_OK) return s;
-  DE_CUDA(h, cudaStreamSynchronize(h->stream));
-  return DE_OK;
+  return read_states(h);
 }
 
 de_status de_eval_noalloc(int32_t precision, int32_t objective, int32_t d, double scale, const double* shift_dev,

@@ -56,3 +56,56 @@ def test_population_after_each_replay(prec, persist, np_, d, gens, monkeypatch):
     finally:
         capi.de_destroy(h)
         capi.de_destroy(ref)
+
+
+def _islands(stream, monkeypatch, mode):
+    monkeypatch.setenv("DE_GB300_FP64_PERSIST", mode)
+    cfg = capi.make_config(16, 8, objective=1, shift=problems.shift(8, seed=2), seed=7, target_error=0.0,
+                           max_generations=10**6)
+    return capi.de_init_islands(cfg, 3, 5, 1, stream)
+
+
+def test_an_island_reset_by_a_graph(monkeypatch):
+    """Its generations are no longer those of the other islands, which the
+    cluster-per-run loop would take for granted."""
+    import torch
+
+    s = torch.cuda.Stream()
+    h, ref = _islands(s.cuda_stream, monkeypatch, "3"), _islands(None, monkeypatch, "1")
+    try:
+        g = _captured(s, lambda: capi.de_reset(h, 1))
+        for n in (7, 4):
+            capi.de_step(h, n)
+            capi.de_step(ref, n)
+            with torch.cuda.stream(s):
+                g.replay()
+            capi.de_reset(ref, 1)
+        capi.de_step(h, 6)
+        capi.de_step(ref, 6)
+        for r in range(3):
+            (x, f), (xr, fr) = capi.de_get_population(h, r), capi.de_get_population(ref, r)
+            assert np.array_equal(x, xr) and np.array_equal(f, fr), r
+        del g
+    finally:
+        capi.de_destroy(h)
+        capi.de_destroy(ref)
+
+
+def test_step_after_one_islands_reset_only_enqueues(monkeypatch):
+    import torch
+
+    s = torch.cuda.Stream()
+    h = _islands(s.cuda_stream, monkeypatch, "3")
+    try:
+        capi.de_step(h, 3)
+        capi.de_reset(h, 1)
+        torch.cuda.synchronize()
+        before = torch.cuda.Event()
+        with torch.cuda.stream(s):
+            torch.cuda._sleep(1_000_000_000)  # about half a second
+            before.record()
+        capi.de_step(h, 4)
+        assert not before.query()
+        assert capi.de_get_best(h, 0)["generations"] == 7
+    finally:
+        capi.de_destroy(h)
