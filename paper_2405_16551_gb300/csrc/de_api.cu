@@ -39,12 +39,20 @@ struct de_handle {
   RunDesc* d_run = nullptr;
   int4* d_items = nullptr;  // FP64 generation kernel work list: (run, tile, first row, rows)
   int nitems = 0;
-  SlicePlan slices;           // FP64 rotations on the tensor cores (de_slice.cuh)
-  int2* d_shares = nullptr;   // sliced generation kernel: the items of each CTA
-  int nshares = 0;
+  SlicePlan slices;           // FP64 rotations on the tensor cores: of the handle's kernels (cooperative, cluster)
+  // the kernels of a single generation take a launch per form of the rotation
+  // (index: SliceForm; 0: the runs that are not sliced)
+  struct FormItems {
+    SlicePlan plan;
+    int4* d_items = nullptr;
+    int2* d_shares = nullptr;  // sliced: the items of each CTA
+    int nitems = 0, nshares = 0;
+    size_t smem = 0;           // not sliced: shared memory of the launch
+    bool variants = false, suite = false;
+  } form[3];
   // every run is sliced plain DE/rand/1/bin of objectives 0..3: the cooperative
-  // launch is k_gen_sliced (unit: every scale is 1)
-  bool sliced_loop = false, unit = true;
+  // launch is k_gen_sliced where its tiles fit (use_sliced; unit: every scale is 1)
+  bool sliced_loop = false, use_sliced = false, unit = true;
   size_t smem_loop = 0;
   int nsm = 1;
   int rows = 8;             // rows per tile of the FP64 generation kernel
@@ -269,6 +277,81 @@ static size_t gen_smem(int rows, int dp, int ncomp = 1) {
 }
 
 constexpr size_t kTileSmemMax = 200 * 1024;
+constexpr int kFormMma = 2;          // SliceForm on mma.sync
+// a tile's work beside its width, in coordinates (a share that counted coordinates
+// alone gave CTAs of D = 10 four times the tiles of CTAs of D = 100)
+constexpr double kShareTile = 300.0;
+
+static void free_form_items(de_handle* h) {
+  for (auto& F : h->form) {
+    if (F.d_items) cudaFree(F.d_items);
+    if (F.d_shares) cudaFree(F.d_shares);
+    F = de_handle::FormItems{};
+  }
+}
+
+// The items of each form of the rotation, and the CTAs' shares of them.
+static de_status build_form_items(de_handle* h, const std::vector<int4>& all) {
+  free_form_items(h);
+  std::vector<int4> items[3];
+  for (const int4& it : all) {
+    const RunDesc& R = h->run[it.x];
+    const int form = R.sl ? slice_form(R.sl_kpad) : 0;
+    auto& F = h->form[form];
+    items[form].push_back(it);
+    F.variants = F.variants || R.strategy != 0 || R.jde;
+    F.suite = F.suite || R.obj >= DE_OBJ_ZAKHAROV;
+    // (sliced rows have no separate term buffers, and a composition function's
+    // components take turns in one)
+    const int bufs = !R.sl ? 0 : R.obj >= DE_OBJ_ZAKHAROV ? 3 : form == kFormMma ? 2 : 4;
+    F.smem = std::max(F.smem, bufs ? (size_t)bufs * R.rows * R.dp * sizeof(double) : gen_smem(R.rows, R.dp, suite_comps(R)));
+    if (R.sl) {
+      if (R.obj >= DE_OBJ_COMPOSITION1) F.smem = std::max(F.smem, slice_group_smem(R.dp));
+      F.plan.kpad = std::max(F.plan.kpad, R.sl_kpad);
+      F.plan.dp_max = std::max(F.plan.dp_max, R.dp);
+    }
+  }
+  for (int form = 0; form < 3; ++form) {
+    auto& F = h->form[form];
+    const auto& v = items[form];
+    F.nitems = (int)v.size();
+    if (!F.nitems) continue;
+    DE_CUDA(h, cudaMalloc(&F.d_items, v.size() * sizeof(int4)));
+    DE_CUDA(h, cudaMemcpyAsync(F.d_items, v.data(), v.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
+    if (form == 0) continue;
+    SlicePlan& p = F.plan;
+    p.on = true;
+    p.form = form;
+    p.cols = slice_kernel_cols(p.kpad);
+    p.smem_op = slice_form_smem(form, p.kpad);
+    p.smem = p.smem_op + F.smem;
+    // contiguous shares of about equal work: a tile is a chain of latencies,
+    // nearly the same whatever its rows and width, times the components of a
+    // composition function
+    const int nct = std::min(F.nitems, h->nsm * k_gen_fp64_tc_per_sm(p, F.variants, F.suite));
+    std::vector<double> acc(v.size() + 1, 0.0);
+    for (size_t k = 0; k < v.size(); ++k) {
+      const RunDesc& R = h->run[v[k].x];
+      acc[k + 1] = acc[k] + suite_comps(R) * (R.d + kShareTile);
+    }
+    std::vector<int2> shares(nct);
+    int at = 0;
+    for (int b = 0; b < nct; ++b) {
+      // at least one item each; the share ends where its work does
+      const double want = acc.back() * (b + 1) / nct;
+      int e = at + 1;
+      while (e < F.nitems - (nct - 1 - b) && 0.5 * (acc[e] + acc[e + 1]) <= want) ++e;
+      if (b == nct - 1) e = F.nitems;
+      shares[b] = make_int2(at, e);
+      at = e;
+    }
+    F.nshares = nct;
+    DE_CUDA(h, cudaMalloc(&F.d_shares, shares.size() * sizeof(int2)));
+    DE_CUDA(h, cudaMemcpyAsync(F.d_shares, shares.data(), shares.size() * sizeof(int2), cudaMemcpyHostToDevice,
+                               h->stream));
+  }
+  return DE_OK;
+}
 
 // Split every run into tiles of at most h->rows targets, of near-equal size.
 static de_status build_items(de_handle* h) {
@@ -290,34 +373,8 @@ static de_status build_items(de_handle* h) {
   h->smem_gen = smem;
   h->nitems = (int)items.size();
   if (h->slices.on) {
-    // contiguous shares of about equal work (a coordinate's FP64 terms, times
-    // the components of a composition function; a row's draws and selection)
-    const int nct = std::min(h->nitems, h->nsm * h->slices.per_sm());
-    std::vector<double> acc(items.size() + 1, 0.0);
-    size_t tiles_smem = smem;
-    for (size_t k = 0; k < items.size(); ++k) {
-      const RunDesc& R = h->run[items[k].x];
-      acc[k + 1] = acc[k] + items[k].w * (suite_comps(R) * (double)R.d + 16.0);
-      if (R.sl && R.obj >= DE_OBJ_COMPOSITION1) tiles_smem = std::max(tiles_smem, slice_group_smem(R.dp));
-    }
-    std::vector<int2> shares(nct);
-    int at = 0;
-    for (int b = 0; b < nct; ++b) {
-      // at least one item each; the share ends where its work does
-      const double want = acc.back() * (b + 1) / nct;
-      int e = at + 1;
-      while (e < h->nitems - (nct - 1 - b) && 0.5 * (acc[e] + acc[e + 1]) <= want) ++e;
-      if (b == nct - 1) e = h->nitems;
-      shares[b] = make_int2(at, e);
-      at = e;
-    }
-    h->nshares = nct;
-    h->slices.smem = h->slices.smem_op + tiles_smem;
-    if (h->d_shares) cudaFree(h->d_shares);
-    h->d_shares = nullptr;
-    DE_CUDA(h, cudaMalloc(&h->d_shares, shares.size() * sizeof(int2)));
-    DE_CUDA(h, cudaMemcpyAsync(h->d_shares, shares.data(), shares.size() * sizeof(int2), cudaMemcpyHostToDevice,
-                               h->stream));
+    const de_status st = build_form_items(h, items);
+    if (st != DE_OK) return st;
   }
   if (h->d_items) cudaFree(h->d_items);
   h->d_items = nullptr;
@@ -356,9 +413,15 @@ static de_status islands_resync(de_handle* h) {
 // Enqueue one generation of every run (the kernels skip stopped runs).
 static de_status launch_generation(de_handle* h, cudaStream_t s) {
   if (h->prec == DE_PREC_FP64) {
-    if (h->slices.on)
-      k_gen_fp64_tc_launch(h->d_run, h->d_items, h->d_shares, h->nshares, h->slices, h->variants, h->suite, s);
-    else
+    if (h->slices.on) {
+      const auto& F0 = h->form[0];
+      if (F0.nitems) k_gen_fp64_launch(h->d_run, F0.d_items, F0.nitems, h->threads, F0.smem, F0.variants, F0.suite, s);
+      for (int form = 1; form < 3; ++form) {
+        const auto& F = h->form[form];
+        if (F.nitems)
+          k_gen_fp64_tc_launch(h->d_run, F.d_items, F.d_shares, F.nshares, F.plan, F.variants, F.suite, s);
+      }
+    } else
       k_gen_fp64_launch(h->d_run, h->d_items, h->nitems, h->threads, h->smem_gen, h->variants, h->suite, s);
     if (h->islands) k_island_launch(h->d_run, h->d_isl, h->stage, h->nruns, true, h->isl.async != 0, s);
   } else {
@@ -430,7 +493,7 @@ static de_status enqueue_generations(de_handle* h, int64_t n) {
       else if (h->fp64_cluster)
         DE_CUDA(h, k_gen_fp64_cluster_launch(h->d_run, h->d_items, h->nitems, h->threads, h->smem_gen, h->variants,
                                              h->suite, h->d_ctl64, g, h->stream, h->slices));
-      else if (h->sliced_loop)
+      else if (h->use_sliced)
         DE_CUDA(h, k_gen_sliced_launch(h->d_run, h->d_items, h->nitems, h->nruns, h->d_ctl64, g, h->slices, h->unit,
                                        h->smem_loop, h->stream, h->test_grid_skip, h->islands ? h->d_isl : nullptr,
                                        h->islands ? &h->stage : nullptr));
@@ -541,13 +604,12 @@ static size_t eval_smem(const de_handle* h, int run0, int n) {
 // 3000 launches, 16 ms, run by run).
 static de_status init_runs(de_handle* h, int run0, int n) {
   h->state_fresh = false;
-  int np_max = 0, dp_max = 0, dp_sliced = 0;
+  int np_max = 0, dp_max = 0;
   bool jde = false, plain = false;
   for (int r = run0; r < run0 + n; ++r) {
     const RunDesc& R = h->run[r];
     np_max = std::max(np_max, R.np);
     dp_max = std::max(dp_max, R.dp);
-    if (R.sl) dp_sliced = std::max(dp_sliced, R.dp);
     jde = jde || R.jde;
     plain = plain || (!R.sl && R.obj != DE_OBJ_ODE);
     if (R.obj == DE_OBJ_ODE && !h->ode_ref_done[r]) {
@@ -568,8 +630,10 @@ static de_status init_runs(de_handle* h, int run0, int n) {
     else
       for (int r = run0; r < run0 + n; ++r) tc_init_eval_launch(h->tc, h->d_run, r, h->run[r], h->stream);
   } else {
-    if (all && h->slices.on)
-      k_eval_pops_tc_launch(h->d_run, h->d_items, h->d_shares, h->nshares, h->slices, dp_sliced, h->stream);
+    for (int form = 1; form < 3 && all; ++form) {
+      const auto& F = h->form[form];
+      if (F.nitems) k_eval_pops_tc_launch(h->d_run, F.d_items, F.d_shares, F.nshares, F.plan, h->stream);
+    }
     if (all && plain) k_eval_pops_launch(h->d_run, run0, n, np_max, eval_smem(h, run0, n), h->stream);
     for (int r = run0; r < run0 + n; ++r) {
       const RunDesc& R = h->run[r];
@@ -615,7 +679,7 @@ static std::string tune_key(const de_handle* h) {
   }
   char b[256];
   // (var, form: which of the kernels apply)
-  snprintf(b, sizeof b, "gen_fp64v6 runs=%d np0=%d d0=%d obj0=%d rot0=%d sumnp=%lld sumnd=%lld var=%d form=%d", h->nruns,
+  snprintf(b, sizeof b, "gen_fp64v7 runs=%d np0=%d d0=%d obj0=%d rot0=%d sumnp=%lld sumnd=%lld var=%d form=%d", h->nruns,
            h->run[0].np, h->run[0].d, h->run[0].obj, h->run[0].rotate, sum_np, sum_d, h->variants ? 1 : 0,
            (h->slices.on ? 1 : 0) + (h->sliced_loop ? 2 : 0) + 4 * h->local.csize);
   return b;
@@ -684,8 +748,8 @@ static int heuristic_rows(const de_handle* h, int nsm) {
   for (auto& R : h->run) np_total += R.np;
   // about one CTA per SM, at most 8 rows (one warp per target)
   int rows = (int)std::max(1LL, std::min(8LL, (np_total + nsm - 1) / nsm));
-  if (h->slices.on) {
-    // the sliced cooperative kernel runs one CTA per SM: the fewest rows
+  if (h->slices.on && (h->sliced_loop || h->slices.form != kFormMma)) {
+    // the cooperative kernels on tcgen05 run one CTA per SM: the fewest rows
     // whose tiles all fit, where there are such
     auto tiles = [&](int r) {
       long long n = 0;
@@ -703,17 +767,19 @@ static int heuristic_rows(const de_handle* h, int nsm) {
 // or islands whose tiles all fit on the device at once (the grid barrier's
 // count, tiles x 2^20 generations per launch, stays below 2^32);
 // DE_GB300_FP64_PERSIST=0 disables it, =1 forces it where it applies.
-static bool fp64_persist_ok(const de_handle* h) {
+static bool fp64_persist_ok(de_handle* h) {
   if (h->prec != DE_PREC_FP64 || h->surr || (h->islands && h->suite) || !h->d_ctl64 || h->nitems >= 4096) return false;
   if (const char* e = getenv("DE_GB300_FP64_PERSIST"))
     if (e[0] == '0') return false;
-  if (h->sliced_loop) return h->nitems <= k_gen_sliced_capacity(h->islands, h->unit, h->slices, h->smem_loop);
+  // (more tiles than SMs: the general loop, two CTAs of which share an SM)
+  h->use_sliced = h->sliced_loop && h->nitems <= k_gen_sliced_capacity(h->islands, h->unit, h->slices, h->smem_loop);
+  if (h->use_sliced) return true;
   return h->nitems <= k_gen_fp64_persist_capacity(h->threads, h->smem_gen, h->variants, h->suite, h->slices,
                                                   h->islands);
 }
 
 // ... and as one thread-block cluster: one run of at most 8 tiles.
-static bool fp64_cluster_ok(const de_handle* h) {
+static bool fp64_cluster_ok(de_handle* h) {
   return h->nruns == 1 && fp64_persist_ok(h) &&
          k_gen_fp64_cluster_fits(h->nitems, h->threads, h->smem_gen, h->variants, h->suite, h->slices);
 }
@@ -1107,7 +1173,7 @@ de_status de_destroy(de_handle* h) {
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   tc_plan_free(h->tc);
   if (h->d_items) cudaFree(h->d_items);
-  if (h->d_shares) cudaFree(h->d_shares);
+  free_form_items(h);
   if (h->d_run) cudaFree(h->d_run);
   if (h->d_ctl64) cudaFree(h->d_ctl64);
   if (h->isl_mem) cudaFree(h->isl_mem);
@@ -1423,14 +1489,16 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
         k_slice_m_launch(R.MT, pairs, c.d, (uint8_t*)R.sl, (int32_t*)R.slx, h->stream);
         h->slices.on = true;
         h->slices.kpad = std::max(h->slices.kpad, R.sl_kpad);
-        h->slices.cols = std::max(h->slices.cols, slice_kernel_cols(R.sl_kpad));
-        h->slices.smem_op = std::max(h->slices.smem_op, slice_kernel_smem(R.sl_kpad));
       }
     } else {
       R.rownorm = 1.0f;
     }
   }
   if (h->slices.on) {
+    h->slices.form = slice_form(h->slices.kpad);
+    h->slices.cols = slice_kernel_cols(h->slices.kpad);
+    for (auto& R : h->run)
+      if (R.sl) h->slices.smem_op = std::max(h->slices.smem_op, slice_form_smem(slice_form(R.sl_kpad), R.sl_kpad));
     // every run's smallest tile has to fit beside the operands
     bool fits = true;
     for (auto& R : h->run) fits = fits && gen_smem(1, R.dp, suite_comps(R)) + h->slices.smem_op <= kTileSmemMax;

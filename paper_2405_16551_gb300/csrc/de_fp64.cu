@@ -314,17 +314,17 @@ constexpr long long kFp64Spin = 1LL << 22;
 
 // ISL: the runs are islands (an instance of its own, so that the other
 // instances keep their register allocation)
-// TC: some run's rotation is sliced (de_slice.cuh); each CTA keeps its run's
-// matrix resident for the whole launch (a composition function's matrices
-// take turns).  kpad, cols: the launch's operand sizes.
-template <bool VAR, bool SUITE, bool ISL, bool TC>
-__global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restrict__ runs,
+// FORM: some run's rotation is sliced (de_slice.cuh, de_slice_mma.cuh); each CTA
+// keeps its run's matrix resident for the whole launch (a composition
+// function's matrices take turns).  kpad, cols: the launch's operand sizes.
+template <bool VAR, bool SUITE, bool ISL, int FORM>
+__global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : FORM == kSliceTc ? 1 : 0) k_gen_fp64_persist(const RunDesc* __restrict__ runs,
                                                           const int4* __restrict__ items, int nruns,
                                                           PersistCtl* ctl, long long gens, int clustered,
                                                           IslandCtl* isl, IslandStage stage, int kpad,
                                                           uint32_t cols) {
   extern __shared__ __align__(1024) uint8_t smem_p[];
-  double* sm = reinterpret_cast<double*>(smem_p + (TC ? slice_smem(kpad) : 0u));
+  double* sm = reinterpret_cast<double*>(smem_p + form_smem<FORM>(kpad));
   __shared__ SliceShared s_sl;
   __shared__ int s_stop, s_best, s_abort, s_done;
   __shared__ unsigned s_below;
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restr
   // (read before the first barrier: no island has advanced)
   const int interval = ISL && islands_together(runs, nruns, true) ? isl->interval : 0;
   SliceCtx sc;
-  if constexpr (TC) slice_begin(sc, smem_p, kpad, cols, s_sl);
+  if constexpr (FORM != kNoSlices) form_begin<FORM>(sc, smem_p, kpad, cols, s_sl);
   unsigned nstopped = 0;  // runs known stopped (thread 0)
   // the failure-detection test (off in normal launches): this CTA may leave
   // out its first arrival, and the barrier may give up sooner
@@ -413,10 +413,10 @@ __global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restr
     const bool live = !s_stop;
     const int64_t g = s_gen + 1;
     if (live) {
-      Best bb = gen_tile<VAR, SUITE, TC>(R, g, it.z, it.w, R.rows, max(s_best, 0), sm, s_fsuite, s_comp, &sc);
+      Best bb = gen_tile<VAR, SUITE, FORM>(R, g, it.z, it.w, R.rows, max(s_best, 0), sm, s_fsuite, s_comp, &sc);
       if (lane == 0) { s_bf[warp] = bb.f; s_bk[warp] = bb.k; s_bi[warp] = bb.i; }
       __syncthreads();
-      if (TC && tid == 0 && s_sl.fail) {
+      if (FORM == kSliceTc && tid == 0 && s_sl.fail) {
         // a wait for the products gave up: every CTA leaves after this
         // generation's barrier (which this one does not join; a cluster's
         // members are told before theirs)
@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restr
     } else if (warp == 0) {
       // arrive, then wait for every CTA of this iteration
       __syncwarp();
-      const bool ok = (!TC || *(volatile int*)&s_abort == 0) && grid_sync();
+      const bool ok = (FORM != kSliceTc || *(volatile int*)&s_abort == 0) && grid_sync();
       if (lane == 0) {
         if (!ok) {
           atomicExch(&ctl->abort, 1);
@@ -547,9 +547,7 @@ __global__ void __launch_bounds__(256) k_gen_fp64_persist(const RunDesc* __restr
       __syncthreads();
     }
   }
-  if constexpr (TC) {
-    slice_end(sc);
-  }
+  if constexpr (FORM != kNoSlices) form_end<FORM>(sc);
 }
 
 }  // namespace de
@@ -559,24 +557,23 @@ namespace de {
 
 // The instance of the cooperative kernel (islands of the suite's objectives
 // run generation by generation).
-static const void* persist_kernel(bool var, bool suite, bool isl, bool tc) {
-  if (tc)
-    return isl ? (var ? (const void*)k_gen_fp64_persist<true, false, true, true>
-                      : (const void*)k_gen_fp64_persist<false, false, true, true>)
-           : var && suite ? (const void*)k_gen_fp64_persist<true, true, false, true>
-           : var          ? (const void*)k_gen_fp64_persist<true, false, false, true>
-           : suite        ? (const void*)k_gen_fp64_persist<false, true, false, true>
-                          : (const void*)k_gen_fp64_persist<false, false, false, true>;
-  return isl ? (var ? (const void*)k_gen_fp64_persist<true, false, true, false>
-                    : (const void*)k_gen_fp64_persist<false, false, true, false>)
-         : var && suite ? (const void*)k_gen_fp64_persist<true, true, false, false>
-         : var          ? (const void*)k_gen_fp64_persist<true, false, false, false>
-         : suite        ? (const void*)k_gen_fp64_persist<false, true, false, false>
-                        : (const void*)k_gen_fp64_persist<false, false, false, false>;
+template <int FORM>
+static const void* persist_kernel_of(bool var, bool suite, bool isl) {
+  return isl ? (var ? (const void*)k_gen_fp64_persist<true, false, true, FORM>
+                    : (const void*)k_gen_fp64_persist<false, false, true, FORM>)
+         : var && suite ? (const void*)k_gen_fp64_persist<true, true, false, FORM>
+         : var          ? (const void*)k_gen_fp64_persist<true, false, false, FORM>
+         : suite        ? (const void*)k_gen_fp64_persist<false, true, false, FORM>
+                        : (const void*)k_gen_fp64_persist<false, false, false, FORM>;
+}
+static const void* persist_kernel(bool var, bool suite, bool isl, int form) {
+  return form == kSliceMma  ? persist_kernel_of<kSliceMma>(var, suite, isl)
+         : form == kSliceTc ? persist_kernel_of<kSliceTc>(var, suite, isl)
+                            : persist_kernel_of<kNoSlices>(var, suite, isl);
 }
 
 // Dynamic shared memory of a cooperative (or one-cluster) launch.  The
-// sliced instances take all of an SM's shared memory: their CTAs wait for one
+// instances on tcgen05 take all of an SM's shared memory: their CTAs wait for one
 // another, so no other kernel that allocates tensor memory may share an SM
 // with them (two such grids, each holding the columns the other waits for,
 // would never finish).
@@ -591,7 +588,9 @@ size_t fp64_exclusive_smem(const void* k, size_t smem) {
   return std::max(smem, (size_t)most - a.sharedSizeBytes);
 }
 
-static size_t persist_smem(const void* k, size_t smem, bool tc) { return tc ? fp64_exclusive_smem(k, smem) : smem; }
+static size_t persist_smem(const void* k, size_t smem, const SlicePlan& sp) {
+  return sp.form == kSliceTc ? fp64_exclusive_smem(k, smem + sp.smem_op) : smem + sp.smem_op;
+}
 
 cudaError_t allow_dynamic_smem(const void* k) {
   cudaFuncAttributes a{};
@@ -611,8 +610,7 @@ void k_configure() {
                         (const void*)k_gen_fp64<false, true>, (const void*)k_gen_fp64<true, true>,
                         (const void*)k_eval_rows, (const void*)k_eval_pops, (const void*)k_best_exact})
     allow_dynamic_smem(k);
-  for (int q = 0; q < 12; ++q)
-    allow_dynamic_smem(persist_kernel((q & 2) != 0, q / 4 == 1, q / 4 == 2, (q & 1) != 0));
+  for (int q = 0; q < 18; ++q) allow_dynamic_smem(persist_kernel(q & 1, (q >> 1) % 3 == 1, (q >> 1) % 3 == 2, q / 6));
   k_tc_configure();
 }
 
@@ -630,8 +628,8 @@ cudaError_t k_gen_fp64_persist_launch(const RunDesc* runs, const int4* items, in
                   (void*)&isl, (void*)&st, (void*)&kpad, (void*)&cols};
   const dim3 grid((unsigned)nitems), block((unsigned)threads);
   if (isl && suite) return cudaErrorInvalidValue;  // islands of the suite's objectives run generation by generation
-  const void* k = persist_kernel(var, suite, isl != nullptr, sp.on);
-  return cudaLaunchCooperativeKernel(k, grid, block, args, persist_smem(k, smem + sp.smem_op, sp.on), s);
+  const void* k = persist_kernel(var, suite, isl != nullptr, sp.form);
+  return cudaLaunchCooperativeKernel(k, grid, block, args, persist_smem(k, smem, sp), s);
 }
 
 // The same kernel as one cluster of nitems CTAs (nitems <= 8, one run).
@@ -656,8 +654,8 @@ cudaError_t k_gen_fp64_cluster_launch(const RunDesc* runs, const int4* items, in
   cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(PersistCtl), s);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[1];
-  const void* k = persist_kernel(var, suite, false, sp.on);
-  cudaLaunchConfig_t cfg = cluster_config(nitems, threads, persist_smem(k, smem + sp.smem_op, sp.on), s, attr);
+  const void* k = persist_kernel(var, suite, false, sp.form);
+  cudaLaunchConfig_t cfg = cluster_config(nitems, threads, persist_smem(k, smem, sp), s, attr);
   int nruns = 1, clustered = 1, kpad = sp.kpad;
   uint32_t cols = sp.cols;
   IslandCtl* isl = nullptr;
@@ -671,8 +669,8 @@ bool k_gen_fp64_cluster_fits(int nitems, int threads, size_t smem, bool var, boo
   if (nitems < 1 || nitems > 8) return false;
   int n = 0;
   cudaLaunchAttribute attr[1];
-  const void* k = persist_kernel(var, suite, false, sp.on);
-  cudaLaunchConfig_t cfg = cluster_config(nitems, threads, persist_smem(k, smem + sp.smem_op, sp.on), 0, attr);
+  const void* k = persist_kernel(var, suite, false, sp.form);
+  cudaLaunchConfig_t cfg = cluster_config(nitems, threads, persist_smem(k, smem, sp), 0, attr);
   if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -685,8 +683,8 @@ int k_gen_fp64_persist_capacity(int threads, size_t smem, bool var, bool suite, 
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (isl && suite) return 0;  // islands of the suite's objectives run generation by generation
-  const void* k = persist_kernel(var, suite, isl, sp.on);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, persist_smem(k, smem + sp.smem_op, sp.on)) !=
+  const void* k = persist_kernel(var, suite, isl, sp.form);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, persist_smem(k, smem, sp)) !=
       cudaSuccess) {
     cudaGetLastError();
     return 0;

@@ -43,7 +43,7 @@
 #include "de_gen_tile.cuh"
 #include "de_internal.cuh"
 #include "de_kernels.h"
-#include "de_slice.cuh"
+#include "de_slice_mma.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -56,12 +56,9 @@ constexpr long long kLocalSpin = 1LL << 22;  // polls of an island counter (each
 // on tcgen05; as digit products on mma.sync (d <= 32).
 enum LocalRot { kRotChain = 0, kRotTc = 1, kRotMma = 2 };
 
-// Operands of the mma.sync form: y's digits as slice_digits writes them (32
-// coordinates), M's digits [digit][8-coordinate group][output < 32] of 16 bytes,
-// the group sums [group][row][output].
-constexpr uint32_t kMmaB = 4u * kSliceKg, kMmaA = (uint32_t)kSlices * 4u * 32u * 16u;
-constexpr int kMmaPst = 36;  // floats per row of the sums (the accumulators' stores meet no bank twice)
-constexpr uint32_t kMmaP = 9u * kSliceRows * kMmaPst * 4u;
+// Bytes of the mma.sync form's operands (de_slice_mma.cuh, width 32).
+constexpr uint32_t kMmaB = mma_b_bytes(32), kMmaA = mma_a_bytes(32), kMmaP = mma_p_bytes(32);
+constexpr int kMmaPst = mma_pst(32);
 
 // Byte offsets of a CTA's dynamic shared memory: operands of the digit
 // products, FP64 rows of y and of the rows that take the chain, the two
@@ -79,70 +76,12 @@ __host__ __device__ inline LocalLayout local_layout(int rot, int kpad, int dp, i
   return L;
 }
 
-__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr)
-               : "memory");
-}
-__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, "
-      "%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// The digit products of outputs 16 mt .. + 15 in groups G0 >= G1 >= G2 (the
-// pairs of digits s of y and t of M with s + t = g; -1: none), into the sums.
-// Integers below 2^23 in FP32: exact.
-template <int G0, int G1, int G2>
-__device__ __forceinline__ void local_products(uint32_t sB, uint32_t sA, float* P, int mt, int lane) {
-  const int i = lane >> 3, r = lane & 7;
-  uint32_t b[kSlices][4];  // per digit of y: the 8-coordinate groups 0 .. 3
-#pragma unroll
-  for (int s = 0; s < kSlices; ++s)
-    if (s <= G0) ldmatrix4(b[s], sB + (uint32_t)i * kSliceKg + (uint32_t)s * 128u + (uint32_t)r * 16u);
-  float c[3][4] = {};
-  const uint32_t a0 = sA + ((uint32_t)(i >> 1) * 32u + (uint32_t)(16 * mt + 8 * (i & 1) + r)) * 16u;
-#pragma unroll
-  for (int t = 0; t < kSlices; ++t) {
-    if (t > G0) continue;
-#pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-      uint32_t a[4];
-      ldmatrix4(a, a0 + (uint32_t)(t * 4 + 2 * ks) * 512u);
-      if (G0 - t >= 0 && G0 - t < kSlices) mma_16816(c[0], a, b[(G0 - t) & 7][2 * ks], b[(G0 - t) & 7][2 * ks + 1]);
-      if (G1 - t >= 0 && G1 - t < kSlices) mma_16816(c[1], a, b[(G1 - t) & 7][2 * ks], b[(G1 - t) & 7][2 * ks + 1]);
-      if (G2 - t >= 0 && G2 - t < kSlices) mma_16816(c[2], a, b[(G2 - t) & 7][2 * ks], b[(G2 - t) & 7][2 * ks + 1]);
-    }
-  }
-  constexpr int G[3] = {G0, G1, G2};
-  const int n = 2 * (lane & 3), j = 16 * mt + (lane >> 2);
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    if (G[q] < 0) continue;
-    float* p = P + (size_t)(G[q] * kSliceRows + n) * kMmaPst + j;
-    p[0] = c[q][0];
-    p[kMmaPst] = c[q][1];
-    p[8] = c[q][2];
-    p[kMmaPst + 8] = c[q][3];
-  }
-}
-
 // M's digits and the zeroed operand of y's, by the whole CTA (which
 // synchronises before the first product).
 __device__ __forceinline__ void local_load_m(const RunDesc& R, uint8_t* smem) {
-  const int tid = threadIdx.x, nkg = R.sl_kpad / 8;
-  for (uint32_t q = tid * 16u; q < kMmaB; q += blockDim.x * 16u)
+  for (uint32_t q = threadIdx.x * 16u; q < kMmaB; q += blockDim.x * 16u)
     *reinterpret_cast<uint4*>(smem + q) = make_uint4(0u, 0u, 0u, 0u);
-  for (int e = tid; e < kSlices * 4 * 32; e += blockDim.x) {
-    const int t = e >> 7, kg = (e >> 5) & 3, r = e & 31;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (kg < nkg)
-      v = __ldg(reinterpret_cast<const uint4*>(R.sl + (size_t)t * slice_bytes(R.sl_kpad) + (size_t)kg * 2048u + r * 16));
-    *reinterpret_cast<uint4*>(smem + kMmaB + (size_t)e * 16u) = v;
-  }
+  mma_copy_m(smem + kMmaB, R.sl, R.sl_kpad);
 }
 
 // z_j (lane j) of the row of y (lane k: y_k) whose digits this warp has
@@ -157,10 +96,10 @@ __device__ __forceinline__ double local_rotate(const RunDesc& R, uint8_t* smem, 
   // a warp takes 16 outputs and 10 to 12 of the 43 pairs of digits
   if (16 * (warp & 1) < d) {
     switch (warp >> 1) {
-      case 0: local_products<8, 3, -1>(sB, sA, sP, warp & 1, lane); break;
-      case 1: local_products<7, 2, -1>(sB, sA, sP, warp & 1, lane); break;
-      case 2: local_products<6, 1, 0>(sB, sA, sP, warp & 1, lane); break;
-      default: local_products<5, 4, -1>(sB, sA, sP, warp & 1, lane); break;
+      case 0: mma_products32<8, 3, -1>(sB, sA, sP, warp & 1, lane); break;
+      case 1: mma_products32<7, 2, -1>(sB, sA, sP, warp & 1, lane); break;
+      case 2: mma_products32<6, 1, 0>(sB, sA, sP, warp & 1, lane); break;
+      default: mma_products32<5, 4, -1>(sB, sA, sP, warp & 1, lane); break;
     }
   }
   __syncthreads();

@@ -369,7 +369,7 @@ int k_gen_sliced_capacity(bool isl, bool unit, const SlicePlan& p, size_t smem) 
 }
 
 size_t sliced_loop_smem(const SlicePlan& p, int dp_max) {
-  return p.smem_op + (size_t)2 * kSliceRows * dp_max * sizeof(double);
+  return slice_smem(p.kpad) + (size_t)2 * kSliceRows * dp_max * sizeof(double);
 }
 
 cudaError_t k_gen_sliced_launch(const RunDesc* runs, const int4* items, int nitems, int nruns, PersistCtl* ctl,

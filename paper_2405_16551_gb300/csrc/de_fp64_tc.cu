@@ -1,14 +1,15 @@
 // de_fp64_tc.cu -- FP64 kernels whose rotation runs as exact digit products on
-// the tensor cores (de_slice.cuh):
+// the tensor cores (de_slice.cuh on tcgen05, de_slice_mma.cuh on mma.sync):
 //
 //   k_slice_m       digit slices and row exponents of a run's matrices (once, at de_init)
-//   k_gen_fp64_tc   one generation of every run: each CTA works through a
-//                   contiguous share of the (run, tile) items and loads a
-//                   run's matrix once
+//   k_gen_fp64_tc   one generation of the runs of one form: each CTA works
+//                   through a contiguous share of the (run, tile) items and
+//                   loads a run's matrix once
 //   k_eval_rows_tc  f of caller rows: one matrix per CTA for all its tiles
 //
-// The persistent kernel's sliced instance is in de_fp64.cu.  All of them use
-// the same tile routines, so a run's numbers do not depend on which one ran.
+// The persistent kernel's sliced instances are in de_fp64.cu.  All of them use
+// the same tile routines, and the products are exact in either form, so a run's
+// numbers do not depend on which one ran.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -52,8 +53,8 @@ __global__ void __launch_bounds__(128) k_slice_m(const double* __restrict__ MT, 
 // buffers.  shares: per CTA the items [x, y).
 constexpr int kCompGroup = 64;  // rows of a composition function per matrix load
 
-template <bool VAR, bool SUITE>
-__global__ void __launch_bounds__(256, 1)
+template <bool VAR, bool SUITE, int FORM>
+__global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : 1)
     k_gen_fp64_tc(const RunDesc* __restrict__ runs, const int4* __restrict__ items, const int2* __restrict__ shares,
                   int kpad, uint32_t cols) {
   extern __shared__ __align__(1024) uint8_t smem_tc[];
@@ -66,11 +67,11 @@ __global__ void __launch_bounds__(256, 1)
   __shared__ int s_bi[8];
   __shared__ double s_fsuite[SUITE ? kCompGroup : 1];
   __shared__ double s_comp[SUITE ? kCompGroup : 1][10];
-  double* sm = reinterpret_cast<double*>(smem_tc + slice_smem(kpad));
+  double* sm = reinterpret_cast<double*>(smem_tc + form_smem<FORM>(kpad));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = blockDim.x >> 5;
   const int2 share = shares[blockIdx.x];
   SliceCtx sc;
-  slice_begin(sc, smem_tc, kpad, cols, s_sl);
+  form_begin<FORM>(sc, smem_tc, kpad, cols, s_sl);
   // only now: the next generation's CTAs must not take tensor memory that a
   // CTA of this one still waits for
   pdl_launch_dependents();
@@ -117,7 +118,7 @@ __global__ void __launch_bounds__(256, 1)
             build_trial_row<false, true>(R, R.X[cur], (uint32_t)(row0 + r), g, lane, T + r * dp, Y + warp * dp);
         }
         __syncthreads();
-        suite_comp_sliced(R, T, dp, nr, Y, Z, s_fsuite, s_comp, sc);
+        suite_comp_sliced<FORM>(R, T, dp, nr, Y, Z, s_fsuite, s_comp, sc);
         for (int r = warp; r < nr; r += nwarps)
           bb.offer(gen_select<VAR>(R, g, row0 + r, s_fsuite[r], T + r * dp, lane), row0 + r);
         __syncthreads();
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(256, 1)
     } else {
       for (int k = i; k < e; ++k) {
         const int4 t = items[k];
-        const Best b = gen_tile<VAR, SUITE, true>(R, g, t.z, t.w, R.rows, s_best, sm, s_fsuite, s_comp, &sc);
+        const Best b = gen_tile<VAR, SUITE, FORM>(R, g, t.z, t.w, R.rows, s_best, sm, s_fsuite, s_comp, &sc);
         bb.take(b.f, b.k, b.i);
         __syncthreads();
       }
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__(256, 1)
         R.part[items[k].y].f = k == i ? bb.f : CUDART_INF;
         R.part[items[k].y].idx = k == i ? bb.i : -1;
       }
-      if (*sc.s_fail) atomicOr(&st->err, kErrTimeout);
+      if (FORM == kSliceTc && *sc.s_fail) atomicOr(&st->err, kErrTimeout);
       __threadfence();
       const uint32_t n = (uint32_t)(e - i);
       s_last = atomicAdd(&st->ticket, n) + n == (uint32_t)R.ntiles;
@@ -152,11 +153,12 @@ __global__ void __launch_bounds__(256, 1)
     }
     i = e;
   }
-  slice_end(sc);
+  form_end<FORM>(sc);
 }
 
 // f of rows r0 .. r1 - 1 of x (row stride ld) with a sliced run; a warp per row
 // of the 8-row tiles.  Y, Z: 8 x dp doubles.
+template <int FORM>
 __device__ __forceinline__ void eval_sliced(const RunDesc& R, SliceCtx& sc, const double* __restrict__ x, int64_t ld,
                                             int r0, int r1, double* __restrict__ fout, uint8_t* __restrict__ fx_out,
                                             double* Y, double* s_f, double (*s_comp)[10]) {
@@ -168,7 +170,7 @@ __device__ __forceinline__ void eval_sliced(const RunDesc& R, SliceCtx& sc, cons
   for (int row0 = r0; row0 < r1; row0 += step) {
     const int nr = min(step, r1 - row0);
     if (suite) {
-      suite_tile<true>(R, x + (size_t)row0 * ld, ld, nr, Y, Z, s_f, s_comp, &sc);
+      suite_tile<FORM>(R, x + (size_t)row0 * ld, ld, nr, Y, Z, s_f, s_comp, &sc);
       for (int r = threadIdx.x; r < nr; r += blockDim.x) {
         fout[row0 + r] = s_f[r];
         if (fx_out) fx_out[row0 + r] = 1;
@@ -190,8 +192,8 @@ __device__ __forceinline__ void eval_sliced(const RunDesc& R, SliceCtx& sc, cons
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
-    if (sc.cur != R.sl) slice_load_m(sc, R.sl, kpad);
-    const double f = slice_fitness(sc, R, Y, Z, nr);
+    if (sc.cur != R.sl) form_load_m<FORM>(sc, R.sl, kpad);
+    const double f = form_fitness<FORM>(sc, R, Y, Z, nr);
     if (warp < nr) {
       if (lane == 0) {
         fout[row0 + warp] = f;
@@ -202,14 +204,15 @@ __device__ __forceinline__ void eval_sliced(const RunDesc& R, SliceCtx& sc, cons
   // a wait that gave up (it should not on a healthy device) cannot be
   // returned by this launch: the rows come back as NaN, the run is marked
   __syncthreads();
-  if (*sc.s_fail) {
+  if (FORM == kSliceTc && *sc.s_fail) {
     for (int r = r0 + (int)threadIdx.x; r < r1; r += blockDim.x) fout[r] = CUDART_NAN;
     if (threadIdx.x == 0) atomicOr(&R.st->err, kErrTimeout);
   }
 }
 
 // n rows of x with run `run`'s objective, in contiguous shares of whole tiles.
-__global__ void __launch_bounds__(256, 1)
+template <int FORM>
+__global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : 1)
     k_eval_rows_tc(const RunDesc* __restrict__ runs, int run, const double* __restrict__ x, int64_t ld, int n,
                    double* __restrict__ fout, uint8_t* __restrict__ fx_out, int kpad, uint32_t cols) {
   extern __shared__ __align__(1024) uint8_t smem_tc[];
@@ -219,17 +222,18 @@ __global__ void __launch_bounds__(256, 1)
   __shared__ double s_comp[kCompGroup][10];
   load_desc(sR, runs + run);
   SliceCtx sc;
-  slice_begin(sc, smem_tc, kpad, cols, s_sl);
-  double* Y = reinterpret_cast<double*>(smem_tc + slice_smem(kpad));
+  form_begin<FORM>(sc, smem_tc, kpad, cols, s_sl);
+  double* Y = reinterpret_cast<double*>(smem_tc + form_smem<FORM>(kpad));
   const int tiles = (n + kSliceRows - 1) / kSliceRows;
   const int r0 = (int)((long long)tiles * blockIdx.x / gridDim.x) * kSliceRows;
   const int r1 = min(n, (int)((long long)tiles * (blockIdx.x + 1) / gridDim.x) * kSliceRows);
-  eval_sliced(sR, sc, x, ld, r0, r1, fout, fx_out, Y, s_f, s_comp);
-  slice_end(sc);
+  eval_sliced<FORM>(sR, sc, x, ld, r0, r1, fout, fx_out, Y, s_f, s_comp);
+  form_end<FORM>(sc);
 }
 
 // The populations X[0] of the sliced runs, in the shares of k_gen_fp64_tc.
-__global__ void __launch_bounds__(256, 1)
+template <int FORM>
+__global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : 1)
     k_eval_pops_tc(const RunDesc* __restrict__ runs, const int4* __restrict__ items, const int2* __restrict__ shares,
                    int kpad, uint32_t cols) {
   extern __shared__ __align__(1024) uint8_t smem_tc[];
@@ -238,8 +242,8 @@ __global__ void __launch_bounds__(256, 1)
   __shared__ double s_f[kCompGroup];
   __shared__ double s_comp[kCompGroup][10];
   SliceCtx sc;
-  slice_begin(sc, smem_tc, kpad, cols, s_sl);
-  double* Y = reinterpret_cast<double*>(smem_tc + slice_smem(kpad));
+  form_begin<FORM>(sc, smem_tc, kpad, cols, s_sl);
+  double* Y = reinterpret_cast<double*>(smem_tc + form_smem<FORM>(kpad));
   const int2 share = shares[blockIdx.x];
   for (int i = share.x; i < share.y;) {
     int e = i + 1;
@@ -248,10 +252,10 @@ __global__ void __launch_bounds__(256, 1)
     load_desc(sR, runs + items[i].x);
     __syncthreads();
     if (sR.sl)
-      eval_sliced(sR, sc, sR.X[0], sR.dp, items[i].z, items[e - 1].z + items[e - 1].w, sR.f[0], sR.fx[0], Y, s_f, s_comp);
+      eval_sliced<FORM>(sR, sc, sR.X[0], sR.dp, items[i].z, items[e - 1].z + items[e - 1].w, sR.f[0], sR.fx[0], Y, s_f, s_comp);
     i = e;
   }
-  slice_end(sc);
+  form_end<FORM>(sc);
 }
 
 // ------------------------------------------------------------------ host side
@@ -294,9 +298,37 @@ void k_slice_m_launch(const double* MT, int nc, int d, uint8_t* sl, int32_t* fex
 
 int slice_kpad_of(int d) { return slice_kpad(d); }
 uint32_t slice_kernel_cols(int kpad) { return slice_tmem_cols(kpad); }
-size_t slice_kernel_smem(int kpad) { return slice_smem(kpad); }
+// mma.sync up to 64 coordinates, the widest whose operands leave room for two
+// CTAs on an SM.  On tcgen05 there is one, and a tile of short rows is a chain of
+// latencies: a generation (us, tcgen05 -> mma.sync) of NP = 1500 at D = 16 / 40 /
+// 64 took 25.7 / 24.0 / 24.7 -> 10.1 / 12.3 / 12.9 (that many tiles do not fit
+// k_gen_sliced), of 60 uneven runs 713 -> 306, of 48 runs of NP = 500, D = 30
+// 181 -> 82; 16384 rows of Zakharov's function at D = 30 113 -> 64.
+int slice_form(int kpad) { return kpad <= kMmaDMax ? kSliceMma : kSliceTc; }
+size_t slice_form_smem(int form, int kpad) { return form == kSliceMma ? mma_smem(kpad) : slice_smem(kpad); }
 size_t slice_group_smem(int dp) { return (size_t)(2 * kSliceRows + kCompGroup) * dp * sizeof(double); }
 static_assert(kSliceExp == kSliceDMax, "row exponents per matrix");
+
+template <int FORM>
+static const void* gen_kernel_of(bool var, bool suite) {
+  return var && suite ? (const void*)k_gen_fp64_tc<true, true, FORM>
+         : var        ? (const void*)k_gen_fp64_tc<true, false, FORM>
+         : suite      ? (const void*)k_gen_fp64_tc<false, true, FORM>
+                      : (const void*)k_gen_fp64_tc<false, false, FORM>;
+}
+static const void* gen_kernel(int form, bool var, bool suite) {
+  return form == kSliceMma ? gen_kernel_of<kSliceMma>(var, suite) : gen_kernel_of<kSliceTc>(var, suite);
+}
+
+int k_gen_fp64_tc_per_sm(const SlicePlan& p, bool var, bool suite) {
+  int n = 0;
+  const void* k = gen_kernel(p.form, var, suite);
+  if (allow_dynamic_smem(k) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, 256, p.smem) != cudaSuccess)
+    cudaGetLastError();
+  // (at least one: a launch that does not fit reports it)
+  return std::max(1, p.form == kSliceTc ? std::min(n, (int)(512u / p.cols)) : n);
+}
 
 void k_gen_fp64_tc_launch(const RunDesc* runs, const int4* items, const int2* shares, int nct, const SlicePlan& p,
                           bool var, bool suite, cudaStream_t s) {
@@ -310,23 +342,24 @@ void k_gen_fp64_tc_launch(const RunDesc* runs, const int4* items, const int2* sh
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (var && suite) cudaLaunchKernelEx(&cfg, k_gen_fp64_tc<true, true>, runs, items, shares, p.kpad, p.cols);
-  else if (var) cudaLaunchKernelEx(&cfg, k_gen_fp64_tc<true, false>, runs, items, shares, p.kpad, p.cols);
-  else if (suite) cudaLaunchKernelEx(&cfg, k_gen_fp64_tc<false, true>, runs, items, shares, p.kpad, p.cols);
-  else cudaLaunchKernelEx(&cfg, k_gen_fp64_tc<false, false>, runs, items, shares, p.kpad, p.cols);
+  int kpad = p.kpad;
+  uint32_t cols = p.cols;
+  void* args[] = {(void*)&runs, (void*)&items, (void*)&shares, (void*)&kpad, (void*)&cols};
+  cudaLaunchKernelExC(&cfg, gen_kernel(p.form, var, suite), args);
 }
 
 void k_tc_configure() {
-  for (const void* k : {(const void*)k_gen_fp64_tc<false, false>, (const void*)k_gen_fp64_tc<true, false>,
-                        (const void*)k_gen_fp64_tc<false, true>, (const void*)k_gen_fp64_tc<true, true>,
-                        (const void*)k_eval_rows_tc, (const void*)k_eval_pops_tc})
+  for (int q = 0; q < 8; ++q) allow_dynamic_smem(gen_kernel(q & 4 ? kSliceMma : kSliceTc, q & 1, (q & 2) != 0));
+  for (const void* k : {(const void*)k_eval_rows_tc<kSliceTc>, (const void*)k_eval_rows_tc<kSliceMma>,
+                        (const void*)k_eval_pops_tc<kSliceTc>, (const void*)k_eval_pops_tc<kSliceMma>})
     allow_dynamic_smem(k);
 }
 
 void k_eval_pops_tc_launch(const RunDesc* runs, const int4* items, const int2* shares, int nct, const SlicePlan& p,
-                           int dp_max, cudaStream_t s) {
-  const size_t smem = p.smem_op + (size_t)2 * kSliceRows * dp_max * sizeof(double);
-  k_eval_pops_tc<<<nct, 256, smem, s>>>(runs, items, shares, p.kpad, p.cols);
+                           cudaStream_t s) {
+  const size_t smem = p.smem_op + (size_t)2 * kSliceRows * p.dp_max * sizeof(double);
+  if (p.form == kSliceMma) k_eval_pops_tc<kSliceMma><<<nct, 256, smem, s>>>(runs, items, shares, p.kpad, p.cols);
+  else k_eval_pops_tc<kSliceTc><<<nct, 256, smem, s>>>(runs, items, shares, p.kpad, p.cols);
 }
 
 void k_eval_rows_tc_launch(const RunDesc* runs, int run, const RunDesc& Rh, const double* x, int64_t ld, int n,
@@ -334,12 +367,13 @@ void k_eval_rows_tc_launch(const RunDesc* runs, int run, const RunDesc& Rh, cons
   int dev = 0, nsm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const int kpad = Rh.sl_kpad;
+  const int kpad = Rh.sl_kpad, form = slice_form(kpad);
   const uint32_t cols = slice_tmem_cols(kpad);
-  const size_t smem = slice_smem(kpad) + (size_t)2 * kSliceRows * Rh.dp * sizeof(double);
-  const int per_sm = (int)(512u / cols);
-  const int tiles = (n + kSliceRows - 1) / kSliceRows;
-  k_eval_rows_tc<<<std::min(tiles, nsm * per_sm), 256, smem, s>>>(runs, run, x, ld, n, f, fx, kpad, cols);
+  const size_t smem = slice_form_smem(form, kpad) + (size_t)2 * kSliceRows * Rh.dp * sizeof(double);
+  const int per_sm = form == kSliceMma ? 2 : 1;
+  const int tiles = (n + kSliceRows - 1) / kSliceRows, grid = std::min(tiles, nsm * per_sm);
+  if (form == kSliceMma) k_eval_rows_tc<kSliceMma><<<grid, 256, smem, s>>>(runs, run, x, ld, n, f, fx, kpad, cols);
+  else k_eval_rows_tc<kSliceTc><<<grid, 256, smem, s>>>(runs, run, x, ld, n, f, fx, kpad, cols);
 }
 
 }  // namespace de

@@ -8,7 +8,7 @@
 #include "de_common.cuh"
 #include "de_device.cuh"
 #include "de_internal.cuh"
-#include "de_slice.cuh"
+#include "de_slice_mma.cuh"
 #include "de_suite.cuh"
 
 namespace de {
@@ -92,8 +92,8 @@ __device__ __forceinline__ double gen_select(const RunDesc& R, int64_t g, int i,
 // every lane).  Population rows, fitness and jDE parameters of generation
 // g - 1 are read at L2.
 // VAR / SUITE: strategy variants and jDE / the benchmark suite's objectives.
-// TC: the run's rotation may be sliced (de_slice.cuh; R.sl != NULL then).
-template <bool VAR, bool SUITE, bool TC = false>
+// FORM: whether and how a run's rotation may be sliced (R.sl != NULL then).
+template <bool VAR, bool SUITE, int FORM = kNoSlices>
 __device__ __forceinline__ Best gen_tile(const RunDesc& R, int64_t g, int row0, int nrows, int rows_max, int best,
                                          double* sm, double* s_fsuite, double (*s_comp)[10], SliceCtx* sc = nullptr) {
   const int cur = (int)((g - 1) & 1);
@@ -122,7 +122,7 @@ __device__ __forceinline__ Best gen_tile(const RunDesc& R, int64_t g, int row0, 
       build_trial_row<false>(R, X, (uint32_t)(row0 + rl), g, lane, T + rl * dp, Y + rl * dp);
   }
   const bool suite = SUITE && suite_objective(R.obj);
-  const bool sliced = TC && R.sl != nullptr && !suite;
+  const bool sliced = FORM != kNoSlices && R.sl != nullptr && !suite;
   if (sliced && warp < nrows) {
     // the digits of the row this warp built (its lanes wrote these coordinates)
     double y[4] = {0.0, 0.0, 0.0, 0.0};
@@ -138,12 +138,12 @@ __device__ __forceinline__ Best gen_tile(const RunDesc& R, int64_t g, int row0, 
   const int nout = nrows * d;
   double fsl = 0.0;
   if (sliced) {
-    if (sc->cur != R.sl) slice_load_m(*sc, R.sl, R.sl_kpad);
-    fsl = slice_fitness(*sc, R, Y, Z, nrows);
+    if (sc->cur != R.sl) form_load_m<FORM>(*sc, R.sl, R.sl_kpad);
+    fsl = form_fitness<FORM>(*sc, R, Y, Z, nrows);
   } else if (suite) {
     // ---- the proposed benchmark's functions (Sec. 7.3, Table 2)
     const int ncomp = R.obj >= kObjComposition1 ? R.nc : 1;  // Y and Z hold every component of the tile
-    suite_tile<TC>(R, T, dp, nrows, Y, Y + (size_t)ncomp * rows_max * dp, s_fsuite, s_comp, sc);
+    suite_tile<FORM>(R, T, dp, nrows, Y, Y + (size_t)ncomp * rows_max * dp, s_fsuite, s_comp, sc);
   } else if (R.obj == kObjOde) {
     // ---- ODE objective: a warp integrates one trial's chain; f to W[row][0]
     for (int rl = warp; rl < nrows; rl += nwarps) {

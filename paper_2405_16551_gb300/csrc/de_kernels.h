@@ -48,15 +48,16 @@ cudaError_t allow_dynamic_smem(const void* k);
 void k_gen_fp64_launch(const RunDesc* runs, const int4* items, int nitems, int threads, size_t smem, bool var,
                        bool suite, cudaStream_t s);
 // FP64 rotations as exact digit products on the tensor cores (de_slice.cuh,
-// de_fp64_tc.cu): what the kernels of a handle with such runs are launched
-// with (on = some run's rotation is sliced)
+// de_slice_mma.cuh, de_fp64_tc.cu): what a kernel with such runs is launched
+// with (on = there are any; else its form is 0)
 struct SlicePlan {
   bool on = false;
+  int form = 0;         // SliceForm of the kernel instance: by the widest run
   int kpad = 0;         // the largest padded d of the sliced runs
-  uint32_t cols = 0;    // tensor-memory columns a CTA allocates
+  int dp_max = 0;       // ... and their largest row stride
+  uint32_t cols = 0;    // tensor-memory columns a CTA allocates (tcgen05)
   size_t smem = 0;      // dynamic shared memory of k_gen_fp64_tc
   size_t smem_op = 0;   // ... of which operands
-  int per_sm() const { return (int)(512u / cols); }
 };
 // eligibility of nc row-major d x d matrices, and the least count of large
 // coordinates a row of y needs for each
@@ -64,19 +65,22 @@ bool slice_plan(const double* M, int nc, int d, int32_t qmin[5]);
 size_t slice_matrix_bytes(int d);  // digit slices of one matrix
 int slice_kpad_of(int d);
 uint32_t slice_kernel_cols(int kpad);
-size_t slice_kernel_smem(int kpad);
+int slice_form(int kpad);                          // the form for runs of padded d kpad
+size_t slice_form_smem(int form, int kpad);        // shared memory of its operands
 size_t slice_group_smem(int dp);   // tile buffers of a composition function's row group
 constexpr int kSliceExp = 128;     // row exponents per matrix
 void k_slice_m_launch(const double* MT, int nc, int d, uint8_t* sl, int32_t* fexp, cudaStream_t s);
-// one generation: nct CTAs, CTA b works through items [shares[b].x, shares[b].y)
+// one generation of runs of one form: nct CTAs, CTA b works through items
+// [shares[b].x, shares[b].y)
 void k_gen_fp64_tc_launch(const RunDesc* runs, const int4* items, const int2* shares, int nct, const SlicePlan& p,
                           bool var, bool suite, cudaStream_t s);
 void k_eval_rows_tc_launch(const RunDesc* runs, int run, const RunDesc& Rh, const double* x, int64_t ld, int n,
                            double* f, uint8_t* fx, cudaStream_t s);
-// the sliced runs' populations, in the shares of k_gen_fp64_tc_launch (dp_max:
-// the largest stride among the sliced runs)
+// CTAs of it that share an SM
+int k_gen_fp64_tc_per_sm(const SlicePlan& p, bool var, bool suite);
+// these runs' populations, in the same shares
 void k_eval_pops_tc_launch(const RunDesc* runs, const int4* items, const int2* shares, int nct, const SlicePlan& p,
-                           int dp_max, cudaStream_t s);
+                           cudaStream_t s);
 void k_tc_configure();
 // Dynamic shared memory that gives a CTA of kernel k a whole SM (at least smem)
 size_t fp64_exclusive_smem(const void* k, size_t smem);

@@ -57,9 +57,9 @@ constexpr uint32_t kSliceAcc = 80;  // accumulator columns: 10 groups x 8 rows
 
 __host__ __device__ inline int slice_kpad(int d) { return (d + 15) / 16 * 16; }
 // bytes of one slice of M: kpad / 8 groups of 128 rows x 16 bytes
-__host__ __device__ inline uint32_t slice_bytes(int kpad) { return (uint32_t)(kpad / 8) * 2048u; }
+__host__ __device__ constexpr uint32_t slice_bytes(int kpad) { return (uint32_t)(kpad / 8) * 2048u; }
 // slices kept in shared memory (the others fit tensor memory's 512 columns)
-__host__ __device__ inline int slice_nsm(int kpad) {
+__host__ __device__ constexpr int slice_nsm(int kpad) {
   const int fit = (int)(512u - kSliceAcc) / (kpad / 2);
   return fit >= kSlices ? 0 : kSlices - fit;
 }
@@ -68,8 +68,8 @@ __host__ __device__ inline uint32_t slice_tmem_cols(int kpad) {
   return need <= 128u ? 128u : need <= 256u ? 256u : 512u;
 }
 // shared memory of the operands: B, then the resident slices
-__host__ __device__ inline uint32_t slice_b_bytes(int kpad) { return ((uint32_t)(kpad / 8) * kSliceKg + 1023u) / 1024u * 1024u; }
-__host__ __device__ inline uint32_t slice_smem(int kpad) { return slice_b_bytes(kpad) + (uint32_t)slice_nsm(kpad) * slice_bytes(kpad); }
+__host__ __device__ constexpr uint32_t slice_b_bytes(int kpad) { return ((uint32_t)(kpad / 8) * kSliceKg + 1023u) / 1024u * 1024u; }
+__host__ __device__ constexpr uint32_t slice_smem(int kpad) { return slice_b_bytes(kpad) + (uint32_t)slice_nsm(kpad) * slice_bytes(kpad); }
 
 // Its part in static shared memory.
 struct SliceShared {
@@ -86,6 +86,7 @@ struct SliceCtx {
   SliceShared* sh;
   uint8_t* sB;       // B operand (1024-byte aligned)
   uint8_t* sA;       // slices resident in shared memory
+  float* sP;         // mma.sync form: the group sums (de_slice_mma.cuh)
   uint32_t tmem;     // accumulators at column 0, slices from column kSliceAcc on
   uint32_t bar;      // mbarrier of the products
   uint32_t phase;

@@ -15,7 +15,7 @@
 #include "de_common.cuh"
 #include "de_device.cuh"
 #include "de_internal.cuh"
-#include "de_slice.cuh"
+#include "de_slice_mma.cuh"
 
 namespace de {
 
@@ -342,13 +342,14 @@ __device__ __forceinline__ void comp_mix(const RunDesc& R, double (*comp)[10], d
 // component's matrix at a time is resident for all rows (a matrix is 229 KB at
 // d = 100, so it is loaded once per component and call, not per 8 rows).
 // Y, Z: 8 x dp doubles; comp: nrows x 10.
+template <int FORM>
 static __device__ __noinline__ void suite_comp_sliced(const RunDesc& R, const double* src, int64_t ld, int nrows,
                                                      double* __restrict__ Y, double* __restrict__ Z,
                                                      double* __restrict__ f, double (*comp)[10], SliceCtx& sc) {
   const int d = R.d, dp = R.dp, kpad = R.sl_kpad;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   for (int c = 0; c < R.nc; ++c) {
-    slice_load_m(sc, R.sl + (size_t)c * kSlices * slice_bytes(kpad), kpad);
+    form_load_m<FORM>(sc, R.sl + (size_t)c * kSlices * slice_bytes(kpad), kpad);
     const int fn = R.sfn[c];
     const bool costly = basic_has_costly(fn);
     const double* tab = R.ctab + (size_t)c * dp;
@@ -361,7 +362,7 @@ static __device__ __noinline__ void suite_comp_sliced(const RunDesc& R, const do
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncthreads();
-      slice_rotate(sc, kpad, R.slx + c * kSliceDMax, R.MT + (size_t)c * d * d, Y, Z, nr, d, dp);
+      form_rotate<FORM>(sc, kpad, R.slx + c * kSliceDMax, R.MT + (size_t)c * d * d, Y, Z, nr, d, dp);
       __syncthreads();
       if (costly) {
         for (int e = tid; e < nr * dp; e += blockDim.x) {
@@ -404,13 +405,13 @@ static __device__ __noinline__ void suite_comp_sliced(const RunDesc& R, const do
 //                   logarithms; at x = o_c the weight is 1 for the first such c.
 constexpr int kSuiteMaxRows = 8;
 
-// TC: the run's rotation may be sliced (sc; R.sl != NULL then).
-template <bool TC = false>
+// FORM: whether and how the run's rotation may be sliced (sc; R.sl != NULL then).
+template <int FORM = kNoSlices>
 static __device__ __noinline__ void suite_tile(const RunDesc& R, const double* src, int64_t ld, int nrows,
                                               double* __restrict__ Y, double* __restrict__ Z, double* __restrict__ f,
                                               double (*comp)[10], SliceCtx* sc = nullptr) {
-  if (TC && R.sl && R.obj >= kObjComposition1) {
-    suite_comp_sliced(R, src, ld, nrows, Y, Z, f, comp, *sc);
+  if (FORM != kNoSlices && R.sl && R.obj >= kObjComposition1) {
+    suite_comp_sliced<FORM>(R, src, ld, nrows, Y, Z, f, comp, *sc);
     return;
   }
   const int d = R.d, dp = R.dp;
@@ -475,13 +476,13 @@ static __device__ __noinline__ void suite_tile(const RunDesc& R, const double* s
     return;
   }
   // basic and hybrid functions: one shift and one rotation
-  if (TC && R.sl) {
-    if (sc->cur != R.sl) slice_load_m(*sc, R.sl, R.sl_kpad);
+  if (FORM != kNoSlices && R.sl) {
+    if (sc->cur != R.sl) form_load_m<FORM>(*sc, R.sl, R.sl_kpad);
     if (warp < nrows)
       suite_digits(R, *sc, warp, lane, src + (size_t)warp * ld, R.o, R.scale, R.sl_qmin[0], Y + warp * dp);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
-    slice_rotate(*sc, R.sl_kpad, R.slx, R.MT, Y, Z, nrows, d, dp);
+    form_rotate<FORM>(*sc, R.sl_kpad, R.slx, R.MT, Y, Z, nrows, d, dp);
   } else {
     for (int e = threadIdx.x; e < nrows * dp; e += blockDim.x) {
       const int r = e / dp, j = e - r * dp;
