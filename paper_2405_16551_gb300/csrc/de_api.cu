@@ -53,6 +53,10 @@ struct de_handle {
   // every run is sliced plain DE/rand/1/bin of objectives 0..3: the cooperative
   // launch is k_gen_sliced where its tiles fit (use_sliced; unit: every scale is 1)
   bool sliced_loop = false, use_sliced = false, unit = true;
+  // every run is a sliced composition function of this many components: the
+  // cooperative launch may take a CTA per tile and component (use_split: it does)
+  int comp_split = 0;
+  bool use_split = false;
   size_t smem_loop = 0;
   int nsm = 1;
   int rows = 8;             // rows per tile of the FP64 generation kernel
@@ -390,6 +394,13 @@ static de_status upload_desc(de_handle* h) {
   return DE_OK;
 }
 
+// Tile buffers of the cooperative launch with a CTA per component (T, Y, Z).
+static size_t split_smem(const de_handle* h) {
+  size_t most = 0;
+  for (const auto& R : h->run) most = std::max(most, (size_t)3 * R.rows * R.dp * sizeof(double));
+  return most;
+}
+
 static void drop_graph(de_handle* h) {
   if (h->graph) cudaGraphExecDestroy(h->graph);
   h->graph = nullptr;
@@ -498,8 +509,9 @@ static de_status enqueue_generations(de_handle* h, int64_t n) {
                                        h->smem_loop, h->stream, h->test_grid_skip, h->islands ? h->d_isl : nullptr,
                                        h->islands ? &h->stage : nullptr));
       else
-        DE_CUDA(h, k_gen_fp64_persist_launch(h->d_run, h->d_items, h->nitems, h->nruns, h->threads, h->smem_gen,
-                                             h->variants, h->suite, h->d_ctl64, g, h->stream, h->slices,
+        DE_CUDA(h, k_gen_fp64_persist_launch(h->d_run, h->d_items, h->nitems, h->nruns, h->threads,
+                                             h->use_split ? split_smem(h) : h->smem_gen, h->variants, h->suite,
+                                             h->d_ctl64, g, h->stream, h->slices, h->use_split ? h->comp_split : 0,
                                              h->test_grid_skip,
                                              h->islands ? h->d_isl : nullptr, h->islands ? &h->stage : nullptr));
     }
@@ -681,7 +693,7 @@ static std::string tune_key(const de_handle* h) {
   // (var, form: which of the kernels apply)
   snprintf(b, sizeof b, "gen_fp64v7 runs=%d np0=%d d0=%d obj0=%d rot0=%d sumnp=%lld sumnd=%lld var=%d form=%d", h->nruns,
            h->run[0].np, h->run[0].d, h->run[0].obj, h->run[0].rotate, sum_np, sum_d, h->variants ? 1 : 0,
-           (h->slices.on ? 1 : 0) + (h->sliced_loop ? 2 : 0) + 4 * h->local.csize);
+           (h->slices.on ? 1 : 0) + (h->sliced_loop ? 2 : 0) + 4 * h->local.csize + 64 * h->comp_split);
   return b;
 }
 
@@ -771,6 +783,11 @@ static bool fp64_persist_ok(de_handle* h) {
   if (h->prec != DE_PREC_FP64 || h->surr || (h->islands && h->suite) || !h->d_ctl64 || h->nitems >= 4096) return false;
   if (const char* e = getenv("DE_GB300_FP64_PERSIST"))
     if (e[0] == '0') return false;
+  // a CTA per (tile, component) wherever they all fit
+  h->use_split = h->comp_split > 0 && !h->islands &&
+                 h->nitems * h->comp_split <= k_gen_fp64_persist_capacity(h->threads, split_smem(h), h->variants, h->suite,
+                                                                          h->slices, false);
+  if (h->use_split) return true;
   // (more tiles than SMs: the general loop, two CTAs of which share an SM)
   h->use_sliced = h->sliced_loop && h->nitems <= k_gen_sliced_capacity(h->islands, h->unit, h->slices, h->smem_loop);
   if (h->use_sliced) return true;
@@ -1273,7 +1290,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
     size_t X0, X1, f0, f1, fx0, fx1, o, MT, Mr, sl, slx;
     bool sliced;
     int32_t qmin[5];
-    size_t st, part, T, ref, jF0, jF1, jC0, jC1, perm, ctab;
+    size_t st, part, T, ref, jF0, jF1, jC0, jC1, perm, ctab, cpart;
     size_t dbg_idx, dbg_jrand, dbg_mask, dbg_trial, dbg_ftrial, dbg_accept, dbg_fp64, dbg_cand;
   };
   std::vector<Offs> offs(nruns);
@@ -1318,6 +1335,8 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
         if (sp.kind != 1 && (sp.fn[q] == DE_OBJ_ELLIPTIC || sp.fn[q] == DE_OBJ_GRIEWANK)) O.ctab = 1;
       if (O.ctab) O.ctab = take((size_t)sp.n * ((c.d + 3) / 4 * 4) * sizeof(double));
     }
+    // (only populations whose tiles can all be resident use it)
+    O.cpart = O.sliced && c.objective >= DE_OBJ_COMPOSITION1 && c.np <= 16 * nsm ? take((size_t)c.np * 5 * sizeof(double2)) : 0;
     if (c.debug_capture) {
       const int nw = (c.d + 31) / 32;
       O.dbg_idx = take((size_t)c.np * 3 * sizeof(int32_t));
@@ -1430,6 +1449,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
       }
     }
     if (O.ctab) R.ctab = (const double*)(A + O.ctab);
+    if (O.cpart) R.cpart = (double2*)(A + O.cpart);
     if (c.jde) {
       R.jF[0] = (double*)(A + O.jF0);
       R.jF[1] = (double*)(A + O.jF1);
@@ -1507,6 +1527,9 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
       for (auto& R : h->run) R.sl = nullptr;
     }
     h->sliced_loop = h->slices.on && !h->variants && !h->suite;
+    h->comp_split = h->slices.on && h->run[0].cpart ? h->run[0].nc : 0;
+    for (auto& R : h->run)
+      if (!R.sl || !R.cpart || R.obj < DE_OBJ_COMPOSITION1 || R.nc != h->comp_split) h->comp_split = 0;
     int dp_max = 0;
     for (auto& R : h->run) {
       // the loop's draws are made before the stop decision, which a debug

@@ -317,12 +317,18 @@ constexpr long long kFp64Spin = 1LL << 22;
 // FORM: some run's rotation is sliced (de_slice.cuh, de_slice_mma.cuh); each CTA
 // keeps its run's matrix resident for the whole launch (a composition
 // function's matrices take turns).  kpad, cols: the launch's operand sizes.
+// split > 0 (every run a sliced composition function of that many components,
+// and the device holds that many CTAs per tile): a CTA per (tile, component), with
+// that component's matrix resident, and one more grid barrier before the mix.  One
+// CTA for all of them loaded every matrix again in every generation, one after
+// another (NP = 250, D = 50, four components: 40.7 us a generation, 24.1 this way;
+// the DFMA chain of all components in one CTA 36.3).
 template <bool VAR, bool SUITE, bool ISL, int FORM>
 __global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : FORM == kSliceTc ? 1 : 0) k_gen_fp64_persist(const RunDesc* __restrict__ runs,
                                                           const int4* __restrict__ items, int nruns,
                                                           PersistCtl* ctl, long long gens, int clustered,
                                                           IslandCtl* isl, IslandStage stage, int kpad,
-                                                          uint32_t cols) {
+                                                          uint32_t cols, int split) {
   extern __shared__ __align__(1024) uint8_t smem_p[];
   double* sm = reinterpret_cast<double*>(smem_p + form_smem<FORM>(kpad));
   __shared__ SliceShared s_sl;
@@ -335,13 +341,17 @@ __global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : FORM == kSliceTc 
   __shared__ int s_bi[8];
   __shared__ double s_fsuite[kSuiteMaxRows];
   __shared__ double s_comp[kSuiteMaxRows][10];
-  const int4 it = items[blockIdx.x];
+  constexpr bool kSplit = SUITE && !ISL && FORM != kNoSlices;
+  const bool sp = kSplit && split > 0;
+  const int part = sp ? (int)blockIdx.x % split : 0;
+  const int4 it = items[sp ? (int)blockIdx.x / split : (int)blockIdx.x];
   __shared__ RunDesc sR;
   load_desc(sR, runs + it.x);
   __syncthreads();
   const RunDesc& R = sR;
   RunState* st = R.st;
   const unsigned nct = gridDim.x;
+  const bool first = it.y == 0 && part == 0;  // this CTA publishes the run's state
   const int ntiles = R.ntiles;
   if (threadIdx.x == 0) {
     s_stop = st->stop;
@@ -353,7 +363,7 @@ __global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : FORM == kSliceTc 
     s_done = 0;
     s_below = 0u;
     if (blockIdx.x == 0) ctl->gen0 = s_gen;
-    if (s_stop && it.y == 0 && nruns > 1) atomicAdd(&ctl->stopped[2], 1u);
+    if (s_stop && first && nruns > 1) atomicAdd(&ctl->stopped[2], 1u);
   }
   __syncthreads();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = blockDim.x >> 5;
@@ -412,8 +422,30 @@ __global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : FORM == kSliceTc 
   for (long long itg = 0; itg < gens; ++itg) {
     const bool live = !s_stop;
     const int64_t g = s_gen + 1;
+    if constexpr (kSplit) {
+      if (sp) {
+        if (live) gen_comp_part<VAR, FORM>(R, g, it.z, it.w, R.rows, max(s_best, 0), sm, part, sc);
+        __syncthreads();
+        if (FORM == kSliceTc && s_sl.fail) {
+          // (as below; nobody joins a barrier this CTA has not reached)
+          if (tid == 0) {
+            atomicExch(&ctl->abort, 1);
+            atomicOr(&st->err, kErrTimeout);
+          }
+          break;
+        }
+        full_sync();
+        if (s_abort) break;
+      }
+    }
     if (live) {
-      Best bb = gen_tile<VAR, SUITE, FORM>(R, g, it.z, it.w, R.rows, max(s_best, 0), sm, s_fsuite, s_comp, &sc);
+      Best bb;
+      bb.init();
+      if (!sp) {
+        bb = gen_tile<VAR, SUITE, FORM>(R, g, it.z, it.w, R.rows, max(s_best, 0), sm, s_fsuite, s_comp, &sc);
+      } else if (part == 0) {
+        if constexpr (kSplit) bb = gen_comp_finish<VAR>(R, g, it.z, it.w, sm, s_fsuite, s_comp);
+      }
       if (lane == 0) { s_bf[warp] = bb.f; s_bk[warp] = bb.k; s_bi[warp] = bb.i; }
       __syncthreads();
       if (FORM == kSliceTc && tid == 0 && s_sl.fail) {
@@ -426,7 +458,7 @@ __global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : FORM == kSliceTc 
         if (clustered)
           for (unsigned q = 0; q < nct; ++q) *cg::this_cluster().map_shared_rank(&s_abort, q) = 1;
       }
-      if (tid == 0) {
+      if (tid == 0 && part == 0) {
         bb.init();
         for (int w = 0; w < nwarps; ++w) bb.take(s_bf[w], s_bk[w], s_bi[w]);
         BestPartial* pp = R.part + (size_t)(g & 1) * ntiles + it.y;
@@ -493,7 +525,7 @@ __global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : FORM == kSliceTc 
         s_evals = evals;
         s_stop = stop;
         s_gen = g;
-        if (it.y == 0) {
+        if (first) {
           if (have) {
             st->best_f = b.f;
             st->best_idx = b.i;
@@ -616,7 +648,7 @@ void k_configure() {
 
 cudaError_t k_gen_fp64_persist_launch(const RunDesc* runs, const int4* items, int nitems, int nruns, int threads,
                                       size_t smem, bool var, bool suite, PersistCtl* ctl, long long gens,
-                                      cudaStream_t s, const SlicePlan& sp, int test_skip, IslandCtl* isl,
+                                      cudaStream_t s, const SlicePlan& sp, int split, int test_skip, IslandCtl* isl,
                                       const IslandStage* stage) {
   cudaError_t e = persist_ctl_reset(ctl, test_skip, s);
   if (e != cudaSuccess) return e;
@@ -625,8 +657,8 @@ cudaError_t k_gen_fp64_persist_launch(const RunDesc* runs, const int4* items, in
   IslandStage st{};
   if (stage) st = *stage;
   void* args[] = {(void*)&runs, (void*)&items, (void*)&nruns, (void*)&ctl, (void*)&gens, (void*)&clustered,
-                  (void*)&isl, (void*)&st, (void*)&kpad, (void*)&cols};
-  const dim3 grid((unsigned)nitems), block((unsigned)threads);
+                  (void*)&isl, (void*)&st, (void*)&kpad, (void*)&cols, (void*)&split};
+  const dim3 grid((unsigned)(nitems * std::max(1, split))), block((unsigned)threads);
   if (isl && suite) return cudaErrorInvalidValue;  // islands of the suite's objectives run generation by generation
   const void* k = persist_kernel(var, suite, isl != nullptr, sp.form);
   return cudaLaunchCooperativeKernel(k, grid, block, args, persist_smem(k, smem, sp), s);
@@ -656,12 +688,12 @@ cudaError_t k_gen_fp64_cluster_launch(const RunDesc* runs, const int4* items, in
   cudaLaunchAttribute attr[1];
   const void* k = persist_kernel(var, suite, false, sp.form);
   cudaLaunchConfig_t cfg = cluster_config(nitems, threads, persist_smem(k, smem, sp), s, attr);
-  int nruns = 1, clustered = 1, kpad = sp.kpad;
+  int nruns = 1, clustered = 1, kpad = sp.kpad, split = 0;
   uint32_t cols = sp.cols;
   IslandCtl* isl = nullptr;
   IslandStage stage{};
   void* args[] = {(void*)&runs, (void*)&items, (void*)&nruns, (void*)&ctl, (void*)&gens, (void*)&clustered,
-                  (void*)&isl, (void*)&stage, (void*)&kpad, (void*)&cols};
+                  (void*)&isl, (void*)&stage, (void*)&kpad, (void*)&cols, (void*)&split};
   return cudaLaunchKernelExC(&cfg, k, args);
 }
 

@@ -157,20 +157,21 @@ __global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : 1)
 }
 
 // f of rows r0 .. r1 - 1 of x (row stride ld) with a sliced run; a warp per row
-// of the 8-row tiles.  Y, Z: 8 x dp doubles.
+// of the 8-row tiles.  Y, Z: 8 x dp doubles, ncomp times that (a composition
+// function's, when the rows are at most 8).
 template <int FORM>
 __device__ __forceinline__ void eval_sliced(const RunDesc& R, SliceCtx& sc, const double* __restrict__ x, int64_t ld,
                                             int r0, int r1, double* __restrict__ fout, uint8_t* __restrict__ fx_out,
-                                            double* Y, double* s_f, double (*s_comp)[10]) {
+                                            double* Y, double* s_f, double (*s_comp)[10], int ncomp) {
   const int d = R.d, dp = R.dp, obj = R.obj, kpad = R.sl_kpad;
-  double* Z = Y + kSliceRows * dp;
+  double* Z = Y + ncomp * kSliceRows * dp;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool suite = suite_objective(obj);
   const int step = suite && obj >= kObjComposition1 ? kCompGroup : kSliceRows;
   for (int row0 = r0; row0 < r1; row0 += step) {
     const int nr = min(step, r1 - row0);
     if (suite) {
-      suite_tile<FORM>(R, x + (size_t)row0 * ld, ld, nr, Y, Z, s_f, s_comp, &sc);
+      suite_tile<FORM>(R, x + (size_t)row0 * ld, ld, nr, Y, Z, s_f, s_comp, &sc, ncomp == 1);
       for (int r = threadIdx.x; r < nr; r += blockDim.x) {
         fout[row0 + r] = s_f[r];
         if (fx_out) fx_out[row0 + r] = 1;
@@ -214,7 +215,7 @@ __device__ __forceinline__ void eval_sliced(const RunDesc& R, SliceCtx& sc, cons
 template <int FORM>
 __global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : 1)
     k_eval_rows_tc(const RunDesc* __restrict__ runs, int run, const double* __restrict__ x, int64_t ld, int n,
-                   double* __restrict__ fout, uint8_t* __restrict__ fx_out, int kpad, uint32_t cols) {
+                   double* __restrict__ fout, uint8_t* __restrict__ fx_out, int kpad, uint32_t cols, int ncomp) {
   extern __shared__ __align__(1024) uint8_t smem_tc[];
   __shared__ SliceShared s_sl;
   __shared__ RunDesc sR;
@@ -227,7 +228,7 @@ __global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : 1)
   const int tiles = (n + kSliceRows - 1) / kSliceRows;
   const int r0 = (int)((long long)tiles * blockIdx.x / gridDim.x) * kSliceRows;
   const int r1 = min(n, (int)((long long)tiles * (blockIdx.x + 1) / gridDim.x) * kSliceRows);
-  eval_sliced<FORM>(sR, sc, x, ld, r0, r1, fout, fx_out, Y, s_f, s_comp);
+  eval_sliced<FORM>(sR, sc, x, ld, r0, r1, fout, fx_out, Y, s_f, s_comp, ncomp);
   form_end<FORM>(sc);
 }
 
@@ -252,7 +253,7 @@ __global__ void __launch_bounds__(256, FORM == kSliceMma ? 2 : 1)
     load_desc(sR, runs + items[i].x);
     __syncthreads();
     if (sR.sl)
-      eval_sliced<FORM>(sR, sc, sR.X[0], sR.dp, items[i].z, items[e - 1].z + items[e - 1].w, sR.f[0], sR.fx[0], Y, s_f, s_comp);
+      eval_sliced<FORM>(sR, sc, sR.X[0], sR.dp, items[i].z, items[e - 1].z + items[e - 1].w, sR.f[0], sR.fx[0], Y, s_f, s_comp, 1);
     i = e;
   }
   form_end<FORM>(sc);
@@ -369,11 +370,14 @@ void k_eval_rows_tc_launch(const RunDesc* runs, int run, const RunDesc& Rh, cons
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int kpad = Rh.sl_kpad, form = slice_form(kpad);
   const uint32_t cols = slice_tmem_cols(kpad);
-  const size_t smem = slice_form_smem(form, kpad) + (size_t)2 * kSliceRows * Rh.dp * sizeof(double);
   const int per_sm = form == kSliceMma ? 2 : 1;
   const int tiles = (n + kSliceRows - 1) / kSliceRows, grid = std::min(tiles, nsm * per_sm);
-  if (form == kSliceMma) k_eval_rows_tc<kSliceMma><<<grid, 256, smem, s>>>(runs, run, x, ld, n, f, fx, kpad, cols);
-  else k_eval_rows_tc<kSliceTc><<<grid, 256, smem, s>>>(runs, run, x, ld, n, f, fx, kpad, cols);
+  // a composition function's components side by side where no CTA has a second
+  // tile (on tcgen05 the loads of the matrices are the longer part: no gain)
+  const int ncomp = form == kSliceMma && tiles <= grid ? suite_comps(Rh) : 1;
+  const size_t smem = slice_form_smem(form, kpad) + (size_t)2 * ncomp * kSliceRows * Rh.dp * sizeof(double);
+  if (form == kSliceMma) k_eval_rows_tc<kSliceMma><<<grid, 256, smem, s>>>(runs, run, x, ld, n, f, fx, kpad, cols, ncomp);
+  else k_eval_rows_tc<kSliceTc><<<grid, 256, smem, s>>>(runs, run, x, ld, n, f, fx, kpad, cols, ncomp);
 }
 
 }  // namespace de

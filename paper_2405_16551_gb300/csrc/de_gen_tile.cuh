@@ -83,29 +83,14 @@ __device__ __forceinline__ double gen_select(const RunDesc& R, int64_t g, int i,
   return fnew;
 }
 
-// One tile of generation g: the trials of targets row0 .. row0 + nrows - 1
-// (a warp per target), their fitness, and greedy selection into the other
-// population buffer.  Shared memory sm: T (trials), Y (shifted trials), Z
-// (rotated), W (second term sum of Ackley), each rows_max x dp doubles.
-// best: the current population's best row (DE/best/1).  Returns the calling
-// warp's best (f, index) over the tile's new population rows (the same in
-// every lane).  Population rows, fitness and jDE parameters of generation
-// g - 1 are read at L2.
-// VAR / SUITE: strategy variants and jDE / the benchmark suite's objectives.
-// FORM: whether and how a run's rotation may be sliced (R.sl != NULL then).
-template <bool VAR, bool SUITE, int FORM = kNoSlices>
-__device__ __forceinline__ Best gen_tile(const RunDesc& R, int64_t g, int row0, int nrows, int rows_max, int best,
-                                         double* sm, double* s_fsuite, double (*s_comp)[10], SliceCtx* sc = nullptr) {
-  const int cur = (int)((g - 1) & 1);
+// The trials of targets row0 .. row0 + nrows - 1 (a warp per target) into T, their
+// shifted rows into Y.
+template <bool VAR>
+__device__ __forceinline__ void gen_trials(const RunDesc& R, int64_t g, int row0, int nrows, int best, double* T,
+                                           double* Y) {
+  const int cur = (int)((g - 1) & 1), dp = R.dp;
   const double* X = R.X[cur];
-  const int d = R.d, dp = R.dp;
-  double* T = sm;
-  double* Y = T + rows_max * dp;
-  double* Z = Y + rows_max * dp;
-  double* W = Z + rows_max * dp;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = blockDim.x >> 5;
-
-  // ---- trials (a warp per target)
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   const bool var = VAR && (R.strategy != 0 || R.jde);
   const double* jFc = VAR && R.jde ? R.jF[cur] : nullptr;
   const double* jCRc = VAR && R.jde ? R.jCR[cur] : nullptr;
@@ -121,16 +106,52 @@ __device__ __forceinline__ Best gen_tile(const RunDesc& R, int64_t g, int row0, 
     for (int rl = warp; rl < nrows; rl += nwarps)
       build_trial_row<false>(R, X, (uint32_t)(row0 + rl), g, lane, T + rl * dp, Y + rl * dp);
   }
+}
+
+// One tile of generation g: the trials of targets row0 .. row0 + nrows - 1
+// (a warp per target), their fitness, and greedy selection into the other
+// population buffer.  Shared memory sm: T (trials), Y (shifted trials), Z
+// (rotated), W (second term sum of Ackley), each rows_max x dp doubles.
+// best: the current population's best row (DE/best/1).  Returns the calling
+// warp's best (f, index) over the tile's new population rows (the same in
+// every lane).  Population rows, fitness and jDE parameters of generation
+// g - 1 are read at L2.
+// VAR / SUITE: strategy variants and jDE / the benchmark suite's objectives.
+// FORM: whether and how a run's rotation may be sliced (R.sl != NULL then).
+template <bool VAR, bool SUITE, int FORM = kNoSlices>
+__device__ __forceinline__ Best gen_tile(const RunDesc& R, int64_t g, int row0, int nrows, int rows_max, int best,
+                                         double* sm, double* s_fsuite, double (*s_comp)[10], SliceCtx* sc = nullptr) {
+  const int d = R.d, dp = R.dp;
+  double* T = sm;
+  double* Y = T + rows_max * dp;
+  double* Z = Y + rows_max * dp;
+  double* W = Z + rows_max * dp;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = blockDim.x >> 5;
+
+  gen_trials<VAR>(R, g, row0, nrows, best, T, Y);
   const bool suite = SUITE && suite_objective(R.obj);
   const bool sliced = FORM != kNoSlices && R.sl != nullptr && !suite;
   if (sliced && warp < nrows) {
-    // the digits of the row this warp built (its lanes wrote these coordinates)
-    double y[4] = {0.0, 0.0, 0.0, 0.0};
-    if (4 * lane < d) {
+    // the digits of the row this warp built, as few coordinates a lane as the
+    // width allows
+    const double* yr = Y + warp * dp;
+    if (FORM == kSliceMma && R.sl_kpad <= 32) {
+      __syncwarp();
+      const double y[1] = {lane < d ? yr[lane] : 0.0};
+      slice_digits(*sc, warp, lane, R.sl_kpad, R.sl_qmin[0], y);
+    } else if (FORM == kSliceMma) {
+      __syncwarp();
+      const double y[2] = {2 * lane < d ? yr[2 * lane] : 0.0, 2 * lane + 1 < d ? yr[2 * lane + 1] : 0.0};
+      slice_digits(*sc, warp, lane, R.sl_kpad, R.sl_qmin[0], y);
+    } else {
+      // (its lanes wrote these coordinates)
+      double y[4] = {0.0, 0.0, 0.0, 0.0};
+      if (4 * lane < d) {
 #pragma unroll
-      for (int m = 0; m < 4; ++m) y[m] = Y[warp * dp + 4 * lane + m];
+        for (int m = 0; m < 4; ++m) y[m] = yr[4 * lane + m];
+      }
+      slice_digits(*sc, warp, lane, R.sl_kpad, R.sl_qmin[0], y);
     }
-    slice_digits(*sc, warp, lane, R.sl_kpad, R.sl_qmin[0], y);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
@@ -224,6 +245,36 @@ __device__ __forceinline__ Best gen_tile(const RunDesc& R, int64_t g, int row0, 
     const double fnew = gen_select<VAR>(R, g, i, ft, T + rl * dp, lane);
     bb.offer(fnew, i);
   }
+  return bb;
+}
+
+// The tile of a composition function whose components run on CTAs of their own,
+// in two steps with a barrier of all of them between: component c's part, and
+// (one of the CTAs) the mix and the selection from all parts.  sm: T, Y, Z.
+template <bool VAR, int FORM>
+__device__ __forceinline__ void gen_comp_part(const RunDesc& R, int64_t g, int row0, int nrows, int rows_max, int best,
+                                              double* sm, int c, SliceCtx& sc) {
+  double* Y = sm + rows_max * R.dp;
+  gen_trials<VAR>(R, g, row0, nrows, best, sm, Y);
+  __syncthreads();
+  suite_comp_part<FORM>(R, sm, R.dp, row0, nrows, Y, Y + rows_max * R.dp, c, sc);
+}
+template <bool VAR>
+__device__ __forceinline__ Best gen_comp_finish(const RunDesc& R, int64_t g, int row0, int nrows, const double* T,
+                                                double* s_f, double (*s_comp)[10]) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  for (int e = threadIdx.x; e < nrows * R.nc; e += blockDim.x) {
+    const int r = e / R.nc, c = e - r * R.nc;
+    const double2 v = __ldcg(R.cpart + (size_t)(row0 + r) * 5 + c);
+    s_comp[r][c] = v.x;
+    s_comp[r][5 + c] = v.y;
+  }
+  __syncthreads();
+  comp_mix(R, s_comp, s_f, nrows);
+  Best bb;
+  bb.init();
+  for (int r = warp; r < nrows; r += nwarps)
+    bb.offer(gen_select<VAR>(R, g, row0 + r, s_f[r], T + r * R.dp, lane), row0 + r);
   return bb;
 }
 

@@ -86,6 +86,7 @@ struct RunDesc {
   // composition functions and basic ones that need it, dp per component:
   // Elliptic's weights, Griewank's 1 / (2 pi sqrt(i)) (k_suite_table)
   const double* ctab;
+  double2* cpart;  // composition functions whose components run on CTAs of their own: (g_c, D_c), 5 a row
   // buffers
   double* X[2];
   double* f[2];

@@ -108,6 +108,8 @@ cudaError_t k_gen_local_launch(const RunDesc* runs, int nruns, const LocalPlan& 
                                cudaStream_t s, int test_skip, IslandCtl* isl, const IslandStage* stage);
 // the generation loop of FP64 runs in one cooperative launch (every item
 // co-resident: nitems <= k_gen_fp64_persist_capacity; gens <= 2^20)
+// split > 0: a CTA per tile and component of a composition function (that many
+// components; nitems * split co-resident CTAs)
 // test_skip > 0: the grid-barrier failure test (PersistCtl::test_skip)
 // isl (NULL without islands): the runs are islands (de_init_islands_ex) whose
 // migrations and common stop run inside the launch
@@ -115,8 +117,8 @@ struct IslandCtl;
 struct IslandStage;
 cudaError_t k_gen_fp64_persist_launch(const RunDesc* runs, const int4* items, int nitems, int nruns, int threads,
                                       size_t smem, bool var, bool suite, PersistCtl* ctl, long long gens,
-                                      cudaStream_t s, const SlicePlan& sp, int test_skip = 0, IslandCtl* isl = nullptr,
-                                      const IslandStage* stage = nullptr);
+                                      cudaStream_t s, const SlicePlan& sp, int split = 0, int test_skip = 0,
+                                      IslandCtl* isl = nullptr, const IslandStage* stage = nullptr);
 // CTAs of the cooperative FP64 kernel that fit at once (isl: the island instance)
 int k_gen_fp64_persist_capacity(int threads, size_t smem, bool var, bool suite, const SlicePlan& sp, bool isl = false);
 // the same loop as one thread-block cluster of nitems CTAs (one run,

@@ -119,10 +119,9 @@ __device__ __forceinline__ bool basic_has_costly(int fn) {
 // i = l + 1; E[l] holds basic_costly of coordinate l, tab the constants.  Called
 // by a whole warp: lane k sums the terms of l = k, k + 32, ... in order, then a
 // fixed xor tree; every lane gets them.
-static __device__ __noinline__ double2 basic_sums_warp(int fn, const double* __restrict__ z,
-                                                       const int32_t* __restrict__ idx, int base, int n, double sc,
-                                                       const double* __restrict__ E, const double* __restrict__ tab,
-                                                       int lane) {
+__device__ __forceinline__ double2 basic_sums(int fn, const double* __restrict__ z,
+                                               const int32_t* __restrict__ idx, int base, int n, double sc,
+                                               const double* __restrict__ E, const double* __restrict__ tab, int lane) {
   auto W = [&](int l) { return sc * z[idx ? idx[base + l] : base + l]; };
   double s1 = 0.0, s2 = 0.0, p = 1.0;
   for (int l = lane; l < n; l += 32) {
@@ -179,7 +178,7 @@ static __device__ __noinline__ double2 basic_sums_warp(int fn, const double* __r
 }
 
 // g of basic function fn on n coordinates from its sums.
-static __device__ __noinline__ double basic_finish(int fn, double s1, double s2, int n) {
+__device__ __forceinline__ double basic_value(int fn, double s1, double s2, int n) {
   switch (fn) {
     case kObjAckley: {
       return 20.0 + 2.718281828459045 - 20.0 * exp(-0.2 * sqrt(s1 / n)) - exp(s2 / n);
@@ -208,10 +207,17 @@ static __device__ __noinline__ double basic_finish(int fn, double s1, double s2,
   }
 }
 
-__device__ __forceinline__ double basic_fn_warp(int fn, const double* z, const int32_t* idx, int base, int n, double sc,
-                                                const double* E, const double* tab, int lane) {
-  const double2 s = basic_sums_warp(fn, z, idx, base, n, sc, E, tab, lane);
-  return basic_finish(fn, s.x, s.y, n);
+static __device__ __noinline__ double2 basic_sums_warp(int fn, const double* z, int n, const double* E,
+                                                       const double* tab, int lane) {
+  return basic_sums(fn, z, nullptr, 0, n, 1.0, E, tab, lane);
+}
+static __device__ __noinline__ double basic_finish(int fn, double s1, double s2, int n) {
+  return basic_value(fn, s1, s2, n);
+}
+static __device__ __noinline__ double basic_fn_warp(int fn, const double* z, const int32_t* idx, int base, int n,
+                                                    double sc, const double* E, const double* tab, int lane) {
+  const double2 s = basic_sums(fn, z, idx, base, n, sc, E, tab, lane);
+  return basic_value(fn, s.x, s.y, n);
 }
 
 // Rotation of the tile's nrows rows with a given transposed matrix: thread
@@ -273,27 +279,38 @@ __device__ __forceinline__ void comp_rotate(const double* __restrict__ MT, const
 }
 
 // y = (x - o) s of tile row r (one warp; src: the row of x), stored as FP64
-// row Yr and as digits of the sliced rotation; returns |x - o|^2 (every lane).
-__device__ __forceinline__ double suite_digits(const RunDesc& R, const SliceCtx& c, int r, int lane, const double* src,
-                                               const double* __restrict__ o, double sc, int qmin,
-                                               double* __restrict__ Yr) {
-  double y[4] = {0.0, 0.0, 0.0, 0.0};
+// row Yr and as digits of the sliced rotation, N coordinates a lane.  DIST: returns
+// |x - o|^2 (every lane).
+template <int N, bool DIST>
+__device__ __forceinline__ double suite_digits_of(const RunDesc& R, const SliceCtx& c, int r, int lane, const double* src,
+                                                  const double* __restrict__ o, double sc, int qmin,
+                                                  double* __restrict__ Yr) {
+  double y[N] = {};
   double dd = 0.0;
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    const int j = 4 * lane + m;
+  for (int m = 0; m < N; ++m) {
+    const int j = N * lane + m;
     if (j < R.d) {
       const double t = __dsub_rn(src[j], o[j]);
-      dd += t * t;
+      if (DIST) dd += t * t;
       y[m] = __dmul_rn(t, sc);
     }
   }
-  if (4 * lane < R.dp) {
-    *reinterpret_cast<double2*>(Yr + 4 * lane) = make_double2(y[0], y[1]);
-    *reinterpret_cast<double2*>(Yr + 4 * lane + 2) = make_double2(y[2], y[3]);
-  }
+  if (N * lane < R.dp) st_coords(Yr + N * lane, y);
   slice_digits(c, r, lane, R.sl_kpad, qmin, y);
-  return warp_sum(dd);
+  return DIST ? warp_sum(dd) : 0.0;
+}
+
+// As few coordinates a lane as the width allows (an FP64 instruction costs the
+// same however few lanes are active), the same in every form: the order of the
+// distance's sum depends on it.
+template <int FORM, bool DIST>
+__device__ __forceinline__ double suite_digits(const RunDesc& R, const SliceCtx& c, int r, int lane, const double* src,
+                                               const double* __restrict__ o, double sc, int qmin,
+                                               double* __restrict__ Yr) {
+  if (R.sl_kpad <= 32) return suite_digits_of<1, DIST>(R, c, r, lane, src, o, sc, qmin, Yr);
+  if (FORM == kSliceMma || R.sl_kpad <= 64) return suite_digits_of<2, DIST>(R, c, r, lane, src, o, sc, qmin, Yr);
+  return suite_digits_of<4, DIST>(R, c, r, lane, src, o, sc, qmin, Yr);
 }
 
 // f[r] of nrows rows of a composition function from g_c (comp[r][0..4]) and
@@ -356,7 +373,7 @@ static __device__ __noinline__ void suite_comp_sliced(const RunDesc& R, const do
     for (int t0 = 0; t0 < nrows; t0 += kSliceRows) {
       const int nr = min(kSliceRows, nrows - t0);
       if (warp < nr) {
-        const double dd = suite_digits(R, sc, warp, lane, src + (size_t)(t0 + warp) * ld, R.o + (size_t)c * dp,
+        const double dd = suite_digits<FORM, true>(R, sc, warp, lane, src + (size_t)(t0 + warp) * ld, R.o + (size_t)c * dp,
                                        R.sscale[c], R.sl_qmin[c], Y + warp * dp);
         if (lane == 0) comp[t0 + warp][5 + c] = dd;
       }
@@ -374,7 +391,7 @@ static __device__ __noinline__ void suite_comp_sliced(const RunDesc& R, const do
         __syncthreads();
       }
       if (warp < nr) {
-        const double2 g = basic_sums_warp(fn, Z + warp * dp, nullptr, 0, d, 1.0, Y + warp * dp, tab, lane);
+        const double2 g = basic_sums_warp(fn, Z + warp * dp, d, Y + warp * dp, tab, lane);
         if (lane == 0) {
           comp[t0 + warp][c] = g.x;
           f[t0 + warp] = g.y;  // until the component is finished
@@ -388,6 +405,90 @@ static __device__ __noinline__ void suite_comp_sliced(const RunDesc& R, const do
   }
   __syncthreads();
   comp_mix(R, comp, f, nrows);
+}
+
+// The same for a tile of at most 8 rows with buffers of every component (Y, Z: nc
+// x nrows x dp doubles): the components' products one after another, all the
+// rest, which is the longer part, once for every (component, row).  With a
+// component's terms, sums and roots between two products a tile was that chain nc
+// times (NP = 50, D = 20, three components: 31.3 us a generation, 26.9 this way).
+template <int FORM>
+static __device__ __noinline__ void suite_comp_tile(const RunDesc& R, const double* src, int64_t ld, int nrows,
+                                                   double* __restrict__ Y, double* __restrict__ Z,
+                                                   double* __restrict__ f, double (*comp)[10], SliceCtx& sc) {
+  const int d = R.d, dp = R.dp, kpad = R.sl_kpad, nc = R.nc, blk = nrows * dp;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  for (int c = 0; c < nc; ++c) {
+    form_load_m<FORM>(sc, R.sl + (size_t)c * kSlices * slice_bytes(kpad), kpad);
+    if (warp < nrows) {
+      const double dd = suite_digits<FORM, true>(R, sc, warp, lane, src + (size_t)warp * ld, R.o + (size_t)c * dp,
+                                                 R.sscale[c], R.sl_qmin[c], Y + (size_t)c * blk + warp * dp);
+      if (lane == 0) comp[warp][5 + c] = dd;
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    form_rotate<FORM>(sc, kpad, R.slx + c * kSliceDMax, R.MT + (size_t)c * d * d, Y + (size_t)c * blk,
+                      Z + (size_t)c * blk, nrows, d, dp);
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nc * blk; e += blockDim.x) {
+    const int c = e / blk, rem = e - c * blk, r = rem / dp, j = rem - r * dp;
+    if (j >= d || !basic_has_costly(R.sfn[c])) continue;
+    const double* zr = Z + (size_t)c * blk + r * dp;
+    Y[e] = basic_costly(R.sfn[c], zr[j], zr[j + 1 < d ? j + 1 : 0], j, d, R.skex[c], R.ctab + (size_t)c * dp);
+  }
+  __syncthreads();
+  for (int p = warp; p < nc * nrows; p += nwarps) {
+    const int c = p / nrows, r = p - c * nrows;
+    double* E = Y + (size_t)c * blk + r * dp;
+    const double2 g = basic_sums_warp(R.sfn[c], Z + (size_t)c * blk + r * dp, d, E, R.ctab + (size_t)c * dp, lane);
+    __syncwarp();  // E has been read
+    if (lane == 0) {
+      comp[r][c] = g.x;
+      E[0] = g.y;  // until the component is finished
+    }
+  }
+  __syncthreads();
+  for (int p = threadIdx.x; p < nc * nrows; p += blockDim.x) {
+    const int c = p / nrows, r = p - c * nrows;
+    comp[r][c] = basic_finish(R.sfn[c], comp[r][c], Y[(size_t)c * blk + r * dp], d);
+  }
+  __syncthreads();
+  comp_mix(R, comp, f, nrows);
+}
+
+// One component's part of a tile, for a CTA that holds component c's matrix:
+// g_c and D_c of row row0 + r to R.cpart.  Y, Z: nrows x dp doubles.
+template <int FORM>
+static __device__ __noinline__ void suite_comp_part(const RunDesc& R, const double* src, int64_t ld, int row0, int nrows,
+                                                   double* __restrict__ Y, double* __restrict__ Z, int c, SliceCtx& sc) {
+  const int d = R.d, dp = R.dp, kpad = R.sl_kpad, fn = R.sfn[c];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint8_t* sl = R.sl + (size_t)c * kSlices * slice_bytes(kpad);
+  const double* tab = R.ctab + (size_t)c * dp;
+  if (sc.cur != sl) form_load_m<FORM>(sc, sl, kpad);
+  double dd = 0.0;
+  if (warp < nrows)
+    dd = suite_digits<FORM, true>(R, sc, warp, lane, src + (size_t)warp * ld, R.o + (size_t)c * dp, R.sscale[c],
+                                  R.sl_qmin[c], Y + warp * dp);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncthreads();
+  form_rotate<FORM>(sc, kpad, R.slx + c * kSliceDMax, R.MT + (size_t)c * d * d, Y, Z, nrows, d, dp);
+  __syncthreads();
+  if (basic_has_costly(fn)) {
+    for (int e = threadIdx.x; e < nrows * dp; e += blockDim.x) {
+      const int r = e / dp, j = e - r * dp;
+      if (j >= d) continue;
+      const double* zr = Z + r * dp;
+      Y[e] = basic_costly(fn, zr[j], zr[j + 1 < d ? j + 1 : 0], j, d, R.skex[c], tab);
+    }
+    __syncthreads();
+  }
+  if (warp < nrows) {
+    const double2 g = basic_sums_warp(fn, Z + warp * dp, d, Y + warp * dp, tab, lane);
+    const double v = basic_finish(fn, g.x, g.y, d);
+    if (lane == 0) R.cpart[(size_t)(row0 + warp) * 5 + c] = make_double2(v, dd);
+  }
 }
 
 // Objective of the suite for nrows rows of src (row stride ld, in shared or
@@ -405,13 +506,16 @@ static __device__ __noinline__ void suite_comp_sliced(const RunDesc& R, const do
 //                   logarithms; at x = o_c the weight is 1 for the first such c.
 constexpr int kSuiteMaxRows = 8;
 
-// FORM: whether and how the run's rotation may be sliced (sc; R.sl != NULL then).
+// FORM: whether and how the run's rotation may be sliced (sc; R.sl != NULL then:
+// for a composition function Y and Z may be 8 x dp doubles, and nrows more than 8,
+// when one says so).
 template <int FORM = kNoSlices>
 static __device__ __noinline__ void suite_tile(const RunDesc& R, const double* src, int64_t ld, int nrows,
                                               double* __restrict__ Y, double* __restrict__ Z, double* __restrict__ f,
-                                              double (*comp)[10], SliceCtx* sc = nullptr) {
+                                              double (*comp)[10], SliceCtx* sc = nullptr, bool one = false) {
   if (FORM != kNoSlices && R.sl && R.obj >= kObjComposition1) {
-    suite_comp_sliced<FORM>(R, src, ld, nrows, Y, Z, f, comp, *sc);
+    if (one) suite_comp_sliced<FORM>(R, src, ld, nrows, Y, Z, f, comp, *sc);
+    else suite_comp_tile<FORM>(R, src, ld, nrows, Y, Z, f, comp, *sc);
     return;
   }
   const int d = R.d, dp = R.dp;
@@ -479,7 +583,7 @@ static __device__ __noinline__ void suite_tile(const RunDesc& R, const double* s
   if (FORM != kNoSlices && R.sl) {
     if (sc->cur != R.sl) form_load_m<FORM>(*sc, R.sl, R.sl_kpad);
     if (warp < nrows)
-      suite_digits(R, *sc, warp, lane, src + (size_t)warp * ld, R.o, R.scale, R.sl_qmin[0], Y + warp * dp);
+      suite_digits<FORM, false>(R, *sc, warp, lane, src + (size_t)warp * ld, R.o, R.scale, R.sl_qmin[0], Y + warp * dp);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     form_rotate<FORM>(*sc, R.sl_kpad, R.slx, R.MT, Y, Z, nrows, d, dp);
