@@ -588,6 +588,14 @@ static de_status read_states(de_handle* h) {
 // captured one.
 static de_status need_states(de_handle* h) { return h->state_fresh && !h->captured ? DE_OK : read_states(h); }
 
+// The end of a call that changes states and returns when it is done: islands are
+// looked at again (whether they still agree).
+static de_status finish_change(de_handle* h) {
+  if (h->islands) return read_states(h);
+  DE_CUDA(h, cudaStreamSynchronize(h->stream));
+  return DE_OK;
+}
+
 static de_status check_device_errors(de_handle* h) {
   for (int r = 0; r < h->nruns; ++r) {
     if (h->h_state[r].err & kErrTimeout) return fail(h, DE_ERR_TIMEOUT, "a device-side wait timed out (run " + std::to_string(r) + ")");
@@ -1548,7 +1556,7 @@ de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_stream,
   for (auto& R : h->run) R.dbuf = h->dbuf ? 1 : 0;
   TRY(build_items(h));
   TRY(upload_desc(h));
-  k_configure();
+  k_configure(h->prec == DE_PREC_FP64, h->slices, h->variants, h->suite);
   if (h->suite) k_suite_table_launch(h->d_run, nruns, h->stream);
   TRY(init_runs(h, 0, nruns));
   if (h->prec == DE_PREC_FP64 && cfgs[0].surrogate_k < 2) {
@@ -1907,8 +1915,7 @@ de_status de_set_population(de_handle* h, int32_t run, const double* x_host, con
   k_best_init_launch(h->d_run, run, 1, h->stream);
   DE_CUDA(h, cudaGetLastError());
   s = islands_resync(h);
-  if (s != DE_OK) return s;
-  return read_states(h);
+  return s == DE_OK ? finish_change(h) : s;
 }
 
 de_status de_set_generation(de_handle* h, int32_t run, int64_t generation) {
@@ -1938,8 +1945,7 @@ de_status de_set_generation(de_handle* h, int32_t run, int64_t generation) {
   k_best_init_launch(h->d_run, run, 1, h->stream);
   DE_CUDA(h, cudaGetLastError());
   s = islands_resync(h);
-  if (s != DE_OK) return s;
-  return read_states(h);
+  return s == DE_OK ? finish_change(h) : s;
 }
 
 de_status de_get_adaptive(de_handle* h, int32_t run, double* f_host, double* cr_host) {
@@ -1984,9 +1990,8 @@ de_status de_get_best(de_handle* h, int32_t run, double* best_f, int32_t* best_i
   if (!h) return fail(nullptr, DE_ERR_INVALID_ARG, "handle is NULL");
   if (run < 0 || run >= h->nruns) return fail(h, DE_ERR_INVALID_ARG, "run out of range");
   const RunDesc& R = h->run[run];
-  de_status s = read_states(h);
-  if (s != DE_OK) return s;
-  s = exact_best(h, run, 1);
+  // (a split precision's best record is made FP64 first, which reads the states)
+  const de_status s = h->prec == DE_PREC_FP64 ? read_states(h) : exact_best(h, run, 1);
   if (s != DE_OK) return s;
   const RunState& st = h->h_state[run];
   if (best_x) {
@@ -2226,8 +2231,7 @@ de_status de_load(de_handle* h, const char* path) {
   }
   DE_CUDA(h, cudaStreamSynchronize(h->stream));
   const de_status s = islands_resync(h);
-  if (s != DE_OK) return s;
-  return read_states(h);
+  return s == DE_OK ? finish_change(h) : s;
 }
 
 de_status de_eval_noalloc(int32_t precision, int32_t objective, int32_t d, double scale, const double* shift_dev,

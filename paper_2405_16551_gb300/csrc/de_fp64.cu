@@ -637,13 +637,15 @@ cudaError_t allow_dynamic_smem(const void* k) {
              : cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
 }
 
-void k_configure() {
-  for (const void* k : {(const void*)k_gen_fp64<false, false>, (const void*)k_gen_fp64<true, false>,
-                        (const void*)k_gen_fp64<false, true>, (const void*)k_gen_fp64<true, true>,
-                        (const void*)k_eval_rows, (const void*)k_eval_pops, (const void*)k_best_exact})
+void k_configure(bool fp64, const SlicePlan& sp, bool var, bool suite) {
+  for (const void* k : {(const void*)k_eval_rows, (const void*)k_eval_pops, (const void*)k_best_exact})
     allow_dynamic_smem(k);
-  for (int q = 0; q < 18; ++q) allow_dynamic_smem(persist_kernel(q & 1, (q >> 1) % 3 == 1, (q >> 1) % 3 == 2, q / 6));
-  k_tc_configure();
+  if (!fp64) return;
+  for (const void* k : {(const void*)k_gen_fp64<false, false>, (const void*)k_gen_fp64<true, false>,
+                        (const void*)k_gen_fp64<false, true>, (const void*)k_gen_fp64<true, true>})
+    allow_dynamic_smem(k);
+  for (int isl = 0; isl < 2; ++isl) allow_dynamic_smem(persist_kernel(var, suite && !isl, isl != 0, sp.form));
+  if (sp.on) k_tc_configure();
 }
 
 cudaError_t k_gen_fp64_persist_launch(const RunDesc* runs, const int4* items, int nitems, int nruns, int threads,

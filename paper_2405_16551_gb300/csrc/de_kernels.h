@@ -37,7 +37,9 @@ struct PersistCtl {
 // failure-detection test (test_skip, and test_spin = 4096 polls)
 cudaError_t persist_ctl_reset(PersistCtl* ctl, int test_skip, cudaStream_t s);
 // FP64 path (de_fp64.cu)
-void k_configure();
+// the FP64 kernels that a handle may launch (allow_dynamic_smem); fp64: its precision
+struct SlicePlan;
+void k_configure(bool fp64, const SlicePlan& sp, bool var, bool suite);
 // Lets kernel k be launched with whatever dynamic shared memory the device
 // allows beside its static part.  The limit belongs to the function, not to a
 // handle: set to one handle's need it would refuse the launches of another,
