@@ -68,7 +68,7 @@ struct de_handle {
   RunState* h_state = nullptr;  // pinned mirror of the device states
   bool state_fresh = false;     // nothing that changes the states was enqueued since the mirror was read
   bool captured = false;        // a call was captured by the caller: its graph changes the states without a call
-  char* h_stage = nullptr;      // pinned staging of small populations (kStageBytes at most)
+  char* h_stage = nullptr;      // pinned staging of small populations (kStageFresh at most)
   size_t stage_bytes = 0;
   cudaGraphExec_t graph = nullptr;
   int graph_gens = 0;
@@ -1793,17 +1793,23 @@ de_status de_get_shape(de_handle* h, int32_t run, int32_t* np, int32_t* d, int32
   return DE_OK;
 }
 
-// Host buffers up to this size come through pinned staging: two asynchronous
-// copies, one wait and a copy by the host.  Straight into pageable memory costs a
-// wait per copy (7 us in all) but no second copy: 64 KB 18 against 22 us, 256 KB
-// 29 against 25 into a kept buffer and 34 against 35 into a new one, 768 KB 63
-// against 30 and 72 against 51.
-static constexpr size_t kStageBytes = (size_t)256 << 10;
-constexpr size_t kMapThreadBytes = (size_t)16 << 20;
+// How a population reaches the caller's pageable buffer (us; 16 cores, 64 KB pages):
+//   through pinned staging, with a copy by the host: 256 KB 29, 768 KB 63;
+//   straight, with a wait per copy: 25, 30; into pages that nobody has touched yet
+//   (a new numpy array) 200 to 1100 for 300 KB to 1 MB (staged 64 to 120), and rows
+//   whose stride differs (d not a multiple of 4) at 1.5 GB/s however many there are,
+//   unless the pages are mapped first: 16 MB 11300 -> 970, 64 MB 43000 -> 3400.
+// So: staged up to kStageBytes, in untouched pages up to kStageFresh; above, rows
+// of another stride have untouched pages mapped, by threads from kMapThreads on
+// (starting them takes 300).
+constexpr size_t kStageBytes = (size_t)256 << 10, kStageFresh = (size_t)2 << 20, kMapThreads = (size_t)16 << 20;
 
 // Whether a page of the buffer has not been touched yet, by a few samples.
-static bool untouched_pages(uintptr_t a, uintptr_t e, size_t page) {
+static bool untouched_pages(const void* p, size_t bytes) {
   constexpr size_t kSamples = 8;
+  const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+  const uintptr_t a = ((uintptr_t)p + page - 1) / page * page, e = ((uintptr_t)p + bytes) / page * page;
+  if (e <= a) return false;
   const size_t n = (e - a) / page, m = std::min(n, kSamples);
   for (size_t k = 0; k < m; ++k) {
     unsigned char v = 1;
@@ -1813,20 +1819,15 @@ static bool untouched_pages(uintptr_t a, uintptr_t e, size_t page) {
   return false;
 }
 
-// Large pageable destinations that the caller has not touched yet (a fresh numpy
-// array): map the pages first.  The copy engine's faults held a 65 MB copy to
-// 1.2 GB/s; mapped, by a few threads, it runs at 40 GB/s.  Buffers that are in use
-// already are left alone (starting the threads alone took 0.3 ms a call), and
-// smaller ones are mapped here.  Only whole pages inside the buffer are touched,
-// and their contents stay.
+// Maps the whole pages inside a buffer; their contents stay.
 static void map_pages(void* p, size_t bytes) {
 #ifndef MADV_POPULATE_WRITE
 #define MADV_POPULATE_WRITE 23
 #endif
   const size_t page = (size_t)sysconf(_SC_PAGESIZE);
   const uintptr_t a = ((uintptr_t)p + page - 1) / page * page, e = ((uintptr_t)p + bytes) / page * page;
-  if (e <= a || !untouched_pages(a, e, page)) return;
-  const int threads = bytes >= kMapThreadBytes ? 8 : 1;
+  if (e <= a) return;
+  const int threads = bytes >= kMapThreads ? 8 : 1;
   const size_t part = ((e - a) / threads + page - 1) / page * page;
   auto touch = [=](int k) {
     const uintptr_t x = a + (size_t)k * part, y = std::min(e, x + part);
@@ -1855,7 +1856,8 @@ de_status de_get_population(de_handle* h, int32_t run, double* x_host, double* f
   const size_t fb = f_host ? (size_t)R.np * sizeof(double) : 0;
   char* xd = (char*)x_host;
   char* fd = (char*)f_host;
-  bool staged = xb + fb <= kStageBytes;
+  const bool fresh = xb > kStageBytes && (xb + fb <= kStageFresh || R.d != R.dp) && untouched_pages(x_host, xb);
+  bool staged = xb + fb <= (fresh ? kStageFresh : kStageBytes);
   if (staged && h->stage_bytes < xb + fb) {
     if (h->h_stage) cudaFreeHost(h->h_stage);
     h->h_stage = nullptr;
@@ -1874,9 +1876,8 @@ de_status de_get_population(de_handle* h, int32_t run, double* x_host, double* f
   if (staged) {
     xd = h->h_stage;
     fd = h->h_stage + xb;
-  } else {
-    if (xb) map_pages(x_host, xb);
-    if (fb) map_pages(f_host, fb);
+  } else if (fresh && R.d != R.dp) {
+    map_pages(x_host, xb);
   }
   if (xb) {
     if (R.d == R.dp)

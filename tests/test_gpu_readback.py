@@ -19,8 +19,9 @@ def _gpu(monkeypatch):
     monkeypatch.setenv("DE_GB300_AUTOTUNE", "0")
 
 
-# (up to 256 KB staged; straight into the buffer; mapped by several threads from 16 MB on)
-@pytest.mark.parametrize("np_,d", [(4, 1), (320, 100), (324, 100), (1000, 99), (5000, 101), (21000, 100), (23000, 99)])
+# (up to 256 KB staged, 2 MB in untouched pages; above, rows of another stride are
+# mapped first, by several threads from 16 MB on)
+@pytest.mark.parametrize("np_,d", [(4, 1), (320, 100), (324, 100), (1000, 99), (3000, 100), (5000, 101), (21000, 100), (23000, 99)])
 def test_the_same_rows_in_every_buffer(np_, d):
     h = capi.de_init(capi.make_config(np_, d, objective=1, shift=problems.shift(d), seed=3, target_error=0.0))
     try:
