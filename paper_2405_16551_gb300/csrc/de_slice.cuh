@@ -15,17 +15,20 @@
 // products of one weight group g = s + t <= 8 stays below 2^24 in size, so
 // its FP32 accumulation in tensor memory is exact:
 //   P_g = sum_k sum_{s + t = g} u_s,k v_t,jk,   z_j = 2^(e + f_j - 76) sum_{g <= 8} 256^(8 - g) P_g
-// with one rounding at the end (in integers; the sum is below 2^83).  What is lost: bits of y_k (M_jk) below
-// 2^-63 of the row's largest, and the groups g >= 9, together about 2^-64 of
-// 2^(e + f_j), where a chain of d DFMAs loses about 2^-52 of the products it
-// sums.
+// with one rounding at the end (in integers; the sum is below 2^83).  What is
+// lost: bits of y_k (M_jk) below 2^-63 of the row's largest, and the groups g >= 9.
+// Of 2^(e + f_j) that is about 2^-64 as a rule, and at most about d 2^-67 (six
+// pairs of digits of 128 in group 9 for every k; 2^-60 at d = 128).  A chain of d
+// DFMAs rounds each of its sums to 2^-53 of it.
 //
 // A row is computed this way only when that comparison holds: with at least
 // qmin = cM + ceil(d / 8) coordinates of size >= 2^-6 max|y| (cM: the most
 // entries below 1/8 of a row of M's largest), every z_j sums at least d / 8
-// products of size >= 2^-9 of the largest possible one.  Other rows (and rows
-// with non-finite, subnormal or extreme values) take the DFMA chain
-// (rows_dfma), and matrices whose cM leaves no room (sparse ones) are not
+// products of size >= 2^-9 of the largest possible one (2^(e + f_j - 2) or more),
+// whose sizes add up to d 2^-14 or more: the chain may lose d 2^-67 in a single
+// rounding of such a sum, as much as is lost here at most.  Other rows (and rows
+// with non-finite, subnormal or extreme values) take the DFMA chain,
+// and matrices whose cM leaves no room (sparse ones) are not
 // sliced at all, so no row is computed less precisely than by the chain.
 //
 // Operands: A = M (128 rows, rows past d zero), one slice per digit t,
