@@ -773,7 +773,12 @@ void k_eval_rows_launch(const RunDesc* runs, int run, const RunDesc& Rh, const d
                         double* f, uint8_t* fx, cudaStream_t s) {
   if (n <= 0) return;
   if (k_eval_few_launch(Rh, x, ld, n, f, fx, s)) return;
-  if (Rh.sl) {
+  // One or two rows of a suite function are a chain of latencies: the DFMA chain
+  // needs no matrix in a CTA before it starts (us, digit products / chain, one row
+  // at D = 100: Zakharov 16.7 / 11.4, F09 58 / 31; four rows of F09 62 /
+  // 93).  Such a row may differ in the last bits from the same row among
+  // more.
+  if (Rh.sl && !(Rh.obj >= DE_OBJ_ZAKHAROV && n <= 2)) {
     k_eval_rows_tc_launch(runs, run, Rh, x, ld, n, f, fx, s);
     return;
   }

@@ -65,3 +65,25 @@ def test_a_cta_that_never_arrives_ends_the_launch(env, monkeypatch):
         assert "timed out" in str(e.value)
     finally:
         capi.de_destroy(h)
+
+
+@pytest.mark.parametrize("obj", [5, 6, 15, 18, 20])
+@pytest.mark.parametrize("d", [30, 64, 100])
+def test_a_few_rows(obj, d):
+    """One and two rows go another way than more."""
+    import torch
+
+    s = problems.suite(obj, d, seed=obj)
+    x = problems.population(5, d, seed=8)
+    xd = torch.from_numpy(x).cuda()
+    fo, S = oracle.evaluate(obj, x, s["shift"], s["rot"], scale=s["scale"], perm=s["perm"])
+    h = capi.de_init(capi.make_config(8, d, objective=obj, shift=s["shift"], rot=s["rot"], perm=s["perm"],
+                                      scale=s["scale"], seed=1))
+    try:
+        for n in (1, 2, 3, 5):
+            f = torch.full((6,), -7.0, dtype=torch.float64, device="cuda")
+            capi.de_eval(h, 0, xd.data_ptr(), d, n, f.data_ptr())
+            f = f.cpu().numpy()
+            assert np.all(np.abs(f[:n] - fo[:n]) <= 1e-12 * (np.abs(fo[:n]) + S[:n])) and np.all(f[n:] == -7.0)
+    finally:
+        capi.de_destroy(h)
