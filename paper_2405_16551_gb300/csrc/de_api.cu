@@ -44,7 +44,7 @@ struct de_handle {
   // (index: SliceForm; 0: the runs that are not sliced)
   struct FormItems {
     SlicePlan plan;
-    int4* d_items = nullptr;
+    int4* d_items = nullptr;   // (the handle's own list where every run has this form)
     int2* d_shares = nullptr;  // sliced: the items of each CTA
     int nitems = 0, nshares = 0;
     size_t smem = 0;           // not sliced: shared memory of the launch
@@ -294,6 +294,10 @@ static void free_form_items(de_handle* h) {
   }
 }
 
+static const int4* form_items(const de_handle* h, int form) {
+  return h->form[form].d_items ? h->form[form].d_items : h->d_items;
+}
+
 // The items of each form of the rotation, and the CTAs' shares of them.
 static de_status build_form_items(de_handle* h, const std::vector<int4>& all) {
   free_form_items(h);
@@ -320,8 +324,10 @@ static de_status build_form_items(de_handle* h, const std::vector<int4>& all) {
     const auto& v = items[form];
     F.nitems = (int)v.size();
     if (!F.nitems) continue;
-    DE_CUDA(h, cudaMalloc(&F.d_items, v.size() * sizeof(int4)));
-    DE_CUDA(h, cudaMemcpyAsync(F.d_items, v.data(), v.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
+    if (v.size() < all.size()) {
+      DE_CUDA(h, cudaMalloc(&F.d_items, v.size() * sizeof(int4)));
+      DE_CUDA(h, cudaMemcpyAsync(F.d_items, v.data(), v.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
+    }
     if (form == 0) continue;
     SlicePlan& p = F.plan;
     p.on = true;
@@ -426,11 +432,11 @@ static de_status launch_generation(de_handle* h, cudaStream_t s) {
   if (h->prec == DE_PREC_FP64) {
     if (h->slices.on) {
       const auto& F0 = h->form[0];
-      if (F0.nitems) k_gen_fp64_launch(h->d_run, F0.d_items, F0.nitems, h->threads, F0.smem, F0.variants, F0.suite, s);
+      if (F0.nitems) k_gen_fp64_launch(h->d_run, form_items(h, 0), F0.nitems, h->threads, F0.smem, F0.variants, F0.suite, s);
       for (int form = 1; form < 3; ++form) {
         const auto& F = h->form[form];
         if (F.nitems)
-          k_gen_fp64_tc_launch(h->d_run, F.d_items, F.d_shares, F.nshares, F.plan, F.variants, F.suite, s);
+          k_gen_fp64_tc_launch(h->d_run, form_items(h, form), F.d_shares, F.nshares, F.plan, F.variants, F.suite, s);
       }
     } else
       k_gen_fp64_launch(h->d_run, h->d_items, h->nitems, h->threads, h->smem_gen, h->variants, h->suite, s);
@@ -652,7 +658,7 @@ static de_status init_runs(de_handle* h, int run0, int n) {
   } else {
     for (int form = 1; form < 3 && all; ++form) {
       const auto& F = h->form[form];
-      if (F.nitems) k_eval_pops_tc_launch(h->d_run, F.d_items, F.d_shares, F.nshares, F.plan, h->stream);
+      if (F.nitems) k_eval_pops_tc_launch(h->d_run, form_items(h, form), F.d_shares, F.nshares, F.plan, h->stream);
     }
     if (all && plain) k_eval_pops_launch(h->d_run, run0, n, np_max, eval_smem(h, run0, n), h->stream);
     for (int r = run0; r < run0 + n; ++r) {
