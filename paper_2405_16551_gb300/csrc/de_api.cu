@@ -1807,8 +1807,10 @@ de_status de_get_shape(de_handle* h, int32_t run, int32_t* np, int32_t* d, int32
 //   unless the pages are mapped first: 16 MB 11300 -> 970, 64 MB 43000 -> 3400.
 // So: staged up to kStageBytes, in untouched pages up to kStageFresh; above, rows
 // of another stride have untouched pages mapped, by threads from kMapThreads on
-// (starting them takes 300).
-constexpr size_t kStageBytes = (size_t)256 << 10, kStageFresh = (size_t)2 << 20, kMapThreads = (size_t)16 << 20;
+// (starting them takes 300), and so have large contiguous copies (a new numpy array
+// asks for huge pages: 65 MB 3290 -> 2940, but 35 MB 1420 -> 2150).
+constexpr size_t kStageBytes = (size_t)256 << 10, kStageFresh = (size_t)2 << 20, kMapThreads = (size_t)16 << 20,
+                 kMapContiguous = (size_t)40 << 20;
 
 // Whether a page of the buffer has not been touched yet, by a few samples.
 static bool untouched_pages(const void* p, size_t bytes) {
@@ -1862,7 +1864,8 @@ de_status de_get_population(de_handle* h, int32_t run, double* x_host, double* f
   const size_t fb = f_host ? (size_t)R.np * sizeof(double) : 0;
   char* xd = (char*)x_host;
   char* fd = (char*)f_host;
-  const bool fresh = xb > kStageBytes && (xb + fb <= kStageFresh || R.d != R.dp) && untouched_pages(x_host, xb);
+  const bool map = R.d != R.dp || xb >= kMapContiguous;
+  const bool fresh = xb > kStageBytes && (xb + fb <= kStageFresh || map) && untouched_pages(x_host, xb);
   bool staged = xb + fb <= (fresh ? kStageFresh : kStageBytes);
   if (staged && h->stage_bytes < xb + fb) {
     if (h->h_stage) cudaFreeHost(h->h_stage);
@@ -1882,7 +1885,7 @@ de_status de_get_population(de_handle* h, int32_t run, double* x_host, double* f
   if (staged) {
     xd = h->h_stage;
     fd = h->h_stage + xb;
-  } else if (fresh && R.d != R.dp) {
+  } else if (fresh && map) {
     map_pages(x_host, xb);
   }
   if (xb) {

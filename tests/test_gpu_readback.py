@@ -21,7 +21,8 @@ def _gpu(monkeypatch):
 
 # (up to 256 KB staged, 2 MB in untouched pages; above, rows of another stride are
 # mapped first, by several threads from 16 MB on)
-@pytest.mark.parametrize("np_,d", [(4, 1), (320, 100), (324, 100), (1000, 99), (3000, 100), (5000, 101), (21000, 100), (23000, 99)])
+@pytest.mark.parametrize("np_,d", [(4, 1), (320, 100), (324, 100), (1000, 99), (3000, 100), (5000, 101), (21000, 100),
+                                  (23000, 99), (55000, 100)])
 def test_the_same_rows_in_every_buffer(np_, d):
     h = capi.de_init(capi.make_config(np_, d, objective=1, shift=problems.shift(d), seed=3, target_error=0.0))
     try:
