@@ -24,7 +24,9 @@
  *   - A handle owns all device memory it allocates.  It issues all of its
  *     work on the CUDA stream given to de_init / de_init_batch (NULL = the
  *     legacy default stream).  Calls that return host data synchronise that
- *     stream; de_step and de_eval only enqueue work.
+ *     stream; de_step and de_eval only enqueue work (so a caller may capture
+ *     them on its own stream; what a captured de_step changes is read anew by
+ *     the calls after a launch of the graph).
  *   - A handle may be used by one host thread at a time.
  *   - Host arrays are dense row-major; "host" and "device" below say which
  *     address space a pointer must be in.
@@ -305,7 +307,9 @@ DE_API de_status de_init_batch(const de_config* cfgs, int32_t nruns, void* cuda_
  * its fitness (and its jDE parameters).  The model stops as a whole: when any
  * island's best is below target_error every island stops with reason
  * DE_STOP_TARGET; the evaluation and generation limits apply per island
- * (the islands advance together).  Results come per island from de_run
+ * (the islands advance together).  Islands that a call has set apart (de_reset
+ * of one, de_set_generation) go on by themselves, without migration, until all
+ * are at one generation again.  Results come per island from de_run
  * (nruns = nislands) and de_get_best.
  * Errors: DE_ERR_INVALID_ARG (nislands outside [2, 4096], interval < 1,
  * migrants outside [1, min(32, np / 2)], run_id + nislands > 2^20, or cfg
@@ -371,8 +375,10 @@ DE_API de_status de_run(de_handle* h, de_result* out);
  * (y = (x - o) scale, z = M y, then the basic, hybrid or composition
  * function).  x_dev: device, n rows of d doubles with row stride ld (>= d)
  * doubles.  f_dev: device, n doubles.  Both caller-owned; enqueued on the
- * stream.  In a split precision, a row whose bounded device-side wait gave up
- * (it should not on a healthy device) comes back as NaN. */
+ * stream.  One or two rows of a suite function (objectives 5..20) may differ in
+ * the last bits from the same rows among more.  In a split precision, a row whose
+ * bounded device-side wait gave up (it should not on a healthy device) comes back
+ * as NaN. */
 DE_API de_status de_eval(de_handle* h, int32_t run, const double* x_dev, int64_t ld, int32_t n, double* f_dev);
 
 /* ---- evaluation without a handle and without allocation ----------------
